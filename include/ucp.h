@@ -164,8 +164,7 @@ int ucp_grad_ke_electrons(ucp_ctx* ctx, double dt_e, int ion_substep_ratio, int6
 int ucp_set_graphs(ucp_ctx* ctx, int enable);
 
 /* Autotuner of the FP32C walk: times, in each launch shape the library has
- * (threads per block x resident blocks per SM, sources through L1 or staged in
- * shared memory), the walks of one block of 10 electron substeps on the current
+ * (resident one-warp blocks per SM, which sets the register budget), the walks of one block of 10 electron substeps on the current
  * state (one walk over every particle and nine over the electrons; best of three
  * after a warm-up) and keeps the fastest shape for this context (returned in
  * *best_shape, that block's walk time in ms in *best_ms; either may be NULL).
@@ -173,8 +172,7 @@ int ucp_set_graphs(ucp_ctx* ctx, int enable);
 int ucp_autotune(ucp_ctx* ctx, double theta, double eps, int* best_shape, float* best_ms);
 
 /* Number of FP32C walk launch shapes, and a call that sets one directly
- * (0 = the default of 128 threads x 7 blocks per SM, leaf sources read
- * through L1; UCP_EINVAL outside
+ * (0 = the default of 24 one-warp blocks per SM; UCP_EINVAL outside
  * [0, UCP_WALK_SHAPES)).  The trial walks of ucp_autotune overwrite the forces and
  * interaction counts read by ucp_get_counts, and the next ucp_step recomputes its
  * first forces. */

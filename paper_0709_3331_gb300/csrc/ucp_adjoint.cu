@@ -325,7 +325,8 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     AdjList& lst = Ls[w];
     const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const float4* __restrict__ F = a.t.f32;
+    const float4* __restrict__ H = a.t.hdr;
+    const float4* __restrict__ LO = a.t.lo;
     const float4* __restrict__ S = a.src32;
     const float eps2 = (float)a.eps2;
 
@@ -337,7 +338,7 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
         const bool valid = lane < ck.y;
         const int t = valid ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
         const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
-        const int end = __float_as_int(F[(size_t)root * kF32 + 1].w);
+        const int end = __float_as_int(LO[root].w);
         float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
         float l[3] = {0.f, 0.f, 0.f};
         float qm = 0.f;
@@ -364,11 +365,10 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
             for (int e = 0; e < npl; ++e) {
                 const int nd = lst.leaf[e];
                 const bool in = (lst.mask[e] >> lane) & 1u;
-                const float4* r = F + (size_t)nd * kF32;
-                const float4 A = r[0], B = r[1], C = r[2];
+                const float4 A = H[nd], B = LO[nd];
                 const float rx = (xh + A.x) + (xl + B.x), ry = (yh + A.y) + (yl + B.y),
                             rz = (zh + A.z) + (zl + B.z);
-                const int jb = __ldg(&a.t.info[nd].x), je = __float_as_int(C.y);
+                const int jb = __ldg(&a.t.info[nd].x), je = __ldg(&a.t.info[nd].y);
                 for (int j = jb; j < je; ++j) {
                     const float4 P = __ldg(S + (j & ~1)), Q = __ldg(S + (j & ~1) + 1);
                     const bool odd = j & 1;
@@ -405,16 +405,16 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
 
         int node = root;
         while (node < end) {
-            const float4* r = F + (size_t)node * kF32;
-            const float4 A = r[0], B = r[1], C = r[2];
+            const float4 A = H[node], B = LO[node];
             const int nxt = __float_as_int(B.w);
-            const bool leaf = __float_as_int(C.y) >= 0;
+            const bool leaf = __float_as_int(A.w) < 0;
+            const float rc2 = fabsf(A.w);
             const bool active = node >= skip;
             const float R[3] = {(xh + A.x) + (xl + B.x), (yh + A.y) + (yl + B.y),
                                 (zh + A.z) + (zl + B.z)};
             const float d2 = dot3f(R, R);
-            bool acc = active && (A.w < d2);
-            if (active && fabsf(d2 - A.w) <= 4e-6f * d2) {
+            bool acc = active && (rc2 < d2);
+            if (active && fabsf(d2 - rc2) <= 4e-6f * d2) {
                 const double* m = a.t.mom + (size_t)node * kMom;
                 double dx = __dsub_rn(a.x[t], m[0]), dy = __dsub_rn(a.y[t], m[1]),
                        dz = __dsub_rn(a.z[t], m[2]);
@@ -442,10 +442,12 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
 #pragma unroll
                 for (int k = 0; k < 12; ++k) src[k] = 0.f;
                 if (acc) {
-                    const float4 D4 = r[3], E4 = r[4];
-                    const float M = C.z;
-                    const float D[3] = {C.w, D4.x, D4.y};
-                    const float Q[6] = {D4.z, D4.w, E4.x, E4.y, E4.z, E4.w};
+                    const float4* r = a.t.rec + (size_t)node * kRec;
+                    const float4 C4 = r[1], D4 = r[2], E4 = r[3];
+                    const float M = r[0].w;
+                    const float D[3] = {C4.x, C4.y, C4.z};
+                    const float Q[6] = {2.f * D4.x, 2.f * D4.y, 2.f * D4.z,
+                                        2.f * D4.w, 2.f * E4.x, 2.f * E4.y};
                     const float g = rsqrt_ftz(d2 + eps2);
                     const float g2 = g * g, g3 = g2 * g, g5 = g3 * g2, g7 = g5 * g2, g9 = g7 * g2;
                     const float Rl = dot3f(R, l), RD = dot3f(R, D), lD = dot3f(l, D);

@@ -47,13 +47,14 @@ inline void count_launch(int k) { g_launches.fetch_add((unsigned long long)k, st
 constexpr int kMom = 16;
 enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MDELTA = 15 };
 
-// One FP32C box record, 5 float4 (80 B):
-//   A = {-ch.x, -ch.y, -ch.z, rcrit2}   ch = fp32(c), cl = fp32(c - ch)
-//   B = {-cl.x, -cl.y, -cl.z, bits(next)}
-//   C = {-tr(Q)/2, bits(end or -1 for a twig), M, D.x}
-//   D = {D.y, D.z, Qxx, Qxy}
-//   E = {Qxz, Qyy, Qyz, Qzz}
-constexpr int kF32 = 5;
+// FP32 box records, written per walk (they hold rcrit2, which depends on theta):
+//   hdr = {-ch.x, -ch.y, -ch.z, +-rcrit2}   ch = fp32(c) relative to the cube's centre;
+//                                           the sign bit of rcrit2 marks a leaf
+// and, in FP32C contexts, read only for boxes that act or are opened,
+//   lo  = {-cl.x, -cl.y, -cl.z, bits(next)} cl = fp32(c - ch)
+//   rec = {-ch.x, -ch.y, -ch.z, M}, {D.x, D.y, D.z, -tr(Q)/2}, {Qxx, Qxy, Qxz, Qyy} / 2,
+//         {Qyz / 2, Qzz / 2, -M, 0}         64 B: four lanes load one box
+constexpr int kRec = 4;
 
 // Box topology {begin, end, next, parent}; depth and leaf flag separately.
 struct Tree {
@@ -64,7 +65,9 @@ struct Tree {
     int* depth_leaf;         // depth | leaf << 8
     unsigned long long* cell;// key prefix of the box at its depth
     double* mom;             // kMom doubles per box
-    float4* f32;             // kF32 float4 per box
+    float4* hdr;             // traversal record per box
+    float4* lo;              // FP32C contexts: low part of the centroid, next
+    float4* rec;             // FP32C contexts: kRec float4 per box
     float* mom32;            // FP32C contexts: 16 floats per box {e xyz, S0, M, D, Q, 0, 0}
     int* child8;             // 8 child slots per box (octant order), -1 = empty
     int* arrive;             // finished children per box (moments' bottom-up sweep)

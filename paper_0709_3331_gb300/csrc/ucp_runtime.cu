@@ -486,7 +486,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     if ((rc = dalloc(c, &c->t.nnodes, 1)) || (rc = dalloc(c, &c->t.maxdepth, 1)) ||
         (rc = dalloc(c, &c->t.info, cz)) || (rc = dalloc(c, &c->t.depth_leaf, cz)) ||
         (rc = dalloc(c, &c->t.cell, cz)) || (rc = dalloc(c, &c->t.mom, cz * kMom)) ||
-        (rc = dalloc(c, &c->t.child8, cz * 8)) || (rc = dalloc(c, &c->t.leaf_list, cz)) ||
+        (rc = dalloc(c, &c->t.hdr, cz)) || (rc = dalloc(c, &c->t.child8, cz * 8)) || (rc = dalloc(c, &c->t.leaf_list, cz)) ||
         (rc = dalloc(c, &c->t.arrive, cz)) ||
         (rc = dalloc(c, &c->t.count, kMaxDepth + 2)))
         return bail(rc);
@@ -506,7 +506,8 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     }
     if (c->precision == UCP_FP32C) {
         // sources in pairs: 2 float4 per pair of particles (padded to an even count)
-        if ((rc = dalloc(c, &c->t.f32, cz * kF32)) || (rc = dalloc(c, &c->src32, n + 1)) ||
+        if ((rc = dalloc(c, &c->t.lo, cz)) || (rc = dalloc(c, &c->t.rec, cz * kRec)) ||
+            (rc = dalloc(c, &c->src32, n + 1)) ||
             (rc = dalloc(c, &c->t.mom32, cz * 16)))
             return bail(rc);
         // the pad slot of an odd count is read (masked) by the pair loop: keep it finite

@@ -4,15 +4,15 @@
 // its expansion about its centroid (monopole, dipole, second moment of the
 // softened kernel); an opened leaf is summed pair by pair.
 //
-// GPU form: one warp walks 32 key-consecutive targets (one per lane).  The
-// per-target criterion is evaluated per lane; the warp descends into a box
-// when any lane opens it, and a lane that accepted an ancestor sits out until
-// the walk passes that ancestor's subtree (pre-order array with skip index
-// "next", no stack).  Lanes that accept a box evaluate its expansion on the
-// spot, reusing R = x_t - c and |R|^2 from the criterion; opened leaves go
-// into a per-warp list in shared memory as (leaf, lane mask) and are summed in
-// bulk, so the pair loop is warp-uniform.  Each lane sums its own target in a
-// fixed order, so results do not depend on scheduling.
+// FP64 form (k_walk_fp64): one warp walks 32 key-consecutive targets (one per
+// lane).  The per-target criterion is evaluated per lane; the warp descends into a
+// box when any lane opens it, and a lane that accepted an ancestor sits out until
+// the walk passes that ancestor's subtree (pre-order array with skip index "next",
+// no stack).  Lanes that accept a box evaluate its expansion on the spot; opened
+// leaves go into a per-warp list in shared memory as (leaf, lane mask) and are
+// summed in bulk.  The FP32C form (k_walk_fp32c) is described at its kernel.  In
+// both, each target's sums are taken in a fixed order, so results do not depend on
+// scheduling.
 #include "ucp_internal.cuh"
 
 #include <math.h>
@@ -22,9 +22,7 @@ namespace ucp {
 namespace {
 
 constexpr int kWalkThreads = 128;
-constexpr int kList = 64;      // opened leaves buffered per warp
-constexpr int kM2PBatch = 32;  // visits whose multipoles are summed in FP32 before a
-                               // compensated add (a power of two)
+constexpr int kList = 64;      // opened leaves buffered per warp (FP64 walk)
 
 struct WarpList {
     int leaf[kList];
@@ -47,44 +45,6 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float v)
     c += (s - ap) + (v - bp);
     s = t;
 }
-
-// ---- bulk copies (TMA) of a leaf's sources into shared memory, completion
-// tracked by an mbarrier (one arrival carrying the byte count)
-__device__ __forceinline__ unsigned int smem_addr(const void* p)
-{
-    return (unsigned int)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_init_fence()
-{
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-// generic-proxy reads of a buffer are ordered before the next bulk copy into it
-__device__ __forceinline__ void async_proxy_fence()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned int bytes,
-                                          unsigned long long* bar)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                 ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned int parity)
-{
-    unsigned int ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                 " selp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(smem_addr(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-constexpr int kStagePairs = 16;          // sources staged per leaf: up to 32 (16 pairs)
-constexpr int kStageSpin = 1 << 20;      // polls of a copy's barrier before giving up
 
 // ------------------------------------------------------------------ FP64
 // Expansion of a box at R = x_t - c, r2 = R.R + eps^2, g = r2^-1/2, u = g^2:
@@ -118,31 +78,6 @@ __device__ __forceinline__ void m2p<double>(double rx, double ry, double rz, dou
     ex += aa * rx - g3 * (Dx + s3 * QRx);
     ey += aa * ry - g3 * (Dy + s3 * QRy);
     ez += aa * rz - g3 * (Dz + s3 * QRz);
-}
-
-// FP32 form; T = -tr(Q)/2 comes with the box record.  kPhi = false: field only.
-template <bool kPhi>
-__device__ __forceinline__ void m2p_f32(float rx, float ry, float rz, float r2, float T, float M,
-                                        float Dx, float Dy, float Dz, float Qxx, float Qxy,
-                                        float Qxz, float Qyy, float Qyz, float Qzz, float& ex,
-                                        float& ey, float& ez, float& ph)
-{
-    float g = rsqrt_ftz(r2);
-    float u = g * g;
-    float g3 = g * u;
-    float QRx = fmaf(Qxx, rx, fmaf(Qxy, ry, Qxz * rz));
-    float QRy = fmaf(Qxy, rx, fmaf(Qyy, ry, Qyz * rz));
-    float QRz = fmaf(Qxz, rx, fmaf(Qyz, ry, Qzz * rz));
-    float RQR = fmaf(rx, QRx, fmaf(ry, QRy, rz * QRz));
-    float w = fmaf(Dx, rx, fmaf(Dy, ry, fmaf(Dz, rz, T)));
-    float h = u * RQR;
-    if (kPhi) ph = fmaf(g, fmaf(u, fmaf(1.5f, h, w), M), ph);
-    float s3 = 3.f * u;
-    float aa = g3 * fmaf(s3, fmaf(2.5f, h, w), M);
-    float mg3 = -g3;
-    ex = fmaf(mg3, fmaf(s3, QRx, Dx), fmaf(aa, rx, ex));
-    ey = fmaf(mg3, fmaf(s3, QRy, Dy), fmaf(aa, ry, ey));
-    ez = fmaf(mg3, fmaf(s3, QRz, Dz), fmaf(aa, rz, ez));
 }
 
 template <bool kKelbg, int kThreads>
@@ -306,50 +241,97 @@ __device__ __forceinline__ void kelbg_pg(float u, float& p, float& g)
     }
 }
 
-// kThreads threads per block, register budget for kBlocks resident blocks per SM.
-// kStage: a leaf's sources (up to 32) are brought into shared memory by a bulk
-// copy issued one list entry ahead (double buffer per warp) instead of being read
-// through L1 by every lane; the arithmetic and its order are the same.
-// kPhi = false (walks whose potential nobody reads, e.g. the electron substeps):
-// the potential terms and their sums are left out; the field is computed by the
-// same operations in the same order, so accelerations are bit-identical.
-template <bool kKelbg, int kThreads, int kBlocks, bool kStage, bool kPhi>
+// One warp walks a chunk of up to 32 key-consecutive targets of one cloud, one per
+// lane, in three parts that alternate:
+//
+// Traversal, lanes over boxes.  A stack holds opened twigs with the mask of the
+// targets that opened them; a step pops up to four and tests their children, one
+// per lane, against the bounding box of the chunk's targets: a child is accepted
+// or opened by every target of its mask when the nearest or the farthest point of
+// that bounding box decides it beyond the criterion's rounding window (four of five
+// children at N = 524,288, theta 0.5), and only the children in between are decided
+// target by target, two per packed operation.  The interaction sets are those of
+// the per-target criterion.
+//
+// Multipoles, lanes over targets.  Accepted boxes wait in a list; 32 at a time their
+// records are brought into shared memory (four lanes per 64-byte record) with the
+// fields of two boxes side by side, and each lane evaluates two boxes per packed
+// FP32x2 instruction (35 of them per pair of boxes).  A lane outside a box's mask
+// takes a zero inverse distance.
+//
+// Direct pairs, lanes over targets: the opened leaves in lists of up to 63, each
+// leaf's sources brought into shared memory while the leaf before it is summed.
+//
+// What bounds it (N = 524,288, theta 0.5, leaves of 32, no potential): per chunk
+// 1,950 children tested in about 70 steps, 1,775 boxes evaluated (68 % of the lanes
+// take part, the others accepted an ancestor) and 162 leaves of 11 sources summed
+// (44 %); of the 2.5 ms of a walk over every particle the multipoles take 1.45 (the
+// FP32 pipe: an FFMA2 holds it for two cycles), the pairs 0.8 and the traversal
+// 0.4.  The form before, a depth-first walk that tested one box per visit in all
+// lanes and evaluated it one box at a time, took 3.75 ms (1.27e5 against 1.81e5 warp
+// instructions per chunk); with the potential 2.7 against 4.1 ms, over the electrons
+// 1.5 against 2.25 ms.  Blocks of one warp keep the shared arrays at constant
+// addresses: 8 % faster than blocks of two to eight warps at the same occupancy.
+//
+// kThreads threads per block (one warp), register budget for kBlocks resident blocks
+// per SM.  kPhi = false (walks whose potential nobody reads, e.g. the electron
+// substeps): the potential terms and their sums are left out; the field is computed
+// by the same operations in the same order, so accelerations are bit-identical.
+constexpr int kStage = 32;           // boxes evaluated per batch (pairs of two)
+constexpr int kStageStride = 36;     // floats per staged pair (32 used; 16-byte aligned)
+// Twigs on the stack: up to kPopWide + 28 while four are popped per step; above
+// kPopWide one is popped per step, which adds at most 7 per level below it.
+constexpr int kPopWide = 64;
+constexpr int kStack = kPopWide + 28 + 7 * (kMaxDepth - 1) + 8;
+
+struct __align__(16) WalkWarp {
+    float stage[kStage / 2 * kStageStride];
+    int2 stack[kStack];              // {twig, mask}
+    int2 acc[2 * kStage];            // {accepted box, mask}
+    int2 leaf[64];                   // {opened leaf, mask}
+};
+
+__device__ __forceinline__ float warp_min(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// Eq. 5 for a target and a box's record m in FP64, rounded like the definition
+__device__ __noinline__ bool accepts_fp64(const double* m, const double* x, const double* y,
+                                          const double* z)
+{
+    const double dx = __dsub_rn(*x, m[0]);
+    const double dy = __dsub_rn(*y, m[1]);
+    const double dz = __dsub_rn(*z, m[2]);
+    return m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+
+__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
+
+template <bool kKelbg, int kThreads, int kBlocks, bool kPhi>
 __global__ void __launch_bounds__(kThreads, kBlocks)
 k_walk_fp32c(WalkArgs a)
 {
-    __shared__ WarpList L[kThreads / 32];
-    __shared__ __align__(16) float4 stage[kStage ? kThreads / 32 : 1][2][2 * kStagePairs];
-    __shared__ __align__(8) unsigned long long stage_bar[kStage ? kThreads / 32 : 1][2];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    WarpList& lst = L[w];
-    unsigned int stage_phase = 0;  // parity to wait for, per buffer (bits 0, 1)
-    bool stage_ok = kStage;        // cleared for good if a copy is not seen to complete
-    if (kStage) {
-        if (lane == 0) {
-            mbar_init(&stage_bar[w][0]);
-            mbar_init(&stage_bar[w][1]);
-            mbar_init_fence();
-        }
-        __syncwarp();
-    }
+    __shared__ WalkWarp shared[kThreads / 32];
+    const int lane = threadIdx.x & 31;
+    WalkWarp& W = shared[threadIdx.x >> 5];
+    const unsigned int lt = (1u << lane) - 1u, me = 1u << lane;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const float4* __restrict__ F = a.t.f32;
+    const float4* __restrict__ H = a.t.hdr;
     const float4* __restrict__ S = a.src32;
     const float eps2 = (float)a.eps2;
 
     for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
          chunk = next_chunk(a.work, lane)) {
-        // up to 32 key-consecutive targets of one cloud, walked through that cloud's tree
         const int4 ck = a.chunks[chunk];
         const int ti = ck.x + lane;
         const bool valid = lane < ck.y;
         const int t = valid ? (a.targets ? a.targets[ti] : ti) : -1;
-        const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
-        const int end = __float_as_int(F[(size_t)root * kF32 + 1].w);
-        // target as an unevaluated float pair: x = xh + xl ({x, y} packed for the
-        // FP32x2 adds), relative to the centre of the cloud's cube like the box
-        // centroids, so that the FP32 errors scale with the cloud's size and not
-        // with its distance from the origin
+        // target as an unevaluated float pair: x = xh + xl, relative to the centre of
+        // the cloud's cube like the box centroids, so that the FP32 errors scale with
+        // the cloud's size and not with its distance from the origin
         float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
         if (valid) {
             const double* cc = a.cubes[ck.z].c;
@@ -357,279 +339,336 @@ k_walk_fp32c(WalkArgs a)
             xh = (float)X; yh = (float)Y; zh = (float)Z;
             xl = (float)(X - (double)xh); yl = (float)(Y - (double)yh); zl = (float)(Z - (double)zh);
         }
-        const float2 xyh = make_float2(xh, yh);
-        // Window of the FP32 criterion (see the traversal): |dm| <= wa d2 + wb
-        // bounds the FP32 error of d2 - rcrit2 for this target, given
-        // |x_t - xh| <= 2^-24 |x_t| and the same for the centroid
+        // Window of the FP32 criterion (see below): |dm| <= wa d2 + wb bounds the FP32
+        // error of d2 - rcrit2 for this target, given |x_t - xh| <= 2^-24 |x_t| and the
+        // same for the centroid
         const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
         const float wa = fmaf(0.5f, bt, 4e-6f), wb = 0.5f * bt;
+        // bounding box of the chunk's targets (centre, half extents), and four times the
+        // widest window of its targets: the centre and extents are rounded too
+        const float xa = warp_min(valid ? xh : INFINITY), xb = -warp_min(valid ? -xh : INFINITY);
+        const float ya = warp_min(valid ? yh : INFINITY), yb = -warp_min(valid ? -yh : INFINITY);
+        const float za = warp_min(valid ? zh : INFINITY), zb = -warp_min(valid ? -zh : INFINITY);
+        const float gx = 0.5f * (xa + xb), gy = 0.5f * (ya + yb), gz = 0.5f * (za + zb);
+        const float ex = fmaxf(xb - gx, gx - xa), ey = fmaxf(yb - gy, gy - ya),
+                    ez = fmaxf(zb - gz, gz - za);
+        const float gwb = 4.f * -warp_min(-wb), gwa = gwb + 1.6e-5f;
         const float qt = valid ? (a.sp[t] ? (float)q1 : (float)q0) : 0.f;
-        const float inv_lambda = (float)(1.0 / a.lambda);
+        const float inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
         const float inv_lambda3 = inv_lambda * inv_lambda * inv_lambda;
-        // compensated totals (sum, correction) and the current multipole batch
+        // compensated totals (sum, correction)
         float sx = 0.f, sy = 0.f, sz = 0.f, sp = 0.f, cx = 0.f, cy = 0.f, cz = 0.f, cp = 0.f;
-        float bx = 0.f, by = 0.f, bz = 0.f, bp = 0.f;
-        int np = 0, nm = 0, vis = 0;
-        int skip = valid ? 0 : 0x7fffffff;
-        int npl = 0;
+        int np = 0, nm = 0;
+        int top = 0, na = 0, nl = 0;
 
-        auto fold_batch = [&]() {
-            two_sum_acc(sx, cx, bx);
-            two_sum_acc(sy, cy, by);
-            two_sum_acc(sz, cz, bz);
-            if (kPhi) two_sum_acc(sp, cp, bp);
-            bx = by = bz = bp = 0.f;
-        };
-
-        // one list entry's pair sum from sources at P0 (paired float4, P0[0] = the
-        // pair that holds source jb)
-        auto leaf_pairs = [&](int nd, const float4* __restrict__ P0) {
-            const float4* r = F + (size_t)nd * kF32;
-            float4 A = r[0], B = r[1], C = r[2];
-            float rx = (xh + A.x) + (xl + B.x);
-            float ry = (yh + A.y) + (yl + B.y);
-            float rz = (zh + A.z) + (zl + B.z);
-            int jb = __ldg(&a.t.info[nd].x), je = __float_as_int(C.y);
-            const float2 rx2 = make_float2(rx, rx), ry2 = make_float2(ry, ry),
-                         rz2 = make_float2(rz, rz), e2 = make_float2(eps2, eps2);
-            float2 px = make_float2(0.f, 0.f), py = px, pz = px, pp = px;
+        // the last cnt <= 32 boxes of the list of accepted boxes
+        auto multipoles = [&](int cnt) {
+            na -= cnt;
+            const int part = lane & 3;
+#pragma unroll
+            for (int it = 0; it < kStage / 8; ++it) {
+                const int e = it * 8 + (lane >> 2);
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (e < cnt) v = __ldg(a.t.rec + (size_t)W.acc[na + e].x * kRec + part);
+                if (part == 3) v.w = __int_as_float(e < cnt ? W.acc[na + e].y : 0);
+                float* d = W.stage + (e >> 1) * kStageStride + part * 8 + (e & 1);
+                d[0] = v.x;
+                d[2] = v.y;
+                d[4] = v.z;
+                d[6] = v.w;
+            }
+            __syncwarp();
+            // With g = (R.R + eps^2)^-1/2, u = g^2, q = Q R / 2, y = D + 5 u q:
+            //   E   = -g^3 [y + u q - (M + 3 u (T + y.R)) R]
+            //   phi = g (M + u (T + y.R - 2 u q.R)),   T = -tr(Q)/2
+            float2 bx = splat(0.f), by = bx, bz = bx, bp = bx;
+            const float2 x2 = splat(xh), y2 = splat(yh), z2 = splat(zh), e2 = splat(eps2);
+            const int pairs = (cnt + 1) >> 1;
 #pragma unroll 2
-            for (int j = jb & ~1; j < je; j += 2) {
-                const float4 P = P0[j - (jb & ~1)], Q = P0[j - (jb & ~1) + 1];
-                float2 dx = __fadd2_rn(rx2, make_float2(P.x, P.y));
-                float2 dy = __fadd2_rn(ry2, make_float2(P.z, P.w));
-                float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
-                float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-                const bool ok0 = j >= jb && j != t;
-                const bool ok1 = j + 1 < je && j + 1 != t;
-                float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f, ok1 ? rsqrt_ftz(r2.y) : 0.f);
-                float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
-                float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
-                px = __ffma2_rn(qr3, dx, px);
-                py = __ffma2_rn(qr3, dy, py);
-                pz = __ffma2_rn(qr3, dz, pz);
-                if (kPhi) pp = __fadd2_rn(pp, qi);
-            }
-            np += (je - jb) - ((t >= jb && t < je) ? 1 : 0);
-            two_sum_acc(sx, cx, px.x + px.y);
-            two_sum_acc(sy, cy, py.x + py.y);
-            two_sum_acc(sz, cz, pz.x + pz.y);
-            if (kPhi) two_sum_acc(sp, cp, pp.x + pp.y);
-        };
-
-        // Staged form: entry e's sources go to buffer e & 1 while entry e - 1 is
-        // summed; entries with more than 32 sources read them from global memory.
-        auto stage_entry = [&](int e) -> bool {
-            const int nd = lst.leaf[e];
-            const int jb = __ldg(&a.t.info[nd].x);
-            const int je = __float_as_int(__ldg(&F[(size_t)nd * kF32 + 2]).y);
-            const int pb = jb >> 1, pe = (je + 1) >> 1;
-            if (!stage_ok || pe - pb > kStagePairs) return false;
-            if (lane == 0) {
-                async_proxy_fence();
-                bulk_load(&stage[w][e & 1][0], S + 2 * (size_t)pb,
-                          (unsigned int)(pe - pb) * 32u, &stage_bar[w][e & 1]);
-            }
-            return true;
-        };
-        auto flush_staged = [&]() {
-            __syncwarp();
-            bool st_cur = npl > 0 ? stage_entry(0) : false;
-            for (int e = 0; e < npl; ++e) {
-                bool st_next = e + 1 < npl ? stage_entry(e + 1) : false;
-                const int nd = lst.leaf[e];
-                const float4* P0;
-                if (st_cur) {
-                    const int b = e & 1;
-                    const unsigned int par = (stage_phase >> b) & 1u;
-                    bool done = false;
-                    for (int it = 0; it < kStageSpin && !done; ++it)
-                        done = mbar_test(&stage_bar[w][b], par);
-                    stage_phase ^= 1u << b;
-                    P0 = &stage[w][b][0];
-                    if (!done) {
-                        // raise the flag, stop staging in this warp and read this
-                        // entry from global memory; the copies still in flight into
-                        // this warp's buffers (this entry's, and the next entry's if
-                        // it was issued) get one more bounded wait each, so that none
-                        // lands after the warp has moved on
-                        if (lane == 0) atomicExch(a.err, 1);
-                        bool late = false;
-                        for (int it = 0; it < kStageSpin && !late; ++it)
-                            late = mbar_test(&stage_bar[w][b], par);
-                        if (st_next) {
-                            const int b1 = b ^ 1;
-                            const unsigned int par1 = (stage_phase >> b1) & 1u;
-                            late = false;
-                            for (int it = 0; it < kStageSpin && !late; ++it)
-                                late = mbar_test(&stage_bar[w][b1], par1);
-                        }
-                        stage_ok = false;
-                        st_next = false;
-                        P0 = S + ((size_t)__ldg(&a.t.info[nd].x) & ~(size_t)1);
-                    }
-                } else {
-                    P0 = S + ((size_t)__ldg(&a.t.info[nd].x) & ~(size_t)1);
+            for (int p = 0; p < pairs; ++p) {
+                const float4* P = reinterpret_cast<const float4*>(W.stage + p * kStageStride);
+                const float4 f0 = P[0], f1 = P[1], f2 = P[2], f3 = P[3], f4 = P[4], f5 = P[5],
+                             f6 = P[6], f7 = P[7];
+                const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
+                const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
+                const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
+                const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __ffma2_rn(rz, rz, e2)));
+                const bool in0 = (__float_as_int(f7.z) & me) != 0;
+                const bool in1 = (__float_as_int(f7.w) & me) != 0;
+                const float2 g = make_float2(in0 ? rsqrt_ftz(r2.x) : 0.f,
+                                             in1 ? rsqrt_ftz(r2.y) : 0.f);
+                nm += in0;
+                nm += in1;
+                const float2 u = __fmul2_rn(g, g);
+                const float2 g3 = __fmul2_rn(g, u);
+                const float2 qxx = make_float2(f4.x, f4.y), qxy = make_float2(f4.z, f4.w),
+                             qxz = make_float2(f5.x, f5.y), qyy = make_float2(f5.z, f5.w),
+                             qyz = make_float2(f6.x, f6.y), qzz = make_float2(f6.z, f6.w);
+                const float2 qx = __ffma2_rn(qxx, rx, __ffma2_rn(qxy, ry, __fmul2_rn(qxz, rz)));
+                const float2 qy = __ffma2_rn(qxy, rx, __ffma2_rn(qyy, ry, __fmul2_rn(qyz, rz)));
+                const float2 qz = __ffma2_rn(qxz, rx, __ffma2_rn(qyz, ry, __fmul2_rn(qzz, rz)));
+                const float2 u5 = __fmul2_rn(splat(5.f), u);
+                const float2 yx = __ffma2_rn(u5, qx, make_float2(f2.x, f2.y));
+                const float2 yy = __ffma2_rn(u5, qy, make_float2(f2.z, f2.w));
+                const float2 yz = __ffma2_rn(u5, qz, make_float2(f3.x, f3.y));
+                const float2 w = __ffma2_rn(yx, rx, __ffma2_rn(yy, ry, __ffma2_rn(yz, rz,
+                                            make_float2(f3.z, f3.w))));
+                const float2 nk = __ffma2_rn(__fmul2_rn(splat(-3.f), u), w,
+                                             make_float2(f7.x, f7.y));
+                bx = __ffma2_rn(g3, __ffma2_rn(nk, rx, __ffma2_rn(u, qx, yx)), bx);
+                by = __ffma2_rn(g3, __ffma2_rn(nk, ry, __ffma2_rn(u, qy, yy)), by);
+                bz = __ffma2_rn(g3, __ffma2_rn(nk, rz, __ffma2_rn(u, qz, yz)), bz);
+                if (kPhi) {
+                    const float2 qr = __ffma2_rn(qx, rx, __ffma2_rn(qy, ry, __fmul2_rn(qz, rz)));
+                    const float2 v = __ffma2_rn(__fmul2_rn(splat(-2.f), u), qr, w);
+                    bp = __ffma2_rn(g, __ffma2_rn(u, v, make_float2(f1.z, f1.w)), bp);
                 }
-                if ((lst.mask[e] >> lane) & 1u) leaf_pairs(nd, P0);
-                __syncwarp();
-                st_cur = st_next;
             }
-            npl = 0;
+            two_sum_acc(sx, cx, -(bx.x + bx.y));
+            two_sum_acc(sy, cy, -(by.x + by.y));
+            two_sum_acc(sz, cz, -(bz.x + bz.y));
+            if (kPhi) two_sum_acc(sp, cp, bp.x + bp.y);
             __syncwarp();
         };
 
-        auto flush = [&]() {
-            if (kStage && !kKelbg) {
-                flush_staged();
-                return;
+        // the last cnt <= 32 leaves of the list of opened leaves, their sources brought
+        // into shared memory one leaf (32 float4: up to 32 sources) ahead
+        auto direct_pairs = [&](int cnt) {
+            nl -= cnt;
+            float4* meta = reinterpret_cast<float4*>(W.stage);   // {-ch, begin}, {-cl, end}
+            float4* buf = meta + 64;                             // 2 x 32 float4
+            if (lane < cnt) {
+                const int nd = W.leaf[nl + lane].x;
+                float4 A = __ldg(H + nd), B = __ldg(a.t.lo + nd);
+                const int2 be = __ldg(reinterpret_cast<const int2*>(a.t.info + nd));
+                A.w = __int_as_float(be.x);
+                B.w = __int_as_float(be.y);
+                meta[2 * lane] = A;
+                meta[2 * lane + 1] = B;
             }
             __syncwarp();
-            for (int e = 0; e < npl; ++e) {
-                int nd = lst.leaf[e];
-                if ((lst.mask[e] >> lane) & 1u) {
-                    const float4* r = F + (size_t)nd * kF32;
-                    float4 A = r[0], B = r[1], C = r[2];
-                    float rx = (xh + A.x) + (xl + B.x);
-                    float ry = (yh + A.y) + (yl + B.y);
-                    float rz = (zh + A.z) + (zl + B.z);
-                    int jb = __ldg(&a.t.info[nd].x), je = __float_as_int(C.y);
+            // float4 s + lane of a leaf's sources, which lie in pairs {x_2p, x_2p+1, y..,
+            // y..}, {z.., z.., q.., q..} as offsets c_leaf - x_j; a pair member outside
+            // [jb, je) is moved far away and takes no charge
+            auto fetch = [&](int jb, int je, int s) -> float4 {
+                const int i = s + lane;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i < ((je + 1) & ~1)) v = __ldg(S + i);
+                if (lane & 1) {
+                    if (i <= jb) v.z = 0.f;
+                    if (i >= je) v.w = 0.f;
+                } else {
+                    if (i < jb) v.x = 1e18f;
+                    if (i + 1 >= je) v.y = 1e18f;
+                }
+                return v;
+            };
+            float2 px = splat(0.f), py = px, pz = px, pp = px;
+            int e = 0, b = 0;
+            int jb = __float_as_int(meta[0].w), je = __float_as_int(meta[1].w), s = jb & ~1;
+            float4 v = fetch(jb, je, s);
+            while (true) {
+                buf[b * 32 + lane] = v;
+                int e1 = e, jb1 = jb, je1 = je, s1 = s + 32;
+                if (s1 >= je) {
+                    ++e1;
+                    if (e1 < cnt) {
+                        jb1 = __float_as_int(meta[2 * e1].w);
+                        je1 = __float_as_int(meta[2 * e1 + 1].w);
+                        s1 = jb1 & ~1;
+                    }
+                }
+                if (e1 < cnt) v = fetch(jb1, je1, s1);
+                __syncwarp();
+                if (W.leaf[nl + e].y & me) {
+                    const float4 A = meta[2 * e], B = meta[2 * e + 1];
+                    const float rx = (xh + A.x) + (xl + B.x);
+                    const float ry = (yh + A.y) + (yl + B.y);
+                    const float rz = (zh + A.z) + (zl + B.z);
+                    const float4* P = buf + b * 32;
+                    const int pairs = (min(s + 32, je + 1) - s) >> 1;
+                    const int lo = max(jb, s), hi = min(je, s + 32);   // sources of this part
+                    const bool self = t >= lo && t < hi;
+                    np += hi - lo - (self ? 1 : 0);
                     if (kKelbg) {
                         // one source at a time: unlike charges (electron-ion) take the
                         // Kelbg form, like charges the softened Coulomb law
-                        float px = 0.f, py = 0.f, pz = 0.f, pp = 0.f;
-                        for (int j = jb; j < je; ++j) {
+                        for (int j = lo; j < hi; ++j) {
                             if (j == t) continue;
-                            const float4 P = __ldg(S + (j & ~1)), Q = __ldg(S + (j & ~1) + 1);
+                            const float4 F = P[(j & ~1) - s], Q = P[(j | 1) - s];
                             const bool odd = j & 1;
-                            float dx = rx + (odd ? P.y : P.x);
-                            float dy = ry + (odd ? P.w : P.z);
+                            float dx = rx + (odd ? F.y : F.x);
+                            float dy = ry + (odd ? F.w : F.z);
                             float dz = rz + (odd ? Q.y : Q.x);
                             float qj = odd ? Q.w : Q.z;
                             if (qj != qt) {
                                 float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                                 if (r2 == 0.f) {
-                                    pp = fmaf(qj, inv_lambda, pp);
+                                    pp.x = fmaf(qj, inv_lambda, pp.x);
                                     continue;
                                 }
                                 float r = sqrtf(r2);
                                 float pf, gf;
                                 kelbg_pg(r * inv_lambda, pf, gf);
                                 float fq = qj * gf * inv_lambda3;
-                                px = fmaf(fq, dx, px);
-                                py = fmaf(fq, dy, py);
-                                pz = fmaf(fq, dz, pz);
-                                pp = fmaf(qj * inv_lambda, pf, pp);
+                                px.x = fmaf(fq, dx, px.x);
+                                py.x = fmaf(fq, dy, py.x);
+                                pz.x = fmaf(fq, dz, pz.x);
+                                pp.x = fmaf(qj * inv_lambda, pf, pp.x);
                             } else {
                                 float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
                                 float ri = rsqrt_ftz(r2);
                                 float qi = qj * ri;
                                 float qr3 = qi * ri * ri;
-                                px = fmaf(qr3, dx, px);
-                                py = fmaf(qr3, dy, py);
-                                pz = fmaf(qr3, dz, pz);
-                                pp += qi;
+                                px.x = fmaf(qr3, dx, px.x);
+                                py.x = fmaf(qr3, dy, py.x);
+                                pz.x = fmaf(qr3, dz, pz.x);
+                                pp.x += qi;
                             }
                         }
-                        np += (je - jb) - ((t >= jb && t < je) ? 1 : 0);
-                        two_sum_acc(sx, cx, px);
-                        two_sum_acc(sy, cy, py);
-                        two_sum_acc(sz, cz, pz);
-                        two_sum_acc(sp, cp, pp);
-                        continue;
-                    }
-                    // sources in pairs {x_2p, x_2p+1, y.., y..}, {z.., z.., q.., q..} as
-                    // offsets c_leaf - x_j; a pair member outside [jb, je) or equal to
-                    // the target gets a zero inverse distance
-                    const float2 rx2 = make_float2(rx, rx), ry2 = make_float2(ry, ry),
-                                 rz2 = make_float2(rz, rz), e2 = make_float2(eps2, eps2);
-                    float2 px = make_float2(0.f, 0.f), py = px, pz = px, pp = px;
+                    } else {
+                        const float2 rx2 = splat(rx), ry2 = splat(ry), rz2 = splat(rz),
+                                     e2 = splat(eps2);
+                        const int tp = self ? t - s : -1;  // the target's own place
 #pragma unroll 2
-                    for (int j = jb & ~1; j < je; j += 2) {
-                        const float4 P = __ldg(S + j), Q = __ldg(S + j + 1);
-                        float2 dx = __fadd2_rn(rx2, make_float2(P.x, P.y));
-                        float2 dy = __fadd2_rn(ry2, make_float2(P.z, P.w));
-                        float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
-                        float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-                        const bool ok0 = j >= jb && j != t;
-                        const bool ok1 = j + 1 < je && j + 1 != t;
-                        float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f, ok1 ? rsqrt_ftz(r2.y) : 0.f);
-                        float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
-                        float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
-                        px = __ffma2_rn(qr3, dx, px);
-                        py = __ffma2_rn(qr3, dy, py);
-                        pz = __ffma2_rn(qr3, dz, pz);
-                        if (kPhi) pp = __fadd2_rn(pp, qi);
+                        for (int p = 0; p < pairs; ++p) {
+                            const float4 F = P[2 * p], Q = P[2 * p + 1];
+                            const float2 dx = __fadd2_rn(rx2, make_float2(F.x, F.y));
+                            const float2 dy = __fadd2_rn(ry2, make_float2(F.z, F.w));
+                            const float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
+                            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy,
+                                                         __ffma2_rn(dz, dz, e2)));
+                            const float2 ri = make_float2(
+                                2 * p != tp ? rsqrt_ftz(r2.x) : 0.f,
+                                2 * p + 1 != tp ? rsqrt_ftz(r2.y) : 0.f);
+                            const float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
+                            const float2 qr3 = __fmul2_rn(qi, __fmul2_rn(ri, ri));
+                            px = __ffma2_rn(qr3, dx, px);
+                            py = __ffma2_rn(qr3, dy, py);
+                            pz = __ffma2_rn(qr3, dz, pz);
+                            if (kPhi) pp = __fadd2_rn(pp, qi);
+                        }
                     }
-                    np += (je - jb) - ((t >= jb && t < je) ? 1 : 0);
+                }
+                // a leaf's pairs are summed in FP32 and enter the total by a compensated
+                // add (folding every fourth leaf only is 1.5 % faster and 1 % less exact)
+                if (e1 != e) {
                     two_sum_acc(sx, cx, px.x + px.y);
                     two_sum_acc(sy, cy, py.x + py.y);
                     two_sum_acc(sz, cz, pz.x + pz.y);
                     if (kPhi) two_sum_acc(sp, cp, pp.x + pp.y);
+                    px = py = pz = pp = splat(0.f);
                 }
+                if (e1 >= cnt) break;
+                e = e1;
+                jb = jb1;
+                je = je1;
+                s = s1;
+                b ^= 1;
             }
-            npl = 0;
             __syncwarp();
         };
 
-        int node = root;
-        while (node < end) {
-            const float4* r = F + (size_t)node * kF32;
-            const float4 A = r[0], B = r[1], C = r[2], D = r[3], E = r[4];
-            const int nxt = __float_as_int(B.w);
-            const bool leaf = __float_as_int(C.y) >= 0;
-            const bool active = node >= skip;
-            // R = x_t - c from the rounded target and centroid (their low parts
-            // enter only the direct pairs): one add per axis on the chain
-            // record -> criterion -> vote -> next box that sets the walk's pace
-            const float2 rxy = __fadd2_rn(xyh, make_float2(A.x, A.y));
-            const float rx = rxy.x, ry = rxy.y;
-            const float rz = zh + A.z;
-            float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            const float dm = d2 - A.w;
-            bool acc = active && dm > 0.f;
-            // Within the FP32 error of d2 - rcrit2 the decision is taken again in
-            // FP64 exactly as the FP64 walk takes it, so both precisions open the
-            // same boxes.  Per axis R is off by at most 2^-23 (|x_t| + |R|), so
-            // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
-            // included) with X_t the target's largest coordinate; with
-            // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
-            // a million at the bench size).
-            if (active && fabsf(dm) <= fmaf(wa, d2, wb)) {
-                const double* m = a.t.mom + (size_t)node * kMom;
-                double dx = __dsub_rn(a.x[t], m[0]);
-                double dy = __dsub_rn(a.y[t], m[1]);
-                double dz = __dsub_rn(a.z[t], m[2]);
-                double dd = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                                      __dmul_rn(dz, dz));
-                acc = m[MR2] < dd;
-            }
-            const bool opn = active && !acc;
-            const unsigned int om = __ballot_sync(0xffffffffu, opn);
-            int next = nxt;
-            if (om) {
-                if (leaf) {
-                    if (lane == 0) {
-                        lst.leaf[npl] = node;
-                        lst.mask[npl] = om;
-                    }
-                    ++npl;
-                } else {
-                    if (acc) skip = nxt;
-                    next = node + 1;
+        // the first step tests the root for every target
+        int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0] : -1;
+        unsigned int mask = __ballot_sync(0xffffffffu, valid);
+        while (true) {
+            const bool has = box >= 0;
+            const float4 h = has ? __ldg(H + box) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const bool leaf = __float_as_int(h.w) < 0;
+            const float rc2 = fabsf(h.w);
+            const float dx = fabsf(gx + h.x), dy = fabsf(gy + h.y), dz = fabsf(gz + h.z);
+            const float nx = fmaxf(dx - ex, 0.f), ny = fmaxf(dy - ey, 0.f), nz = fmaxf(dz - ez, 0.f);
+            const float fx = dx + ex, fy = dy + ey, fz = dz + ez;
+            const float near2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
+            const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+            const bool all_acc = near2 - rc2 > fmaf(gwa, near2, gwb);
+            const bool all_opn = rc2 - far2 > fmaf(gwa, far2, gwb);
+            unsigned int am = has && all_acc ? mask : 0u;   // targets that accept the box
+            const bool some = has && !all_acc && !all_opn;
+            const unsigned int between = __ballot_sync(0xffffffffu, some);
+            if (between) {
+                // decided target by target, two boxes per packed operation: pairs of
+                // {-c} x, y, z, {-rcrit2}, {box, mask}, side by side
+                const int slot = some ? __popc(between & lt) : -1;
+                const int cnt = __popc(between);
+                if (some) {
+                    float* d = W.stage + (slot >> 1) * 12 + (slot & 1);
+                    d[0] = h.x;
+                    d[2] = h.y;
+                    d[4] = h.z;
+                    d[6] = -rc2;
+                    d[8] = __int_as_float(box);
+                    d[10] = __int_as_float((int)mask);
                 }
+                if (lane == 0 && (cnt & 1)) {
+                    float* d = W.stage + (cnt >> 1) * 12 + 1;
+                    d[0] = d[2] = d[4] = d[6] = d[8] = d[10] = 0.f;
+                }
+                __syncwarp();
+                const float2 x2 = splat(xh), y2 = splat(yh), z2 = splat(zh);
+                for (int p = 0; 2 * p < cnt; ++p) {
+                    const float4* P = reinterpret_cast<const float4*>(W.stage + p * 12);
+                    const float4 f0 = P[0], f1 = P[1], f2 = P[2];
+                    const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
+                    const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
+                    const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
+                    const float2 d2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+                    const float2 dm = __fadd2_rn(d2, make_float2(f1.z, f1.w));
+                    const float2 win = __ffma2_rn(splat(wa), d2, splat(wb));
+                    const bool in0 = (__float_as_int(f2.z) & me) != 0;
+                    const bool in1 = (__float_as_int(f2.w) & me) != 0;
+                    bool acc0 = in0 && dm.x > 0.f, acc1 = in1 && dm.y > 0.f;
+                    // Within the FP32 error of d2 - rcrit2 the decision is taken again in
+                    // FP64 exactly as the FP64 walk takes it, so both precisions open the
+                    // same boxes.  Per axis R is off by at most 2^-23 (|x_t| + |R|), so
+                    // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
+                    // included) with X_t the target's largest coordinate; with
+                    // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
+                    // a million at the bench size).
+                    const bool again0 = in0 && fabsf(dm.x) <= win.x;
+                    const bool again1 = in1 && fabsf(dm.y) <= win.y;
+                    if (again0)
+                        acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + t,
+                                            a.y + t, a.z + t);
+                    if (again1)
+                        acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kMom, a.x + t,
+                                            a.y + t, a.z + t);
+                    const unsigned int am0 = __ballot_sync(0xffffffffu, acc0);
+                    const unsigned int am1 = __ballot_sync(0xffffffffu, acc1);
+                    if (slot == 2 * p) am = am0;
+                    if (slot == 2 * p + 1) am = am1;
+                }
+                __syncwarp();
             }
-            if (acc) {
-                m2p_f32<kPhi>(rx, ry, rz, d2 + eps2, C.x, C.z, C.w, D.x, D.y, D.z, D.w, E.x, E.y, E.z,
-                        E.w, bx, by, bz, bp);
-                ++nm;
+            const unsigned int om = has ? mask & ~am : 0u;  // targets that open it
+            const unsigned int A = __ballot_sync(0xffffffffu, am != 0u);
+            const unsigned int OL = __ballot_sync(0xffffffffu, om != 0u && leaf);
+            const unsigned int OT = __ballot_sync(0xffffffffu, om != 0u && !leaf);
+            if (am) W.acc[na + __popc(A & lt)] = make_int2(box, (int)am);
+            if (om) {
+                if (leaf) W.leaf[nl + __popc(OL & lt)] = make_int2(box, (int)om);
+                else W.stack[top + __popc(OT & lt)] = make_int2(box, (int)om);
             }
-            if ((++vis & (kM2PBatch - 1)) == 0) fold_batch();
-            node = next;
-            if (npl == kList) flush();
+            na += __popc(A);
+            nl += __popc(OL);
+            top += __popc(OT);
+            __syncwarp();
+            const bool done = top == 0;
+            while (na >= kStage || (done && na > 0)) multipoles(min(na, kStage));
+            while (nl >= 32 || (done && nl > 0)) direct_pairs(min(nl, 32));
+            if (done) break;
+            const int pop = top > kPopWide ? 1 : min(top, 4);
+            box = -1;
+            mask = 0u;
+            if ((lane >> 3) < pop) {
+                const int2 e = W.stack[top - 1 - (lane >> 3)];
+                box = __ldg(a.t.child8 + (size_t)e.x * 8 + (lane & 7));
+                mask = (unsigned int)e.y;
+            }
+            top -= pop;
+            __syncwarp();
         }
-        flush();
-        fold_batch();
 
         if (valid) {
             const int s = a.sp[t];
@@ -673,24 +712,25 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
             r2 = INFINITY;
         }
         m[MR2] = r2;
+        // the centroid, relative to the cube's centre as the walk's targets are,
+        // enters negated (x_t - c as a sum); the trace term of the expansion as
+        // one value
+        const double ux = m[0] - cb.c[0], uy = m[1] - cb.c[1], uz = m[2] - cb.c[2];
+        const float chx = (float)ux, chy = (float)uy, chz = (float)uz;
+        const float rc2 = (float)r2;
+        t.hdr[nd] = make_float4(-chx, -chy, -chz, (dl & 256) ? -rc2 : rc2);
         if (want_f32) {
-            int4 inf = t.info[nd];
-            float4* r = t.f32 + (size_t)nd * kF32;
-            // the centroid, relative to the cube's centre as the walk's targets are,
-            // enters negated (x_t - c as a sum); the trace term of the expansion as
-            // one value
-            const double ux = m[0] - cb.c[0], uy = m[1] - cb.c[1], uz = m[2] - cb.c[2];
-            float chx = (float)ux, chy = (float)uy, chz = (float)uz;
-            r[0] = make_float4(-chx, -chy, -chz, (float)r2);
-            r[1] = make_float4((float)((double)chx - ux), (float)((double)chy - uy),
-                               (float)((double)chz - uz), __int_as_float(inf.z));
+            t.lo[nd] = make_float4((float)((double)chx - ux), (float)((double)chy - uy),
+                                   (float)((double)chz - uz), __int_as_float(t.info[nd].z));
             const float qxx = (float)m[MQ], qyy = (float)m[MQ + 3], qzz = (float)m[MQ + 5];
-            r[2] = make_float4(-0.5f * ((qxx + qyy) + qzz),
-                               __int_as_float((dl & 256) ? inf.y : -1), (float)m[MM],
-                               (float)m[MD]);
-            r[3] = make_float4((float)m[MD + 1], (float)m[MD + 2], (float)m[MQ], (float)m[MQ + 1]);
-            r[4] = make_float4((float)m[MQ + 2], (float)m[MQ + 3], (float)m[MQ + 4],
-                               (float)m[MQ + 5]);
+            const float M = (float)m[MM];
+            float4* r = t.rec + (size_t)nd * kRec;
+            r[0] = make_float4(-chx, -chy, -chz, M);
+            r[1] = make_float4((float)m[MD], (float)m[MD + 1], (float)m[MD + 2],
+                               -0.5f * ((qxx + qyy) + qzz));
+            r[2] = make_float4(0.5f * qxx, 0.5f * (float)m[MQ + 1], 0.5f * (float)m[MQ + 2],
+                               0.5f * qyy);
+            r[3] = make_float4(0.5f * (float)m[MQ + 4], 0.5f * qzz, -M, 0.f);
         }
     }
 }
@@ -740,26 +780,30 @@ void launch_walk_fp64(const WalkArgs& a, int nsm, cudaStream_t s)
     }
 }
 
-// Launch shapes of the FP32C walk that the autotuner chooses from: threads per
-// block, resident blocks per SM, which also sets the register budget (28 warps
-// per SM at 72 registers, 32 at 64), and whether leaf sources are staged in
-// shared memory by bulk copies.  The persistent grid takes 32-target
-// chunks from a counter, so the shape changes the schedule, never a result.
-static const int kShapes[][3] = {{128, 7, 0}, {896, 1, 0}, {128, 8, 0}, {1024, 1, 0},
-                                 {256, 4, 0}, {512, 2, 0}, {128, 7, 1}, {896, 1, 1},
-                                 {128, 8, 1}, {256, 4, 1}};
+// Launch shapes of the FP32C walk that the autotuner chooses from: blocks of one
+// warp, and how many of them are resident per SM, which sets the register budget,
+// {threads, blocks, 0}.  The persistent grid takes 32-target chunks from a counter,
+// so the shape changes the schedule, never a result.
+static const int kShapes[][3] = {{32, 24, 0}, {32, 20, 0}, {32, 28, 0}, {32, 32, 0},
+                                 {32, 16, 0}, {32, 18, 0}, {32, 22, 0}, {32, 26, 0},
+                                 {32, 14, 0}, {32, 12, 0}};
 int walk_shape_count() { return (int)(sizeof(kShapes) / sizeof(kShapes[0])); }
 
-template <bool kKelbg, bool kStage, bool kPhi>
-static void walk_fp32c_shape(const WalkArgs& a, int th, int per_sm, int b, cudaStream_t s)
+template <bool kKelbg, bool kPhi>
+static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, cudaStream_t s)
 {
-    if (th == 32) k_walk_fp32c<kKelbg, 32, 24, false, kPhi><<<b, 32, 0, s>>>(a);
-    else if (th == 896) k_walk_fp32c<kKelbg, 896, 1, kStage, kPhi><<<b, 896, 0, s>>>(a);
-    else if (th == 1024) k_walk_fp32c<kKelbg, 1024, 1, false, kPhi><<<b, 1024, 0, s>>>(a);
-    else if (th == 256) k_walk_fp32c<kKelbg, 256, 4, kStage, kPhi><<<b, 256, 0, s>>>(a);
-    else if (th == 512) k_walk_fp32c<kKelbg, 512, 2, false, kPhi><<<b, 512, 0, s>>>(a);
-    else if (per_sm >= 8) k_walk_fp32c<kKelbg, 128, 8, kStage, kPhi><<<b, 128, 0, s>>>(a);
-    else k_walk_fp32c<kKelbg, 128, 7, kStage, kPhi><<<b, 128, 0, s>>>(a);
+    switch (per_sm) {
+    case 12: k_walk_fp32c<kKelbg, 32, 12, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 14: k_walk_fp32c<kKelbg, 32, 14, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 16: k_walk_fp32c<kKelbg, 32, 16, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 18: k_walk_fp32c<kKelbg, 32, 18, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 20: k_walk_fp32c<kKelbg, 32, 20, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 22: k_walk_fp32c<kKelbg, 32, 22, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 26: k_walk_fp32c<kKelbg, 32, 26, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 28: k_walk_fp32c<kKelbg, 32, 28, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 32: k_walk_fp32c<kKelbg, 32, 32, kPhi><<<b, 32, 0, s>>>(a); break;
+    default: k_walk_fp32c<kKelbg, 32, 24, kPhi><<<b, 32, 0, s>>>(a); break;
+    }
 }
 
 void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
@@ -767,19 +811,13 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
     count_launch(1);
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     if (shape < 0 || shape >= walk_shape_count()) shape = 0;
-    int th = kShapes[shape][0], b;
     const int per_sm = kShapes[shape][1];
-    // the Kelbg pair law reads its sources directly
-    const bool stage = kShapes[shape][2] != 0 && !a.kelbg;
-    walk_grid(a.nchunks, nsm, &th, per_sm, &b);
+    const int b = walk_blocks(a.nchunks, nsm, per_sm, 1);
     // the potential is computed only when the caller reads it (the Kelbg form
     // always computes it)
-    const bool phi = a.phi != nullptr;
-    if (a.kelbg) walk_fp32c_shape<true, false, true>(a, th, per_sm, b, s);
-    else if (stage && phi) walk_fp32c_shape<false, true, true>(a, th, per_sm, b, s);
-    else if (stage) walk_fp32c_shape<false, true, false>(a, th, per_sm, b, s);
-    else if (phi) walk_fp32c_shape<false, false, true>(a, th, per_sm, b, s);
-    else walk_fp32c_shape<false, false, false>(a, th, per_sm, b, s);
+    if (a.kelbg) walk_fp32c_shape<true, true>(a, per_sm, b, s);
+    else if (a.phi) walk_fp32c_shape<false, true>(a, per_sm, b, s);
+    else walk_fp32c_shape<false, false>(a, per_sm, b, s);
 }
 
 }  // namespace ucp

@@ -21,10 +21,9 @@ UCP_FP64, UCP_FP32C = 0, 1
 UCP_ION, UCP_ELECTRON = 0, 1
 UCP_POT_PLUMMER, UCP_POT_KELBG = 0, 1
 UCP_WALK_SHAPES = 10
-# (threads per block, blocks per SM, leaf sources staged by bulk copies) of each
-# FP32C walk launch shape
-WALK_SHAPE_TABLE = ((128, 7, 0), (896, 1, 0), (128, 8, 0), (1024, 1, 0), (256, 4, 0), (512, 2, 0),
-                    (128, 7, 1), (896, 1, 1), (128, 8, 1), (256, 4, 1))
+# (threads per block, blocks per SM, 0) of each FP32C walk launch shape
+WALK_SHAPE_TABLE = ((32, 24, 0), (32, 20, 0), (32, 28, 0), (32, 32, 0), (32, 16, 0), (32, 18, 0),
+                    (32, 22, 0), (32, 26, 0), (32, 14, 0), (32, 12, 0))
 
 EXPORTS = ("ucp_create", "ucp_destroy", "ucp_set_state", "ucp_get_state", "ucp_tree_build",
            "ucp_tree_force", "ucp_step", "ucp_energy", "ucp_stats", "ucp_get_cube",
