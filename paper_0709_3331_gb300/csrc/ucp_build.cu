@@ -747,7 +747,7 @@ __device__ __forceinline__ void box_centre(const Cube& cb, unsigned long long ce
 // (z when S0 = 0); shifting to c: D = sum q y - M e,
 // Q = sum q y y^T - (sum q y) e^T - e (sum q y)^T + M e e^T.  delta = |e|.
 __device__ __forceinline__ void finish_box(const double* a, const double z[3],
-                                           double* __restrict__ m)
+                                           double* __restrict__ m, double* __restrict__ delta)
 {
     double S0 = a[0], M = a[1];
     double e[3];
@@ -768,8 +768,9 @@ __device__ __forceinline__ void finish_box(const double* a, const double z[3],
     double ex = __dsub_rn(m[MC + 0], z[0]);
     double ey = __dsub_rn(m[MC + 1], z[1]);
     double ez = __dsub_rn(m[MC + 2], z[2]);
-    m[MDELTA] = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)),
-                                     __dmul_rn(ez, ez)));
+    *delta = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)),
+                                  __dmul_rn(ez, ez)));
+    m[MT] = -0.5 * (m[MQ] + m[MQ + 3] + m[MQ + 5]);
 }
 
 __global__ void k_clear_children(Tree t)
@@ -819,7 +820,7 @@ __device__ void twig_combine_f64(const Cube* __restrict__ cube, const Tree& t, i
         a[13] += qk[5] + (2.0 * dk[2] + me2) * e[2];
     }
     double rec[kMom];
-    finish_box(a, zp, rec);
+    finish_box(a, zp, rec, t.delta + p);
     double* pm = t.mom + (size_t)p * kMom;
 #pragma unroll
     for (int k = 0; k < kMom; ++k) pm[k] = rec[k];
@@ -910,7 +911,7 @@ k_moments_leaves(const double* __restrict__ x, const double* __restrict__ y,
             a[13] += qj * yv[2] * yv[2];
         }
         double rec[kMom];
-        finish_box(a, zc, rec);
+        finish_box(a, zc, rec, t.delta + node);
         double* m = t.mom + (size_t)node * kMom;
 #pragma unroll
         for (int k = 0; k < kMom; ++k) m[k] = rec[k];
@@ -937,7 +938,8 @@ k_moments_leaves(const double* __restrict__ x, const double* __restrict__ y,
 // about that same point.  Compact per-box record mom32 = {e xyz, S0, M, D xyz,
 // Q xx xy xz yy yz zz, 0, 0} feeds the twig combine.
 __device__ __forceinline__ void finish_box_f32(const float* a, const double z[3], float* m32,
-                                               double* __restrict__ m64)
+                                               double* __restrict__ m64,
+                                               double* __restrict__ delta)
 {
     float S0 = a[0], M = a[1];
     float inv = S0 > 0.f ? 1.f / S0 : 0.f;
@@ -963,7 +965,7 @@ __device__ __forceinline__ void finish_box_f32(const float* a, const double z[3]
     for (int k = 0; k < 3; ++k) m64[MD + k] = d[k];
     for (int k = 0; k < 6; ++k) m64[MQ + k] = q[k];
     m64[MS0] = S0;
-    m64[MDELTA] = sqrtf(fmaf(e[0], e[0], fmaf(e[1], e[1], e[2] * e[2])));
+    *delta = sqrtf(fmaf(e[0], e[0], fmaf(e[1], e[1], e[2] * e[2])));
 }
 
 // Child slot o of twig p shifted to the twig's centre (zeros for an empty slot).
@@ -1029,7 +1031,7 @@ __device__ void twig_combine_f32(const Cube* __restrict__ cube, const Tree& t, i
 #pragma unroll
     for (int k = 0; k < 14; ++k) w[k] = u[k] + v[k];
     float m32[16];
-    finish_box_f32(w, zp, m32, t.mom + (size_t)p * kMom);
+    finish_box_f32(w, zp, m32, t.mom + (size_t)p * kMom, t.delta + p);
     float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)p * 16);
     for (int k = 0; k < 4; ++k)
         w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
@@ -1077,7 +1079,7 @@ k_moments_leaves_f32(const double* __restrict__ x, const double* __restrict__ y,
         }
         float m32[16];
         double* m = t.mom + (size_t)node * kMom;
-        finish_box_f32(a, zc, m32, m);
+        finish_box_f32(a, zc, m32, m, t.delta + node);
         float4* r32 = reinterpret_cast<float4*>(t.mom32 + (size_t)node * 16);
         for (int k = 0; k < 4; ++k)
             r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);

@@ -42,10 +42,10 @@ extern std::atomic<unsigned long long> g_launches;
 inline void count_launch(int k) { g_launches.fetch_add((unsigned long long)k, std::memory_order_relaxed); }
 
 // One FP64 box record, 16 doubles (128 B), read by the FP64 walk.
-// {c.x, c.y, c.z, rcrit2, M, D.x, D.y, D.z, Qxx, Qxy, Qxz, Qyy, Qyz, Qzz, S0, delta}
+// {c.x, c.y, c.z, rcrit2, M, D.x, D.y, D.z, Qxx, Qxy, Qxz, Qyy, Qyz, Qzz, S0, -tr(Q)/2}
 // rcrit2 = (s/theta + delta)^2 is filled per walk (it depends on theta).
 constexpr int kMom = 16;
-enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MDELTA = 15 };
+enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
 
 // FP32 box records, written per walk (they hold rcrit2, which depends on theta):
 //   hdr = {-ch.x, -ch.y, -ch.z, +-rcrit2}   ch = fp32(c) relative to the cube's centre;
@@ -65,6 +65,7 @@ struct Tree {
     int* depth_leaf;         // depth | leaf << 8
     unsigned long long* cell;// key prefix of the box at its depth
     double* mom;             // kMom doubles per box
+    double* delta;           // |centroid - geometric centre| per box
     float4* hdr;             // traversal record per box
     float4* lo;              // FP32C contexts: low part of the centroid, next
     float4* rec;             // FP32C contexts: kRec float4 per box

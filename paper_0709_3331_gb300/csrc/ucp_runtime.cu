@@ -280,9 +280,11 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
         if (f32) launch_walk_fp32c(a, c->nsm, c->s, c->walk_shape);
         else launch_walk_fp64(a, c->nsm, c->s);
         prof_end(c);
-        // the next walk over the same targets takes its chunks longest-first
-        launch_chunk_order(electrons_only ? c->chunks_e : c->chunks_all, a.nchunks, a.targets,
-                           c->cnt_p2p, c->cnt_m2p, c->chunk_cost, c->chunk_tmp, c->s);
+        // the next walk over the same targets takes its chunks longest-first (the FP64
+        // walk takes one target at a time: its end is as even without)
+        if (f32)
+            launch_chunk_order(electrons_only ? c->chunks_e : c->chunks_all, a.nchunks, a.targets,
+                               c->cnt_p2p, c->cnt_m2p, c->chunk_cost, c->chunk_tmp, c->s);
         c->walk_targets += a.ntargets;
         c->walk_launches += 1;
     }
@@ -298,35 +300,19 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
 // Walk chunks: up to 32 consecutive targets of one cloud.  All-particle chunks
 // cover each cloud's segment; electron chunks cover each cloud's run in the
 // compacted electron list (electrons keep their cloud order under sorting).
-// Targets per walk chunk: 32 (one per lane).  An FP64 context too small to give
-// every SM two chunks takes narrower chunks (down to 8 targets), so more warps
-// share the latency-bound FP64 walk; its sums do not depend on which targets
-// share a warp, so the results are the same.  The FP32C walk's batched sums do
-// depend on the warp's company, so it keeps 32.
-static int chunk_width(ucp_ctx* c)
-{
-    if (c->precision != UCP_FP64) return 32;
-    int w = 32;
-    while (w > 8) {
-        int64_t nch = 0;
-        for (int cl = 0; cl < c->n_clouds; ++cl)
-            nch += (c->cloud_start_h[cl + 1] - c->cloud_start_h[cl] + w - 1) / w;
-        if (nch >= 2 * (int64_t)c->nsm) break;
-        w /= 2;
-    }
-    return w;
-}
+constexpr int kChunk = 32;
 
 int build_chunks(ucp_ctx* c, const std::vector<int>& ne_per_cloud)
 {
     std::vector<int4> all, el;
     int e0 = 0;
-    const int W = chunk_width(c);
     for (int cl = 0; cl < c->n_clouds; ++cl) {
         int b = c->cloud_start_h[cl], e = c->cloud_start_h[cl + 1];
-        for (int t = b; t < e; t += W) all.push_back(make_int4(t, std::min(W, e - t), cl, 0));
+        for (int t = b; t < e; t += kChunk)
+            all.push_back(make_int4(t, std::min(kChunk, e - t), cl, 0));
         int ne = ne_per_cloud[cl];
-        for (int t = 0; t < ne; t += W) el.push_back(make_int4(e0 + t, std::min(W, ne - t), cl, 0));
+        for (int t = 0; t < ne; t += kChunk)
+            el.push_back(make_int4(e0 + t, std::min(kChunk, ne - t), cl, 0));
         e0 += ne;
     }
     if ((int)all.size() > c->n_chunks_all_cap || (int)el.size() > c->n_chunks_all_cap)
@@ -486,6 +472,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     if ((rc = dalloc(c, &c->t.nnodes, 1)) || (rc = dalloc(c, &c->t.maxdepth, 1)) ||
         (rc = dalloc(c, &c->t.info, cz)) || (rc = dalloc(c, &c->t.depth_leaf, cz)) ||
         (rc = dalloc(c, &c->t.cell, cz)) || (rc = dalloc(c, &c->t.mom, cz * kMom)) ||
+        (rc = dalloc(c, &c->t.delta, cz)) ||
         (rc = dalloc(c, &c->t.hdr, cz)) || (rc = dalloc(c, &c->t.child8, cz * 8)) || (rc = dalloc(c, &c->t.leaf_list, cz)) ||
         (rc = dalloc(c, &c->t.arrive, cz)) ||
         (rc = dalloc(c, &c->t.count, kMaxDepth + 2)))
@@ -550,7 +537,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
             c->t.cloud = c->cloud;
         }
         int64_t nch = 0;
-        for (int i = 0; i < n_clouds; ++i) nch += (sizes[i] + 7) / 8;  // chunks of >= 8
+        for (int i = 0; i < n_clouds; ++i) nch += (sizes[i] + kChunk - 1) / kChunk;
         c->n_chunks_all_cap = (int)nch;
         if ((rc = dalloc(c, &c->chunks_all, (size_t)nch)) ||
             (rc = dalloc(c, &c->chunks_e, (size_t)nch)) ||
@@ -1365,12 +1352,13 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
     std::vector<int4> info(nn);
     std::vector<int> dl(nn);
     std::vector<unsigned long long> cell(nn);
-    std::vector<double> mom((size_t)nn * kMom);
+    std::vector<double> mom((size_t)nn * kMom), delta(nn);
     CK(cudaMemcpyAsync(info.data(), c->t.info, sizeof(int4) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(dl.data(), c->t.depth_leaf, sizeof(int) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(cell.data(), c->t.cell, 8 * (size_t)nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(mom.data(), c->t.mom, sizeof(double) * kMom * nn, cudaMemcpyDeviceToHost,
                        c->s));
+    CK(cudaMemcpyAsync(delta.data(), c->t.delta, sizeof(double) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaStreamSynchronize(c->s));
     for (int i = 0; i < nn; ++i) {
         int d = dl[i] & 255;
@@ -1401,7 +1389,7 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
             for (int a = 0; a < 3; ++a) g[6 + a] = m[MC + a];
             for (int a = 0; a < 3; ++a) g[9 + a] = m[MD + a];
             for (int a = 0; a < 6; ++a) g[12 + a] = m[MQ + a];
-            g[18] = m[MDELTA];
+            g[18] = delta[i];
             g[19] = 0.0;
         }
     }

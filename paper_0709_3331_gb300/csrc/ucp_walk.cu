@@ -4,15 +4,10 @@
 // its expansion about its centroid (monopole, dipole, second moment of the
 // softened kernel); an opened leaf is summed pair by pair.
 //
-// FP64 form (k_walk_fp64): one warp walks 32 key-consecutive targets (one per
-// lane).  The per-target criterion is evaluated per lane; the warp descends into a
-// box when any lane opens it, and a lane that accepted an ancestor sits out until
-// the walk passes that ancestor's subtree (pre-order array with skip index "next",
-// no stack).  Lanes that accept a box evaluate its expansion on the spot; opened
-// leaves go into a per-warp list in shared memory as (leaf, lane mask) and are
-// summed in bulk.  The FP32C form (k_walk_fp32c) is described at its kernel.  In
-// both, each target's sums are taken in a fixed order, so results do not depend on
-// scheduling.
+// FP64 contexts walk one target per warp (k_walk_fp64), FP32C contexts 32
+// key-consecutive targets per warp (k_walk_fp32c); each is described at its kernel.
+// In both, each target's sums are taken in a fixed order, so results do not depend
+// on scheduling.
 #include "ucp_internal.cuh"
 
 #include <math.h>
@@ -20,14 +15,6 @@
 namespace ucp {
 
 namespace {
-
-constexpr int kWalkThreads = 128;
-constexpr int kList = 64;      // opened leaves buffered per warp (FP64 walk)
-
-struct WarpList {
-    int leaf[kList];
-    unsigned int mask[kList];
-};
 
 __device__ __forceinline__ int next_chunk(int* work, int lane)
 {
@@ -47,175 +34,220 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float v)
 }
 
 // ------------------------------------------------------------------ FP64
-// Expansion of a box at R = x_t - c, r2 = R.R + eps^2, g = r2^-1/2, u = g^2:
-//   phi = g (M + u (D.R - tr(Q)/2 + (3/2) u R.Q.R))
-//   E   = g^3 (M + 3u (D.R - tr(Q)/2 + (5/2) u R.Q.R)) R - g^3 (D + 3u Q R)
-// (the Taylor expansion of the softened kernel through second order, with the
-// terms of each power of u collected).
-template <class T>
-__device__ __forceinline__ void m2p(T rx, T ry, T rz, T r2, T M, T Dx, T Dy, T Dz, T Qxx, T Qxy,
-                                    T Qxz, T Qyy, T Qyz, T Qzz, T& ex, T& ey, T& ez, T& ph);
+// Twigs on the stack: up to kPopWide + 28 while four are popped per step; above
+// kPopWide one is popped per step, which adds at most 7 per level below it.
+constexpr int kPopWide = 64;
+constexpr int kStack = kPopWide + 28 + 7 * (kMaxDepth - 1) + 8;
 
-template <>
-__device__ __forceinline__ void m2p<double>(double rx, double ry, double rz, double r2, double M,
-                                            double Dx, double Dy, double Dz, double Qxx,
-                                            double Qxy, double Qxz, double Qyy, double Qyz,
-                                            double Qzz, double& ex, double& ey, double& ez,
-                                            double& ph)
+// Eq. 5 for a target and a box's record m in FP64, rounded like the definition
+__device__ __noinline__ bool accepts_fp64(const double* m, const double* x, const double* y,
+                                          const double* z)
 {
-    double g = rsqrt(r2);
-    double u = g * g;
-    double g3 = g * u;
-    double QRx = Qxx * rx + Qxy * ry + Qxz * rz;
-    double QRy = Qxy * rx + Qyy * ry + Qyz * rz;
-    double QRz = Qxz * rx + Qyz * ry + Qzz * rz;
-    double RQR = rx * QRx + ry * QRy + rz * QRz;
-    double w = Dx * rx + Dy * ry + Dz * rz - 0.5 * (Qxx + Qyy + Qzz);
-    double h = u * RQR;
-    ph += g * (M + u * (w + 1.5 * h));
-    double s3 = 3.0 * u;
-    double aa = g3 * (M + s3 * (w + 2.5 * h));
-    ex += aa * rx - g3 * (Dx + s3 * QRx);
-    ey += aa * ry - g3 * (Dy + s3 * QRy);
-    ez += aa * rz - g3 * (Dz + s3 * QRz);
+    const double dx = __dsub_rn(*x, m[0]);
+    const double dy = __dsub_rn(*y, m[1]);
+    const double dz = __dsub_rn(*z, m[2]);
+    return m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-template <bool kKelbg, int kThreads>
-__global__ void __launch_bounds__(kThreads)
+// One warp walks one target; its lanes are boxes and sources.  A step of the
+// traversal pops up to four opened twigs from a stack and tests their children, one
+// per lane; accepted boxes and the particles of opened leaves wait in two lists and
+// are evaluated 32 at a time, one per lane.  The criterion is taken in FP32 on the
+// traversal records and again in FP64 within its rounding window (see the FP32C
+// walk), so the decisions are those of FP64.
+//
+// What bounds it: the FP64 pipe, which takes a warp instruction for 16 cycles
+// however many of its lanes are active (2 multiply-adds per clock and SM).  One
+// target per warp keeps all lanes at work in both lists (of 32 targets in a warp
+// 65 % took part in a multipole and 35 % in a direct pair) and the FP32 criterion
+// leaves the pipe to the interactions: @@FIG@@.  A target's sums
+// are over its own boxes and sources in an order set by the tree alone, so they do
+// not depend on the launch.
+//
+// Expansion of a box at R = x_t - c, r2 = R.R + eps^2, g = r2^-1/2, u = g^2,
+// w = D.R - tr(Q)/2, h = u R.Q.R:
+//   phi = g (M + u (w + (3/2) h))
+//   E   = g^3 [(M + 3u (w + (5/2) h)) R - (D + 3u Q R)]
+// (the Taylor expansion of the softened kernel through second order, with the
+// terms of each power of u collected).
+template <bool kKelbg, bool kPhi>
+__global__ void __launch_bounds__(32, 16)
 k_walk_fp64(WalkArgs a)
 {
-    __shared__ WarpList L[kThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    WarpList& lst = L[w];
+    __shared__ int stack[kStack], acc[64], src[64];
+    const int lane = threadIdx.x;
+    const unsigned int lt = (1u << lane) - 1u;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const double* __restrict__ mom = a.t.mom;
-    const int4* __restrict__ info = a.t.info;
-    const int* __restrict__ dlf = a.t.depth_leaf;
+    const float4* __restrict__ H = a.t.hdr;
     const double* __restrict__ X = a.x;
     const double* __restrict__ Y = a.y;
     const double* __restrict__ Z = a.z;
     const int8_t* __restrict__ SP = a.sp;
+    unsigned long long sum_p = 0, sum_m = 0;
 
-    for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
-         chunk = next_chunk(a.work, lane)) {
-        // up to 32 key-consecutive targets of one cloud, walked through that cloud's tree
-        const int4 ck = a.chunks[chunk];
-        const int ti = ck.x + lane;
-        const bool valid = lane < ck.y;
-        const int t = valid ? (a.targets ? a.targets[ti] : ti) : -1;
-        const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
-        const int end = info[root].z;
-        const double xt = valid ? X[t] : 0.0, yt = valid ? Y[t] : 0.0, zt = valid ? Z[t] : 0.0;
-        const int8_t st = valid ? SP[t] : 0;
-        // multipole and direct-pair sums kept apart: each is then a sum over this
-        // target's own boxes in pre-order, whichever targets share the warp
+    while (true) {
+        const unsigned int item = (unsigned int)next_chunk(a.work, lane);
+        if ((item >> 5) >= (unsigned int)a.nchunks) break;
+        const int4 ck = a.chunks[item >> 5];
+        const int place = (int)(item & 31u);
+        if (place >= ck.y) continue;
+        const int ti = ck.x + place;
+        const int t = a.targets ? a.targets[ti] : ti;
+        const double xt = X[t], yt = Y[t], zt = Z[t];
+        const int8_t st = SP[t];
+        const double* cc = a.cubes[ck.z].c;
+        const float xh = (float)(xt - cc[0]), yh = (float)(yt - cc[1]), zh = (float)(zt - cc[2]);
+        const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
+        const float wa = fmaf(0.5f, bt, 4e-6f), wb = 0.5f * bt;
         double ex = 0.0, ey = 0.0, ez = 0.0, ph = 0.0;
-        double pex = 0.0, pey = 0.0, pez = 0.0, pph = 0.0;
-        int np = 0, nm = 0;
-        int skip = valid ? 0 : 0x7fffffff;
-        int npl = 0;
+        int top = 0, na = 0, nq = 0, np = 0, nm = 0;
 
-        auto flush = [&]() {
-            __syncwarp();
-            for (int e = 0; e < npl; ++e) {
-                int nd = lst.leaf[e];
-                if ((lst.mask[e] >> lane) & 1u) {
-                    int4 inf = info[nd];
-                    for (int j = inf.x; j < inf.y; ++j) {
-                        if (j == t) continue;
-                        double qj = SP[j] ? q1 : q0;
-                        double dx = xt - X[j], dy = yt - Y[j], dz = zt - Z[j];
-                        if (kKelbg && SP[j] != st) {
-                            // Sec. 2.1 Eq. 3: qj (1 - e)/r, e = exp(-r/lambda);
-                            // E = qj r_vec [(1 - e)/r^3 - e/(lambda r^2)]
-                            double r = sqrt(dx * dx + dy * dy + dz * dz);
-                            ++np;
-                            if (r == 0.0) {
-                                pph += qj / a.lambda;
-                                continue;
-                            }
-                            double u = r / a.lambda;
-                            double e = exp(-u), ome = -expm1(-u);
-                            double f = ome / (r * r * r) - e / (a.lambda * r * r);
-                            pex += qj * dx * f;
-                            pey += qj * dy * f;
-                            pez += qj * dz * f;
-                            pph += qj * ome / r;
-                            continue;
-                        }
-                        double r2 = dx * dx + dy * dy + dz * dz + a.eps2;
-                        double ri = rsqrt(r2);
-                        double qr3 = qj * ri * ri * ri;
-                        pex += qr3 * dx;
-                        pey += qr3 * dy;
-                        pez += qr3 * dz;
-                        pph += qj * ri;
-                        ++np;
-                    }
-                }
+        // the last cnt <= 32 accepted boxes
+        auto multipoles = [&](int cnt) {
+            na -= cnt;
+            if (lane < cnt) {
+                const double2* m =
+                    reinterpret_cast<const double2*>(a.t.mom + (size_t)acc[na + lane] * kMom);
+                const double2 m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3], m4 = m[4], m5 = m[5],
+                              m6 = m[6], m7 = m[7];
+                const double rx = xt - m0.x, ry = yt - m0.y, rz = zt - m1.x;
+                const double r2 = rx * rx + (ry * ry + (rz * rz + a.eps2));
+                const double M = m2.x;
+                const double g = rsqrt(r2);
+                const double u = g * g;
+                const double g3 = g * u;
+                const double qx = m4.x * rx + m4.y * ry + m5.x * rz;
+                const double qy = m4.y * rx + m5.y * ry + m6.x * rz;
+                const double qz = m5.x * rx + m6.x * ry + m6.y * rz;
+                const double rqr = rx * qx + ry * qy + rz * qz;
+                const double w = m2.y * rx + (m3.x * ry + (m3.y * rz + m7.y));
+                const double h = u * rqr;
+                const double s3 = 3.0 * u;
+                const double k = M + s3 * (w + 2.5 * h);
+                ex += g3 * (k * rx - (m2.y + s3 * qx));
+                ey += g3 * (k * ry - (m3.x + s3 * qy));
+                ez += g3 * (k * rz - (m3.y + s3 * qz));
+                if (kPhi) ph += g * (M + u * (w + 1.5 * h));
             }
-            npl = 0;
             __syncwarp();
         };
-
-        int node = root;
-        while (node < end) {
-            const double* m = mom + (size_t)node * kMom;
-            const int4 inf = info[node];
-            const bool leaf = (dlf[node] & 256) != 0;
-            const bool active = node >= skip;
-            // Eq. 5 as (s/theta + delta)^2 < |x_t - c|^2, rounded like the definition
-            double dx = __dsub_rn(xt, m[0]);
-            double dy = __dsub_rn(yt, m[1]);
-            double dz = __dsub_rn(zt, m[2]);
-            double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                                  __dmul_rn(dz, dz));
-            const bool acc = active && (m[MR2] < d2);
-            const bool opn = active && !acc;
-            const unsigned int om = __ballot_sync(0xffffffffu, opn);
-            int next = inf.z;
-            if (om) {
-                if (leaf) {
-                    if (lane == 0) {
-                        lst.leaf[npl] = node;
-                        lst.mask[npl] = om;
+        // the last cnt <= 32 sources
+        auto direct_pairs = [&](int cnt) {
+            nq -= cnt;
+            const int j = lane < cnt ? src[nq + lane] : t;
+            if (j != t) {
+                const double qj = SP[j] ? q1 : q0;
+                const double dx = xt - X[j], dy = yt - Y[j], dz = zt - Z[j];
+                if (kKelbg && SP[j] != st) {
+                    // Sec. 2.1 Eq. 3: qj (1 - e)/r, e = exp(-r/lambda);
+                    // E = qj r_vec [(1 - e)/r^3 - e/(lambda r^2)]
+                    const double r = sqrt(dx * dx + dy * dy + dz * dz);
+                    if (r == 0.0) {
+                        ph += qj / a.lambda;
+                    } else {
+                        const double u = r / a.lambda;
+                        const double e = exp(-u), ome = -expm1(-u);
+                        const double f = ome / (r * r * r) - e / (a.lambda * r * r);
+                        ex += qj * dx * f;
+                        ey += qj * dy * f;
+                        ez += qj * dz * f;
+                        ph += qj * ome / r;
                     }
-                    ++npl;
                 } else {
-                    if (acc) skip = inf.z;
-                    next = node + 1;
+                    const double ri = rsqrt(dx * dx + (dy * dy + (dz * dz + a.eps2)));
+                    const double qi = qj * ri;
+                    const double qr3 = qi * (ri * ri);
+                    ex += qr3 * dx;
+                    ey += qr3 * dy;
+                    ez += qr3 * dz;
+                    if (kPhi) ph += qi;
                 }
             }
-            if (acc) {
-                m2p<double>(dx, dy, dz, d2 + a.eps2, m[MM], m[MD], m[MD + 1], m[MD + 2], m[MQ],
-                            m[MQ + 1], m[MQ + 2], m[MQ + 3], m[MQ + 4], m[MQ + 5], ex, ey, ez, ph);
-                ++nm;
-            }
-            node = next;
-            if (npl == kList) flush();
-        }
-        flush();
+            np += __popc(__ballot_sync(0xffffffffu, j != t));
+        };
 
-        if (valid) {
-            const int s = SP[t];
-            const double qm = (s ? q1 : q0) / a.msp[s];
-            a.ax[t] = qm * (ex + pex);
-            a.ay[t] = qm * (ey + pey);
-            a.az[t] = qm * (ez + pez);
-            if (a.phi) a.phi[t] = ph + pph;
+        int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0] : -1;
+        while (true) {
+            const bool has = box >= 0;
+            const float4 h = has ? __ldg(H + box) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const bool leaf = __float_as_int(h.w) < 0;
+            const float rx = xh + h.x, ry = yh + h.y, rz = zh + h.z;
+            const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+            const float dm = d2 - fabsf(h.w);
+            bool ok = has && dm > 0.f;
+            if (has && fabsf(dm) <= fmaf(wa, d2, wb))
+                ok = accepts_fp64(a.t.mom + (size_t)box * kMom, X + t, Y + t, Z + t);
+            const unsigned int A = __ballot_sync(0xffffffffu, ok);
+            const unsigned int OL = __ballot_sync(0xffffffffu, has && !ok && leaf);
+            const unsigned int OT = __ballot_sync(0xffffffffu, has && !ok && !leaf);
+            if (ok) acc[na + __popc(A & lt)] = box;
+            if (has && !ok && !leaf) stack[top + __popc(OT & lt)] = box;
+            na += __popc(A);
+            nm += __popc(A);
+            top += __popc(OT);
+            __syncwarp();
+            const bool done = top == 0;
+            while (na >= 32 || (done && na > 0)) multipoles(min(na, 32));
+            if (OL) {
+                // the opened leaves' particles, in one run over the lanes
+                int2 be = make_int2(0, 0);
+                if ((OL >> lane) & 1u) be = __ldg(reinterpret_cast<const int2*>(a.t.info + box));
+                int end = be.y - be.x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, end, o);
+                    if (lane >= o) end += v;
+                }
+                const int total = __shfl_sync(0xffffffffu, end, 31);
+                const int first = be.y - end;      // particle f of the run in this leaf: first + f
+                for (int base = 0; base < total; base += 32) {
+                    const int f = base + lane;
+                    int owner = 0;                 // lanes whose leaf ends at or before f
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+                        if (__shfl_sync(0xffffffffu, end, owner + o - 1) <= f) owner += o;
+                    const int j = __shfl_sync(0xffffffffu, first, owner) + f;
+                    if (f < total) src[nq + lane] = j;
+                    nq += min(32, total - base);
+                    __syncwarp();
+                    if (nq >= 32) direct_pairs(32);
+                    __syncwarp();
+                }
+            }
+            if (done) {
+                if (nq > 0) direct_pairs(nq);
+                break;
+            }
+            const int pop = top > kPopWide ? 1 : min(top, 4);
+            box = -1;
+            if ((lane >> 3) < pop)
+                box = __ldg(a.t.child8 + (size_t)stack[top - 1 - (lane >> 3)] * 8 + (lane & 7));
+            top -= pop;
+            __syncwarp();
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            ex += __shfl_xor_sync(0xffffffffu, ex, o);
+            ey += __shfl_xor_sync(0xffffffffu, ey, o);
+            ez += __shfl_xor_sync(0xffffffffu, ez, o);
+            if (kPhi) ph += __shfl_xor_sync(0xffffffffu, ph, o);
+        }
+        if (lane == 0) {
+            const double qm = (st ? q1 : q0) / a.msp[st];
+            a.ax[t] = qm * ex;
+            a.ay[t] = qm * ey;
+            a.az[t] = qm * ez;
+            if (kPhi && a.phi) a.phi[t] = ph;
             a.cnt_p2p[t] = np;
             a.cnt_m2p[t] = nm;
         }
-        unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
-            sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
-        }
-        if (lane == 0) {
-            atomicAdd(&a.stats[0], sp2);
-            atomicAdd(&a.stats[1], sm2);
-        }
+        sum_p += (unsigned long long)np;
+        sum_m += (unsigned long long)nm;
+    }
+    if (lane == 0) {
+        atomicAdd(&a.stats[0], sum_p);
+        atomicAdd(&a.stats[1], sum_m);
     }
 }
 
@@ -279,11 +311,6 @@ __device__ __forceinline__ void kelbg_pg(float u, float& p, float& g)
 // by the same operations in the same order, so accelerations are bit-identical.
 constexpr int kStage = 32;           // boxes evaluated per batch (pairs of two)
 constexpr int kStageStride = 36;     // floats per staged pair (32 used; 16-byte aligned)
-// Twigs on the stack: up to kPopWide + 28 while four are popped per step; above
-// kPopWide one is popped per step, which adds at most 7 per level below it.
-constexpr int kPopWide = 64;
-constexpr int kStack = kPopWide + 28 + 7 * (kMaxDepth - 1) + 8;
-
 struct __align__(16) WalkWarp {
     float stage[kStage / 2 * kStageStride];
     int2 stack[kStack];              // {twig, mask}
@@ -296,16 +323,6 @@ __device__ __forceinline__ float warp_min(float v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
-}
-
-// Eq. 5 for a target and a box's record m in FP64, rounded like the definition
-__device__ __noinline__ bool accepts_fp64(const double* m, const double* x, const double* y,
-                                          const double* z)
-{
-    const double dx = __dsub_rn(*x, m[0]);
-    const double dy = __dsub_rn(*y, m[1]);
-    const double dz = __dsub_rn(*z, m[2]);
-    return m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
 __device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
@@ -706,7 +723,7 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
         double s = ldexp(L, -(dl & 255));
         double r2;
         if (theta > 0.0) {
-            double rc = __dadd_rn(__ddiv_rn(s, theta), m[MDELTA]);
+            double rc = __dadd_rn(__ddiv_rn(s, theta), t.delta[nd]);
             r2 = __dmul_rn(rc, rc);
         } else {
             r2 = INFINITY;
@@ -744,40 +761,23 @@ void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, cu
     k_mac_prepare<<<blocks, 256, 0, s>>>(t, cube, theta, want_f32);
 }
 
-static int walk_blocks(int nchunks, int nsm, int per_sm, int warps_per_block)
+// blocks of one warp: per_sm on every SM, or one per work item
+static int walk_blocks(int64_t items, int nsm, int per_sm)
 {
-    int blocks = nsm * per_sm;
-    int need = (nchunks + warps_per_block - 1) / warps_per_block;
-    if (blocks > need) blocks = need;
+    const int blocks = nsm * per_sm < items ? nsm * per_sm : (int)items;
     return blocks < 1 ? 1 : blocks;
-}
-
-// Grid of th-thread blocks, per_sm resident per SM.  When the chunks cannot give
-// every SM a block (small clouds), blocks narrow to one warp so the same warps
-// spread over more SMs.  Each warp walks whole chunks, so no shape changes a result.
-static void walk_grid(int nchunks, int nsm, int* th, int per_sm, int* blocks)
-{
-    const int wpb = *th / 32;
-    *blocks = walk_blocks(nchunks, nsm, per_sm, wpb);
-    if (*blocks < nsm && wpb > 1) {
-        *th = 32;
-        *blocks = walk_blocks(nchunks, nsm, per_sm * wpb, 1);
-    }
 }
 
 void launch_walk_fp64(const WalkArgs& a, int nsm, cudaStream_t s)
 {
     count_launch(1);
-    int th = kWalkThreads, b;
-    walk_grid(a.nchunks, nsm, &th, 8, &b);
+    const int b = walk_blocks((int64_t)a.nchunks * 32, nsm, 16);
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
-    if (a.kelbg) {
-        if (th == 32) k_walk_fp64<true, 32><<<b, 32, 0, s>>>(a);
-        else k_walk_fp64<true, kWalkThreads><<<b, kWalkThreads, 0, s>>>(a);
-    } else {
-        if (th == 32) k_walk_fp64<false, 32><<<b, 32, 0, s>>>(a);
-        else k_walk_fp64<false, kWalkThreads><<<b, kWalkThreads, 0, s>>>(a);
-    }
+    // the potential is computed only when the caller reads it
+    if (a.kelbg && a.phi) k_walk_fp64<true, true><<<b, 32, 0, s>>>(a);
+    else if (a.kelbg) k_walk_fp64<true, false><<<b, 32, 0, s>>>(a);
+    else if (a.phi) k_walk_fp64<false, true><<<b, 32, 0, s>>>(a);
+    else k_walk_fp64<false, false><<<b, 32, 0, s>>>(a);
 }
 
 // Launch shapes of the FP32C walk that the autotuner chooses from: blocks of one
@@ -812,7 +812,7 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     if (shape < 0 || shape >= walk_shape_count()) shape = 0;
     const int per_sm = kShapes[shape][1];
-    const int b = walk_blocks(a.nchunks, nsm, per_sm, 1);
+    const int b = walk_blocks(a.nchunks, nsm, per_sm);
     // the potential is computed only when the caller reads it (the Kelbg form
     // always computes it)
     if (a.kelbg) walk_fp32c_shape<true, true>(a, per_sm, b, s);
