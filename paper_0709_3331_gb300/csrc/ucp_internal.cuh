@@ -192,10 +192,13 @@ void launch_scatter3(const double* ax, const double* ay, const double* az, const
                      int n, double* out, cudaStream_t s);
 void launch_scatter1(const double* a, const unsigned int* id, int n, double* out, cudaStream_t s);
 void launch_scatter_int(const int* a, const unsigned int* id, int n, int* out, cudaStream_t s);
-void launch_deinterleave(const double* aos, int n, double* x, double* y, double* z,
-                         cudaStream_t s);
-void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n, int* flags,
-                        cudaStream_t s);
-void launch_iota(unsigned int* a, int n, cudaStream_t s);
+void launch_load_state(const double* pos, const double* vel, const int8_t* sp, int n,
+                       double* const* st6, int8_t* sp_slot, int8_t* sp_caller, unsigned int* id,
+                       cudaStream_t s);
+// flags: {non-finite, bad species, electrons of cloud 0, 1, ...}, zeroed before
+void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n,
+                        const unsigned char* cloud, int* flags, cudaStream_t s);
+void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
+                   int4* chunks, cudaStream_t s);
 
 }  // namespace ucp

@@ -168,34 +168,71 @@ __global__ void k_scatter_int(const int* __restrict__ a, const unsigned int* __r
     if (i < n) out[id[i]] = a[i];
 }
 
-__global__ void k_deinterleave(const double* __restrict__ aos, int n, double* __restrict__ x,
-                               double* __restrict__ y, double* __restrict__ z)
+// Caller-order state (N x 3 arrays, vel may be NULL: zeros) into the context's
+// arrays: six streams, species (twice: in the slots' order and in the caller's) and
+// the identity as caller indices.
+__global__ void k_load_state(const double* __restrict__ pos, const double* __restrict__ vel,
+                             const int8_t* __restrict__ sp, int n, double* __restrict__ x,
+                             double* __restrict__ y, double* __restrict__ z,
+                             double* __restrict__ vx, double* __restrict__ vy,
+                             double* __restrict__ vz, int8_t* __restrict__ sp_slot,
+                             int8_t* __restrict__ sp_caller, unsigned int* __restrict__ id)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    x[i] = aos[3 * (size_t)i];
-    y[i] = aos[3 * (size_t)i + 1];
-    z[i] = aos[3 * (size_t)i + 2];
+    const size_t b = 3 * (size_t)i;
+    x[i] = pos[b];
+    y[i] = pos[b + 1];
+    z[i] = pos[b + 2];
+    vx[i] = vel ? vel[b] : 0.0;
+    vy[i] = vel ? vel[b + 1] : 0.0;
+    vz[i] = vel ? vel[b + 2] : 0.0;
+    const int8_t s = sp[i];
+    sp_slot[i] = s;
+    if (sp_caller) sp_caller[i] = s;
+    id[i] = (unsigned int)i;
 }
 
 // flags[0] |= 1 on a non-finite position or velocity, flags[1] |= 1 on a
-// species code other than 0 or 1.
+// species code other than 0 or 1, flags[2 + c] += electrons of cloud c.
 __global__ void k_check_state(const double* __restrict__ pos, const double* __restrict__ vel,
-                              const int8_t* __restrict__ sp, int n, int* __restrict__ flags)
+                              const int8_t* __restrict__ sp, int n,
+                              const unsigned char* __restrict__ cloud, int* __restrict__ flags)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    bool bad = false;
-    for (int a = 0; a < 3; ++a)
-        bad |= !isfinite(pos[3 * (size_t)i + a]) || !isfinite(vel[3 * (size_t)i + a]);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    bool bad = false, wrong = false, electron = false;
+    int c = 0;
+    if (i < n) {
+        for (int a = 0; a < 3; ++a)
+            bad |= !isfinite(pos[3 * (size_t)i + a]) || !isfinite(vel[3 * (size_t)i + a]);
+        wrong = sp[i] != 0 && sp[i] != 1;
+        electron = sp[i] == 1;
+        if (cloud) c = cloud[i];
+    }
     if (bad) atomicOr(&flags[0], 1);
-    if (sp[i] != 0 && sp[i] != 1) atomicOr(&flags[1], 1);
+    if (wrong) atomicOr(&flags[1], 1);
+    // electrons: one count per warp and cloud
+    const unsigned int e = __ballot_sync(0xffffffffu, electron);
+    const unsigned int peers = __match_any_sync(0xffffffffu, c) & e;
+    if (electron && lane == __ffs(peers) - 1) atomicAdd(&flags[2 + c], __popc(peers));
 }
 
-__global__ void k_iota(unsigned int* a, int n)
+// Walk chunks of up to `width` consecutive targets, cloud by cloud: cloud c's run of
+// targets is [first[c], first[c + 1]), its chunks start at place[c].
+__global__ void k_chunks(const int* __restrict__ first, const int* __restrict__ place, int n_clouds,
+                         int width, int nchunks, int4* __restrict__ chunks)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] = (unsigned int)i;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= nchunks) return;
+    int lo = 0, hi = n_clouds;          // the cloud whose chunks hold i
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (place[mid] <= i) lo = mid;
+        else hi = mid;
+    }
+    const int b = first[lo] + (i - place[lo]) * width;
+    chunks[i] = make_int4(b, min(width, first[lo + 1] - b), lo, 0);
 }
 
 inline int nb(int n) { return (n + kT - 1) / kT > 0 ? (n + kT - 1) / kT : 1; }
@@ -263,23 +300,28 @@ void launch_scatter_int(const int* a, const unsigned int* id, int n, int* out, c
     k_scatter_int<<<nb(n), kT, 0, s>>>(a, id, n, out);
 }
 
-void launch_deinterleave(const double* aos, int n, double* x, double* y, double* z, cudaStream_t s)
+void launch_load_state(const double* pos, const double* vel, const int8_t* sp, int n,
+                       double* const* st6, int8_t* sp_slot, int8_t* sp_caller, unsigned int* id,
+                       cudaStream_t s)
 {
     count_launch(1);
-    k_deinterleave<<<nb(n), kT, 0, s>>>(aos, n, x, y, z);
+    k_load_state<<<nb(n), kT, 0, s>>>(pos, vel, sp, n, st6[0], st6[1], st6[2], st6[3], st6[4],
+                                      st6[5], sp_slot, sp_caller, id);
 }
 
-void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n, int* flags,
-                        cudaStream_t s)
+void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n,
+                        const unsigned char* cloud, int* flags, cudaStream_t s)
 {
     count_launch(1);
-    k_check_state<<<nb(n), kT, 0, s>>>(pos, vel, sp, n, flags);
+    k_check_state<<<nb(n), kT, 0, s>>>(pos, vel, sp, n, cloud, flags);
 }
 
-void launch_iota(unsigned int* a, int n, cudaStream_t s)
+void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
+                   int4* chunks, cudaStream_t s)
 {
+    if (nchunks < 1) return;
     count_launch(1);
-    k_iota<<<nb(n), kT, 0, s>>>(a, n);
+    k_chunks<<<nb(nchunks), kT, 0, s>>>(first, place, n_clouds, width, nchunks, chunks);
 }
 
 }  // namespace ucp

@@ -57,7 +57,11 @@ struct ucp_ctx {
     double* en_part = nullptr;
     int en_nblk = 1;
     double* en_out = nullptr;
-    int* flags = nullptr;
+    int* flags = nullptr;              // set_state: bad values, electrons per cloud
+    int* chunk_table = nullptr;        // 2 (n_clouds + 1): runs of targets, first chunks
+    // host side of those (page-locked: small copies that do not wait for a staging copy)
+    int* host_flags = nullptr;
+    int* host_table = nullptr;
     double* stage = nullptr;  // n x 6 doubles for host transfers and layout changes
     int8_t* stage_sp = nullptr;
     int8_t* sp_caller = nullptr;  // species in caller order
@@ -109,7 +113,11 @@ struct ucp_ctx {
     int64_t prof_launches = 0;
 
     std::string err;
-    std::vector<void*> allocs;
+    // device arrays: one slab, the place of each noted by dalloc
+    struct Slot { void** p; size_t offset; };
+    std::vector<Slot> slots;
+    size_t slab_bytes = 0;
+    void* slab = nullptr;
 };
 
 namespace {
@@ -134,17 +142,25 @@ int check_launch(ucp_ctx* c, const char* where)
     return UCP_OK;
 }
 
+// The context's device memory is one allocation: dalloc notes an array, commit
+// allocates them all and sets the pointers (60 separate cudaMallocs took most of
+// ucp_create).
 template <class T>
-int dalloc(ucp_ctx* c, T** p, size_t count)
+void dalloc(ucp_ctx* c, T** p, size_t count)
 {
-    void* q = nullptr;
-    cudaError_t e = cudaMalloc(&q, (count ? count : 1) * sizeof(T));
+    c->slots.push_back({reinterpret_cast<void**>(p), (size_t)c->slab_bytes});
+    c->slab_bytes += ((count ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+}
+
+int commit(ucp_ctx* c)
+{
+    cudaError_t e = cudaMalloc(&c->slab, c->slab_bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        c->slab = nullptr;
         return fail(c, UCP_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     }
-    c->allocs.push_back(q);
-    *p = (T*)q;
+    for (auto& s : c->slots) *s.p = static_cast<char*>(c->slab) + s.offset;
     return UCP_OK;
 }
 
@@ -302,29 +318,26 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
 // compacted electron list (electrons keep their cloud order under sorting).
 constexpr int kChunk = 32;
 
-int build_chunks(ucp_ctx* c, const std::vector<int>& ne_per_cloud)
+// Chunk lists from the first target of every cloud (n_clouds + 1 values): the counts
+// are the host's, the lists are written on the device.  table: room for 2 (n_clouds
+// + 1) ints on the host (its contents are uploaded) and on the device.
+int build_chunks(ucp_ctx* c, const int* first, int* host_table, int* table, int4* chunks,
+                 int* n_chunks)
 {
-    std::vector<int4> all, el;
-    int e0 = 0;
-    for (int cl = 0; cl < c->n_clouds; ++cl) {
-        int b = c->cloud_start_h[cl], e = c->cloud_start_h[cl + 1];
-        for (int t = b; t < e; t += kChunk)
-            all.push_back(make_int4(t, std::min(kChunk, e - t), cl, 0));
-        int ne = ne_per_cloud[cl];
-        for (int t = 0; t < ne; t += kChunk)
-            el.push_back(make_int4(e0 + t, std::min(kChunk, ne - t), cl, 0));
-        e0 += ne;
+    const int nc = c->n_clouds;
+    int* place = host_table + nc + 1;
+    int total = 0;
+    for (int cl = 0; cl < nc; ++cl) {
+        host_table[cl] = first[cl];
+        place[cl] = total;
+        total += (first[cl + 1] - first[cl] + kChunk - 1) / kChunk;
     }
-    if ((int)all.size() > c->n_chunks_all_cap || (int)el.size() > c->n_chunks_all_cap)
-        return fail(c, UCP_EINVAL, "internal: chunk capacity");
-    c->n_chunks_all = (int)all.size();
-    c->n_chunks_e = (int)el.size();
-    CK(cudaMemcpyAsync(c->chunks_all, all.data(), sizeof(int4) * all.size(), cudaMemcpyHostToDevice,
-                       c->s));
-    if (!el.empty())
-        CK(cudaMemcpyAsync(c->chunks_e, el.data(), sizeof(int4) * el.size(),
-                           cudaMemcpyHostToDevice, c->s));
-    CK(cudaStreamSynchronize(c->s));
+    host_table[nc] = first[nc];
+    place[nc] = total;
+    if (total > c->n_chunks_all_cap) return fail(c, UCP_EINVAL, "internal: chunk capacity");
+    CK(cudaMemcpyAsync(table, host_table, sizeof(int) * 2 * (nc + 1), cudaMemcpyHostToDevice, c->s));
+    launch_chunks(table, table + nc + 1, nc, kChunk, total, chunks, c->s);
+    *n_chunks = total;
     return UCP_OK;
 }
 
@@ -371,7 +384,8 @@ void ucp_destroy(ucp_ctx* c)
     if (!c) return;
     if (c->s) cudaStreamSynchronize(c->s);
     else cudaDeviceSynchronize();
-    for (void* p : c->allocs) cudaFree(p);
+    if (c->slab) cudaFree(c->slab);
+    if (c->host_flags) cudaFreeHost(c->host_flags);
     for (auto& e : c->ev) {
         cudaEventDestroy(e.first);
         cudaEventDestroy(e.second);
@@ -441,42 +455,43 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     };
     if (cudaGetDevice(&c->device) != cudaSuccess) return bail(UCP_ECUDA);
     cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device);
-    size_t n = (size_t)c->n;
+    const size_t n = (size_t)c->n;
     for (int b = 0; b < 2; ++b) {
-        for (int a = 0; a < 6; ++a)
-            if ((rc = dalloc(c, &c->st[b][a], n))) return bail(rc);
-        if ((rc = dalloc(c, &c->sp[b], n))) return bail(rc);
-        if ((rc = dalloc(c, &c->id[b], n))) return bail(rc);
-        if ((rc = dalloc(c, &c->key[b], n))) return bail(rc);
-        if ((rc = dalloc(c, &c->val[b], n))) return bail(rc);
+        for (int a = 0; a < 6; ++a) dalloc(c, &c->st[b][a], n);
+        dalloc(c, &c->sp[b], n);
+        dalloc(c, &c->id[b], n);
+        dalloc(c, &c->key[b], n);
+        dalloc(c, &c->val[b], n);
     }
-    if ((rc = dalloc(c, &c->ax, n)) || (rc = dalloc(c, &c->ay, n)) || (rc = dalloc(c, &c->az, n)) ||
-        (rc = dalloc(c, &c->phi, n)))
-        return bail(rc);
-    if ((rc = dalloc(c, &c->sort.ghist, 8 * 256 + 9)) || (rc = dalloc(c, &c->sort.goff, 8 * 256)) ||
-        (rc = dalloc(c, &c->sort.status, sort_status_words(c->n))) ||
-        (rc = dalloc(c, &c->sort.err, 1)) || (rc = dalloc(c, &c->sort.epoch, 1)) ||
-        (rc = dalloc(c, &c->sort.test_epoch, 1)) ||
-        (rc = dalloc(c, &c->sort.test_keys, sort_test_words())) ||
-        (rc = dalloc(c, &c->sort.test_vals, sort_test_words())))
-        return bail(rc);
-    if (cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) != cudaSuccess ||
-        cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) != cudaSuccess ||
-        cudaMemsetAsync(c->sort.epoch, 0, sizeof(unsigned int), c->s) != cudaSuccess)
-        return bail(UCP_ECUDA);
-    size_t spw = scan_partials_words(c->n);
-    if ((rc = dalloc(c, &c->scan_part, spw))) return bail(rc);
-    if ((rc = dalloc(c, &c->pos_cnt, n)) || (rc = dalloc(c, &c->pos_off, n))) return bail(rc);
+    dalloc(c, &c->ax, n);
+    dalloc(c, &c->ay, n);
+    dalloc(c, &c->az, n);
+    dalloc(c, &c->phi, n);
+    dalloc(c, &c->sort.ghist, 8 * 256 + 9);
+    dalloc(c, &c->sort.goff, 8 * 256);
+    dalloc(c, &c->sort.status, sort_status_words(c->n));
+    dalloc(c, &c->sort.err, 1);
+    dalloc(c, &c->sort.epoch, 1);
+    dalloc(c, &c->sort.test_epoch, 1);
+    dalloc(c, &c->sort.test_keys, sort_test_words());
+    dalloc(c, &c->sort.test_vals, sort_test_words());
+    dalloc(c, &c->scan_part, scan_partials_words(c->n));
+    dalloc(c, &c->pos_cnt, n);
+    dalloc(c, &c->pos_off, n);
+    const size_t cz = (size_t)cap;
     c->t.cap = (int)cap;
-    size_t cz = (size_t)cap;
-    if ((rc = dalloc(c, &c->t.nnodes, 1)) || (rc = dalloc(c, &c->t.maxdepth, 1)) ||
-        (rc = dalloc(c, &c->t.info, cz)) || (rc = dalloc(c, &c->t.depth_leaf, cz)) ||
-        (rc = dalloc(c, &c->t.cell, cz)) || (rc = dalloc(c, &c->t.mom, cz * kMom)) ||
-        (rc = dalloc(c, &c->t.delta, cz)) ||
-        (rc = dalloc(c, &c->t.hdr, cz)) || (rc = dalloc(c, &c->t.child8, cz * 8)) || (rc = dalloc(c, &c->t.leaf_list, cz)) ||
-        (rc = dalloc(c, &c->t.arrive, cz)) ||
-        (rc = dalloc(c, &c->t.count, kMaxDepth + 2)))
-        return bail(rc);
+    dalloc(c, &c->t.nnodes, 1);
+    dalloc(c, &c->t.maxdepth, 1);
+    dalloc(c, &c->t.info, cz);
+    dalloc(c, &c->t.depth_leaf, cz);
+    dalloc(c, &c->t.cell, cz);
+    dalloc(c, &c->t.mom, cz * kMom);
+    dalloc(c, &c->t.delta, cz);
+    dalloc(c, &c->t.hdr, cz);
+    dalloc(c, &c->t.child8, cz * 8);
+    dalloc(c, &c->t.leaf_list, cz);
+    dalloc(c, &c->t.arrive, cz);
+    dalloc(c, &c->t.count, kMaxDepth + 2);
     {
         // twigs of depth d: at most min(8^d, n / (leaf_cap + 1)); none at the depth cap
         int64_t off = 0, pow8 = 1;
@@ -489,19 +504,16 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
                 }
             if (pow8 < ((int64_t)1 << 40)) pow8 *= 8;
         }
-        if ((rc = dalloc(c, &c->t.twig_list, (size_t)(off > 0 ? off : 1)))) return bail(rc);
+        dalloc(c, &c->t.twig_list, (size_t)(off > 0 ? off : 1));
     }
     if (c->precision == UCP_FP32C) {
+        dalloc(c, &c->t.lo, cz);
+        dalloc(c, &c->t.rec, cz * kRec);
+        dalloc(c, &c->t.mom32, cz * 16);
         // sources in pairs: 2 float4 per pair of particles (padded to an even count)
-        if ((rc = dalloc(c, &c->t.lo, cz)) || (rc = dalloc(c, &c->t.rec, cz * kRec)) ||
-            (rc = dalloc(c, &c->src32, n + 1)) ||
-            (rc = dalloc(c, &c->t.mom32, cz * 16)))
-            return bail(rc);
-        // the pad slot of an odd count is read (masked) by the pair loop: keep it finite
-        if (cudaMemsetAsync(c->src32, 0, sizeof(float4) * (n + 1), c->s) != cudaSuccess)
-            return bail(UCP_ECUDA);
+        dalloc(c, &c->src32, n + 1);
     }
-    if ((rc = dalloc(c, &c->cube, (size_t)n_clouds))) return bail(rc);
+    dalloc(c, &c->cube, (size_t)n_clouds);
     {
         int64_t biggest = 0;
         for (int i = 0; i < n_clouds; ++i) biggest = sizes[i] > biggest ? sizes[i] : biggest;
@@ -513,56 +525,66 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     c->en_nblk = (int)((n + 2047) / 2048);
     if (c->en_nblk > 4 * c->nsm) c->en_nblk = 4 * c->nsm;
     if (c->en_nblk < 1) c->en_nblk = 1;
-    if ((rc = dalloc(c, &c->bbox_part, (size_t)n_clouds * c->bbox_nblk * 6)) ||
-        (rc = dalloc(c, &c->en_part, (size_t)c->en_nblk * 6)) ||
-        (rc = dalloc(c, &c->en_out, (size_t)6 * n_clouds)))
-        return bail(rc);
-    {
-        // clouds: segment starts, the (static) cloud of every slot, walk chunk capacity
-        if ((rc = dalloc(c, &c->cloud_start, (size_t)n_clouds + 1))) return bail(rc);
-        if (cudaMemcpyAsync(c->cloud_start, c->cloud_start_h.data(), sizeof(int) * (n_clouds + 1),
-                            cudaMemcpyHostToDevice, c->s) != cudaSuccess)
-            return bail(UCP_ECUDA);
-        c->t.cloud_start = c->cloud_start;
-        c->t.cloud = nullptr;
-        if (n_clouds > 1) {
-            std::vector<unsigned char> cl(n);
-            for (int i = 0; i < n_clouds; ++i)
-                for (int j = c->cloud_start_h[i]; j < c->cloud_start_h[i + 1]; ++j)
-                    cl[j] = (unsigned char)i;
-            if ((rc = dalloc(c, &c->cloud, n))) return bail(rc);
-            if (cudaMemcpyAsync(c->cloud, cl.data(), n, cudaMemcpyHostToDevice, c->s) != cudaSuccess ||
-                cudaStreamSynchronize(c->s) != cudaSuccess)
-                return bail(UCP_ECUDA);
-            c->t.cloud = c->cloud;
-        }
-        int64_t nch = 0;
-        for (int i = 0; i < n_clouds; ++i) nch += (sizes[i] + kChunk - 1) / kChunk;
-        c->n_chunks_all_cap = (int)nch;
-        if ((rc = dalloc(c, &c->chunks_all, (size_t)nch)) ||
-            (rc = dalloc(c, &c->chunks_e, (size_t)nch)) ||
-            (rc = dalloc(c, &c->chunk_cost, (size_t)nch)) ||
-            (rc = dalloc(c, &c->chunk_tmp, (size_t)nch)))
-            return bail(rc);
+    dalloc(c, &c->bbox_part, (size_t)n_clouds * c->bbox_nblk * 6);
+    dalloc(c, &c->en_part, (size_t)c->en_nblk * 6);
+    dalloc(c, &c->en_out, (size_t)6 * n_clouds);
+    // clouds: segment starts, the (static) cloud of every slot, walk chunk capacity
+    dalloc(c, &c->cloud_start, (size_t)n_clouds + 1);
+    if (n_clouds > 1) dalloc(c, &c->cloud, n);
+    int64_t nch = 0;
+    for (int i = 0; i < n_clouds; ++i) nch += (sizes[i] + kChunk - 1) / kChunk;
+    c->n_chunks_all_cap = (int)nch;
+    dalloc(c, &c->chunks_all, (size_t)nch);
+    dalloc(c, &c->chunks_e, (size_t)nch);
+    dalloc(c, &c->chunk_cost, (size_t)nch);
+    dalloc(c, &c->chunk_tmp, (size_t)nch);
+    dalloc(c, &c->qsp, 2);
+    dalloc(c, &c->msp, 2);
+    dalloc(c, &c->tlist, n);
+    dalloc(c, &c->tcount, 1);
+    dalloc(c, &c->cnt_p2p, n);
+    dalloc(c, &c->cnt_m2p, n);
+    dalloc(c, &c->work, 1);
+    dalloc(c, &c->stats, 2);
+    dalloc(c, &c->flags, 2 + (size_t)n_clouds);
+    dalloc(c, &c->chunk_table, 2 * ((size_t)n_clouds + 1));
+    dalloc(c, &c->stage, 6 * n);
+    dalloc(c, &c->stage_sp, n);
+    dalloc(c, &c->sp_caller, n);
+    dalloc(c, &c->stage_int, 2 * n);
+    if ((rc = commit(c))) return bail(rc);
+
+    c->t.cloud_start = c->cloud_start;
+    c->t.cloud = c->cloud;
+    std::vector<unsigned char> cl;
+    if (n_clouds > 1) {
+        cl.resize(n);
+        for (int i = 0; i < n_clouds; ++i)
+            for (int j = c->cloud_start_h[i]; j < c->cloud_start_h[i + 1]; ++j)
+                cl[j] = (unsigned char)i;
     }
-    if ((rc = dalloc(c, &c->qsp, 2)) || (rc = dalloc(c, &c->msp, 2))) return bail(rc);
-    if ((rc = dalloc(c, &c->tlist, n)) || (rc = dalloc(c, &c->tcount, 1)))
-        return bail(rc);
-    if ((rc = dalloc(c, &c->cnt_p2p, n)) || (rc = dalloc(c, &c->cnt_m2p, n)) ||
-        (rc = dalloc(c, &c->work, 1)) || (rc = dalloc(c, &c->stats, 2)) ||
-        (rc = dalloc(c, &c->flags, 2)))
-        return bail(rc);
-    if ((rc = dalloc(c, &c->stage, 6 * n)) || (rc = dalloc(c, &c->stage_sp, n)) ||
-        (rc = dalloc(c, &c->sp_caller, n)) ||
-        (rc = dalloc(c, &c->stage_int, 2 * n)))
-        return bail(rc);
-    if (cudaMemcpyAsync(c->qsp, c->q, 2 * sizeof(double), cudaMemcpyHostToDevice, c->s) ||
+    if (cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) ||
+        cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) ||
+        cudaMemsetAsync(c->sort.epoch, 0, sizeof(unsigned int), c->s) ||
+        // the pad slot of an odd count is read (masked) by the pair loop: keep it finite
+        (c->src32 && cudaMemsetAsync(c->src32, 0, sizeof(float4) * (n + 1), c->s)) ||
+        cudaMemcpyAsync(c->cloud_start, c->cloud_start_h.data(), sizeof(int) * (n_clouds + 1),
+                        cudaMemcpyHostToDevice, c->s) ||
+        (c->cloud && cudaMemcpyAsync(c->cloud, cl.data(), n, cudaMemcpyHostToDevice, c->s)) ||
+        cudaMemcpyAsync(c->qsp, c->q, 2 * sizeof(double), cudaMemcpyHostToDevice, c->s) ||
         cudaMemcpyAsync(c->msp, c->m, 2 * sizeof(double), cudaMemcpyHostToDevice, c->s) ||
         cudaMemsetAsync(c->stats, 0, 2 * sizeof(unsigned long long), c->s) ||
-        cudaStreamSynchronize(c->s)) {
+        cudaHostAlloc(&c->host_flags, sizeof(int) * (3 + 2 * UCP_MAX_CLOUDS + 2 * (UCP_MAX_CLOUDS + 1)),
+                      0)) {
         c->err = "initial copies failed";
         return bail(UCP_ECUDA);
     }
+    c->host_table = c->host_flags + 3 + 2 * UCP_MAX_CLOUDS;
+    // the chunks over every particle follow from the sizes alone
+    if ((rc = build_chunks(c, c->cloud_start_h.data(), c->host_table, c->chunk_table, c->chunks_all,
+                           &c->n_chunks_all)))
+        return bail(rc);
+    if (cudaStreamSynchronize(c->s) || check_launch(c, "create")) return bail(UCP_ECUDA);
     *out = c;
     return UCP_OK;
 }
@@ -572,65 +594,43 @@ int ucp_set_state(ucp_ctx* c, const double* pos, const double* vel, const int8_t
 {
     if (!c) return UCP_EINVAL;
     if (!pos || !vel || !species) return fail(c, UCP_EINVAL, "null pointer");
-    size_t n = (size_t)c->n;
+    const size_t n = (size_t)c->n;
     const double* dpos = pos;
     const double* dvel = vel;
     const int8_t* dsp = species;
-    int k = c->cur;
-    std::vector<int8_t> host_sp;
+    const int k = c->cur, nc = c->n_clouds;
     if (!on_device) {
-        int ne = 0;
-        for (size_t i = 0; i < n; ++i) {
-            for (int a = 0; a < 3; ++a)
-                if (!std::isfinite(pos[3 * i + a]) || !std::isfinite(vel[3 * i + a]))
-                    return fail(c, UCP_ENONFINITE, "non-finite position or velocity");
-            if (species[i] != 0 && species[i] != 1)
-                return fail(c, UCP_EINVAL, "species must be 0 (ion) or 1 (electron)");
-            ne += species[i] == 1;
-        }
         CK(cudaMemcpyAsync(c->stage, pos, 3 * n * sizeof(double), cudaMemcpyHostToDevice, c->s));
         CK(cudaMemcpyAsync(c->stage + 3 * n, vel, 3 * n * sizeof(double), cudaMemcpyHostToDevice,
                            c->s));
-        CK(cudaMemcpyAsync(c->sp[k], species, n, cudaMemcpyHostToDevice, c->s));
+        CK(cudaMemcpyAsync(c->stage_sp, species, n, cudaMemcpyHostToDevice, c->s));
         dpos = c->stage;
         dvel = c->stage + 3 * n;
-        c->n_e = ne;
-    } else {
-        CK(cudaMemsetAsync(c->flags, 0, 2 * sizeof(int), c->s));
-        launch_check_state(pos, vel, species, c->n, c->flags, c->s);
-        int fl[2] = {0, 0};
-        CK(cudaMemcpyAsync(fl, c->flags, sizeof(fl), cudaMemcpyDeviceToHost, c->s));
-        CK(cudaStreamSynchronize(c->s));
-        if (fl[0]) return fail(c, UCP_ENONFINITE, "non-finite position or velocity");
-        if (fl[1]) return fail(c, UCP_EINVAL, "species must be 0 (ion) or 1 (electron)");
-        CK(cudaMemcpyAsync(c->sp[k], dsp, n, cudaMemcpyDeviceToDevice, c->s));
-        host_sp.resize(n);
-        CK(cudaMemcpyAsync(host_sp.data(), dsp, n, cudaMemcpyDeviceToHost, c->s));
-        CK(cudaStreamSynchronize(c->s));
-        species = host_sp.data();
-        int ne = 0;
-        for (size_t i = 0; i < n; ++i) ne += species[i] == 1;
-        c->n_e = ne;
+        dsp = c->stage_sp;
     }
-    {
-        std::vector<int> ne_cl(c->n_clouds, 0);
-        for (int cl = 0; cl < c->n_clouds; ++cl)
-            for (int i = c->cloud_start_h[cl]; i < c->cloud_start_h[cl + 1]; ++i)
-                ne_cl[cl] += species[i] == 1;
-        int rc = build_chunks(c, ne_cl);
-        if (rc) return rc;
-    }
-    launch_deinterleave(dpos, c->n, c->st[k][0], c->st[k][1], c->st[k][2], c->s);
-    launch_deinterleave(dvel, c->n, c->st[k][3], c->st[k][4], c->st[k][5], c->s);
-    launch_iota(c->id[k], c->n, c->s);
-    CK(cudaMemcpyAsync(c->sp_caller, c->sp[k], n, cudaMemcpyDeviceToDevice, c->s));
+    // checks and electron counts on the device, one small copy back; nothing of the
+    // context's state changes before they are known
+    CK(cudaMemsetAsync(c->flags, 0, (2 + nc) * sizeof(int), c->s));
+    launch_check_state(dpos, dvel, dsp, c->n, c->cloud, c->flags, c->s);
+    int* fl = c->host_flags;
+    CK(cudaMemcpyAsync(fl, c->flags, (2 + nc) * sizeof(int), cudaMemcpyDeviceToHost, c->s));
+    CK(cudaStreamSynchronize(c->s));
+    if (fl[0]) return fail(c, UCP_ENONFINITE, "non-finite position or velocity");
+    if (fl[1]) return fail(c, UCP_EINVAL, "species must be 0 (ion) or 1 (electron)");
+    int* first = c->host_flags + 2 + UCP_MAX_CLOUDS;   // of every cloud in the electron list
+    first[0] = 0;
+    for (int cl = 0; cl < nc; ++cl) first[cl + 1] = first[cl] + fl[2 + cl];
+    c->n_e = first[nc];
+    int rc = build_chunks(c, first, c->host_table, c->chunk_table, c->chunks_e, &c->n_chunks_e);
+    if (rc) return rc;
+    launch_load_state(dpos, dvel, dsp, c->n, c->st[k], c->sp[k], c->sp_caller, c->id[k], c->s);
     CK(cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s));
     c->have_state = true;
     c->tree_valid = false;
     c->acc_valid = false;
     c->phi_valid = false;
     c->steps = 0;
-    int rc = check_launch(c, "set_state");
+    rc = check_launch(c, "set_state");
     if (rc) return rc;
     if (!on_device) CK(cudaStreamSynchronize(c->s));
     return UCP_OK;
@@ -967,14 +967,11 @@ int ucp_step(ucp_ctx* c, double dt_e, int kk, int64_t n_electron_steps, double t
 }
 
 // Replace the positions and velocities (device, caller order) without the
-// checks of ucp_set_state; species stay as set.
+// checks of ucp_set_state; species stay as set (dvel NULL: zero velocities).
 static void load_state(ucp_ctx* c, const double* dpos, const double* dvel)
 {
     int k = c->cur;
-    launch_deinterleave(dpos, c->n, c->st[k][0], c->st[k][1], c->st[k][2], c->s);
-    launch_deinterleave(dvel, c->n, c->st[k][3], c->st[k][4], c->st[k][5], c->s);
-    cudaMemcpyAsync(c->sp[k], c->sp_caller, (size_t)c->n, cudaMemcpyDeviceToDevice, c->s);
-    launch_iota(c->id[k], c->n, c->s);
+    launch_load_state(dpos, dvel, c->sp_caller, c->n, c->st[k], c->sp[k], nullptr, c->id[k], c->s);
     c->tree_valid = false;
     c->acc_valid = false;
     c->phi_valid = false;
@@ -997,9 +994,9 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
     const int64_t nseg = (S + C - 1) / C;
     // working memory of this call: checkpoints, one segment of positions, lambdas
     double *ck = nullptr, *seg = nullptr, *lx = nullptr, *lv = nullptr, *lam = nullptr,
-           *lsorted = nullptr, *mu = nullptr, *adj = nullptr, *dloss = nullptr, *zero = nullptr;
+           *lsorted = nullptr, *mu = nullptr, *adj = nullptr, *dloss = nullptr;
     auto freeall = [&]() {
-        for (double* p : {ck, seg, lx, lv, lam, lsorted, mu, adj, dloss, zero})
+        for (double* p : {ck, seg, lx, lv, lam, lsorted, mu, adj, dloss})
             if (p) cudaFree(p);
     };
     size_t adj_words = (size_t)c->t.cap * 12;
@@ -1007,8 +1004,7 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
         cudaMalloc(&seg, sizeof(double) * n3 * (C + 1)) || cudaMalloc(&lx, sizeof(double) * n3) ||
         cudaMalloc(&lv, sizeof(double) * n3) || cudaMalloc(&lam, sizeof(double) * n3) ||
         cudaMalloc(&lsorted, sizeof(double) * n3) || cudaMalloc(&mu, sizeof(double) * n3) ||
-        cudaMalloc(&adj, sizeof(double) * adj_words) || cudaMalloc(&dloss, sizeof(double)) ||
-        cudaMalloc(&zero, sizeof(double) * n3)) {
+        cudaMalloc(&adj, sizeof(double) * adj_words) || cudaMalloc(&dloss, sizeof(double))) {
         cudaGetLastError();
         freeall();
         return fail(c, UCP_ENOMEM, "adjoint working memory");
@@ -1039,7 +1035,6 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
     launch_ke_seed(ck + 2 * n3 * nseg + n3, c->sp_caller, c->n, c->m[UCP_ELECTRON], lv, dloss,
                    c->s);
     cudaMemsetAsync(lx, 0, sizeof(double) * n3, c->s);
-    cudaMemsetAsync(zero, 0, sizeof(double) * n3, c->s);
     WalkArgs a;
     // reverse: for g = S .. 1: adjoint of the kicks at X_g, then of drift g; X_0 last
     for (int64_t sgi = nseg - 1; sgi >= 0 && !rc; --sgi) {
@@ -1058,7 +1053,7 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
             const bool endp = g == 0 || g == S;
             const double ce = (endp ? 1.0 : 2.0) * h_e;
             const double ci = (g % kk == 0) ? (endp ? 1.0 : 2.0) * h_i : 0.0;
-            load_state(c, seg + n3 * (size_t)j, zero);
+            load_state(c, seg + n3 * (size_t)j, nullptr);
             if ((rc = build(c))) break;
             const int f32 = c->precision == UCP_FP32C;
             launch_mac_prepare(c->t, c->cube, theta, f32, c->s);
