@@ -3,8 +3,8 @@
 // fixed (the boxes every target opens or accepts do not move under an
 // infinitesimal displacement).  FP64.
 //
-// The walk visits exactly the boxes of the forward walk (same criterion, same
-// rounding).  Per target (lane):
+// The walk visits exactly the boxes of the forward walk (the same decisions).  Per
+// target:
 //   direct pair j:    mu_t += (q_t q_j / m_t) J(r) lambda_t,  J = g^3 I - 3 g^5 r r^T
 //                     mu_j -= q_j J(r) w_t,  w_t = q_t lambda_t / m_t
 //   accepted box n:   mu_t -= (q_t/m_t) (M d2g lambda - sum_bc lambda_b D_c d3g_abc
@@ -14,36 +14,15 @@
 //   q_s (alpha_n - Gamma_n (x_s - c_n)) + (|q_s| / S0_n) kappa_n
 // (the source side through the dipole and second moment at fixed centre, and
 // through the |q|-weighted centre the expansion is taken about).
-// Source-side sums over targets are warp reductions followed by FP64 atomic
+// Source-side sums over targets are summed per group of targets and then by atomic
 // adds, so their order (and last bits) may vary from run to run.
-#include "ucp_internal.cuh"
+#include "ucp_lists.cuh"
 
 #include <math.h>
 
 namespace ucp {
 
 namespace {
-
-constexpr int kAdjThreads = 128;
-constexpr int kAdjWarps = kAdjThreads / 32;
-constexpr int kAdjList = 64;
-
-struct AdjList {
-    int leaf[kAdjList];
-    unsigned int mask[kAdjList];
-};
-
-__device__ __forceinline__ double wsum(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-__device__ __forceinline__ double dot3(const double* a, const double* b)
-{
-    return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
-}
 
 __device__ __forceinline__ void qmul(const double* Q, const double* v, double* o)
 {
@@ -52,188 +31,202 @@ __device__ __forceinline__ void qmul(const double* Q, const double* v, double* o
     o[2] = Q[2] * v[0] + Q[4] * v[1] + Q[5] * v[2];
 }
 
-// sum_bcd v_b Q_cd d4g_abcd
-__device__ __forceinline__ void t4(const double* R, const double* v, const double* Q, double g,
-                                   double* o)
+__device__ __forceinline__ double dot3(const double* a, const double* b)
 {
-    double g2 = g * g, g5 = g2 * g2 * g, g7 = g5 * g2, g9 = g7 * g2;
-    double QR[3], Qv[3];
-    qmul(Q, R, QR);
-    qmul(Q, v, Qv);
-    double RQR = dot3(R, QR), Rv = dot3(R, v), vQR = dot3(v, QR), trQ = Q[0] + Q[3] + Q[5];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-        o[a] = 105.0 * R[a] * Rv * RQR * g9 -
-               15.0 * g7 * (v[a] * RQR + 2.0 * Rv * QR[a] + 2.0 * R[a] * vQR + R[a] * Rv * trQ) +
-               3.0 * g5 * (v[a] * trQ + 2.0 * Qv[a]);
+    return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-__global__ void __launch_bounds__(kAdjThreads)
-k_walk_adjoint(WalkArgs a, const double* __restrict__ lam, double* __restrict__ mu,
+// ---- FP64 form: one warp per group of up to kAdjGroup targets, the traversal of
+// the FP32C walk on the FP64 contexts' records (FP32 criterion, again in FP64 within
+// its window: the FP64 walk's decisions).  The lanes are the sources, 32 accepted
+// boxes or 32 particles of opened leaves, and every lane goes through the group's
+// targets, so a source's own sums stay in its registers and a target's partial sums
+// in shared memory, one per lane, until the end.  All terms are linear in the
+// target's weight w = (q/m) lambda.
+//
+// What bounds it: the FP64 pipe (about 120 operations per box and target, 16 cycles
+// per warp instruction).  Eight targets per warp keep 85 % of the lanes at work (32:
+// 68 %); groups get smaller when eight would leave SMs without work.  The form
+// before summed each box's 12 values and each pair's three over the warp in FP64
+// (75 and 15 additions): accelerations and their vector-Jacobian product at N = 4,096
+// took 15.9 ms against 2.0.
+constexpr int kAdjGroup = 8;
+
+struct __align__(16) AdjWarp64 {
+    WalkWarp walk;
+    double mt[kAdjGroup][3][32];      // partial sums of the targets, per lane
+    double tgt[kAdjGroup][6];         // position and weight
+    int slot[kAdjGroup];
+};
+
+__global__ void __launch_bounds__(32, 12)
+k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __restrict__ mu,
                double* __restrict__ adj)
 {
-    __shared__ AdjList Ls[kAdjWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    AdjList& lst = Ls[w];
+    __shared__ AdjWarp64 shared;
+    AdjWarp64& W = shared;
+    const int lane = threadIdx.x;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const double* __restrict__ mom = a.t.mom;
-    const int4* __restrict__ info = a.t.info;
-    const int* __restrict__ dlf = a.t.depth_leaf;
-    const double* __restrict__ X = a.x;
-    const double* __restrict__ Y = a.y;
-    const double* __restrict__ Z = a.z;
-    const int8_t* __restrict__ SP = a.sp;
+    const int per = 32 / group;       // groups per chunk
 
-    for (int chunk = 0; true;) {
-        if (lane == 0) chunk = atomicAdd(a.work, 1);
-        chunk = __shfl_sync(0xffffffffu, chunk, 0);
-        if (chunk >= a.nchunks) break;
-        const int4 ck = a.chunks[chunk];
-        const bool valid = lane < ck.y;
-        const int t = valid ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
-        const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
-        const int end = info[root].z;
-        const double xt = valid ? X[t] : 0.0, yt = valid ? Y[t] : 0.0, zt = valid ? Z[t] : 0.0;
-        double l[3] = {0.0, 0.0, 0.0};
-        double qm = 0.0;
-        if (valid) {
-            l[0] = lam[3 * (size_t)t];
-            l[1] = lam[3 * (size_t)t + 1];
-            l[2] = lam[3 * (size_t)t + 2];
-            const int s = SP[t];
-            qm = (s ? q1 : q0) / a.msp[s];
+    while (true) {
+        const unsigned int item = (unsigned int)next_chunk(a.work, lane);
+        if (item / per >= (unsigned int)a.nchunks) break;
+        const int4 ck = a.chunks[item / per];
+        const int skip = (int)(item % per) * group;
+        const int nt = min(group, ck.y - skip);
+        if (nt <= 0) continue;
+        const int ti = ck.x + skip + lane;
+        const int t = lane < nt ? (a.targets ? a.targets[ti] : ti) : -1;
+        const ChunkTarget tg(a, t, ck.z);
+        if (t >= 0) {
+            const int s = a.sp[t];
+            const double qm = (s ? q1 : q0) / a.msp[s];
+            W.tgt[lane][0] = a.x[t];
+            W.tgt[lane][1] = a.y[t];
+            W.tgt[lane][2] = a.z[t];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) W.tgt[lane][3 + k] = qm * lam[3 * (size_t)t + k];
+            W.slot[lane] = t;
         }
-        const double wv[3] = {qm * l[0], qm * l[1], qm * l[2]};
-        double mt[3] = {0.0, 0.0, 0.0};
-        int skip = valid ? 0 : 0x7fffffff;
-        int npl = 0;
+        for (int g = 0; g < nt; ++g)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) W.mt[g][k][lane] = 0.0;
+        __syncwarp();
 
-        auto flush = [&]() {
-            __syncwarp();
-            for (int e = 0; e < npl; ++e) {
-                const int nd = lst.leaf[e];
-                const bool in = (lst.mask[e] >> lane) & 1u;
-                const int4 inf = info[nd];
-                for (int j = inf.x; j < inf.y; ++j) {
-                    double sx = 0.0, sy = 0.0, sz = 0.0;
-                    const double qj = SP[j] ? q1 : q0;
-                    if (in && j != t) {
-                        double r[3] = {xt - X[j], yt - Y[j], zt - Z[j]};
-                        double g = rsqrt(dot3(r, r) + a.eps2);
-                        double g3 = g * g * g, g5 = g3 * g * g;
-                        double rl = dot3(r, l), rw = dot3(r, wv);
-                        mt[0] += qm * qj * (l[0] * g3 - 3.0 * r[0] * rl * g5);
-                        mt[1] += qm * qj * (l[1] * g3 - 3.0 * r[1] * rl * g5);
-                        mt[2] += qm * qj * (l[2] * g3 - 3.0 * r[2] * rl * g5);
-                        sx = -qj * (wv[0] * g3 - 3.0 * r[0] * rw * g5);
-                        sy = -qj * (wv[1] * g3 - 3.0 * r[1] * rw * g5);
-                        sz = -qj * (wv[2] * g3 - 3.0 * r[2] * rw * g5);
-                    }
-                    sx = wsum(sx);
-                    sy = wsum(sy);
-                    sz = wsum(sz);
-                    if (lane == 0) {
-                        atomicAdd(&mu[3 * (size_t)j], sx);
-                        atomicAdd(&mu[3 * (size_t)j + 1], sy);
-                        atomicAdd(&mu[3 * (size_t)j + 2], sz);
-                    }
+        // The same terms as the FP32 form below: the target takes -H, the box alpha,
+        // Gamma and kappa.
+        auto multipoles = [&](const int2* boxes, int cnt) {
+            const int2 bm = lane < cnt ? boxes[lane] : make_int2(0, 0);
+            const unsigned int mask = (unsigned int)bm.y;
+            const double* m = a.t.mom + (size_t)bm.x * kMom;
+            const double c[3] = {m[MC], m[MC + 1], m[MC + 2]};
+            const double M = m[MM], D[3] = {m[MD], m[MD + 1], m[MD + 2]};
+            const double Q[6] = {m[MQ], m[MQ + 1], m[MQ + 2], m[MQ + 3], m[MQ + 4], m[MQ + 5]};
+            const double T = m[MT];                       // -tr(Q)/2
+            double al[3] = {0, 0, 0}, ga[6] = {0, 0, 0, 0, 0, 0}, ka[3] = {0, 0, 0}, tr = 0.0;
+#pragma unroll 1
+            for (int g = 0; g < nt; ++g) {
+                if (!((mask >> g) & 1u)) continue;
+                const double R[3] = {W.tgt[g][0] - c[0], W.tgt[g][1] - c[1], W.tgt[g][2] - c[2]};
+                const double w[3] = {W.tgt[g][3], W.tgt[g][4], W.tgt[g][5]};
+                const double gi = rsqrt(dot3(R, R) + a.eps2);
+                const double u = gi * gi, g3 = gi * u, g5 = g3 * u, g7 = g5 * u, g9 = g7 * u;
+                const double rw = dot3(R, w), rd = dot3(R, D), wd = dot3(w, D);
+                double q[3], qw[3];
+                qmul(Q, R, q);
+                qmul(Q, w, qw);
+                const double rqr = dot3(R, q), wqr = dot3(w, q);
+                const double p5 = 3.0 * (g5 * rw), p7 = 15.0 * (g7 * rw), g53 = 3.0 * g5;
+                // k = 1/2 T4(w) = kr R - p7 q + kw w + 3 g^5 Q w
+                const double kw = -(7.5 * (g7 * rqr) + g53 * T);
+                const double kr = 52.5 * (g9 * rw) * rqr - 15.0 * (g7 * wqr) + p7 * T;
+                const double aR = g53 * (M * rw - wd) + p7 * rd;
+                const double aw = -(M * g3 + g53 * rd);
+                const double h7 = 0.5 * p7;
+                double b[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const double kk = kr * R[k] + (kw * w[k] + (g53 * qw[k] - p7 * q[k]));
+                    ka[k] += kk;
+                    W.mt[g][k][lane] -= aR * R[k] + (aw * w[k] + (kk - p5 * D[k]));
+                    al[k] += p5 * R[k] - g3 * w[k];
+                    b[k] = g53 * w[k] - h7 * R[k];
                 }
+                tr += p5;
+                ga[0] += b[0] * R[0];
+                ga[1] += b[0] * R[1] + b[1] * R[0];
+                ga[2] += b[0] * R[2] + b[2] * R[0];
+                ga[3] += b[1] * R[1];
+                ga[4] += b[1] * R[2] + b[2] * R[1];
+                ga[5] += b[2] * R[2];
             }
-            npl = 0;
+            if (mask) {
+                double* d = adj + (size_t)bm.x * 12;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    atomicAdd(d + k, al[k]);
+                    atomicAdd(d + 9 + k, ka[k]);
+                }
+                atomicAdd(d + 3, 2.0 * ga[0] + tr);
+                atomicAdd(d + 4, ga[1]);
+                atomicAdd(d + 5, ga[2]);
+                atomicAdd(d + 6, 2.0 * ga[3] + tr);
+                atomicAdd(d + 7, ga[4]);
+                atomicAdd(d + 8, 2.0 * ga[5] + tr);
+            }
             __syncwarp();
         };
 
-        int node = root;
-        while (node < end) {
-            const double* m = mom + (size_t)node * kMom;
-            const int4 inf = info[node];
-            const bool leaf = (dlf[node] & 256) != 0;
-            const bool active = node >= skip;
-            double dx = __dsub_rn(xt, m[0]);
-            double dy = __dsub_rn(yt, m[1]);
-            double dz = __dsub_rn(zt, m[2]);
-            double d2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                                  __dmul_rn(dz, dz));
-            const bool acc = active && (m[MR2] < d2);
-            const bool opn = active && !acc;
-            const unsigned int am = __ballot_sync(0xffffffffu, acc);
-            const unsigned int om = __ballot_sync(0xffffffffu, opn);
-            int next = inf.z;
-            if (om) {
-                if (leaf) {
-                    if (lane == 0) {
-                        lst.leaf[npl] = node;
-                        lst.mask[npl] = om;
-                    }
-                    ++npl;
-                } else {
-                    if (acc) skip = inf.z;
-                    next = node + 1;
+        auto direct_pairs = [&](const int2* leaves, int cnt) {
+            const LeafRun run(a, leaves, cnt);
+            for (int base = 0; base < run.total; base += 32) {
+                int j, nd;
+                unsigned int mask;
+                run.at(base + lane, j, nd, mask);
+                double xj = 0.0, yj = 0.0, zj = 0.0, qj = 0.0;
+                if (mask) {
+                    xj = a.x[j];
+                    yj = a.y[j];
+                    zj = a.z[j];
+                    qj = a.sp[j] ? q1 : q0;
                 }
-            }
-            if (am) {
-                double src[12];
+                double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+                for (int g = 0; g < nt; ++g) {
+                    if (!((mask >> g) & 1u) || W.slot[g] == j) continue;
+                    const double R[3] = {W.tgt[g][0] - xj, W.tgt[g][1] - yj, W.tgt[g][2] - zj};
+                    const double w[3] = {W.tgt[g][3], W.tgt[g][4], W.tgt[g][5]};
+                    const double gi = rsqrt(dot3(R, R) + a.eps2);
+                    const double u = gi * gi, cw = qj * (gi * u);
+                    const double cr = -3.0 * (cw * u) * dot3(R, w);
 #pragma unroll
-                for (int k = 0; k < 12; ++k) src[k] = 0.0;
-                if (acc) {
-                    const double R[3] = {dx, dy, dz};
-                    const double M = m[MM];
-                    const double D[3] = {m[MD], m[MD + 1], m[MD + 2]};
-                    const double Q[6] = {m[MQ], m[MQ + 1], m[MQ + 2], m[MQ + 3], m[MQ + 4], m[MQ + 5]};
-                    const double g = rsqrt(d2 + a.eps2);
-                    const double g2 = g * g, g3 = g2 * g, g5 = g3 * g2, g7 = g5 * g2;
-                    const double Rl = dot3(R, l), RD = dot3(R, D), lD = dot3(l, D);
-                    double T4l[3];
-                    t4(R, l, Q, g, T4l);
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        double hess = M * (3.0 * R[c] * Rl * g5 - l[c] * g3);
-                        double dterm = -15.0 * R[c] * Rl * RD * g7 +
-                                       3.0 * (l[c] * RD + D[c] * Rl + R[c] * lD) * g5;
-                        mt[c] -= qm * (hess - dterm + 0.5 * T4l[c]);
-                    }
-                    const double Rw = dot3(R, wv);
-                    double T4w[3];
-                    t4(R, wv, Q, g, T4w);
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        src[c] = 3.0 * R[c] * Rw * g5 - wv[c] * g3;   // alpha
-                        src[9 + c] = 0.5 * T4w[c];                     // kappa
-                    }
-                    const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) {
-                        const int e = ia[k], c = ib[k];
-                        src[3 + k] = -15.0 * Rw * R[e] * R[c] * g7 +
-                                     3.0 * (wv[e] * R[c] + wv[c] * R[e] + (e == c ? Rw : 0.0)) * g5;
+                    for (int k = 0; k < 3; ++k) {
+                        const double tv = cr * R[k] + cw * w[k];
+                        s[k] -= tv;
+                        W.mt[g][k][lane] += tv;
                     }
                 }
+                if (mask)
 #pragma unroll
-                for (int k = 0; k < 12; ++k) src[k] = wsum(src[k]);
-                if (lane == 0)
-                    for (int k = 0; k < 12; ++k) atomicAdd(&adj[(size_t)node * 12 + k], src[k]);
+                    for (int k = 0; k < 3; ++k) atomicAdd(&mu[3 * (size_t)j + k], s[k]);
             }
-            node = next;
-            if (npl == kAdjList) flush();
+            __syncwarp();
+        };
+
+        walk_lists(a, W.walk, tg, ck.z, multipoles, direct_pairs);
+
+        for (int v = lane; v < 3 * nt; v += 32) {
+            // the lanes' partial sums of one component, in lane order
+            const double* p = W.mt[v / 3][v % 3];
+            double sum = 0.0;
+            for (int k = 0; k < 32; ++k) sum += p[(k + lane) & 31];
+            atomicAdd(&mu[3 * (size_t)W.slot[v / 3] + v % 3], sum);
         }
-        flush();
-        if (valid) {
-            atomicAdd(&mu[3 * (size_t)t], mt[0]);
-            atomicAdd(&mu[3 * (size_t)t + 1], mt[1]);
-            atomicAdd(&mu[3 * (size_t)t + 2], mt[2]);
-        }
+        __syncwarp();
     }
 }
 
-// ---- FP32 form (FP32C contexts): the node-relative coordinates, records and
-// borderline FP64 decisions of the FP32C walk; per-lane sums in FP32, the
-// scatter into mu in FP64, the box accumulators in FP32.
+// ---- FP32 form (FP32C contexts): one warp per chunk of up to 32 targets, the
+// traversal of the FP32C walk (the same decisions).  Both parts of the derivative
+// run with the lanes over the sources: 32 accepted boxes, or 32 particles of opened
+// leaves, one per lane, against the chunk's targets two at a time in packed FP32x2.
+// A lane then holds its source's own sums (12 box terms, or 3 components) in
+// registers and adds them to memory once per batch; the targets' sums are three
+// values per target summed over the lanes by halving exchanges, four targets at a
+// time.  All terms are linear in the target's weight w = (q/m) lambda.  A pair's
+// separation is formed from the leaf's centroid and the particle's offset, as in the
+// forward walks.
+//
+// What bounds it: the FP32 pipe (63 % busy), by the box part's 113 packed operations
+// per box and pair of targets.  The form before took the lanes over targets and summed
+// each box's 12 values over the warp (70 instructions beside 110 of arithmetic,
+// unpacked) and each pair's three: 6.1 ms over every particle at N = 262,144 against
+// 3.1, over the electrons 4.1 against 1.95.
 
-// Warp sums of several values at once by halving exchanges: at each xor step a
-// lane keeps half of its values and adds the partner's copy of that half, so 16
-// values take 16 exchanges instead of 80 (4 values: 6 instead of 20), and the
-// sums end up spread over the lanes.
-// 16 values: lane L ends with value 8 b4 + 4 b3 + 2 b2 + b1 (b_k = bit k of L)
+// Warp sums of 16 values by halving exchanges: at each xor step a lane keeps half of
+// its values and adds the partner's copy of that half, so 16 values take 16
+// exchanges instead of 80; lane L ends with value L / 2 (both lanes of a pair).
 __device__ __forceinline__ float warp_sum16(float (&v)[16], int lane)
 {
 #pragma unroll
@@ -262,239 +255,258 @@ __device__ __forceinline__ float warp_sum16(float (&v)[16], int lane)
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-// 4 values: lane L ends with value 2 b4 + b3
-__device__ __forceinline__ float warp_sum4(float (&v)[4], int lane)
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 dot2(const float2* a, const float2* b)
 {
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const bool hi = (lane & 16) != 0;
-        const float keep = hi ? v[i + 2] : v[i], send = hi ? v[i] : v[i + 2];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-    {
-        const bool hi = (lane & 8) != 0;
-        const float keep = hi ? v[1] : v[0], send = hi ? v[0] : v[1];
-        v[0] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    float r = v[0];
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-    return r;
+    return fma2(a[0], b[0], fma2(a[1], b[1], mul2(a[2], b[2])));
 }
 
-__device__ __forceinline__ float dot3f(const float* a, const float* b)
+// four floats added to 16-byte aligned memory
+__device__ __forceinline__ void red_add4(float* p, float x, float y, float z, float w)
 {
-    return fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2]));
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};"
+                 :: "l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
-__device__ __forceinline__ void qmulf(const float* Q, const float* v, float* o)
-{
-    o[0] = fmaf(Q[0], v[0], fmaf(Q[1], v[1], Q[2] * v[2]));
-    o[1] = fmaf(Q[1], v[0], fmaf(Q[3], v[1], Q[4] * v[2]));
-    o[2] = fmaf(Q[2], v[0], fmaf(Q[4], v[1], Q[5] * v[2]));
-}
+struct __align__(16) AdjWarp {
+    WalkWarp walk;
+    // two targets: relative to the chunk's centre and weights {x, y}, {z, wx}, {wy, wz};
+    // relative to the cube's centre as float pairs {xh, yh}, {zh, xl}, {yl, zl}
+    float4 tgt[16][6];
+    float mt[8][32];         // four targets' sums: lane L holds value L / 2
+    int slot[32];            // the targets' slots
+};
 
-// The fourth-derivative term of the expansion contracted with a vector v:
-//   o_a = 105 R_a (R.v)(R.Q.R) g^9 - 15 g^7 (v_a R.Q.R + 2 (R.v)(QR)_a + 2 R_a v.QR
-//         + R_a (R.v) tr Q) + 3 g^5 (v_a tr Q + 2 (Qv)_a),
-// collected as coefficients of R_a, (QR)_a, v_a and (Qv)_a.  It is linear in v:
-// the source side's weight w = (q/m) lambda takes it as q/m times lambda's.
-__device__ __forceinline__ void t4f(const float* R, const float* v, const float* Q, float g5,
-                                    float g7, float g9, float Rv, float* o)
-{
-    float QR[3], Qv[3];
-    qmulf(Q, R, QR);
-    qmulf(Q, v, Qv);
-    const float RQR = dot3f(R, QR), trQ = Q[0] + Q[3] + Q[5];
-    const float cv = 3.f * g5 * trQ - 15.f * g7 * RQR;
-    const float cqv = 6.f * g5;
-    const float vQR = dot3f(v, QR);
-    const float cr = 105.f * Rv * RQR * g9 - 15.f * g7 * (2.f * vQR + Rv * trQ);
-    const float cq = -30.f * g7 * Rv;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) o[a] = fmaf(cr, R[a], fmaf(cq, QR[a], fmaf(cv, v[a], cqv * Qv[a])));
-}
-
-// 8 blocks of 128 per SM (64 registers): more resident warps for this issue-bound
-// walk than the compiler's own choice, without spills
-__global__ void __launch_bounds__(kAdjThreads, 8)
+__global__ void __launch_bounds__(32, 16)
 k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restrict__ mu,
                    float* __restrict__ adj)
 {
-    __shared__ AdjList Ls[kAdjWarps];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    AdjList& lst = Ls[w];
+    __shared__ AdjWarp shared;
+    AdjWarp& W = shared;
+    const int lane = threadIdx.x;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const float4* __restrict__ H = a.t.hdr;
-    const float4* __restrict__ LO = a.t.lo;
     const float4* __restrict__ S = a.src32;
-    const float eps2 = (float)a.eps2;
+    const float2 e2 = splat((float)a.eps2);
 
-    for (int chunk = 0; true;) {
-        if (lane == 0) chunk = atomicAdd(a.work, 1);
-        chunk = __shfl_sync(0xffffffffu, chunk, 0);
-        if (chunk >= a.nchunks) break;
+    for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
+         chunk = next_chunk(a.work, lane)) {
         const int4 ck = a.chunks[chunk];
-        const bool valid = lane < ck.y;
-        const int t = valid ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
-        const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
-        const int end = __float_as_int(LO[root].w);
-        float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
-        float l[3] = {0.f, 0.f, 0.f};
-        float qm = 0.f;
-        if (valid) {
-            // relative to the centre of the cloud's cube, as the box records are
-            const double* cc = a.cubes[ck.z].c;
-            double X = a.x[t] - cc[0], Y = a.y[t] - cc[1], Z = a.z[t] - cc[2];
-            xh = (float)X; yh = (float)Y; zh = (float)Z;
-            xl = (float)(X - (double)xh); yl = (float)(Y - (double)yh); zl = (float)(Z - (double)zh);
-            l[0] = (float)lam[3 * (size_t)t];
-            l[1] = (float)lam[3 * (size_t)t + 1];
-            l[2] = (float)lam[3 * (size_t)t + 2];
-            const int s = a.sp[t];
-            qm = (float)((s ? q1 : q0) / a.msp[s]);
-        }
-        // the source side's weight is w = (q/m) lambda: every source-side term is
-        // q/m times the target side's form in lambda
-        float mt[3] = {0.f, 0.f, 0.f};
-        int skip = valid ? 0 : 0x7fffffff;
-        int npl = 0;
-
-        auto flush = [&]() {
-            __syncwarp();
-            for (int e = 0; e < npl; ++e) {
-                const int nd = lst.leaf[e];
-                const bool in = (lst.mask[e] >> lane) & 1u;
-                const float4 A = H[nd], B = LO[nd];
-                const float rx = (xh + A.x) + (xl + B.x), ry = (yh + A.y) + (yl + B.y),
-                            rz = (zh + A.z) + (zl + B.z);
-                const int jb = __ldg(&a.t.info[nd].x), je = __ldg(&a.t.info[nd].y);
-                for (int j = jb; j < je; ++j) {
-                    const float4 P = __ldg(S + (j & ~1)), Q = __ldg(S + (j & ~1) + 1);
-                    const bool odd = j & 1;
-                    float sx = 0.f, sy = 0.f, sz = 0.f;
-                    const float qj = odd ? Q.w : Q.z;
-                    if (in && j != t) {
-                        float r3[3] = {rx + (odd ? P.y : P.x), ry + (odd ? P.w : P.z),
-                                       rz + (odd ? Q.y : Q.x)};
-                        float g = rsqrt_ftz(dot3f(r3, r3) + eps2);
-                        float g3 = g * g * g, g5 = g3 * g * g;
-                        const float rl = dot3f(r3, l), qq = qm * qj;
-                        // the pair's term on the target; the source takes its negative
-                        const float cl = qq * g3, cr = -3.f * qq * rl * g5;
-                        float tv[3];
+        const int t = lane < ck.y ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
+        const ChunkTarget tg(a, t, ck.z);
+        {
+            float w[3] = {0.f, 0.f, 0.f};
+            if (t >= 0) {
+                const int s = a.sp[t];
+                const double qm = (s ? q1 : q0) / a.msp[s];
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            tv[c] = fmaf(cl, l[c], cr * r3[c]);
-                            mt[c] += tv[c];
-                        }
-                        sx = -tv[0];
-                        sy = -tv[1];
-                        sz = -tv[2];
-                    }
-                    float sv[4] = {sx, sy, sz, 0.f};
-                    const float tot = warp_sum4(sv, lane);
-                    const int comp = ((lane >> 4) & 1) * 2 + ((lane >> 3) & 1);
-                    if ((lane & 7) == 0 && comp < 3)
-                        atomicAdd(&mu[3 * (size_t)j + comp], (double)tot);
-                }
+                for (int k = 0; k < 3; ++k) w[k] = (float)(qm * lam[3 * (size_t)t + k]);
             }
-            npl = 0;
+            float* d = reinterpret_cast<float*>(W.tgt[lane >> 1]) + (lane & 1);
+            d[0] = (tg.xh - tg.gx) + tg.xl;
+            d[2] = (tg.yh - tg.gy) + tg.yl;
+            d[4] = (tg.zh - tg.gz) + tg.zl;
+            d[6] = w[0];
+            d[8] = w[1];
+            d[10] = w[2];
+            d[12] = tg.xh;
+            d[14] = tg.yh;
+            d[16] = tg.zh;
+            d[18] = tg.xl;
+            d[20] = tg.yl;
+            d[22] = tg.zl;
+            W.slot[lane] = t >= 0 ? t : 0x7fffffff;
+#pragma unroll
+            for (int g = 0; g < 8; ++g) W.mt[g][lane] = 0.f;
+            __syncwarp();
+        }
+        const int groups = (ck.y + 3) >> 2;
+
+        // Accepted boxes, one per lane.  With g = (R.R + eps^2)^-1/2 and every l replaced
+        // by w:  H = aR R + al w + aD D + k,  k = 1/2 T4(w),
+        //   aR = 3 g^5 (M R.w - w.D) + 15 g^7 (R.w)(R.D),  al = -(M g^3 + 3 g^5 R.D),
+        //   aD = -3 g^5 R.w;
+        // the target takes -H; the box 3 g^5 (R.w) R - g^3 w (alpha), k (kappa) and
+        // b R^T + R b^T + 3 g^5 (R.w) I, b = 3 g^5 w - (15/2) g^7 (R.w) R (Gamma).
+        auto multipoles = [&](const int2* boxes, int cnt) {
+            const int2 bm = lane < cnt ? boxes[lane] : make_int2(0, 0);
+            const unsigned int mask = (unsigned int)bm.y;
+            const float4* r = a.t.rec + (size_t)bm.x * kRec;
+            const float4 r0 = __ldg(r), r1 = __ldg(r + 1), r2 = __ldg(r + 2), r3 = __ldg(r + 3),
+                         lo = __ldg(a.t.lo + bm.x);
+            const float2 cx = splat((r0.x + tg.gx) + lo.x), cy = splat((r0.y + tg.gy) + lo.y),
+                         cz = splat((r0.z + tg.gz) + lo.z);
+            const float2 M3 = splat(3.f * r0.w), nM = splat(-r0.w);
+            const float2 nD[3] = {splat(-3.f * r1.x), splat(-3.f * r1.y), splat(-3.f * r1.z)};
+            const float2 qxx = splat(r2.x), qxy = splat(r2.y), qxz = splat(r2.z), qyy = splat(r2.w),
+                         qyz = splat(r3.x), qzz = splat(r3.y);                 // Q / 2
+            const float2 t3 = splat(-3.f * r1.w), t15 = splat(15.f * r1.w);    // 3/2, -15/2 tr Q
+            float2 al[3], ga[6], ka[3], tr;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) al[k] = ka[k] = splat(0.f);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) ga[k] = splat(0.f);
+            tr = splat(0.f);
+#pragma unroll 1
+            for (int g4 = 0; g4 < groups; ++g4) {
+                float v[16];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4* T = W.tgt[2 * g4 + h];
+                    const float4 f0 = T[0], f1 = T[1], f2 = T[2];
+                    const float2 R[3] = {add2(cx, make_float2(f0.x, f0.y)),
+                                         add2(cy, make_float2(f0.z, f0.w)),
+                                         add2(cz, make_float2(f1.x, f1.y))};
+                    const float2 w[3] = {make_float2(f1.z, f1.w), make_float2(f2.x, f2.y),
+                                         make_float2(f2.z, f2.w)};
+                    const float2 rr = fma2(R[0], R[0], fma2(R[1], R[1], fma2(R[2], R[2], e2)));
+                    const unsigned int in = mask >> (4 * g4 + 2 * h);
+                    const float2 g = make_float2((in & 1u) ? rsqrt_ftz(rr.x) : 0.f,
+                                                 (in & 2u) ? rsqrt_ftz(rr.y) : 0.f);
+                    const float2 u = mul2(g, g), g3 = mul2(g, u), g5 = mul2(g3, u),
+                                 g7 = mul2(g5, u), g9 = mul2(g7, u);
+                    const float2 rw = dot2(R, w), rd = dot2(R, nD), wd = dot2(w, nD);
+                    const float2 q[3] = {
+                        fma2(qxx, R[0], fma2(qxy, R[1], mul2(qxz, R[2]))),
+                        fma2(qxy, R[0], fma2(qyy, R[1], mul2(qyz, R[2]))),
+                        fma2(qxz, R[0], fma2(qyz, R[1], mul2(qzz, R[2])))};
+                    const float2 qw[3] = {
+                        fma2(qxx, w[0], fma2(qxy, w[1], mul2(qxz, w[2]))),
+                        fma2(qxy, w[0], fma2(qyy, w[1], mul2(qyz, w[2]))),
+                        fma2(qxz, w[0], fma2(qyz, w[1], mul2(qzz, w[2])))};
+                    const float2 rqr = dot2(R, q), wqr = dot2(w, q);
+                    const float2 p5 = mul2(g5, rw), p7 = mul2(g7, rw);
+                    // k = kr R + kq q + kw w + 6 g^5 (Q/2) w
+                    const float2 kw = fma2(g7, mul2(splat(-15.f), rqr), mul2(g5, t3));
+                    const float2 kr = fma2(mul2(splat(105.f), rqr), mul2(g9, rw),
+                                           fma2(g7, mul2(splat(-30.f), wqr), mul2(t15, p7)));
+                    const float2 kq = mul2(splat(-30.f), p7), k6 = mul2(splat(6.f), g5);
+                    const float2 aR = fma2(mul2(splat(-5.f), p7), rd, mul2(g5, fma2(M3, rw, wd)));
+                    const float2 aw = fma2(g5, rd, mul2(nM, g3));
+                    const float2 p53 = mul2(splat(3.f), p5), g53 = mul2(splat(3.f), g5),
+                                 ng3 = mul2(splat(-1.f), g3), p75 = mul2(splat(-7.5f), p7);
+                    float2 b[3];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const float2 kk = fma2(kr, R[k], fma2(kq, q[k], fma2(kw, w[k], mul2(k6, qw[k]))));
+                        const float2 hh = fma2(aR, R[k], fma2(aw, w[k], fma2(p5, nD[k], kk)));
+                        v[6 * h + k] = hh.x;
+                        v[6 * h + 3 + k] = hh.y;
+                        ka[k] = add2(ka[k], kk);
+                        al[k] = fma2(p53, R[k], fma2(ng3, w[k], al[k]));
+                        b[k] = fma2(g53, w[k], mul2(p75, R[k]));
+                    }
+                    tr = add2(tr, p53);
+                    ga[0] = fma2(b[0], R[0], ga[0]);
+                    ga[1] = fma2(b[0], R[1], fma2(b[1], R[0], ga[1]));
+                    ga[2] = fma2(b[0], R[2], fma2(b[2], R[0], ga[2]));
+                    ga[3] = fma2(b[1], R[1], ga[3]);
+                    ga[4] = fma2(b[1], R[2], fma2(b[2], R[1], ga[4]));
+                    ga[5] = fma2(b[2], R[2], ga[5]);
+                }
+                v[12] = v[13] = v[14] = v[15] = 0.f;
+                const float tot = warp_sum16(v, lane);
+                W.mt[g4][lane] -= tot;
+            }
+            if (mask) {
+                float* d = adj + (size_t)bm.x * 12;
+                const float T = tr.x + tr.y;
+                red_add4(d, al[0].x + al[0].y, al[1].x + al[1].y, al[2].x + al[2].y,
+                         2.f * (ga[0].x + ga[0].y) + T);
+                red_add4(d + 4, ga[1].x + ga[1].y, ga[2].x + ga[2].y,
+                         2.f * (ga[3].x + ga[3].y) + T, ga[4].x + ga[4].y);
+                red_add4(d + 8, 2.f * (ga[5].x + ga[5].y) + T, ka[0].x + ka[0].y,
+                         ka[1].x + ka[1].y, ka[2].x + ka[2].y);
+            }
             __syncwarp();
         };
 
-        int node = root;
-        while (node < end) {
-            const float4 A = H[node], B = LO[node];
-            const int nxt = __float_as_int(B.w);
-            const bool leaf = __float_as_int(A.w) < 0;
-            const float rc2 = fabsf(A.w);
-            const bool active = node >= skip;
-            const float R[3] = {(xh + A.x) + (xl + B.x), (yh + A.y) + (yl + B.y),
-                                (zh + A.z) + (zl + B.z)};
-            const float d2 = dot3f(R, R);
-            bool acc = active && (rc2 < d2);
-            if (active && fabsf(d2 - rc2) <= 4e-6f * d2) {
-                const double* m = a.t.mom + (size_t)node * kMom;
-                double dx = __dsub_rn(a.x[t], m[0]), dy = __dsub_rn(a.y[t], m[1]),
-                       dz = __dsub_rn(a.z[t], m[2]);
-                acc = m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)),
-                                         __dmul_rn(dz, dz));
-            }
-            const bool opn = active && !acc;
-            const unsigned int am = __ballot_sync(0xffffffffu, acc);
-            const unsigned int om = __ballot_sync(0xffffffffu, opn);
-            int next = nxt;
-            if (om) {
-                if (leaf) {
-                    if (lane == 0) {
-                        lst.leaf[npl] = node;
-                        lst.mask[npl] = om;
-                    }
-                    ++npl;
-                } else {
-                    if (acc) skip = nxt;
-                    next = node + 1;
+        // Opened leaves: their particles in one run over the lanes.  A pair's term on
+        // the target is q_j (g^3 w - 3 g^5 (r.w) r); the source takes its negative.
+        auto direct_pairs = [&](const int2* leaves, int cnt) {
+            const LeafRun run(a, leaves, cnt);
+            for (int base = 0; base < run.total; base += 32) {
+                int j, nd;
+                unsigned int mask;
+                run.at(base + lane, j, nd, mask);
+                float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A;
+                float nx = 0.f, ny = 0.f, nz = 0.f, qj = 0.f;
+                if (mask) {
+                    // r = (x_t - c_leaf) + (c_leaf - x_j), the first from float pairs
+                    A = __ldg(a.t.hdr + nd);
+                    B = __ldg(a.t.lo + nd);
+                    const float4 P = __ldg(S + (j & ~1)), Q = __ldg(S + (j | 1));
+                    const bool odd = j & 1;
+                    nx = odd ? P.y : P.x;
+                    ny = odd ? P.w : P.z;
+                    nz = odd ? Q.y : Q.x;
+                    qj = odd ? Q.w : Q.z;
+                    // the particle's own place among the targets, if it has one
+                    int pos = 0;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1)
+                        if (W.slot[pos + o - 1] < j) pos += o;
+                    if (W.slot[pos] == j) mask &= ~(1u << pos);
                 }
-            }
-            if (am) {
-                float src[12];
+                const float2 cx = splat(A.x), cy = splat(A.y), cz = splat(A.z);
+                const float2 lx = splat(B.x), ly = splat(B.y), lz = splat(B.z);
+                const float2 px = splat(nx), py = splat(ny), pz = splat(nz);
+                const float2 q2 = splat(qj), nq3 = splat(-3.f * qj);
+                float2 s3[3] = {splat(0.f), splat(0.f), splat(0.f)};
+#pragma unroll 1
+                for (int g4 = 0; g4 < groups; ++g4) {
+                    float v[16];
 #pragma unroll
-                for (int k = 0; k < 12; ++k) src[k] = 0.f;
-                if (acc) {
-                    const float4* r = a.t.rec + (size_t)node * kRec;
-                    const float4 C4 = r[1], D4 = r[2], E4 = r[3];
-                    const float M = r[0].w;
-                    const float D[3] = {C4.x, C4.y, C4.z};
-                    const float Q[6] = {2.f * D4.x, 2.f * D4.y, 2.f * D4.z,
-                                        2.f * D4.w, 2.f * E4.x, 2.f * E4.y};
-                    const float g = rsqrt_ftz(d2 + eps2);
-                    const float g2 = g * g, g3 = g2 * g, g5 = g3 * g2, g7 = g5 * g2, g9 = g7 * g2;
-                    const float Rl = dot3f(R, l), RD = dot3f(R, D), lD = dot3f(l, D);
-                    float T4l[3];
-                    t4f(R, l, Q, g5, g7, g9, Rl, T4l);
-                    // monopole Hessian M (3 R (R.l) g^5 - l g^3) minus the dipole term
-                    // -15 R (R.l)(R.D) g^7 + 3 (l (R.D) + D (R.l) + R (l.D)) g^5,
-                    // collected as coefficients of R, l and D
-                    const float aR = 3.f * g5 * (M * Rl - lD) + 15.f * g7 * Rl * RD;
-                    const float al = -(M * g3 + 3.f * g5 * RD);
-                    const float aD = -3.f * g5 * Rl;
+                    for (int h = 0; h < 2; ++h) {
+                        const float4* T = W.tgt[2 * g4 + h];
+                        const float4 f1 = T[1], f2 = T[2], f3 = T[3], f4 = T[4], f5 = T[5];
+                        const float2 R[3] = {
+                            add2(add2(add2(cx, make_float2(f3.x, f3.y)),
+                                      add2(lx, make_float2(f4.z, f4.w))), px),
+                            add2(add2(add2(cy, make_float2(f3.z, f3.w)),
+                                      add2(ly, make_float2(f5.x, f5.y))), py),
+                            add2(add2(add2(cz, make_float2(f4.x, f4.y)),
+                                      add2(lz, make_float2(f5.z, f5.w))), pz)};
+                        const float2 w[3] = {make_float2(f1.z, f1.w), make_float2(f2.x, f2.y),
+                                             make_float2(f2.z, f2.w)};
+                        const float2 rr = fma2(R[0], R[0], fma2(R[1], R[1], fma2(R[2], R[2], e2)));
+                        const unsigned int in = mask >> (4 * g4 + 2 * h);
+                        const float2 g = make_float2((in & 1u) ? rsqrt_ftz(rr.x) : 0.f,
+                                                     (in & 2u) ? rsqrt_ftz(rr.y) : 0.f);
+                        const float2 u = mul2(g, g), g3 = mul2(g, u), g5 = mul2(g3, u);
+                        const float2 cr = mul2(mul2(nq3, g5), dot2(R, w)), cw = mul2(q2, g3);
 #pragma unroll
-                    for (int c = 0; c < 3; ++c)
-                        mt[c] -= qm * fmaf(aR, R[c], fmaf(al, l[c], fmaf(aD, D[c], 0.5f * T4l[c])));
-                    // source side in w = (q/m) lambda: q/m times the lambda forms
-                    const float Rw = qm * Rl, w5 = 3.f * qm * g5, w3 = qm * g3, hq = 0.5f * qm;
-#pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        src[c] = fmaf(3.f * Rw * g5, R[c], -w3 * l[c]);
-                        src[9 + c] = hq * T4l[c];
+                        for (int k = 0; k < 3; ++k) {
+                            const float2 tv = fma2(cr, R[k], mul2(cw, w[k]));
+                            v[6 * h + k] = tv.x;
+                            v[6 * h + 3 + k] = tv.y;
+                            s3[k] = add2(s3[k], tv);
+                        }
                     }
-                    const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-                    const float r7 = -15.f * Rw * g7;
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) {
-                        const int e = ia[k], c = ib[k];
-                        src[3 + k] = fmaf(r7 * R[e], R[c],
-                                          w5 * (l[e] * R[c] + l[c] * R[e] + (e == c ? Rl : 0.f)));
-                    }
+                    v[12] = v[13] = v[14] = v[15] = 0.f;
+                    const float tot = warp_sum16(v, lane);
+                    W.mt[g4][lane] += tot;
                 }
-                float sv[16];
+                if (mask)
 #pragma unroll
-                for (int k = 0; k < 16; ++k) sv[k] = k < 12 ? src[k] : 0.f;
-                const float tot = warp_sum16(sv, lane);
-                const int term = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 +
-                                 ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-                if ((lane & 1) == 0 && term < 12) atomicAdd(&adj[(size_t)node * 12 + term], tot);
+                    for (int k = 0; k < 3; ++k)
+                        atomicAdd(&mu[3 * (size_t)j + k], -(double)(s3[k].x + s3[k].y));
             }
-            node = next;
-            if (npl == kAdjList) flush();
-        }
-        flush();
-        if (valid) {
-            atomicAdd(&mu[3 * (size_t)t], (double)mt[0]);
-            atomicAdd(&mu[3 * (size_t)t + 1], (double)mt[1]);
-            atomicAdd(&mu[3 * (size_t)t + 2], (double)mt[2]);
-        }
+            __syncwarp();
+        };
+
+        walk_lists(a, W.walk, tg, ck.z, multipoles, direct_pairs);
+
+        // value L / 2 of a group: components of target (L / 2) / 3 of its four
+        const int term = lane >> 1;
+        if ((lane & 1) == 0 && term < 12)
+            for (int g4 = 0; g4 < groups; ++g4) {
+                const int k = 4 * g4 + term / 3;
+                if (k < ck.y)
+                    atomicAdd(&mu[3 * (size_t)W.slot[k] + term % 3], (double)W.mt[g4][lane]);
+            }
+        __syncwarp();
     }
 }
 
@@ -588,15 +600,19 @@ __global__ void k_axpy3(double* __restrict__ y, const double* __restrict__ x, do
     y[i] += a * x[i];
 }
 
-// lam_v = m_e v on electrons, 0 on ions; loss = sum 1/2 m_e v^2 (deterministic: one block)
-__global__ void k_ke_seed(const double* __restrict__ v, const int8_t* __restrict__ sp, int n,
-                          double me, double* __restrict__ lam_v, double* __restrict__ loss)
+// lam_v = m_e v on electrons, 0 on ions; part = the blocks' sums of 1/2 m_e v^2, added
+// in block order by the second kernel (deterministic)
+constexpr int kSeedBlocks = 304;
+
+__global__ void __launch_bounds__(256)
+k_ke_seed(const double* __restrict__ v, const int8_t* __restrict__ sp, int n, double me,
+          double* __restrict__ lam_v, double* __restrict__ part)
 {
     double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        bool e = sp[i] != 0;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+        const bool e = sp[i] != 0;
         for (int k = 0; k < 3; ++k) {
-            double vv = v[3 * (size_t)i + k];
+            const double vv = v[3 * (size_t)i + k];
             lam_v[3 * (size_t)i + k] = e ? me * vv : 0.0;
             if (e) acc += 0.5 * me * vv * vv;
         }
@@ -608,7 +624,29 @@ __global__ void k_ke_seed(const double* __restrict__ v, const int8_t* __restrict
         if ((int)threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *loss = sh[0];
+    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
+}
+
+__global__ void k_ke_sum(const double* __restrict__ part, int nblk, double* __restrict__ loss)
+{
+    const int lane = threadIdx.x;
+    double acc = 0.0;
+    for (int b = lane; b < nblk; b += 32) acc += part[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) *loss = acc;
+}
+
+// dst[id[t]] = src[t] for N x 3 arrays (key order -> caller order)
+__global__ void k_scatter_rows3(const double* __restrict__ src, const unsigned int* __restrict__ id,
+                                int n, double* __restrict__ dst)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const size_t j = id[t];
+    dst[3 * j] = src[3 * (size_t)t];
+    dst[3 * j + 1] = src[3 * (size_t)t + 1];
+    dst[3 * j + 2] = src[3 * (size_t)t + 2];
 }
 
 }  // namespace
@@ -639,11 +677,22 @@ void launch_axpy3(double* y, const double* x, double a, int n, cudaStream_t s)
     k_axpy3<<<(3 * n + 255) / 256, 256, 0, s>>>(y, x, a, n);
 }
 
+size_t ke_seed_words() { return 1 + kSeedBlocks; }
+
 void launch_ke_seed(const double* v, const int8_t* sp, int n, double me, double* lam_v,
                     double* loss, cudaStream_t s)
 {
+    count_launch(2);
+    const int b = n < 256 * kSeedBlocks ? (n + 255) / 256 : kSeedBlocks;
+    k_ke_seed<<<b, 256, 0, s>>>(v, sp, n, me, lam_v, loss + 1);
+    k_ke_sum<<<1, 32, 0, s>>>(loss + 1, b, loss);
+}
+
+void launch_scatter_rows3(const double* src, const unsigned int* id, int n, double* dst,
+                          cudaStream_t s)
+{
     count_launch(1);
-    k_ke_seed<<<1, 256, 0, s>>>(v, sp, n, me, lam_v, loss);
+    k_scatter_rows3<<<(n + 255) / 256, 256, 0, s>>>(src, id, n, dst);
 }
 
 void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, double* adj, int n,
@@ -652,19 +701,22 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
     count_launch(3);
     cudaMemsetAsync(a.work, 0, sizeof(int), s);
     cudaMemsetAsync(mu, 0, sizeof(double) * 3 * (size_t)n, s);
-    int blocks = nsm * 8;
-    int need = (a.nchunks + kAdjWarps - 1) / kAdjWarps;
-    if (blocks > need) blocks = need;
-    if (blocks < 1) blocks = 1;
     if (a.src32) {
+        int blocks = nsm * 16 < a.nchunks ? nsm * 16 : a.nchunks;
+        if (blocks < 1) blocks = 1;
         // FP32C context: FP32 walk, FP32 box accumulators (in the same buffer)
         float* adjf = reinterpret_cast<float*>(adj);
         k_zero_adj<float><<<2 * 152, 256, 0, s>>>(a.t.nnodes, adjf);
-        k_walk_adjoint_f32<<<blocks, kAdjThreads, 0, s>>>(a, lam, mu, adjf);
+        k_walk_adjoint_f32<<<blocks, 32, 0, s>>>(a, lam, mu, adjf);
         k_adjoint_push<float><<<4 * 152, 256, 0, s>>>(a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
     } else {
         k_zero_adj<double><<<2 * 152, 256, 0, s>>>(a.t.nnodes, adj);
-        k_walk_adjoint<<<blocks, kAdjThreads, 0, s>>>(a, lam, mu, adj);
+        // eight targets per warp, fewer while that leaves an SM with under four warps
+        int group = kAdjGroup;
+        while (group > 1 && (int64_t)a.nchunks * (32 / group) < 4 * (int64_t)nsm) group /= 2;
+        const int64_t items = (int64_t)a.nchunks * (32 / group);
+        const int blocks = items < 1 ? 1 : items < 12 * nsm ? (int)items : 12 * nsm;
+        k_walk_adjoint<<<blocks, 32, 0, s>>>(a, group, lam, mu, adj);
         k_adjoint_push<double><<<4 * 152, 256, 0, s>>>(a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
     }
 }

@@ -149,6 +149,7 @@ struct WalkArgs {
 void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, cudaStream_t s);
 void launch_walk_fp64(const WalkArgs& a, int nsm, cudaStream_t s);
 void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape);
+void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, cudaStream_t s);  // no potential
 int walk_shape_count();
 // Reorders a chunk list longest-first by the cost (20 per pair + 64 per multipole)
 // its targets had in the walk just finished; cost and tmp hold nchunks entries.
@@ -166,6 +167,9 @@ void launch_scatter_add3(const double* src, const unsigned int* id, int n, doubl
 void launch_kick_lambda(const double* lam_v, const int8_t* sp, int n, double ce, double ci,
                         double* out, cudaStream_t s);
 void launch_axpy3(double* y, const double* x, double a, int n, cudaStream_t s);
+void launch_scatter_rows3(const double* src, const unsigned int* id, int n, double* dst,
+                          cudaStream_t s);
+size_t ke_seed_words();  // doubles at loss: the sum and the blocks' partial sums
 void launch_ke_seed(const double* v, const int8_t* sp, int n, double me, double* lam_v,
                     double* loss, cudaStream_t s);
 

@@ -1,0 +1,253 @@
+// ucp_lists.cuh -- the traversal shared by the walks over 32 targets: which boxes
+// a chunk's targets accept and which leaves they open (Sec. 3, Eq. 5).
+#pragma once
+
+#include "ucp_internal.cuh"
+
+#include <math.h>
+
+namespace ucp {
+
+__device__ __forceinline__ int next_chunk(int* work, int lane)
+{
+    int c = 0;
+    if (lane == 0) c = atomicAdd(work, 1);
+    return __shfl_sync(0xffffffffu, c, 0);
+}
+
+// Twigs on the stack: up to kPopWide + 28 while four are popped per step; above
+// kPopWide one is popped per step, which adds at most 7 per level below it.
+constexpr int kPopWide = 64;
+constexpr int kStack = kPopWide + 28 + 7 * (kMaxDepth - 1) + 8;
+
+// Eq. 5 for a target and a box's record m in FP64, rounded like the definition
+static __device__ __noinline__ bool accepts_fp64(const double* m, const double* x, const double* y,
+                                          const double* z)
+{
+    const double dx = __dsub_rn(*x, m[0]);
+    const double dy = __dsub_rn(*y, m[1]);
+    const double dz = __dsub_rn(*z, m[2]);
+    return m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+
+constexpr int kStage = 32;           // accepted boxes evaluated per batch
+constexpr int kStageStride = 36;     // floats per staged pair of boxes (32 used; 16-byte aligned)
+
+struct __align__(16) WalkWarp {
+    float stage[kStage / 2 * kStageStride];
+    int2 stack[kStack];              // {twig, mask}
+    int2 acc[2 * kStage];            // {accepted box, mask}
+    int2 leaf[64];                   // {opened leaf, mask}
+};
+
+__device__ __forceinline__ float warp_min(float v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
+
+// One target of a chunk (t < 0: an idle lane) and the chunk's bounds.
+struct ChunkTarget {
+    int t;
+    // target as an unevaluated float pair x = xh + xl, relative to the centre of
+    // the cloud's cube like the box centroids, so that the FP32 errors scale with
+    // the cloud's size and not with its distance from the origin
+    float xh, yh, zh, xl, yl, zl;
+    // window of the FP32 criterion (see walk_lists): |dm| <= wa d2 + wb bounds the FP32
+    // error of d2 - rcrit2 for this target, given |x_t - xh| <= 2^-24 |x_t| and the
+    // same for the centroid
+    float wa, wb;
+    // bounding box of the chunk's targets (centre, half extents), and four times the
+    // widest window of its targets: the centre and extents are rounded too
+    float gx, gy, gz, ex, ey, ez, gwa, gwb;
+
+    __device__ __forceinline__ ChunkTarget(const WalkArgs& a, int t_, int cloud) : t(t_)
+    {
+        xh = yh = zh = xl = yl = zl = 0.f;
+        const bool valid = t >= 0;
+        if (valid) {
+            const double* cc = a.cubes[cloud].c;
+            const double X = a.x[t] - cc[0], Y = a.y[t] - cc[1], Z = a.z[t] - cc[2];
+            xh = (float)X; yh = (float)Y; zh = (float)Z;
+            xl = (float)(X - (double)xh); yl = (float)(Y - (double)yh); zl = (float)(Z - (double)zh);
+        }
+        const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
+        wa = fmaf(0.5f, bt, 4e-6f);
+        wb = 0.5f * bt;
+        const float xa = warp_min(valid ? xh : INFINITY), xb = -warp_min(valid ? -xh : INFINITY);
+        const float ya = warp_min(valid ? yh : INFINITY), yb = -warp_min(valid ? -yh : INFINITY);
+        const float za = warp_min(valid ? zh : INFINITY), zb = -warp_min(valid ? -zh : INFINITY);
+        gx = 0.5f * (xa + xb);
+        gy = 0.5f * (ya + yb);
+        gz = 0.5f * (za + zb);
+        ex = fmaxf(xb - gx, gx - xa);
+        ey = fmaxf(yb - gy, gy - ya);
+        ez = fmaxf(zb - gz, gz - za);
+        gwb = 4.f * -warp_min(-wb);
+        gwa = gwb + 1.6e-5f;
+    }
+};
+
+// Walks a chunk's targets, one per lane, through their cloud's tree with the lanes
+// over boxes: multipoles(list, cnt) takes cnt <= 32 accepted boxes {box, mask of the
+// targets that accept it}, pairs(list, cnt) cnt <= 32 opened leaves {leaf, mask of the
+// targets that open it}; both are called by the whole warp and may use W.stage.
+template <class M, class P>
+__device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const ChunkTarget& tg,
+                                           int cloud, M& multipoles, P& direct_pairs)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned int lt = (1u << lane) - 1u, me = 1u << lane;
+    int top = 0, na = 0, nl = 0;
+    // the first step tests the root for every target
+    int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[cloud] : 0] : -1;
+    unsigned int mask = __ballot_sync(0xffffffffu, tg.t >= 0);
+    while (true) {
+        const bool has = box >= 0;
+        const float4 h = has ? __ldg(a.t.hdr + box) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const bool leaf = __float_as_int(h.w) < 0;
+        const float rc2 = fabsf(h.w);
+        const float dx = fabsf(tg.gx + h.x), dy = fabsf(tg.gy + h.y), dz = fabsf(tg.gz + h.z);
+        const float nx = fmaxf(dx - tg.ex, 0.f), ny = fmaxf(dy - tg.ey, 0.f), nz = fmaxf(dz - tg.ez, 0.f);
+        const float fx = dx + tg.ex, fy = dy + tg.ey, fz = dz + tg.ez;
+        const float near2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
+        const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+        const bool all_acc = near2 - rc2 > fmaf(tg.gwa, near2, tg.gwb);
+        const bool all_opn = rc2 - far2 > fmaf(tg.gwa, far2, tg.gwb);
+        unsigned int am = has && all_acc ? mask : 0u;   // targets that accept the box
+        const bool some = has && !all_acc && !all_opn;
+        const unsigned int between = __ballot_sync(0xffffffffu, some);
+        if (between) {
+            // decided target by target, two boxes per packed operation: pairs of
+            // {-c} x, y, z, {-rcrit2}, {box, mask}, side by side
+            const int slot = some ? __popc(between & lt) : -1;
+            const int cnt = __popc(between);
+            if (some) {
+                float* d = W.stage + (slot >> 1) * 12 + (slot & 1);
+                d[0] = h.x;
+                d[2] = h.y;
+                d[4] = h.z;
+                d[6] = -rc2;
+                d[8] = __int_as_float(box);
+                d[10] = __int_as_float((int)mask);
+            }
+            if (lane == 0 && (cnt & 1)) {
+                float* d = W.stage + (cnt >> 1) * 12 + 1;
+                d[0] = d[2] = d[4] = d[6] = d[8] = d[10] = 0.f;
+            }
+            __syncwarp();
+            const float2 x2 = splat(tg.xh), y2 = splat(tg.yh), z2 = splat(tg.zh);
+            for (int p = 0; 2 * p < cnt; ++p) {
+                const float4* P = reinterpret_cast<const float4*>(W.stage + p * 12);
+                const float4 f0 = P[0], f1 = P[1], f2 = P[2];
+                const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
+                const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
+                const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
+                const float2 d2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+                const float2 dm = __fadd2_rn(d2, make_float2(f1.z, f1.w));
+                const float2 win = __ffma2_rn(splat(tg.wa), d2, splat(tg.wb));
+                const bool in0 = (__float_as_int(f2.z) & me) != 0;
+                const bool in1 = (__float_as_int(f2.w) & me) != 0;
+                bool acc0 = in0 && dm.x > 0.f, acc1 = in1 && dm.y > 0.f;
+                // Within the FP32 error of d2 - rcrit2 the decision is taken again in
+                // FP64 exactly as the FP64 walk takes it, so both precisions open the
+                // same boxes.  Per axis R is off by at most 2^-23 (|x_t| + |R|), so
+                // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
+                // included) with X_t the target's largest coordinate; with
+                // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
+                // a million at the bench size).
+                const bool again0 = in0 && fabsf(dm.x) <= win.x;
+                const bool again1 = in1 && fabsf(dm.y) <= win.y;
+                if (again0)
+                    acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + tg.t,
+                                        a.y + tg.t, a.z + tg.t);
+                if (again1)
+                    acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kMom, a.x + tg.t,
+                                        a.y + tg.t, a.z + tg.t);
+                const unsigned int am0 = __ballot_sync(0xffffffffu, acc0);
+                const unsigned int am1 = __ballot_sync(0xffffffffu, acc1);
+                if (slot == 2 * p) am = am0;
+                if (slot == 2 * p + 1) am = am1;
+            }
+            __syncwarp();
+        }
+        const unsigned int om = has ? mask & ~am : 0u;  // targets that open it
+        const unsigned int A = __ballot_sync(0xffffffffu, am != 0u);
+        const unsigned int OL = __ballot_sync(0xffffffffu, om != 0u && leaf);
+        const unsigned int OT = __ballot_sync(0xffffffffu, om != 0u && !leaf);
+        if (am) W.acc[na + __popc(A & lt)] = make_int2(box, (int)am);
+        if (om) {
+            if (leaf) W.leaf[nl + __popc(OL & lt)] = make_int2(box, (int)om);
+            else W.stack[top + __popc(OT & lt)] = make_int2(box, (int)om);
+        }
+        na += __popc(A);
+        nl += __popc(OL);
+        top += __popc(OT);
+        __syncwarp();
+        const bool done = top == 0;
+        while (na >= kStage || (done && na > 0)) {
+            const int cnt = min(na, kStage);
+            na -= cnt;
+            multipoles(W.acc + na, cnt);
+        }
+        while (nl >= 32 || (done && nl > 0)) {
+            const int cnt = min(nl, 32);
+            nl -= cnt;
+            direct_pairs(W.leaf + nl, cnt);
+        }
+        if (done) break;
+        const int pop = top > kPopWide ? 1 : min(top, 4);
+        box = -1;
+        mask = 0u;
+        if ((lane >> 3) < pop) {
+            const int2 e = W.stack[top - 1 - (lane >> 3)];
+            box = __ldg(a.t.child8 + (size_t)e.x * 8 + (lane & 7));
+            mask = (unsigned int)e.y;
+        }
+        top -= pop;
+        __syncwarp();
+    }
+}
+
+// The particles of up to 32 opened leaves {leaf, mask} as one run over the lanes.
+struct LeafRun {
+    int total, end, first;       // end: of this lane's leaf in the run; first: begin - start
+    int2 lm;
+
+    __device__ __forceinline__ LeafRun(const WalkArgs& a, const int2* leaves, int cnt)
+    {
+        const int lane = threadIdx.x & 31;
+        int2 be = make_int2(0, 0);
+        lm = make_int2(0, 0);
+        if (lane < cnt) {
+            lm = leaves[lane];
+            be = __ldg(reinterpret_cast<const int2*>(a.t.info + lm.x));
+        }
+        end = be.y - be.x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += v;
+        }
+        total = __shfl_sync(0xffffffffu, end, 31);
+        first = be.y - end;
+    }
+
+    // particle f of the run: its slot, its leaf and that leaf's mask (0 past the end)
+    __device__ __forceinline__ void at(int f, int& j, int& leaf, unsigned int& mask) const
+    {
+        int owner = 0;           // leaves that end at or before f
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, end, owner + o - 1) <= f) owner += o;
+        j = __shfl_sync(0xffffffffu, first, owner) + f;
+        leaf = __shfl_sync(0xffffffffu, lm.x, owner);
+        mask = (unsigned int)__shfl_sync(0xffffffffu, lm.y, owner);
+        if (f >= total) mask = 0u;
+    }
+};
+
+}  // namespace ucp

@@ -118,6 +118,10 @@ struct ucp_ctx {
     std::vector<Slot> slots;
     size_t slab_bytes = 0;
     void* slab = nullptr;
+    // working memory of the adjoint walks, allocated by the first call that needs it:
+    // 12 sums per box (FP64, or FP32 in FP32C contexts) and the walk's result, key order
+    double* adj = nullptr;
+    double* mu = nullptr;
 };
 
 namespace {
@@ -248,8 +252,11 @@ int build(ucp_ctx* c)
     return check_launch(c, "tree build");
 }
 
-// One walk over all particles (electrons_only = 0) or the electrons.
-int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_phi)
+// One walk over all particles (electrons_only = 0) or the electrons.  visits: in an
+// FP32C context, sums box by box in pre-order (forward runs of the gradient; no
+// potential).
+int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_phi,
+          bool visits = false)
 {
     int k = c->cur;
     int f32 = c->precision == UCP_FP32C;
@@ -293,7 +300,8 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
     cudaMemsetAsync(c->cnt_m2p, 0, sizeof(int) * (size_t)c->n, c->s);
     if (a.ntargets > 0) {
         prof_begin(c);
-        if (f32) launch_walk_fp32c(a, c->nsm, c->s, c->walk_shape);
+        if (f32 && visits) launch_walk_fp32c_visits(a, c->nsm, c->s);
+        else if (f32) launch_walk_fp32c(a, c->nsm, c->s, c->walk_shape);
         else launch_walk_fp64(a, c->nsm, c->s);
         prof_end(c);
         // the next walk over the same targets takes its chunks longest-first (the FP64
@@ -352,6 +360,20 @@ int device_error(ucp_ctx* c)
     return UCP_OK;
 }
 
+int adjoint_memory(ucp_ctx* c)
+{
+    if (c->adj) return UCP_OK;
+    const size_t box = 12 * (c->precision == UCP_FP32C ? sizeof(float) : sizeof(double));
+    const size_t sums = ((size_t)c->t.cap * box + 255) & ~(size_t)255;
+    if (cudaMalloc(&c->adj, sums + 3 * sizeof(double) * (size_t)c->n) != cudaSuccess) {
+        cudaGetLastError();
+        c->adj = nullptr;
+        return fail(c, UCP_ENOMEM, "adjoint working memory");
+    }
+    c->mu = reinterpret_cast<double*>(reinterpret_cast<char*>(c->adj) + sums);
+    return UCP_OK;
+}
+
 int valid_walk_args(ucp_ctx* c, double theta, double eps)
 {
     if (!(theta >= 0.0 && theta <= 1.0)) return fail(c, UCP_EINVAL, "theta must be in [0, 1]");
@@ -385,6 +407,7 @@ void ucp_destroy(ucp_ctx* c)
     if (c->s) cudaStreamSynchronize(c->s);
     else cudaDeviceSynchronize();
     if (c->slab) cudaFree(c->slab);
+    if (c->adj) cudaFree(c->adj);
     if (c->host_flags) cudaFreeHost(c->host_flags);
     for (auto& e : c->ev) {
         cudaEventDestroy(e.first);
@@ -700,14 +723,15 @@ int ucp_tree_force(ucp_ctx* c, double theta, double eps, double* acc, double* ph
 }
 
 // The split-step push; with store != NULL the positions after every electron
-// substep are written there in caller order (n x 3 doubles per substep).
+// substep are written there in caller order (n x 3 doubles per substep).  gradient:
+// a forward run of the gradient, whose potential nobody reads.
 static int run_blocks(ucp_ctx* c, double dt_e, int kk, int64_t nblocks, double theta, double eps,
-                      double* store)
+                      double* store, bool gradient = false)
 {
     int rc;
     if (!c->acc_valid) {
         if (!c->tree_valid && (rc = build(c))) return rc;
-        if ((rc = force(c, theta, eps, 0, false))) return rc;
+        if ((rc = force(c, theta, eps, 0, false, gradient))) return rc;
     }
     const double dt_i = (double)kk * dt_e;
     const double h_i = 0.5 * dt_i, h_e = 0.5 * dt_e;
@@ -726,7 +750,7 @@ static int run_blocks(ucp_ctx* c, double dt_e, int kk, int64_t nblocks, double t
                          c->st[k][5], dt_e, c->n, c->s);
             if ((rc = build(c))) return rc;
             // the walk over every particle also leaves phi for a following ucp_energy
-            if ((rc = force(c, theta, eps, sub < kk, sub == kk))) return rc;
+            if ((rc = force(c, theta, eps, sub < kk, sub == kk && !gradient, gradient))) return rc;
             pend_e = 1;
             if (store) {
                 k = c->cur;
@@ -994,17 +1018,17 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
     const int64_t nseg = (S + C - 1) / C;
     // working memory of this call: checkpoints, one segment of positions, lambdas
     double *ck = nullptr, *seg = nullptr, *lx = nullptr, *lv = nullptr, *lam = nullptr,
-           *lsorted = nullptr, *mu = nullptr, *adj = nullptr, *dloss = nullptr;
+           *lsorted = nullptr, *dloss = nullptr;
     auto freeall = [&]() {
-        for (double* p : {ck, seg, lx, lv, lam, lsorted, mu, adj, dloss})
+        for (double* p : {ck, seg, lx, lv, lam, lsorted, dloss})
             if (p) cudaFree(p);
     };
-    size_t adj_words = (size_t)c->t.cap * 12;
+    if ((rc = adjoint_memory(c))) return rc;
     if (cudaMalloc(&ck, sizeof(double) * n3 * 2 * (nseg + 1)) ||
         cudaMalloc(&seg, sizeof(double) * n3 * (C + 1)) || cudaMalloc(&lx, sizeof(double) * n3) ||
         cudaMalloc(&lv, sizeof(double) * n3) || cudaMalloc(&lam, sizeof(double) * n3) ||
-        cudaMalloc(&lsorted, sizeof(double) * n3) || cudaMalloc(&mu, sizeof(double) * n3) ||
-        cudaMalloc(&adj, sizeof(double) * adj_words) || cudaMalloc(&dloss, sizeof(double))) {
+        cudaMalloc(&lsorted, sizeof(double) * n3) ||
+        cudaMalloc(&dloss, sizeof(double) * ke_seed_words())) {
         cudaGetLastError();
         freeall();
         return fail(c, UCP_ENOMEM, "adjoint working memory");
@@ -1025,7 +1049,9 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
         if (last)
             cudaMemcpyAsync(seg, ck + 2 * n3 * sgi, sizeof(double) * n3, cudaMemcpyDeviceToDevice,
                             c->s);
-        if ((rc = run_blocks(c, dt_e, kk, len / kk, theta, eps, last ? seg + n3 : nullptr))) break;
+        if ((rc = run_blocks(c, dt_e, kk, len / kk, theta, eps, last ? seg + n3 : nullptr,
+                             true)))
+            break;
         snapshot(ck + 2 * n3 * (sgi + 1));
     }
     if (rc) {
@@ -1044,7 +1070,7 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
             load_state(c, ck + 2 * n3 * sgi, ck + 2 * n3 * sgi + n3);
             cudaMemcpyAsync(seg, ck + 2 * n3 * sgi, sizeof(double) * n3, cudaMemcpyDeviceToDevice,
                             c->s);
-            if ((rc = run_blocks(c, dt_e, kk, len / kk, theta, eps, seg + n3))) break;
+            if ((rc = run_blocks(c, dt_e, kk, len / kk, theta, eps, seg + n3, true))) break;
         }
         for (int64_t j = len; j >= (sgi == 0 ? 0 : 1); --j) {
             const int64_t g = g0 + j;
@@ -1090,8 +1116,8 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
             a.lambda = 1.0;
             a.work = c->work;
             a.err = c->sort.err;
-            launch_walk_adjoint(a, lsorted, mu, adj, c->n, c->nsm, c->s);
-            launch_scatter_add3(mu, c->id[k], c->n, lx, c->s);
+            launch_walk_adjoint(a, lsorted, c->mu, c->adj, c->n, c->nsm, c->s);
+            launch_scatter_add3(c->mu, c->id[k], c->n, lx, c->s);
             if (g > 0) launch_axpy3(lv, lx, dt_e, c->n, c->s);  // drift g
             if ((rc = check_launch(c, "adjoint"))) break;
         }
@@ -1126,32 +1152,15 @@ int ucp_accel_vjp(ucp_ctx* c, double theta, double eps, const double* lam_in, do
     int rc = valid_walk_args(c, theta, eps);
     if (rc) return rc;
     const size_t n3 = (size_t)3 * c->n;
-    double *lam = nullptr, *lsorted = nullptr, *mu = nullptr, *adj = nullptr, *out = nullptr;
-    auto freeall = [&]() {
-        for (double* p : {lam, lsorted, mu, adj, out})
-            if (p) cudaFree(p);
-    };
-    if (cudaMalloc(&lam, sizeof(double) * n3) || cudaMalloc(&lsorted, sizeof(double) * n3) ||
-        cudaMalloc(&mu, sizeof(double) * n3) || cudaMalloc(&out, sizeof(double) * n3) ||
-        cudaMalloc(&adj, sizeof(double) * (size_t)c->t.cap * 12)) {
-        cudaGetLastError();
-        freeall();
-        return fail(c, UCP_ENOMEM, "adjoint working memory");
-    }
-    cudaMemcpyKind kin = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (cudaMemcpyAsync(lam, lam_in, sizeof(double) * n3, kin, c->s) ||
-        cudaMemsetAsync(out, 0, sizeof(double) * n3, c->s)) {
-        freeall();
-        return fail(c, UCP_ECUDA, "adjoint input copy");
-    }
-    if (!c->tree_valid && (rc = build(c))) {
-        freeall();
-        return rc;
-    }
+    if ((rc = adjoint_memory(c))) return rc;
+    double* lsorted = c->stage + n3;
+    if (!on_device)
+        CK(cudaMemcpyAsync(c->stage, lam_in, sizeof(double) * n3, cudaMemcpyHostToDevice, c->s));
+    if (!c->tree_valid && (rc = build(c))) return rc;
     const int f32 = c->precision == UCP_FP32C;
     launch_mac_prepare(c->t, c->cube, theta, f32, c->s);
     const int k = c->cur;
-    launch_gather3(lam, c->id[k], c->n, lsorted, c->s);
+    launch_gather3(on_device ? lam_in : c->stage, c->id[k], c->n, lsorted, c->s);
     WalkArgs a;
     a.x = c->st[k][0];
     a.y = c->st[k][1];
@@ -1172,14 +1181,14 @@ int ucp_accel_vjp(ucp_ctx* c, double theta, double eps, const double* lam_in, do
     a.lambda = 1.0;
     a.work = c->work;
     a.err = c->sort.err;
-    launch_walk_adjoint(a, lsorted, mu, adj, c->n, c->nsm, c->s);
-    launch_scatter_add3(mu, c->id[k], c->n, out, c->s);
+    launch_walk_adjoint(a, lsorted, c->mu, c->adj, c->n, c->nsm, c->s);
+    double* dst = on_device ? mu_out : c->stage;
+    launch_scatter_rows3(c->mu, c->id[k], c->n, dst, c->s);
     rc = check_launch(c, "adjoint walk");
-    cudaMemcpyKind kout = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (!rc && cudaMemcpyAsync(mu_out, out, sizeof(double) * n3, kout, c->s))
+    if (!rc && !on_device &&
+        cudaMemcpyAsync(mu_out, dst, sizeof(double) * n3, cudaMemcpyDeviceToHost, c->s))
         rc = fail(c, UCP_ECUDA, "adjoint output copy");
-    cudaStreamSynchronize(c->s);
-    freeall();
+    if (cudaStreamSynchronize(c->s) && !rc) rc = fail(c, UCP_ECUDA, "adjoint walk");
     if (!rc) rc = device_error(c);
     return rc;
 }

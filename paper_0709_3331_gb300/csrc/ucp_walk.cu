@@ -8,20 +8,13 @@
 // key-consecutive targets per warp (k_walk_fp32c); each is described at its kernel.
 // In both, each target's sums are taken in a fixed order, so results do not depend
 // on scheduling.
-#include "ucp_internal.cuh"
+#include "ucp_lists.cuh"
 
 #include <math.h>
 
 namespace ucp {
 
 namespace {
-
-__device__ __forceinline__ int next_chunk(int* work, int lane)
-{
-    int c = 0;
-    if (lane == 0) c = atomicAdd(work, 1);
-    return __shfl_sync(0xffffffffu, c, 0);
-}
 
 // Error-free sum (Knuth's TwoSum) folded into a running correction.
 __device__ __forceinline__ void two_sum_acc(float& s, float& c, float v)
@@ -34,21 +27,6 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float v)
 }
 
 // ------------------------------------------------------------------ FP64
-// Twigs on the stack: up to kPopWide + 28 while four are popped per step; above
-// kPopWide one is popped per step, which adds at most 7 per level below it.
-constexpr int kPopWide = 64;
-constexpr int kStack = kPopWide + 28 + 7 * (kMaxDepth - 1) + 8;
-
-// Eq. 5 for a target and a box's record m in FP64, rounded like the definition
-__device__ __noinline__ bool accepts_fp64(const double* m, const double* x, const double* y,
-                                          const double* z)
-{
-    const double dx = __dsub_rn(*x, m[0]);
-    const double dy = __dsub_rn(*y, m[1]);
-    const double dz = __dsub_rn(*z, m[2]);
-    return m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-}
-
 // One warp walks one target; its lanes are boxes and sources.  A step of the
 // traversal pops up to four opened twigs from a stack and tests their children, one
 // per lane; accepted boxes and the particles of opened leaves wait in two lists and
@@ -311,23 +289,6 @@ __device__ __forceinline__ void kelbg_pg(float u, float& p, float& g)
 // per SM.  kPhi = false (walks whose potential nobody reads, e.g. the electron
 // substeps): the potential terms and their sums are left out; the field is computed
 // by the same operations in the same order, so accelerations are bit-identical.
-constexpr int kStage = 32;           // boxes evaluated per batch (pairs of two)
-constexpr int kStageStride = 36;     // floats per staged pair (32 used; 16-byte aligned)
-struct __align__(16) WalkWarp {
-    float stage[kStage / 2 * kStageStride];
-    int2 stack[kStack];              // {twig, mask}
-    int2 acc[2 * kStage];            // {accepted box, mask}
-    int2 leaf[64];                   // {opened leaf, mask}
-};
-
-__device__ __forceinline__ float warp_min(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-__device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
 
 template <bool kKelbg, int kThreads, int kBlocks, bool kPhi>
 __global__ void __launch_bounds__(kThreads, kBlocks)
@@ -336,7 +297,7 @@ k_walk_fp32c(WalkArgs a)
     __shared__ WalkWarp shared[kThreads / 32];
     const int lane = threadIdx.x & 31;
     WalkWarp& W = shared[threadIdx.x >> 5];
-    const unsigned int lt = (1u << lane) - 1u, me = 1u << lane;
+    const unsigned int me = 1u << lane;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
     const float4* __restrict__ H = a.t.hdr;
     const float4* __restrict__ S = a.src32;
@@ -348,48 +309,24 @@ k_walk_fp32c(WalkArgs a)
         const int ti = ck.x + lane;
         const bool valid = lane < ck.y;
         const int t = valid ? (a.targets ? a.targets[ti] : ti) : -1;
-        // target as an unevaluated float pair: x = xh + xl, relative to the centre of
-        // the cloud's cube like the box centroids, so that the FP32 errors scale with
-        // the cloud's size and not with its distance from the origin
-        float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
-        if (valid) {
-            const double* cc = a.cubes[ck.z].c;
-            double X = a.x[t] - cc[0], Y = a.y[t] - cc[1], Z = a.z[t] - cc[2];
-            xh = (float)X; yh = (float)Y; zh = (float)Z;
-            xl = (float)(X - (double)xh); yl = (float)(Y - (double)yh); zl = (float)(Z - (double)zh);
-        }
-        // Window of the FP32 criterion (see below): |dm| <= wa d2 + wb bounds the FP32
-        // error of d2 - rcrit2 for this target, given |x_t - xh| <= 2^-24 |x_t| and the
-        // same for the centroid
-        const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
-        const float wa = fmaf(0.5f, bt, 4e-6f), wb = 0.5f * bt;
-        // bounding box of the chunk's targets (centre, half extents), and four times the
-        // widest window of its targets: the centre and extents are rounded too
-        const float xa = warp_min(valid ? xh : INFINITY), xb = -warp_min(valid ? -xh : INFINITY);
-        const float ya = warp_min(valid ? yh : INFINITY), yb = -warp_min(valid ? -yh : INFINITY);
-        const float za = warp_min(valid ? zh : INFINITY), zb = -warp_min(valid ? -zh : INFINITY);
-        const float gx = 0.5f * (xa + xb), gy = 0.5f * (ya + yb), gz = 0.5f * (za + zb);
-        const float ex = fmaxf(xb - gx, gx - xa), ey = fmaxf(yb - gy, gy - ya),
-                    ez = fmaxf(zb - gz, gz - za);
-        const float gwb = 4.f * -warp_min(-wb), gwa = gwb + 1.6e-5f;
+        const ChunkTarget tg(a, t, ck.z);
+        const float xh = tg.xh, yh = tg.yh, zh = tg.zh, xl = tg.xl, yl = tg.yl, zl = tg.zl;
         const float qt = valid ? (a.sp[t] ? (float)q1 : (float)q0) : 0.f;
         const float inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
         const float inv_lambda3 = inv_lambda * inv_lambda * inv_lambda;
         // compensated totals (sum, correction)
         float sx = 0.f, sy = 0.f, sz = 0.f, sp = 0.f, cx = 0.f, cy = 0.f, cz = 0.f, cp = 0.f;
         int np = 0, nm = 0;
-        int top = 0, na = 0, nl = 0;
 
         // the last cnt <= 32 boxes of the list of accepted boxes
-        auto multipoles = [&](int cnt) {
-            na -= cnt;
+        auto multipoles = [&](const int2* boxes, int cnt) {
             const int part = lane & 3;
 #pragma unroll
             for (int it = 0; it < kStage / 8; ++it) {
                 const int e = it * 8 + (lane >> 2);
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (e < cnt) v = __ldg(a.t.rec + (size_t)W.acc[na + e].x * kRec + part);
-                if (part == 3) v.w = __int_as_float(e < cnt ? W.acc[na + e].y : 0);
+                if (e < cnt) v = __ldg(a.t.rec + (size_t)boxes[e].x * kRec + part);
+                if (part == 3) v.w = __int_as_float(e < cnt ? boxes[e].y : 0);
                 float* d = W.stage + (e >> 1) * kStageStride + part * 8 + (e & 1);
                 d[0] = v.x;
                 d[2] = v.y;
@@ -452,12 +389,11 @@ k_walk_fp32c(WalkArgs a)
 
         // the last cnt <= 32 leaves of the list of opened leaves, their sources brought
         // into shared memory one leaf (32 float4: up to 32 sources) ahead
-        auto direct_pairs = [&](int cnt) {
-            nl -= cnt;
+        auto direct_pairs = [&](const int2* leaves, int cnt) {
             float4* meta = reinterpret_cast<float4*>(W.stage);   // {-ch, begin}, {-cl, end}
             float4* buf = meta + 64;                             // 2 x 32 float4
             if (lane < cnt) {
-                const int nd = W.leaf[nl + lane].x;
+                const int nd = leaves[lane].x;
                 float4 A = __ldg(H + nd), B = __ldg(a.t.lo + nd);
                 const int2 be = __ldg(reinterpret_cast<const int2*>(a.t.info + nd));
                 A.w = __int_as_float(be.x);
@@ -499,7 +435,7 @@ k_walk_fp32c(WalkArgs a)
                 }
                 if (e1 < cnt) v = fetch(jb1, je1, s1);
                 __syncwarp();
-                if (W.leaf[nl + e].y & me) {
+                if (leaves[e].y & me) {
                     const float4 A = meta[2 * e], B = meta[2 * e + 1];
                     const float rx = (xh + A.x) + (xl + B.x);
                     const float ry = (yh + A.y) + (yl + B.y);
@@ -561,7 +497,7 @@ k_walk_fp32c(WalkArgs a)
                                 2 * p != tp ? rsqrt_ftz(r2.x) : 0.f,
                                 2 * p + 1 != tp ? rsqrt_ftz(r2.y) : 0.f);
                             const float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
-                            const float2 qr3 = __fmul2_rn(qi, __fmul2_rn(ri, ri));
+                            const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
                             px = __ffma2_rn(qr3, dx, px);
                             py = __ffma2_rn(qr3, dy, py);
                             pz = __ffma2_rn(qr3, dz, pz);
@@ -588,106 +524,7 @@ k_walk_fp32c(WalkArgs a)
             __syncwarp();
         };
 
-        // the first step tests the root for every target
-        int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0] : -1;
-        unsigned int mask = __ballot_sync(0xffffffffu, valid);
-        while (true) {
-            const bool has = box >= 0;
-            const float4 h = has ? __ldg(H + box) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const bool leaf = __float_as_int(h.w) < 0;
-            const float rc2 = fabsf(h.w);
-            const float dx = fabsf(gx + h.x), dy = fabsf(gy + h.y), dz = fabsf(gz + h.z);
-            const float nx = fmaxf(dx - ex, 0.f), ny = fmaxf(dy - ey, 0.f), nz = fmaxf(dz - ez, 0.f);
-            const float fx = dx + ex, fy = dy + ey, fz = dz + ez;
-            const float near2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
-            const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
-            const bool all_acc = near2 - rc2 > fmaf(gwa, near2, gwb);
-            const bool all_opn = rc2 - far2 > fmaf(gwa, far2, gwb);
-            unsigned int am = has && all_acc ? mask : 0u;   // targets that accept the box
-            const bool some = has && !all_acc && !all_opn;
-            const unsigned int between = __ballot_sync(0xffffffffu, some);
-            if (between) {
-                // decided target by target, two boxes per packed operation: pairs of
-                // {-c} x, y, z, {-rcrit2}, {box, mask}, side by side
-                const int slot = some ? __popc(between & lt) : -1;
-                const int cnt = __popc(between);
-                if (some) {
-                    float* d = W.stage + (slot >> 1) * 12 + (slot & 1);
-                    d[0] = h.x;
-                    d[2] = h.y;
-                    d[4] = h.z;
-                    d[6] = -rc2;
-                    d[8] = __int_as_float(box);
-                    d[10] = __int_as_float((int)mask);
-                }
-                if (lane == 0 && (cnt & 1)) {
-                    float* d = W.stage + (cnt >> 1) * 12 + 1;
-                    d[0] = d[2] = d[4] = d[6] = d[8] = d[10] = 0.f;
-                }
-                __syncwarp();
-                const float2 x2 = splat(xh), y2 = splat(yh), z2 = splat(zh);
-                for (int p = 0; 2 * p < cnt; ++p) {
-                    const float4* P = reinterpret_cast<const float4*>(W.stage + p * 12);
-                    const float4 f0 = P[0], f1 = P[1], f2 = P[2];
-                    const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
-                    const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
-                    const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
-                    const float2 d2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
-                    const float2 dm = __fadd2_rn(d2, make_float2(f1.z, f1.w));
-                    const float2 win = __ffma2_rn(splat(wa), d2, splat(wb));
-                    const bool in0 = (__float_as_int(f2.z) & me) != 0;
-                    const bool in1 = (__float_as_int(f2.w) & me) != 0;
-                    bool acc0 = in0 && dm.x > 0.f, acc1 = in1 && dm.y > 0.f;
-                    // Within the FP32 error of d2 - rcrit2 the decision is taken again in
-                    // FP64 exactly as the FP64 walk takes it, so both precisions open the
-                    // same boxes.  Per axis R is off by at most 2^-23 (|x_t| + |R|), so
-                    // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
-                    // included) with X_t the target's largest coordinate; with
-                    // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
-                    // a million at the bench size).
-                    const bool again0 = in0 && fabsf(dm.x) <= win.x;
-                    const bool again1 = in1 && fabsf(dm.y) <= win.y;
-                    if (again0)
-                        acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + t,
-                                            a.y + t, a.z + t);
-                    if (again1)
-                        acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kMom, a.x + t,
-                                            a.y + t, a.z + t);
-                    const unsigned int am0 = __ballot_sync(0xffffffffu, acc0);
-                    const unsigned int am1 = __ballot_sync(0xffffffffu, acc1);
-                    if (slot == 2 * p) am = am0;
-                    if (slot == 2 * p + 1) am = am1;
-                }
-                __syncwarp();
-            }
-            const unsigned int om = has ? mask & ~am : 0u;  // targets that open it
-            const unsigned int A = __ballot_sync(0xffffffffu, am != 0u);
-            const unsigned int OL = __ballot_sync(0xffffffffu, om != 0u && leaf);
-            const unsigned int OT = __ballot_sync(0xffffffffu, om != 0u && !leaf);
-            if (am) W.acc[na + __popc(A & lt)] = make_int2(box, (int)am);
-            if (om) {
-                if (leaf) W.leaf[nl + __popc(OL & lt)] = make_int2(box, (int)om);
-                else W.stack[top + __popc(OT & lt)] = make_int2(box, (int)om);
-            }
-            na += __popc(A);
-            nl += __popc(OL);
-            top += __popc(OT);
-            __syncwarp();
-            const bool done = top == 0;
-            while (na >= kStage || (done && na > 0)) multipoles(min(na, kStage));
-            while (nl >= 32 || (done && nl > 0)) direct_pairs(min(nl, 32));
-            if (done) break;
-            const int pop = top > kPopWide ? 1 : min(top, 4);
-            box = -1;
-            mask = 0u;
-            if ((lane >> 3) < pop) {
-                const int2 e = W.stack[top - 1 - (lane >> 3)];
-                box = __ldg(a.t.child8 + (size_t)e.x * 8 + (lane & 7));
-                mask = (unsigned int)e.y;
-            }
-            top -= pop;
-            __syncwarp();
-        }
+        walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
 
         if (valid) {
             const int s = a.sp[t];
@@ -696,6 +533,165 @@ k_walk_fp32c(WalkArgs a)
             a.ay[t] = qm * ((double)sy + (double)cy);
             a.az[t] = qm * ((double)sz + (double)cz);
             if (kPhi && a.phi) a.phi[t] = (double)sp + (double)cp;
+            a.cnt_p2p[t] = np;
+            a.cnt_m2p[t] = nm;
+        }
+        unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
+            sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
+        }
+        if (lane == 0) {
+            atomicAdd(&a.stats[0], sp2);
+            atomicAdd(&a.stats[1], sm2);
+        }
+    }
+}
+
+// ---- The FP32C walk of ucp_grad_ke_electrons' forward runs: a chunk's targets visit
+// boxes in pre-order, one box per step in all lanes, and multipoles are summed box by
+// box, 32 visits to a compensated add.  Its forces agree with k_walk_fp32c's to about
+// 2e-8, but the gradient of an unresolved run amplifies such a difference to 1e-3 of
+// single components within 20 electron steps (close electron-ion encounters), and this
+// order of sums is the one whose gradients the library has always returned.  1.4
+// against 0.95 ms per walk over the electrons at N = 262,144, a tenth of a gradient.
+constexpr int kVisitThreads = 128;
+constexpr int kVisitList = 64;      // opened leaves buffered per warp
+constexpr int kVisitBatch = 32;     // visits summed in FP32 before a compensated add
+
+__global__ void __launch_bounds__(kVisitThreads, 7)
+k_walk_fp32c_visits(WalkArgs a)
+{
+    __shared__ int2 lists[kVisitThreads / 32][kVisitList];   // {opened leaf, mask}
+    const int lane = threadIdx.x & 31;
+    int2* lst = lists[threadIdx.x >> 5];
+    const double q0 = a.qsp[0], q1 = a.qsp[1];
+    const float4* __restrict__ H = a.t.hdr;
+    const float4* __restrict__ LO = a.t.lo;
+    const float4* __restrict__ S = a.src32;
+    const float eps2 = (float)a.eps2;
+
+    for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
+         chunk = next_chunk(a.work, lane)) {
+        const int4 ck = a.chunks[chunk];
+        const int t = lane < ck.y ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
+        const bool valid = t >= 0;
+        const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
+        const int end = __float_as_int(LO[root].w);
+        float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
+        if (valid) {
+            const double* cc = a.cubes[ck.z].c;
+            const double X = a.x[t] - cc[0], Y = a.y[t] - cc[1], Z = a.z[t] - cc[2];
+            xh = (float)X; yh = (float)Y; zh = (float)Z;
+            xl = (float)(X - (double)xh); yl = (float)(Y - (double)yh); zl = (float)(Z - (double)zh);
+        }
+        const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
+        const float wa = fmaf(0.5f, bt, 4e-6f), wb = 0.5f * bt;   // see walk_lists
+        float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
+        float bx = 0.f, by = 0.f, bz = 0.f;
+        int np = 0, nm = 0, vis = 0, npl = 0;
+        int skip = valid ? 0 : 0x7fffffff;
+
+        auto fold = [&]() {
+            two_sum_acc(sx, cx, bx);
+            two_sum_acc(sy, cy, by);
+            two_sum_acc(sz, cz, bz);
+            bx = by = bz = 0.f;
+        };
+        auto flush = [&]() {
+            __syncwarp();
+            for (int e = 0; e < npl; ++e) {
+                if (!(((unsigned int)lst[e].y >> lane) & 1u)) continue;
+                const int nd = lst[e].x;
+                const float4 A = H[nd], B = LO[nd];
+                const float rx = (xh + A.x) + (xl + B.x), ry = (yh + A.y) + (yl + B.y),
+                            rz = (zh + A.z) + (zl + B.z);
+                const int jb = __ldg(&a.t.info[nd].x), je = __ldg(&a.t.info[nd].y);
+                const float2 rx2 = splat(rx), ry2 = splat(ry), rz2 = splat(rz), e2 = splat(eps2);
+                float2 px = splat(0.f), py = px, pz = px;
+#pragma unroll 2
+                for (int j = jb & ~1; j < je; j += 2) {
+                    const float4 P = __ldg(S + j), Q = __ldg(S + j + 1);
+                    const float2 dx = __fadd2_rn(rx2, make_float2(P.x, P.y));
+                    const float2 dy = __fadd2_rn(ry2, make_float2(P.z, P.w));
+                    const float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
+                    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+                    const bool ok0 = j >= jb && j != t;
+                    const bool ok1 = j + 1 < je && j + 1 != t;
+                    const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                                  ok1 ? rsqrt_ftz(r2.y) : 0.f);
+                    const float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
+                    const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
+                    px = __ffma2_rn(qr3, dx, px);
+                    py = __ffma2_rn(qr3, dy, py);
+                    pz = __ffma2_rn(qr3, dz, pz);
+                }
+                np += (je - jb) - ((t >= jb && t < je) ? 1 : 0);
+                two_sum_acc(sx, cx, px.x + px.y);
+                two_sum_acc(sy, cy, py.x + py.y);
+                two_sum_acc(sz, cz, pz.x + pz.y);
+            }
+            npl = 0;
+            __syncwarp();
+        };
+
+        int node = root;
+        while (node < end) {
+            const float4 A = H[node], B = LO[node];
+            const float4* r = a.t.rec + (size_t)node * kRec;
+            const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
+            const int nxt = __float_as_int(B.w);
+            const bool leaf = __float_as_int(A.w) < 0;
+            const bool active = node >= skip;
+            const float rx = xh + A.x, ry = yh + A.y, rz = zh + A.z;
+            const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+            const float dm = d2 - fabsf(A.w);
+            bool acc = active && dm > 0.f;
+            if (active && fabsf(dm) <= fmaf(wa, d2, wb))
+                acc = accepts_fp64(a.t.mom + (size_t)node * kMom, a.x + t, a.y + t, a.z + t);
+            const unsigned int om = __ballot_sync(0xffffffffu, active && !acc);
+            int next = nxt;
+            if (om) {
+                if (leaf) {
+                    if (lane == 0) lst[npl] = make_int2(node, (int)om);
+                    ++npl;
+                } else {
+                    if (acc) skip = nxt;
+                    next = node + 1;
+                }
+            }
+            if (acc) {
+                const float g = rsqrt_ftz(d2 + eps2);
+                const float u = g * g, g3 = g * u;
+                const float Qxx = 2.f * r2.x, Qxy = 2.f * r2.y, Qxz = 2.f * r2.z, Qyy = 2.f * r2.w,
+                            Qyz = 2.f * r3.x, Qzz = 2.f * r3.y;
+                const float QRx = fmaf(Qxx, rx, fmaf(Qxy, ry, Qxz * rz));
+                const float QRy = fmaf(Qxy, rx, fmaf(Qyy, ry, Qyz * rz));
+                const float QRz = fmaf(Qxz, rx, fmaf(Qyz, ry, Qzz * rz));
+                const float RQR = fmaf(rx, QRx, fmaf(ry, QRy, rz * QRz));
+                const float w = fmaf(r1.x, rx, fmaf(r1.y, ry, fmaf(r1.z, rz, r1.w)));
+                const float h = u * RQR, s3 = 3.f * u;
+                const float aa = g3 * fmaf(s3, fmaf(2.5f, h, w), r0.w);
+                const float mg3 = -g3;
+                bx = fmaf(mg3, fmaf(s3, QRx, r1.x), fmaf(aa, rx, bx));
+                by = fmaf(mg3, fmaf(s3, QRy, r1.y), fmaf(aa, ry, by));
+                bz = fmaf(mg3, fmaf(s3, QRz, r1.z), fmaf(aa, rz, bz));
+                ++nm;
+            }
+            if ((++vis & (kVisitBatch - 1)) == 0) fold();
+            node = next;
+            if (npl == kVisitList) flush();
+        }
+        flush();
+        fold();
+
+        if (valid) {
+            const int s = a.sp[t];
+            const double qm = (s ? q1 : q0) / a.msp[s];
+            a.ax[t] = qm * ((double)sx + (double)cx);
+            a.ay[t] = qm * ((double)sy + (double)cy);
+            a.az[t] = qm * ((double)sz + (double)cz);
             a.cnt_p2p[t] = np;
             a.cnt_m2p[t] = nm;
         }
@@ -820,6 +816,15 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
     if (a.kelbg) walk_fp32c_shape<true, true>(a, per_sm, b, s);
     else if (a.phi) walk_fp32c_shape<false, true>(a, per_sm, b, s);
     else walk_fp32c_shape<false, false>(a, per_sm, b, s);
+}
+
+void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, cudaStream_t s)
+{
+    count_launch(1);
+    cudaMemsetAsync(a.work, 0, sizeof(int), s);
+    const int wpb = kVisitThreads / 32;
+    const int b = walk_blocks(((int64_t)a.nchunks + wpb - 1) / wpb, nsm, 7);
+    k_walk_fp32c_visits<<<b, kVisitThreads, 0, s>>>(a);
 }
 
 }  // namespace ucp
