@@ -5,7 +5,7 @@
 // Arithmetic that decides an integer (cube, cell coordinates, box centre) is
 // written with explicit round-to-nearest intrinsics in the order of the
 // definition, so that no multiply-add contraction changes a cell.
-#include "ucp_internal.cuh"
+#include "ucp_scan.cuh"
 
 #include <math.h>
 
@@ -16,37 +16,6 @@ namespace {
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
-
-__device__ __forceinline__ int warp_incl_scan(int v, int lane)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += u;
-    }
-    return v;
-}
-
-// Exclusive scan of one value per thread over a block of kScanThreads.
-__device__ int block_excl_scan(int v, int* total)
-{
-    __shared__ int warp_sums[32];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int inc = warp_incl_scan(v, lane);
-    if (lane == 31) warp_sums[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        int nw = blockDim.x >> 5;
-        int s = lane < nw ? warp_sums[lane] : 0;
-        int si = warp_incl_scan(s, lane);
-        if (lane < nw) warp_sums[lane] = si - s;
-        if (lane == 31) *total = si;
-    }
-    __syncthreads();
-    int r = warp_sums[w] + inc - v;
-    __syncthreads();
-    return r;
-}
 
 __global__ void k_scan_reduce(const int* __restrict__ in, int n, int* __restrict__ part)
 {
@@ -98,44 +67,6 @@ __global__ void k_scan_apply(const int* __restrict__ in, int* __restrict__ out, 
         int i = base + threadIdx.x * kScanItems + k;
         if (i < n) out[i] = off;
         off += v[k];
-    }
-}
-
-// Target selection: the slots whose species is `species`, in slot order.  The
-// count per tile and the write pass take the flag straight from the species.
-__global__ void k_select_count(const int8_t* __restrict__ sp, int species, int n,
-                               int* __restrict__ part)
-{
-    int base = blockIdx.x * kScanTile;
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int i = base + threadIdx.x * kScanItems + k;
-        if (i < n) s += sp[i] == species;
-    }
-    __shared__ int tot;
-    block_excl_scan(s, &tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-__global__ void k_select_write(const int8_t* __restrict__ sp, int species, int n,
-                               const int* __restrict__ part, int* __restrict__ list)
-{
-    int base = blockIdx.x * kScanTile;
-    int v[kScanItems];
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int i = base + threadIdx.x * kScanItems + k;
-        v[k] = i < n && sp[i] == species;
-        s += v[k];
-    }
-    __shared__ int tot;
-    int off = block_excl_scan(s, &tot) + part[blockIdx.x];
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int i = base + threadIdx.x * kScanItems + k;
-        if (v[k]) list[off++] = i;
     }
 }
 
@@ -193,8 +124,17 @@ __global__ void k_bbox_partial(const double* __restrict__ x, const double* __res
 // Sec. 3: the cube that encloses every particle.  Centre = (min + max) / 2 per
 // axis; side = largest extent * (1 + 2^-20) so that the maximum falls inside;
 // side 1 when all particles coincide.
-__global__ void k_bbox_final(const double* __restrict__ part, int nblk, Cube* cubes)
+// Block 0 also clears the build's counters and advances the tag of the published words.
+__global__ void k_bbox_final(const double* __restrict__ part, int nblk, Cube* cubes, BuildCtl ctl)
 {
+    if (blockIdx.x == 0) {
+        for (int i = threadIdx.x; i < kCtlWords; i += blockDim.x) ctl.words[i] = 0;
+        // every build's published words carry a tag 16 above the previous build's, kept
+        // on the device so that a captured graph replays with fresh tags (every word of
+        // a region is rewritten each build, so a stale word always carries an older
+        // tag, also across 30-bit wrap-around)
+        if (threadIdx.x == 0) *ctl.epoch = (*ctl.epoch + 16u) & 0x3fffffffu;
+    }
     part += (size_t)blockIdx.x * nblk * 6;  // cloud blockIdx.x
     Cube* cube = cubes + blockIdx.x;
     // min and max taken on the ordered integer images, as in k_bbox_partial
@@ -255,208 +195,36 @@ __device__ __forceinline__ unsigned int cell_coord(double x, double lo, double k
     return (unsigned int)min(max(k, 0), 2097151);
 }
 
-__global__ void k_keys(const double* __restrict__ x, const double* __restrict__ y,
-                       const double* __restrict__ z, int n, const Cube* __restrict__ cubes,
-                       const unsigned char* __restrict__ cloud,
-                       unsigned long long* __restrict__ key, unsigned int* __restrict__ val)
+__device__ __forceinline__ unsigned long long morton_key(double x, double y, double z,
+                                                         const Cube* __restrict__ cube)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const Cube* cube = cubes + (cloud ? cloud[i] : 0);
-    double ks = cube->kscale;
-    unsigned int kx = cell_coord(x[i], cube->lo[0], ks);
-    unsigned int ky = cell_coord(y[i], cube->lo[1], ks);
-    unsigned int kz = cell_coord(z[i], cube->lo[2], ks);
-    key[i] = spread3(kx) | (spread3(ky) << 1) | (spread3(kz) << 2);
-    val[i] = (unsigned int)i;
+    const double ks = cube->kscale;
+    return spread3(cell_coord(x, cube->lo[0], ks)) | (spread3(cell_coord(y, cube->lo[1], ks)) << 1) |
+           (spread3(cell_coord(z, cube->lo[2], ks)) << 2);
 }
 
-// ---------------------------------------------------------------- sort
-constexpr int kSortThreads = 256;
-constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortChunks = 8;                              // 32-key chunks per warp
-constexpr int kSortTile = kSortThreads * kSortChunks;       // 2048 keys per block
-constexpr int kRadix = 256;
-constexpr int kSortSpinLimit = 1 << 20;  // polls of a predecessor's word before giving up
-constexpr int kLook = 8;                  // predecessors read per look-back round trip
-
-// Digit histograms of all eight passes in one read of the keys.
-__global__ void __launch_bounds__(kSortThreads)
-k_sort_hist_all(const unsigned long long* __restrict__ key, int n, unsigned int* __restrict__ ghist)
+// Keys, and the digit counts of every pass of the sort (the passes' digits are the
+// key's top 8 passes bits).
+constexpr int kKeyThreads = 256;
+__global__ void __launch_bounds__(kKeyThreads)
+k_keys(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
+       int n, const Cube* __restrict__ cubes, const unsigned char* __restrict__ cloud,
+       unsigned long long* __restrict__ key, int passes, int* __restrict__ hist)
 {
-    __shared__ unsigned int h[8][kRadix];
-    for (int i = threadIdx.x; i < 8 * kRadix; i += kSortThreads) (&h[0][0])[i] = 0;
+    __shared__ int h[kSortPassesMax][kRadix];
+    for (int i = threadIdx.x; i < passes * kRadix; i += kKeyThreads) (&h[0][0])[i] = 0;
     __syncthreads();
-    for (int i = blockIdx.x * kSortThreads + threadIdx.x; i < n; i += gridDim.x * kSortThreads) {
-        unsigned long long k = key[i];
-#pragma unroll
-        for (int p = 0; p < 8; ++p) atomicAdd(&h[p][(unsigned int)(k >> (8 * p)) & 0xffu], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 8 * kRadix; i += kSortThreads) {
-        unsigned int v = (&h[0][0])[i];
-        if (v) atomicAdd(&ghist[i], v);
-    }
-}
-
-// goff[p][d] = number of keys whose pass-p digit is below d.
-// Also advances the sort's tag: every build's published words carry a tag 16
-// above the previous build's, kept on the device so that a captured graph
-// replays with fresh tags (every word of a pass region is rewritten each build,
-// so a stale word always carries an older tag, also across 30-bit wrap-around).
-__global__ void __launch_bounds__(kRadix) k_sort_offsets(const unsigned int* __restrict__ ghist,
-                                                         unsigned int* __restrict__ goff,
-                                                         unsigned int* __restrict__ epoch)
-{
-    __shared__ int tot;
-    if (threadIdx.x == 0) *epoch = (*epoch + 16u) & 0x3fffffffu;
-    for (int p = 0; p < 8; ++p) {
-        int v = (int)ghist[p * kRadix + threadIdx.x];
-        goff[p * kRadix + threadIdx.x] = (unsigned int)block_excl_scan(v, &tot);
-    }
-}
-
-// One stable LSD pass in a single kernel (decoupled look-back).  A block takes
-// the next tile from a counter, ranks its keys stably (each warp owns a
-// contiguous quarter-tile and ranks it chunk by chunk with match_any), and
-// publishes its per-digit count; the digit offset of the tile is the sum of
-// the counts of all earlier tiles, read back through their published words
-// {epoch, flag (1 = count of the tile, 2 = inclusive prefix), value}.  A block
-// waits only on tiles taken before its own, whose blocks are running, and
-// every wait is bounded: past spin_limit polls it raises *err, keeps its keys
-// where they are and leaves (the host reports UCP_ETIMEOUT).
-__global__ void __launch_bounds__(kSortThreads)
-k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __restrict__ vin,
-           unsigned long long* __restrict__ kout, unsigned int* __restrict__ vout, int n,
-           int shift, const unsigned int* __restrict__ goff, unsigned long long* status,
-           int* tile_ctr, const unsigned int* __restrict__ epoch_dev, unsigned int pass, int* err,
-           int spin_limit, const unsigned char* __restrict__ digit_of_val)
-{
-    const unsigned int epoch = (*epoch_dev + pass) & 0x3fffffffu;
-    __shared__ int cnt[kSortWarps][kRadix];
-    __shared__ int s_tile, s_fail;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        s_tile = atomicAdd(tile_ctr, 1);
-        s_fail = 0;
-    }
-    for (int d = lane; d < kRadix; d += 32) cnt[w][d] = 0;
-    __syncthreads();
-    const int tile = s_tile;
-    const int base = tile * kSortTile + w * (kSortTile / kSortWarps);
-    unsigned long long kk[kSortChunks];
-    unsigned int vv[kSortChunks];
-    int dig[kSortChunks], rank[kSortChunks];
-    const unsigned int lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int c = 0; c < kSortChunks; ++c) {
-        int i = base + c * 32 + lane;
-        bool ok = i < n;
-        kk[c] = ok ? kin[i] : 0ull;
-        vv[c] = ok ? vin[i] : 0u;
-        // digit: 8 key bits, or (cloud pass) the cloud of the element's previous slot
-        int d = ok ? (digit_of_val ? (int)digit_of_val[vv[c]] : (int)((kk[c] >> shift) & 0xffu))
-                   : kRadix + lane;  // invalid lanes unique
-        dig[c] = d;
-        unsigned int peers = __match_any_sync(0xffffffffu, d);
-        int leader = __ffs(peers) - 1;
-        int before = 0;
-        if (ok && lane == leader) {
-            before = cnt[w][d];
-            cnt[w][d] = before + __popc(peers);
-        }
-        before = __shfl_sync(0xffffffffu, before, leader);
-        rank[c] = before + __popc(peers & lt);
-        __syncwarp();
+    const int low = kKeyBits - 8 * passes;
+    for (int i = blockIdx.x * kKeyThreads + threadIdx.x; i < n; i += gridDim.x * kKeyThreads) {
+        const unsigned long long k = morton_key(x[i], y[i], z[i], cubes + (cloud ? cloud[i] : 0));
+        key[i] = k;
+        for (int p = 0; p < passes; ++p)
+            atomicAdd(&h[p][(unsigned int)(k >> (low + 8 * p)) & 0xffu], 1);
     }
     __syncthreads();
-    {
-        const int d = threadIdx.x;  // kSortThreads == kRadix
-        int total = 0;
-        for (int ww = 0; ww < kSortWarps; ++ww) {
-            int t = cnt[ww][d];
-            cnt[ww][d] = total;
-            total += t;
-        }
-        const unsigned long long tag = (unsigned long long)epoch << 34;
-        unsigned long long* mine = status + (size_t)tile * kRadix + d;
-        unsigned int prefix = 0;
-        if (tile > 0) {
-            atomicExch(mine, tag | (1ull << 32) | (unsigned int)total);
-            // kLook predecessors' words per round trip (independent loads), taken in
-            // order j, j - 1, ... up to the first inclusive prefix or the first word
-            // not yet published, which is polled again
-            int j = tile - 1, spins = 0;
-            bool done = false;
-            while (!done) {
-                unsigned long long v[kLook];
-#pragma unroll
-                for (int u = 0; u < kLook; ++u)
-                    v[u] = j - u >= 0 ? __ldcv(status + (size_t)(j - u) * kRadix + d) : 0ull;
-                int used = 0;
-                bool blocked = false;
-#pragma unroll
-                for (int u = 0; u < kLook; ++u) {
-                    if (done || blocked || j - u < 0) continue;
-                    const unsigned int flag = (unsigned int)(v[u] >> 32) & 3u;
-                    if ((v[u] >> 34) != (unsigned long long)epoch || flag == 0u) {
-                        blocked = true;
-                        continue;
-                    }
-                    prefix += (unsigned int)v[u];
-                    ++used;
-                    if (flag == 2u) done = true;
-                }
-                j -= used;
-                if (done || j < 0) break;  // (tile 0 publishes an inclusive prefix)
-                if (blocked) {
-                    if (++spins > spin_limit) {
-                        atomicOr(err, 1);
-                        s_fail = 1;
-                        break;
-                    }
-                    __nanosleep(64);
-                }
-            }
-        }
-        atomicExch(mine, tag | (2ull << 32) | (prefix + (unsigned int)total));
-        const int off = (int)(goff[d] + prefix);
-        for (int ww = 0; ww < kSortWarps; ++ww) cnt[ww][d] += off;
-    }
-    __syncthreads();
-    const bool fail = s_fail != 0;
-#pragma unroll
-    for (int c = 0; c < kSortChunks; ++c) {
-        int i = base + c * 32 + lane;
-        if (i < n) {
-            int p = fail ? i : cnt[w][dig[c]] + rank[c];
-            kout[p] = kk[c];
-            vout[p] = vv[c];
-        }
-    }
-}
-
-// Equal keys must come out ordered by caller index (ties by particle index):
-// the run starting at i is insertion-sorted by ids[perm[.]].  Runs are rare and
-// short except when particles coincide (depth-21 boxes).
-__global__ void k_tiefix(const unsigned long long* __restrict__ key, unsigned int* __restrict__ perm,
-                         const unsigned int* __restrict__ ids, int n)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1) return;
-    unsigned long long k = key[i];
-    if (key[i + 1] != k || (i > 0 && key[i - 1] == k)) return;
-    int e = i + 1;
-    while (e < n && key[e] == k) ++e;
-    for (int a = i + 1; a < e; ++a) {
-        unsigned int pv = perm[a];
-        unsigned int idv = ids[pv];
-        int b = a - 1;
-        while (b >= i && ids[perm[b]] > idv) {
-            perm[b + 1] = perm[b];
-            --b;
-        }
-        perm[b + 1] = pv;
+    for (int i = threadIdx.x; i < passes * kRadix; i += kKeyThreads) {
+        const int v = (&h[0][0])[i];
+        if (v) atomicAdd(&hist[i], v);
     }
 }
 
@@ -775,7 +543,10 @@ __device__ __forceinline__ void finish_box(const double* a, const double z[3],
 
 __global__ void k_clear_children(Tree t)
 {
-    int total = *t.nnodes * 8;
+    const int nn = *t.nnodes;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x)
+        t.arrive[i] = 0;
+    const int total = nn * 8;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x)
         t.child8[i] = -1;
 }
@@ -1113,109 +884,29 @@ void launch_scan(const int* in, int* out, int n, int* partials, int* total, cuda
     k_scan_apply<<<nb, kScanThreads, 0, s>>>(in, out, n, partials);
 }
 
-void launch_select(const int8_t* sp, int species, int n, int* list, int* partials, int* count,
-                   cudaStream_t s)
-{
-    count_launch(3);
-    int nb = (n + kScanTile - 1) / kScanTile;
-    if (nb < 1) nb = 1;
-    k_select_count<<<nb, kScanThreads, 0, s>>>(sp, species, n, partials);
-    k_scan_partials<<<1, kScanThreads, 0, s>>>(partials, nb, count);
-    k_select_write<<<nb, kScanThreads, 0, s>>>(sp, species, n, partials, list);
-}
-
 void launch_bbox(const double* x, const double* y, const double* z, int n, double* partials,
-                 int nblk, Cube* cubes, const int* cloud_start, int n_clouds, cudaStream_t s)
+                 int nblk, Cube* cubes, const int* cloud_start, int n_clouds, BuildCtl ctl,
+                 cudaStream_t s)
 {
     count_launch(2);
     k_bbox_partial<<<dim3(nblk, n_clouds), 256, 0, s>>>(x, y, z, n, partials, cloud_start);
-    k_bbox_final<<<n_clouds, 256, 0, s>>>(partials, nblk, cubes);
+    k_bbox_final<<<n_clouds, 256, 0, s>>>(partials, nblk, cubes, ctl);
 }
 
 void launch_keys(const double* x, const double* y, const double* z, int n, const Cube* cubes,
-                 const unsigned char* cloud, unsigned long long* key, unsigned int* val,
+                 const unsigned char* cloud, unsigned long long* key, int passes, BuildCtl ctl,
                  cudaStream_t s)
 {
     count_launch(1);
-    k_keys<<<(n + 255) / 256, 256, 0, s>>>(x, y, z, n, cubes, cloud, key, val);
-}
-
-size_t sort_test_words() { return 4 * (size_t)kSortTile; }
-
-size_t sort_status_words(int n)
-{
-    int nb = (n + kSortTile - 1) / kSortTile;
-    return (size_t)9 * kRadix * (size_t)(nb > 0 ? nb : 1);
-}
-
-int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, SortScratch sc,
-                const unsigned int* ids_in, const unsigned char* cloud,
-                const int* cloud_start, int n_clouds, cudaStream_t s)
-{
-    count_launch(11 + (n_clouds > 1 ? 1 : 0));
-    const int nb = (n + kSortTile - 1) / kSortTile;
-    cudaMemsetAsync(sc.ghist, 0, sizeof(unsigned int) * (8 * kRadix + 9), s);  // + tile counters
-    int hb = (n + 4 * kSortThreads - 1) / (4 * kSortThreads);
-    if (hb > 2 * 152) hb = 2 * 152;
-    k_sort_hist_all<<<hb > 0 ? hb : 1, kSortThreads, 0, s>>>(key[0], n, sc.ghist);
-    k_sort_offsets<<<1, kRadix, 0, s>>>(sc.ghist, sc.goff, sc.epoch);
-    int* tiles = reinterpret_cast<int*>(sc.ghist + 8 * kRadix);
-    int cur = 0;
-    for (int p = 0; p < 8; ++p) {
-        k_onesweep<<<nb, kSortThreads, 0, s>>>(key[cur], val[cur], key[cur ^ 1], val[cur ^ 1], n,
-                                               8 * p, sc.goff + p * kRadix,
-                                               sc.status + (size_t)p * nb * kRadix, tiles + p,
-                                               sc.epoch, (unsigned int)p, sc.err, kSortSpinLimit,
-                                               nullptr);
-        cur ^= 1;
-    }
-    if (n_clouds > 1) {
-        // a ninth stable pass by cloud: (cloud, key) order, each cloud back in its
-        // fixed segment; the offsets of a cloud are its segment start
-        k_onesweep<<<nb, kSortThreads, 0, s>>>(key[cur], val[cur], key[cur ^ 1], val[cur ^ 1], n,
-                                               0, reinterpret_cast<const unsigned int*>(cloud_start),
-                                               sc.status + (size_t)8 * nb * kRadix, tiles + 8,
-                                               sc.epoch, 8u, sc.err, kSortSpinLimit, cloud);
-        cur ^= 1;
-    }
-    k_tiefix<<<(n + 255) / 256, 256, 0, s>>>(key[cur], val[cur], ids_in, n);
-    return cur;
-}
-
-int sort_selftest_timeout(SortScratch sc, cudaStream_t s)
-{
-    // a lone block that takes tile 1 while tile 0 never publishes: its bounded
-    // wait must run out, raise *err and leave the keys where they are
-    count_launch(1);
-    static const int one = 1;
-    int* tiles = reinterpret_cast<int*>(sc.ghist + 8 * kRadix);
-    if (cudaMemsetAsync(sc.status, 0, sizeof(unsigned long long) * 2 * kRadix, s) != cudaSuccess ||
-        cudaMemcpyAsync(tiles, &one, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(sc.goff, 0, sizeof(unsigned int) * kRadix, s) != cudaSuccess ||
-        cudaMemcpyAsync(sc.test_epoch, &one, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemsetAsync(sc.test_keys, 0, sizeof(unsigned long long) * 4 * kSortTile, s) != cudaSuccess ||
-        cudaMemsetAsync(sc.test_vals, 0, sizeof(unsigned int) * 4 * kSortTile, s) != cudaSuccess)
-        return -1;
-    // input: tiles 0-1 of the test buffers; output: tiles 2-3
-    k_onesweep<<<1, kSortThreads, 0, s>>>(sc.test_keys, sc.test_vals, sc.test_keys + 2 * kSortTile,
-                                          sc.test_vals + 2 * kSortTile, 2 * kSortTile, 0, sc.goff,
-                                          sc.status, tiles, sc.test_epoch, 0u, sc.err, 2000, nullptr);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-void launch_tiefix(const unsigned long long* key, unsigned int* perm, const unsigned int* ids,
-                   int n, cudaStream_t s)
-{
-    count_launch(1);
-    k_tiefix<<<(n + 255) / 256, 256, 0, s>>>(key, perm, ids, n);
+    int nb = (n + kKeyThreads - 1) / kKeyThreads;
+    if (nb > 8 * 152) nb = 8 * 152;
+    k_keys<<<nb, kKeyThreads, 0, s>>>(x, y, z, n, cubes, cloud, key, passes, ctl.words + kCtlHist);
 }
 
 void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* pos_cnt,
                      int* pos_off, int* scan_part, Tree t, cudaStream_t s)
 {
     count_launch(3);
-    cudaMemsetAsync(t.maxdepth, 0, sizeof(int), s);
-    cudaMemsetAsync(t.count, 0, sizeof(int) * (kMaxDepth + 2), s);
     const int nb = (n + kTopoThreads - 1) / kTopoThreads;
     const bool win = leaf_cap <= kTopoWin;
     if (win) k_topo_count_win<<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, t);
@@ -1233,7 +924,6 @@ void launch_moments(const double* x, const double* y, const double* z, const int
     // leaves from their particles, then every twig as its last child finishes
     // (bottom-up sweep with arrival counters), in one launch
     count_launch(1);
-    cudaMemsetAsync(t.arrive, 0, sizeof(int) * (size_t)t.cap, s);
     // small blocks spread the leaf threads (about one per eight particles) evenly
     // over the SMs
     int blocks = (n + kMomThreads - 1) / kMomThreads;

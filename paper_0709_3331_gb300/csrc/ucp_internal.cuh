@@ -89,31 +89,56 @@ struct Cube {                // enclosing cube: centre, side, lower corner, 2^21
     double kscale;
 };
 
-// ---- build (ucp_build.cu) ----
+// ---- build (ucp_build.cu, ucp_sort.cu) ----
+constexpr int kKeyBits = 63;
+constexpr int kRadix = 256;
+constexpr int kSortPassesMax = 4;        // passes over the key's top digits (sort_passes)
+// Counters of one build, cleared together at its start.
+enum CtlIdx {
+    kCtlHist = 0,                                  // digit counts of every pass
+    kCtlTile = kCtlHist + kSortPassesMax * kRadix, // tile counters: passes, then the clouds' pass
+    kCtlLong = kCtlTile + kSortPassesMax + 1,      // raised: a run too long for the run sort
+    kCtlBarrier,                                   // arrivals at the full sort's barrier
+    kCtlMaxDepth,
+    kCtlCount,                                     // kMaxDepth + 2 list counters
+    kCtlWords = kCtlCount + kMaxDepth + 2
+};
+struct BuildCtl {
+    int* words;              // kCtlWords
+    unsigned int* epoch;     // tag of the published words, advanced every build
+};
 void launch_bbox(const double* x, const double* y, const double* z, int n, double* partials,
-                 int nblk, Cube* cubes, const int* cloud_start, int n_clouds, cudaStream_t s);
+                 int nblk, Cube* cubes, const int* cloud_start, int n_clouds, BuildCtl ctl,
+                 cudaStream_t s);
 void launch_keys(const double* x, const double* y, const double* z, int n, const Cube* cubes,
-                 const unsigned char* cloud, unsigned long long* key, unsigned int* val,
+                 const unsigned char* cloud, unsigned long long* key, int passes, BuildCtl ctl,
                  cudaStream_t s);
 struct SortScratch {
-    unsigned int* ghist;           // 8 x 256 digit counts, then 9 tile counters
-    unsigned int* goff;            // 8 x 256 digit offsets
-    unsigned long long* status;    // 9 passes x tiles x 256 published words
+    unsigned long long* status;    // passes x tiles x 256 published words
     int* err;                      // raised by a wait that gave up
-    unsigned int* epoch;           // tag of the published words, advanced every build
+    int* full_counts;              // full sort: 2 x blocks x 256 digit counts
     unsigned int* test_epoch;      // tag used by the bounded-wait self-test (1)
+    int* test_ctl;                 // its tile counter and 256 zero offsets
     unsigned long long* test_keys; // 4 tiles, for the bounded-wait self-test
     unsigned int* test_vals;
 };
+int sort_passes(int64_t largest_cloud);
 size_t sort_status_words(int n);
 size_t sort_test_words();
-// returns the buffer (0 or 1) that holds the sorted keys and permutation
-int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, SortScratch sc,
-                const unsigned int* ids_in, const unsigned char* cloud,
-                const int* cloud_start, int n_clouds, cudaStream_t s);
-int sort_selftest_timeout(SortScratch sc, cudaStream_t s);
-void launch_tiefix(const unsigned long long* key, unsigned int* perm, const unsigned int* ids,
-                   int n, cudaStream_t s);
+size_t sort_full_words();
+// Particle state of one order: six streams, species, caller index.
+struct StateRef {
+    double* f[6];
+    int8_t* sp;
+    unsigned int* id;
+};
+// Sorts key[0] (unsorted keys of the slots of `in`) and moves the state into key order
+// (`out`); returns the buffer (0 or 1) that holds the sorted keys.
+int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int passes,
+                const SortScratch& sc, BuildCtl ctl, const StateRef& in, const StateRef& out,
+                const unsigned char* cloud, const int* cloud_start, int n_clouds, int nsm,
+                cudaStream_t s);
+int sort_selftest_timeout(const SortScratch& sc, cudaStream_t s);
 void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* pos_cnt,
                      int* pos_off, int* scan_part, Tree t, cudaStream_t s);
 void launch_moments(const double* x, const double* y, const double* z, const int8_t* sp,
@@ -174,16 +199,14 @@ void launch_ke_seed(const double* v, const int8_t* sp, int n, double me, double*
                     double* loss, cudaStream_t s);
 
 // ---- push and reductions (ucp_push.cu) ----
-void launch_permute(const unsigned int* perm, int n, const double* const* src6, double* const* dst6,
-                    const int8_t* sp_in, int8_t* sp_out, const unsigned int* id_in,
-                    unsigned int* id_out, cudaStream_t s);
 void launch_kick(double* vx, double* vy, double* vz, const double* ax, const double* ay,
                  const double* az, const int8_t* sp, int species, double h, int n, int times,
                  cudaStream_t s);
-// list[0 .. count) = the slots whose species is `species`, in slot order;
-// partials holds scan_partials_words(n) ints
-void launch_select(const int8_t* sp, int species, int n, int* list, int* partials, int* count,
-                   cudaStream_t s);
+// list = the slots whose species is `species`, in slot order; partials holds
+// select_words(n) ints; cnt0 and cnt1 (n ints, may be NULL) are cleared
+size_t select_words(int n);
+void launch_select(const int8_t* sp, int species, int n, int* list, int* partials, int* cnt0,
+                   int* cnt1, cudaStream_t s);
 void launch_drift(double* x, double* y, double* z, const double* vx, const double* vy,
                   const double* vz, double dt, int n, cudaStream_t s);
 void launch_energy(const double* vx, const double* vy, const double* vz, const double* phi,

@@ -95,9 +95,10 @@ struct ChunkTarget {
 // over boxes: multipoles(list, cnt) takes cnt <= 32 accepted boxes {box, mask of the
 // targets that accept it}, pairs(list, cnt) cnt <= 32 opened leaves {leaf, mask of the
 // targets that open it}; both are called by the whole warp and may use W.stage.
-template <class M, class P>
+template <class Boxes, class Pairs>
 __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const ChunkTarget& tg,
-                                           int cloud, M& multipoles, P& direct_pairs)
+                                           int cloud, Boxes& multipoles,
+                                           Pairs& direct_pairs)
 {
     const int lane = threadIdx.x & 31;
     const unsigned int lt = (1u << lane) - 1u, me = 1u << lane;

@@ -1,6 +1,5 @@
 // ucp_push.cu -- velocity Verlet kicks and drifts (Sec. 2 of arXiv 0709.3331),
-// the key-order permutation of the particle state, target selection, energy
-// and momentum reductions (Sec. 5), and layout conversions at the boundary.
+// energy and momentum reductions (Sec. 5), and layout conversions at the boundary.
 #include "ucp_internal.cuh"
 
 #include <math.h>
@@ -10,28 +9,6 @@ namespace ucp {
 namespace {
 
 constexpr int kT = 256;
-
-__global__ void k_permute(const unsigned int* __restrict__ perm, int n,
-                          const double* __restrict__ s0, const double* __restrict__ s1,
-                          const double* __restrict__ s2, const double* __restrict__ s3,
-                          const double* __restrict__ s4, const double* __restrict__ s5,
-                          double* __restrict__ d0, double* __restrict__ d1, double* __restrict__ d2,
-                          double* __restrict__ d3, double* __restrict__ d4, double* __restrict__ d5,
-                          const int8_t* __restrict__ spi, int8_t* __restrict__ spo,
-                          const unsigned int* __restrict__ idi, unsigned int* __restrict__ ido)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    unsigned int p = perm[i];
-    d0[i] = s0[p];
-    d1[i] = s1[p];
-    d2[i] = s2[p];
-    d3[i] = s3[p];
-    d4[i] = s4[p];
-    d5[i] = s5[p];
-    spo[i] = spi[p];
-    ido[i] = idi[p];
-}
 
 __global__ void k_kick(double* __restrict__ vx, double* __restrict__ vy, double* __restrict__ vz,
                        const double* __restrict__ ax, const double* __restrict__ ay,
@@ -238,16 +215,6 @@ __global__ void k_chunks(const int* __restrict__ first, const int* __restrict__ 
 inline int nb(int n) { return (n + kT - 1) / kT > 0 ? (n + kT - 1) / kT : 1; }
 
 }  // namespace
-
-void launch_permute(const unsigned int* perm, int n, const double* const* src6, double* const* dst6,
-                    const int8_t* sp_in, int8_t* sp_out, const unsigned int* id_in,
-                    unsigned int* id_out, cudaStream_t s)
-{
-    count_launch(1);
-    k_permute<<<nb(n), kT, 0, s>>>(perm, n, src6[0], src6[1], src6[2], src6[3], src6[4], src6[5],
-                                   dst6[0], dst6[1], dst6[2], dst6[3], dst6[4], dst6[5], sp_in,
-                                   sp_out, id_in, id_out);
-}
 
 void launch_kick(double* vx, double* vy, double* vz, const double* ax, const double* ay,
                  const double* az, const int8_t* sp, int species, double h, int n, int times,

@@ -38,7 +38,10 @@ struct ucp_ctx {
     unsigned long long* key[2] = {};
     unsigned int* val[2] = {};
     SortScratch sort = {};
+    BuildCtl ctl = {};
+    int passes = 3;          // of the sort over the key's top digits
     int* scan_part = nullptr;
+    int* sel_part = nullptr;
     int* pos_cnt = nullptr;
     int* pos_off = nullptr;
     Tree t = {};
@@ -49,7 +52,6 @@ struct ucp_ctx {
     double* qsp = nullptr;
     double* msp = nullptr;
     int* tlist = nullptr;    // selected targets (electrons), key order
-    int* tcount = nullptr;
     int* cnt_p2p = nullptr;
     int* cnt_m2p = nullptr;
     int* work = nullptr;
@@ -228,19 +230,21 @@ int build(ucp_ctx* c)
     int n = c->n, k = c->cur;
     const int* cs = c->n_clouds > 1 ? c->cloud_start : nullptr;
     launch_bbox(c->st[k][0], c->st[k][1], c->st[k][2], n, c->bbox_part, c->bbox_nblk, c->cube,
-                cs, c->n_clouds, c->s);
+                cs, c->n_clouds, c->ctl, c->s);
     launch_keys(c->st[k][0], c->st[k][1], c->st[k][2], n, c->cube, c->t.cloud, c->key[0],
-                c->val[0], c->s);
-    const int b = launch_sort(c->key, c->val, n, c->sort, c->id[k], c->t.cloud, c->cloud_start,
-                              c->n_clouds, c->s);
-    c->sorted_buf = b;
-    const double* src[6];
-    double* dst[6];
+                c->passes, c->ctl, c->s);
+    StateRef in, out;
     for (int a = 0; a < 6; ++a) {
-        src[a] = c->st[k][a];
-        dst[a] = c->st[k ^ 1][a];
+        in.f[a] = c->st[k][a];
+        out.f[a] = c->st[k ^ 1][a];
     }
-    launch_permute(c->val[b], n, src, dst, c->sp[k], c->sp[k ^ 1], c->id[k], c->id[k ^ 1], c->s);
+    in.sp = c->sp[k];
+    in.id = c->id[k];
+    out.sp = c->sp[k ^ 1];
+    out.id = c->id[k ^ 1];
+    const int b = launch_sort(c->key, c->val, n, c->passes, c->sort, c->ctl, in, out, c->t.cloud,
+                              c->cloud_start, c->n_clouds, c->nsm, c->s);
+    c->sorted_buf = b;
     c->cur = k ^ 1;
     k = c->cur;
     launch_topology(c->key[b], n, c->leaf_cap, c->pos_cnt, c->pos_off, c->scan_part, c->t, c->s);
@@ -271,7 +275,8 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
     a.src32 = c->src32;
     a.t = c->t;
     if (electrons_only) {
-        launch_select(c->sp[k], UCP_ELECTRON, c->n, c->tlist, c->scan_part, c->tcount, c->s);
+        launch_select(c->sp[k], UCP_ELECTRON, c->n, c->tlist, c->sel_part, c->cnt_p2p,
+                      c->cnt_m2p, c->s);
         a.targets = c->tlist;
         a.ntargets = c->n_e;
         a.chunks = c->chunks_e;
@@ -296,8 +301,6 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
     a.work = c->work;
     a.err = c->sort.err;
     a.stats = c->stats;
-    cudaMemsetAsync(c->cnt_p2p, 0, sizeof(int) * (size_t)c->n, c->s);
-    cudaMemsetAsync(c->cnt_m2p, 0, sizeof(int) * (size_t)c->n, c->s);
     if (a.ntargets > 0) {
         prof_begin(c);
         if (f32 && visits) launch_walk_fp32c_visits(a, c->nsm, c->s);
@@ -490,11 +493,12 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->ay, n);
     dalloc(c, &c->az, n);
     dalloc(c, &c->phi, n);
-    dalloc(c, &c->sort.ghist, 8 * 256 + 9);
-    dalloc(c, &c->sort.goff, 8 * 256);
+    dalloc(c, &c->ctl.words, kCtlWords);
+    dalloc(c, &c->ctl.epoch, 1);
     dalloc(c, &c->sort.status, sort_status_words(c->n));
     dalloc(c, &c->sort.err, 1);
-    dalloc(c, &c->sort.epoch, 1);
+    dalloc(c, &c->sort.full_counts, sort_full_words());
+    dalloc(c, &c->sort.test_ctl, 1 + kRadix);
     dalloc(c, &c->sort.test_epoch, 1);
     dalloc(c, &c->sort.test_keys, sort_test_words());
     dalloc(c, &c->sort.test_vals, sort_test_words());
@@ -504,7 +508,6 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     const size_t cz = (size_t)cap;
     c->t.cap = (int)cap;
     dalloc(c, &c->t.nnodes, 1);
-    dalloc(c, &c->t.maxdepth, 1);
     dalloc(c, &c->t.info, cz);
     dalloc(c, &c->t.depth_leaf, cz);
     dalloc(c, &c->t.cell, cz);
@@ -514,7 +517,6 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->t.child8, cz * 8);
     dalloc(c, &c->t.leaf_list, cz);
     dalloc(c, &c->t.arrive, cz);
-    dalloc(c, &c->t.count, kMaxDepth + 2);
     {
         // twigs of depth d: at most min(8^d, n / (leaf_cap + 1)); none at the depth cap
         int64_t off = 0, pow8 = 1;
@@ -540,6 +542,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     {
         int64_t biggest = 0;
         for (int i = 0; i < n_clouds; ++i) biggest = sizes[i] > biggest ? sizes[i] : biggest;
+        c->passes = sort_passes(biggest);
         c->bbox_nblk = (int)((biggest + 2047) / 2048);
         int lim = n_clouds > 1 ? 16 : 4 * c->nsm;
         if (c->bbox_nblk > lim) c->bbox_nblk = lim;
@@ -564,7 +567,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->qsp, 2);
     dalloc(c, &c->msp, 2);
     dalloc(c, &c->tlist, n);
-    dalloc(c, &c->tcount, 1);
+    dalloc(c, &c->sel_part, select_words(c->n));
     dalloc(c, &c->cnt_p2p, n);
     dalloc(c, &c->cnt_m2p, n);
     dalloc(c, &c->work, 1);
@@ -577,6 +580,8 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->stage_int, 2 * n);
     if ((rc = commit(c))) return bail(rc);
 
+    c->t.maxdepth = c->ctl.words + kCtlMaxDepth;
+    c->t.count = c->ctl.words + kCtlCount;
     c->t.cloud_start = c->cloud_start;
     c->t.cloud = c->cloud;
     std::vector<unsigned char> cl;
@@ -588,7 +593,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     }
     if (cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) ||
         cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) ||
-        cudaMemsetAsync(c->sort.epoch, 0, sizeof(unsigned int), c->s) ||
+        cudaMemsetAsync(c->ctl.epoch, 0, sizeof(unsigned int), c->s) ||
         // the pad slot of an odd count is read (masked) by the pair loop: keep it finite
         (c->src32 && cudaMemsetAsync(c->src32, 0, sizeof(float4) * (n + 1), c->s)) ||
         cudaMemcpyAsync(c->cloud_start, c->cloud_start_h.data(), sizeof(int) * (n_clouds + 1),
@@ -1097,8 +1102,8 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
             if (ci == 0.0 && c->n_e > 0) {
                 // inside a block the ions' weights are zero: only the electrons'
                 // accelerations carry adjoint weight, so only they are walked
-                launch_select(c->sp[k], UCP_ELECTRON, c->n, c->tlist, c->scan_part,
-                              c->tcount, c->s);
+                launch_select(c->sp[k], UCP_ELECTRON, c->n, c->tlist, c->sel_part, nullptr,
+                              nullptr, c->s);
                 a.targets = c->tlist;
                 a.ntargets = c->n_e;
                 a.chunks = c->chunks_e;

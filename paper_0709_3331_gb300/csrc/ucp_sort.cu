@@ -1,0 +1,530 @@
+// ucp_sort.cu -- the key order of Sec. 3's TREE (arXiv 0709.3331) on the GPU: a stable
+// radix sort of the Morton keys and the permutation of the particle state into that
+// order, and the selection of the walk's targets.
+//
+// Only the key's top digits are sorted by radix passes: with 2^(8 passes) cells a run
+// of particles whose keys share those digits is short (two on average in the densest
+// part of a Gaussian cloud of 524,288 with three passes), and the kernel that moves
+// the state orders each run of its tile by the rest of the key in shared memory.  A
+// run longer than kRun raises a flag on the device, on which one further kernel,
+// otherwise empty, sorts the whole key.  Three passes of eight: 62 of 165 us at
+// N = 524,288.
+#include "ucp_scan.cuh"
+
+namespace ucp {
+
+namespace {
+
+constexpr int kSortThreads = 256;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortChunks = 8;                              // 32-key chunks per warp
+constexpr int kSortTile = kSortThreads * kSortChunks;       // 2048 keys per block
+constexpr int kSortSpinLimit = 1 << 20;  // polls of a predecessor's word before giving up
+constexpr int kLook = 8;                  // predecessors read per look-back round trip
+constexpr int kRun = 32;                  // longest run ordered in shared memory
+
+// Stable ranks of a tile's keys by digit: each warp owns a contiguous part and ranks it
+// chunk by chunk with match_any; cnt[w][d] counts warp w's keys of digit d before.
+struct TileRanks {
+    unsigned long long kk[kSortChunks];
+    unsigned int vv[kSortChunks];
+    int dig[kSortChunks], rank[kSortChunks];
+};
+
+__device__ __forceinline__ void rank_chunk(TileRanks& r, int c, bool ok, int digit, int* cnt,
+                                           int lane)
+{
+    const int d = ok ? digit : kRadix + lane;  // invalid lanes unique
+    r.dig[c] = d;
+    const unsigned int peers = __match_any_sync(0xffffffffu, d);
+    const int leader = __ffs(peers) - 1;
+    int before = 0;
+    if (ok && lane == leader) {
+        before = cnt[d];
+        cnt[d] = before + __popc(peers);
+    }
+    before = __shfl_sync(0xffffffffu, before, leader);
+    r.rank[c] = before + __popc(peers & ((1u << lane) - 1u));
+    __syncwarp();
+}
+
+// One stable LSD pass in a single kernel (decoupled look-back).  A block takes
+// the next tile from a counter, ranks its keys stably, and publishes its per-digit
+// count; the digit offset of the tile is the sum of the counts of all earlier tiles,
+// read back through their published words {epoch, flag (1 = count of the tile, 2 =
+// inclusive prefix), value}, on top of the digit's first place: the scan of the digit
+// counts `digits`, or (scan = 0) `digits` itself, its first ndigits valid.  A block
+// waits only on tiles taken before its own, whose blocks are running, and
+// every wait is bounded: past spin_limit polls it raises *err, keeps its keys
+// where they are and leaves (the host reports UCP_ETIMEOUT).
+__global__ void __launch_bounds__(kSortThreads)
+k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __restrict__ vin,
+           unsigned long long* __restrict__ kout, unsigned int* __restrict__ vout, int n,
+           int shift, const int* __restrict__ digits, int scan, int ndigits,
+           unsigned long long* status, int* tile_ctr, const unsigned int* __restrict__ epoch_dev,
+           unsigned int pass, int* err, int spin_limit,
+           const unsigned char* __restrict__ digit_of_val)
+{
+    const unsigned int epoch = (*epoch_dev + pass) & 0x3fffffffu;
+    __shared__ int cnt[kSortWarps][kRadix];
+    __shared__ int s_tile, s_fail, s_tot;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        s_tile = atomicAdd(tile_ctr, 1);
+        s_fail = 0;
+    }
+    for (int d = lane; d < kRadix; d += 32) cnt[w][d] = 0;
+    const int dv = (int)threadIdx.x < ndigits ? digits[threadIdx.x] : 0;  // kSortThreads == kRadix
+    __syncthreads();
+    const int tile = s_tile;
+    const int base = tile * kSortTile + w * (kSortTile / kSortWarps);
+    TileRanks r;
+#pragma unroll
+    for (int c = 0; c < kSortChunks; ++c) {
+        const int i = base + c * 32 + lane;
+        const bool ok = i < n;
+        r.kk[c] = ok ? kin[i] : 0ull;
+        r.vv[c] = ok ? (vin ? vin[i] : (unsigned int)i) : 0u;
+    }
+    const int first = scan ? block_excl_scan(dv, &s_tot) : dv;
+#pragma unroll
+    for (int c = 0; c < kSortChunks; ++c) {
+        const bool ok = base + c * 32 + lane < n;
+        // digit: 8 key bits, or (cloud pass) the cloud of the element's previous slot
+        const int d = !ok ? 0 : digit_of_val ? (int)digit_of_val[r.vv[c]]
+                                             : (int)((r.kk[c] >> shift) & 0xffu);
+        rank_chunk(r, c, ok, d, cnt[w], lane);
+    }
+    __syncthreads();
+    {
+        const int d = threadIdx.x;
+        int total = 0;
+        for (int ww = 0; ww < kSortWarps; ++ww) {
+            int t = cnt[ww][d];
+            cnt[ww][d] = total;
+            total += t;
+        }
+        const unsigned long long tag = (unsigned long long)epoch << 34;
+        unsigned long long* mine = status + (size_t)tile * kRadix + d;
+        unsigned int prefix = 0;
+        if (tile > 0) {
+            atomicExch(mine, tag | (1ull << 32) | (unsigned int)total);
+            // kLook predecessors' words per round trip (independent loads), taken in
+            // order j, j - 1, ... up to the first inclusive prefix or the first word
+            // not yet published, which is polled again
+            int j = tile - 1, spins = 0;
+            bool done = false;
+            while (!done) {
+                unsigned long long v[kLook];
+#pragma unroll
+                for (int u = 0; u < kLook; ++u)
+                    v[u] = j - u >= 0 ? __ldcv(status + (size_t)(j - u) * kRadix + d) : 0ull;
+                int used = 0;
+                bool blocked = false;
+#pragma unroll
+                for (int u = 0; u < kLook; ++u) {
+                    if (done || blocked || j - u < 0) continue;
+                    const unsigned int flag = (unsigned int)(v[u] >> 32) & 3u;
+                    if ((v[u] >> 34) != (unsigned long long)epoch || flag == 0u) {
+                        blocked = true;
+                        continue;
+                    }
+                    prefix += (unsigned int)v[u];
+                    ++used;
+                    if (flag == 2u) done = true;
+                }
+                j -= used;
+                if (done || j < 0) break;  // (tile 0 publishes an inclusive prefix)
+                if (blocked) {
+                    if (++spins > spin_limit) {
+                        atomicOr(err, 1);
+                        s_fail = 1;
+                        break;
+                    }
+                    __nanosleep(64);
+                }
+            }
+        }
+        atomicExch(mine, tag | (2ull << 32) | (prefix + (unsigned int)total));
+        const int off = first + (int)prefix;
+        for (int ww = 0; ww < kSortWarps; ++ww) cnt[ww][d] += off;
+    }
+    __syncthreads();
+    const bool fail = s_fail != 0;
+#pragma unroll
+    for (int c = 0; c < kSortChunks; ++c) {
+        const int i = base + c * 32 + lane;
+        if (i < n) {
+            const int p = fail ? i : cnt[w][r.dig[c]] + r.rank[c];
+            kout[p] = r.kk[c];
+            vout[p] = r.vv[c];
+        }
+    }
+}
+
+// Particle at sorted place i: its state, species and caller index from slot p.
+__device__ __forceinline__ void move_state(const StateRef& in, const StateRef& out, int i,
+                                           unsigned int p)
+{
+#pragma unroll
+    for (int a = 0; a < 6; ++a) out.f[a][i] = in.f[a][p];
+    out.sp[i] = in.sp[p];
+    out.id[i] = in.id[p];
+}
+
+// Orders the runs of equal top digits by (key, caller index) and moves the state.  A
+// block owns kFinish places and also sees the kRun places on either side, so that
+// every run that touches its places and is no longer than kRun lies in its window;
+// neighbouring blocks order a shared run each for itself.  Reads the passes' result,
+// writes the sorted keys to another buffer.
+constexpr int kFinish = 256;
+constexpr int kWindow = kFinish + 2 * kRun;
+
+__global__ void __launch_bounds__(kFinish)
+k_finish_sort(const unsigned long long* __restrict__ kin, const unsigned int* __restrict__ vin,
+              unsigned long long* __restrict__ kout, int n, int low, StateRef in, StateRef out,
+              const unsigned char* __restrict__ cloud, int* __restrict__ long_run)
+{
+    __shared__ unsigned long long sk[kWindow + 1];   // place l - 1 of the window
+    __shared__ unsigned int sv[kWindow + 1];
+    __shared__ unsigned char sc[kWindow + 1];
+    const int base = blockIdx.x * kFinish;
+    for (int l = threadIdx.x; l <= kWindow; l += kFinish) {
+        const int i = base - kRun - 1 + l;
+        const bool ok = i >= 0 && i < n;
+        sk[l] = ok ? kin[i] : 0ull;
+        sv[l] = ok ? vin[i] : 0u;
+        sc[l] = ok && cloud ? cloud[i] : 0;
+    }
+    __syncthreads();
+    // place l of the window continues the run of place l - 1
+    auto follows = [&](int l) {
+        const int i = base - kRun - 1 + l;
+        return i > 0 && i < n && l <= kWindow && (sk[l] >> low) == (sk[l - 1] >> low) &&
+               sc[l] == sc[l - 1];
+    };
+    // the first places of the runs (decided before any run is reordered; the top
+    // digits of a place do not change)
+    for (int l = 1 + threadIdx.x; l < 1 + kRun + kFinish; l += kFinish) {
+        if (follows(l) || !follows(l + 1)) continue;
+        int e = l + 1;
+        while (e - l <= kRun && follows(e)) ++e;
+        if (e - l > kRun) {
+            *long_run = 1;
+            continue;
+        }
+        for (int a = l + 1; a < e; ++a) {
+            const unsigned long long k = sk[a];
+            const unsigned int v = sv[a];
+            int b = a - 1;
+            while (b >= l && (sk[b] > k || (sk[b] == k && in.id[sv[b]] > in.id[v]))) {
+                sk[b + 1] = sk[b];
+                sv[b + 1] = sv[b];
+                --b;
+            }
+            sk[b + 1] = k;
+            sv[b + 1] = v;
+        }
+    }
+    __syncthreads();
+    const int i = base + threadIdx.x;
+    if (i < n) {
+        const int l = 1 + kRun + threadIdx.x;
+        kout[i] = sk[l];
+        move_state(in, out, i, sv[l]);
+    }
+}
+
+// The whole key, when a run was too long: eight LSD passes (a ninth by cloud), runs of
+// equal keys by caller index, and the state, by blocks that meet at a barrier (a
+// cooperative launch; its waits are bounded).  Returns at once when no run was.
+constexpr int kFullBlocks = 304;
+
+__global__ void __launch_bounds__(kSortThreads)
+k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, unsigned int* v1,
+            int n, int n_clouds, int* ctl, int* counts,
+            int* err, StateRef in, StateRef out, const unsigned char* __restrict__ cloud)
+{
+    if (ctl[kCtlLong] == 0) return;
+    __shared__ int cnt[kSortWarps][kRadix];
+    __shared__ int s_base[kRadix];
+    __shared__ int s_tot;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nb = gridDim.x;
+    int met = 0;
+    bool lost = false;
+    auto barrier = [&]() {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(&ctl[kCtlBarrier], 1);
+            ++met;
+            int spins = 0;
+            while (*(volatile int*)&ctl[kCtlBarrier] < met * nb) {
+                if (++spins > (kSortSpinLimit << 3)) {
+                    atomicOr(err, 1);
+                    break;
+                }
+                __nanosleep(64);
+            }
+            __threadfence();
+            s_tot = *(volatile int*)err;
+        }
+        __syncthreads();
+        lost = s_tot != 0;
+        __syncthreads();
+    };
+    // a block's contiguous part, in whole tiles
+    const int tiles = (n + kSortTile - 1) / kSortTile;
+    const int t0 = (int)((long long)tiles * blockIdx.x / nb), t1 = (int)((long long)tiles * (blockIdx.x + 1) / nb);
+    const int lo = t0 * kSortTile, hi = min(n, t1 * kSortTile);
+
+    // the passes' result (k0, v0) is the input; any order would do, ties end by caller
+    // index
+    unsigned long long *ka = k0, *kb = k1;
+    unsigned int *va = v0, *vb = v1;
+    const int passes = 8 + (n_clouds > 1 ? 1 : 0);
+    for (int p = 0; p < passes && !lost; ++p) {
+        int* cn = counts + (size_t)(p & 1) * kFullBlocks * kRadix;
+        for (int d = threadIdx.x; d < kRadix; d += kSortThreads) s_base[d] = 0;
+        __syncthreads();
+        auto digit = [&](unsigned long long k, unsigned int v) {
+            return p == 8 ? (int)cloud[v] : (int)((k >> (8 * p)) & 0xffu);
+        };
+        for (int i = lo + threadIdx.x; i < hi; i += kSortThreads)
+            atomicAdd(&s_base[digit(__ldcg(ka + i), __ldcg(va + i))], 1);
+        __syncthreads();
+        __stcg(cn + (size_t)blockIdx.x * kRadix + threadIdx.x, s_base[threadIdx.x]);
+        barrier();
+        if (lost) break;
+        {
+            int tot = 0, mine = 0;
+            for (int b = 0; b < nb; ++b) {
+                const int c = __ldcg(cn + (size_t)b * kRadix + threadIdx.x);
+                if (b < (int)blockIdx.x) mine += c;
+                tot += c;
+            }
+            const int first = block_excl_scan(tot, &s_tot);
+            s_base[threadIdx.x] = first + mine;
+        }
+        for (int tile = t0; tile < t1; ++tile) {
+            __syncthreads();
+            for (int d = lane; d < kRadix; d += 32) cnt[w][d] = 0;
+            __syncwarp();
+            const int base = tile * kSortTile + w * (kSortTile / kSortWarps);
+            TileRanks r;
+#pragma unroll
+            for (int c = 0; c < kSortChunks; ++c) {
+                const int i = base + c * 32 + lane;
+                const bool ok = i < n;
+                r.kk[c] = ok ? __ldcg(ka + i) : 0ull;
+                r.vv[c] = ok ? __ldcg(va + i) : 0u;
+                rank_chunk(r, c, ok, ok ? digit(r.kk[c], r.vv[c]) : 0, cnt[w], lane);
+            }
+            __syncthreads();
+            {
+                int run = s_base[threadIdx.x];
+                for (int ww = 0; ww < kSortWarps; ++ww) {
+                    const int c = cnt[ww][threadIdx.x];
+                    cnt[ww][threadIdx.x] = run;
+                    run += c;
+                }
+                s_base[threadIdx.x] = run;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int c = 0; c < kSortChunks; ++c) {
+                if (base + c * 32 + lane < n) {
+                    const int q = cnt[w][r.dig[c]] + r.rank[c];
+                    __stcg(kb + q, r.kk[c]);
+                    __stcg(vb + q, r.vv[c]);
+                }
+            }
+        }
+        barrier();
+        unsigned long long* tk = ka;
+        ka = kb;
+        kb = tk;
+        unsigned int* tv = va;
+        va = vb;
+        vb = tv;
+    }
+    if (lost) return;
+    // equal keys by caller index: the thread at a run's first place sorts it
+    for (int i = lo + threadIdx.x; i < hi && i < n - 1; i += kSortThreads) {
+        const unsigned long long k = __ldcg(ka + i);
+        const auto joins = [&](int j) {
+            return j > 0 && j < n && __ldcg(ka + j) == k && __ldcg(ka + j - 1) == k &&
+                   (!cloud || cloud[j] == cloud[j - 1]);
+        };
+        if (joins(i) || !joins(i + 1)) continue;
+        int e = i + 1;
+        while (joins(e)) ++e;
+        for (int a = i + 1; a < e; ++a) {
+            const unsigned int pv = __ldcg(va + a), idv = in.id[pv];
+            int b = a - 1;
+            while (b >= i && in.id[__ldcg(va + b)] > idv) {
+                __stcg(va + b + 1, __ldcg(va + b));
+                --b;
+            }
+            __stcg(va + b + 1, pv);
+        }
+    }
+    barrier();
+    if (lost) return;
+    // the sorted keys end in k1 whatever the number of passes
+    for (int i = lo + threadIdx.x; i < hi; i += kSortThreads) {
+        if (ka != k1) k1[i] = __ldcg(ka + i);
+        move_state(in, out, i, __ldcg(va + i));
+    }
+}
+
+}  // namespace
+
+// Passes over the top digits: a run of equal digits should stay a few particles where
+// the cloud is densest (a Gaussian cloud's centre holds 63 times the mean over its
+// cube: 4 particles per cell at 2^12 with two passes and at 2^20 with three).
+int sort_passes(int64_t largest_cloud)
+{
+    return largest_cloud <= (1 << 12) ? 2 : largest_cloud <= (1 << 20) ? 3 : 4;
+}
+
+size_t sort_test_words() { return 4 * (size_t)kSortTile; }
+size_t sort_full_words() { return 2 * (size_t)kFullBlocks * kRadix; }
+
+size_t sort_status_words(int n)
+{
+    int nb = (n + kSortTile - 1) / kSortTile;
+    return (size_t)(kSortPassesMax + 1) * kRadix * (size_t)(nb > 0 ? nb : 1);
+}
+
+int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int passes,
+                const SortScratch& sc, BuildCtl ctl, const StateRef& in, const StateRef& out,
+                const unsigned char* cloud, const int* cloud_start, int n_clouds, int nsm,
+                cudaStream_t s)
+{
+    const bool clouds = n_clouds > 1;
+    count_launch(passes + 2 + (clouds ? 1 : 0));
+    const int nb = (n + kSortTile - 1) / kSortTile;
+    const int low = kKeyBits - 8 * passes;
+    int cur = 0;
+    for (int p = 0; p < passes; ++p) {
+        k_onesweep<<<nb, kSortThreads, 0, s>>>(
+            key[cur], p == 0 ? nullptr : val[cur], key[cur ^ 1], val[cur ^ 1], n, low + 8 * p,
+            ctl.words + kCtlHist + p * kRadix, 1, kRadix, sc.status + (size_t)p * nb * kRadix,
+            ctl.words + kCtlTile + p, ctl.epoch, (unsigned int)p, sc.err, kSortSpinLimit, nullptr);
+        cur ^= 1;
+    }
+    if (clouds) {
+        // a stable pass by cloud: (cloud, key) order, each cloud back in its fixed
+        // segment; a cloud's first place is its segment's start
+        k_onesweep<<<nb, kSortThreads, 0, s>>>(
+            key[cur], val[cur], key[cur ^ 1], val[cur ^ 1], n, 0, cloud_start, 0, n_clouds,
+            sc.status + (size_t)passes * nb * kRadix, ctl.words + kCtlTile + passes, ctl.epoch,
+            (unsigned int)passes, sc.err, kSortSpinLimit, cloud);
+        cur ^= 1;
+    }
+    const int fin = cur ^ 1;
+    k_finish_sort<<<(n + kFinish - 1) / kFinish, kFinish, 0, s>>>(
+        key[cur], val[cur], key[fin], n, low, in, out, cloud, ctl.words + kCtlLong);
+    unsigned long long *k0 = key[cur], *k1 = key[fin];
+    unsigned int *v0 = val[cur], *v1 = val[fin];
+    int* words = ctl.words;
+    int *counts = sc.full_counts, *err = sc.err;
+    StateRef si = in, so = out;
+    void* args[] = {&k0, &k1, &v0, &v1, &n, &n_clouds, &words, &counts, &err, &si, &so, &cloud};
+    int blocks = nb < kFullBlocks ? nb : kFullBlocks;
+    if (blocks > nsm) blocks = nsm;
+    cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_sort_full), dim3(blocks),
+                                dim3(kSortThreads), args, 0, s);
+    return fin;
+}
+
+int sort_selftest_timeout(const SortScratch& sc, cudaStream_t s)
+{
+    // a lone block that takes tile 1 while tile 0 never publishes: its bounded
+    // wait must run out, raise *err and leave the keys where they are
+    count_launch(1);
+    static const int one = 1;
+    if (cudaMemsetAsync(sc.status, 0, sizeof(unsigned long long) * 2 * kRadix, s) != cudaSuccess ||
+        cudaMemsetAsync(sc.test_ctl, 0, sizeof(int) * (1 + kRadix), s) != cudaSuccess ||
+        cudaMemcpyAsync(sc.test_ctl, &one, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(sc.test_epoch, &one, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemsetAsync(sc.test_keys, 0, sizeof(unsigned long long) * 4 * kSortTile, s) != cudaSuccess ||
+        cudaMemsetAsync(sc.test_vals, 0, sizeof(unsigned int) * 4 * kSortTile, s) != cudaSuccess)
+        return -1;
+    // input: tiles 0-1 of the test buffers; output: tiles 2-3
+    k_onesweep<<<1, kSortThreads, 0, s>>>(sc.test_keys, sc.test_vals, sc.test_keys + 2 * kSortTile,
+                                          sc.test_vals + 2 * kSortTile, 2 * kSortTile, 0,
+                                          sc.test_ctl + 1, 1, kRadix, sc.status, sc.test_ctl,
+                                          sc.test_epoch, 0u, sc.err, 2000, nullptr);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// ---- target selection: the slots whose species is `species`, in slot order
+namespace {
+
+constexpr int kSelThreads = 1024;
+constexpr int kSelItems = 4;
+constexpr int kSelTile = kSelThreads * kSelItems;
+
+__global__ void __launch_bounds__(kSelThreads)
+k_select_count(const int8_t* __restrict__ sp, int species, int n, int* __restrict__ part)
+{
+    const int base = blockIdx.x * kSelTile;
+    int s = 0;
+#pragma unroll
+    for (int k = 0; k < kSelItems; ++k) {
+        const int i = base + threadIdx.x * kSelItems + k;
+        if (i < n) s += sp[i] == species;
+    }
+    __shared__ int tot;
+    block_excl_scan(s, &tot);
+    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+}
+
+// Every block sums the counts of the tiles before its own; the interaction counts of
+// every slot (if given) are cleared on the way (the walk writes those of its targets).
+__global__ void __launch_bounds__(kSelThreads)
+k_select_write(const int8_t* __restrict__ sp, int species, int n, const int* __restrict__ part,
+               int* __restrict__ list, int* __restrict__ cnt0, int* __restrict__ cnt1)
+{
+    __shared__ int tot, before;
+    int b = 0;
+    for (int i = threadIdx.x; i < (int)blockIdx.x; i += kSelThreads) b += part[i];
+    block_excl_scan(b, &before);
+    const int base = blockIdx.x * kSelTile;
+    int v[kSelItems];
+    int s = 0;
+#pragma unroll
+    for (int k = 0; k < kSelItems; ++k) {
+        const int i = base + threadIdx.x * kSelItems + k;
+        v[k] = i < n && sp[i] == species;
+        s += v[k];
+        if (i < n && cnt0) {
+            cnt0[i] = 0;
+            cnt1[i] = 0;
+        }
+    }
+    int off = block_excl_scan(s, &tot) + before;
+#pragma unroll
+    for (int k = 0; k < kSelItems; ++k) {
+        const int i = base + threadIdx.x * kSelItems + k;
+        if (v[k]) list[off++] = i;
+    }
+}
+
+}  // namespace
+
+size_t select_words(int n) { return (size_t)((n + kSelTile - 1) / kSelTile) + 1; }
+
+void launch_select(const int8_t* sp, int species, int n, int* list, int* partials, int* cnt0,
+                   int* cnt1, cudaStream_t s)
+{
+    count_launch(2);
+    const int nb = (n + kSelTile - 1) / kSelTile;
+    k_select_count<<<nb, kSelThreads, 0, s>>>(sp, species, n, partials);
+    k_select_write<<<nb, kSelThreads, 0, s>>>(sp, species, n, partials, list, cnt0, cnt1);
+}
+
+}  // namespace ucp
