@@ -518,9 +518,10 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
                                const double* __restrict__ qsp, Tree t,
                                const TA* __restrict__ adj, double* __restrict__ mu)
 {
-    const int nl = t.count[kMaxDepth + 1];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nl; i += gridDim.x * blockDim.x) {
-        const int leaf = t.leaf_list[i];
+    const int nn = *t.nnodes;
+    for (int leaf = blockIdx.x * blockDim.x + threadIdx.x; leaf < nn;
+         leaf += gridDim.x * blockDim.x) {
+        if (!(t.depth_leaf[leaf] & 256)) continue;
         double A[3] = {0, 0, 0}, G[6] = {0, 0, 0, 0, 0, 0}, Cc[3] = {0, 0, 0}, K[3] = {0, 0, 0};
         for (int nd = leaf; nd >= 0; nd = t.info[nd].w) {
             double r[12];
@@ -529,7 +530,8 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
             double c[3] = {m[MC], m[MC + 1], m[MC + 2]};
             double Gc[3];
             qmul(r + 3, c, Gc);
-            const double inv = m[MS0] > 0.0 ? 1.0 / m[MS0] : 0.0;
+            const double S0 = t.mom32 ? (double)t.mom32[(size_t)nd * 16 + 3] : m[MS0];
+            const double inv = S0 > 0.0 ? 1.0 / S0 : 0.0;
             for (int k = 0; k < 3; ++k) {
                 A[k] += r[k];
                 Cc[k] += Gc[k];

@@ -13,63 +13,6 @@ namespace ucp {
 
 namespace {
 
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-__global__ void k_scan_reduce(const int* __restrict__ in, int n, int* __restrict__ part)
-{
-    int base = blockIdx.x * kScanTile;
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int i = base + threadIdx.x * kScanItems + k;
-        if (i < n) s += in[i];
-    }
-    __shared__ int tot;
-    block_excl_scan(s, &tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-__global__ void k_scan_partials(int* part, int nb, int* total)
-{
-    // one block: each thread scans a contiguous chunk of the partials
-    int per = (nb + blockDim.x - 1) / blockDim.x;
-    int b0 = threadIdx.x * per;
-    int s = 0;
-    for (int b = b0; b < b0 + per && b < nb; ++b) s += part[b];
-    __shared__ int tot;
-    int off = block_excl_scan(s, &tot);
-    for (int b = b0; b < b0 + per && b < nb; ++b) {
-        int v = part[b];
-        part[b] = off;
-        off += v;
-    }
-    if (threadIdx.x == 0 && total) *total = tot;
-}
-
-__global__ void k_scan_apply(const int* __restrict__ in, int* __restrict__ out, int n,
-                             const int* __restrict__ part)
-{
-    int base = blockIdx.x * kScanTile;
-    int v[kScanItems];
-    int s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int i = base + threadIdx.x * kScanItems + k;
-        v[k] = i < n ? in[i] : 0;
-        s += v[k];
-    }
-    __shared__ int tot;
-    int off = block_excl_scan(s, &tot) + part[blockIdx.x];
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int i = base + threadIdx.x * kScanItems + k;
-        if (i < n) out[i] = off;
-        off += v[k];
-    }
-}
-
 // ---------------------------------------------------------------- cube
 // Ordered integer image of a finite double: comparing the images compares the
 // values, so min/max run on the integer ALU instead of the (scarce) FP64 pipe.
@@ -303,29 +246,19 @@ __device__ __forceinline__ void segment_of(const Tree& t, int n, int i, int& lo,
 // those of depth >= first_depth(i) down to the first leaf.  A box exists iff
 // its parent holds more than leaf_cap particles.  Emitting boxes in order of
 // (start position, depth) gives pre-order with children in octant order.
-__global__ void k_topo_count(const unsigned long long* __restrict__ K, int n, int leaf_cap,
-                             int* __restrict__ cnt, Tree t)
+__device__ int count_by_search(const unsigned long long* __restrict__ K, int lo, int hi, int i,
+                               int leaf_cap)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int lo, hi;
-    segment_of(t, n, i, lo, hi);
-    int d0 = first_depth(K, lo, i);
+    const int d0 = first_depth(K, lo, i);
+    if (d0 > kMaxDepth) return 0;
+    if (d0 > 0 && box_end(K, hi, i, d0 - 1) - box_begin(K, lo, i, d0 - 1) <= leaf_cap) return 0;
     int c = 0;
-    if (d0 <= kMaxDepth) {
-        bool ok = true;
-        if (d0 > 0) {
-            int pb = box_begin(K, lo, i, d0 - 1), pe = box_end(K, hi, i, d0 - 1);
-            ok = pe - pb > leaf_cap;
-        }
-        if (ok)
-            for (int d = d0; d <= kMaxDepth; ++d) {
-                int e = box_end(K, hi, i, d);
-                ++c;
-                if (e - i <= leaf_cap || d == kMaxDepth) break;
-            }
+    for (int d = d0; d <= kMaxDepth; ++d) {
+        const int e = box_end(K, hi, i, d);
+        ++c;
+        if (e - i <= leaf_cap || d == kMaxDepth) break;
     }
-    cnt[i] = c;
+    return c;
 }
 
 // ---- the same counts by a window of sorted positions (leaf_cap <= kTopoWin).
@@ -379,102 +312,163 @@ __device__ __forceinline__ int leaf_depth_win(const unsigned char* fd, int li, i
     return min(best, kMaxDepth);
 }
 
-__global__ void __launch_bounds__(kTopoThreads)
-k_topo_count_win(const unsigned long long* __restrict__ K, int n, int leaf_cap,
-                 int* __restrict__ cnt, Tree t)
-{
-    __shared__ unsigned char fd[kTopoThreads + 2 * kTopoWin];
-    const int base = blockIdx.x * kTopoThreads;
-    load_fd_window(K, t, n, base, fd);
-    __syncthreads();
-    const int i = base + threadIdx.x;
-    if (i >= n) return;
-    const int li = threadIdx.x + kTopoWin;
-    const int d0 = fd[li];
-    int c = 0;
-    if (d0 <= kMaxDepth) {
-        const int lv = leaf_depth_win(fd, li, leaf_cap);
-        if (lv >= d0) c = lv - d0 + 1;
-    }
-    cnt[i] = c;
-}
-
-// atomicAdd(ctr, 1) for every calling lane, one atomic per distinct counter in
-// the warp (the lanes that add to the same counter take consecutive slots)
-__device__ __forceinline__ int warp_inc(int* ctr)
-{
-    const unsigned int active = __activemask();
-    const unsigned int peers = __match_any_sync(active, (unsigned long long)ctr);
-    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(ctr, __popc(peers));
-    base = __shfl_sync(peers, base, leader);
-    return base + __popc(peers & ((1u << lane) - 1u));
-}
+// Box counts of every position and their exclusive prefix sums in one kernel
+// (decoupled look-back over tiles taken from a counter, as in the key sort; waits
+// bounded), which gives every box its place; a tile also clears the child slots and
+// arrival counters of the boxes that start in it.
+constexpr int kTopoSpinLimit = 1 << 20;
 
 template <bool kWin>
 __global__ void __launch_bounds__(kTopoThreads)
-k_topo_emit(const unsigned long long* __restrict__ K, int n, int leaf_cap,
-            const int* __restrict__ cnt, const int* __restrict__ off, Tree t)
+k_topo_scan(const unsigned long long* __restrict__ K, int n, int leaf_cap, int* __restrict__ cnt,
+            int* __restrict__ off, Tree t, BuildCtl ctl, unsigned long long* status, int* err)
 {
-    // with kWin the leaf's end comes from the window of first depths (a leaf
-    // holds at most leaf_cap <= kTopoWin positions unless it is a depth-cap box)
     __shared__ unsigned char fd[kWin ? kTopoThreads + 2 * kTopoWin : 1];
+    __shared__ int s_tile, s_tot, s_prefix;
+    if (threadIdx.x == 0) s_tile = atomicAdd(&ctl.words[kCtlTopoTile], 1);
+    __syncthreads();
+    const int tile = s_tile, base = tile * kTopoThreads;
+    const int i = base + threadIdx.x;
+    int c = 0;
     if (kWin) {
-        load_fd_window(K, t, n, blockIdx.x * kTopoThreads, fd);
+        load_fd_window(K, t, n, base, fd);
         __syncthreads();
-    }
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int c = cnt[i];
-    // the capacity bounds the box count of sorted keys; clamp in case it ever did not
-    int nn = min(*t.nnodes, t.cap);
-    if (i == 0 && *t.nnodes > t.cap) *t.nnodes = t.cap;
-    if (c == 0) return;
-    int lo, hi;
-    segment_of(t, n, i, lo, hi);
-    int d0 = first_depth(K, lo, i);
-    int node = off[i];
-    int parent = -1;
-    if (d0 > 0) {
-        int pb = box_begin(K, lo, i, d0 - 1);
-        parent = off[pb] + (d0 - 1 - first_depth(K, lo, pb));
-    }
-    int dmax = 0;
-    for (int j = 0; j < c; ++j) {
-        int d = d0 + j;
-        // the boxes above the last one at this position hold more than leaf_cap
-        // particles (the count stops at the first that does not): twigs, whose end
-        // and skip index are their last child's, filled in by the moments' bottom-up
-        // sweep; only the last box's end is looked up here
-        int e = -1, nx = -1;
-        bool leaf = false;
-        if (j == c - 1) {
-            if (kWin) {
-                // the leaf: its end within the window, else (a bigger depth-cap box) search
-                const int li = threadIdx.x + kTopoWin;
-                for (int m = 1; m <= leaf_cap && e < 0; ++m)
-                    if (fd[li + m] <= d) e = i + m;
-            }
-            if (e < 0) e = box_end(K, hi, i, d);
-            leaf = (e - i <= leaf_cap) || d == kMaxDepth;
-            nx = e < n ? off[e] : nn;
+        const int li = threadIdx.x + kTopoWin;
+        const int d0 = fd[li];
+        if (i < n && d0 <= kMaxDepth) {
+            const int lv = leaf_depth_win(fd, li, leaf_cap);
+            if (lv >= d0) c = lv - d0 + 1;
         }
-        if (node >= t.cap) break;  // cannot happen: the capacity bounds the box count
-        unsigned long long pre = prefix_at(K[i], d);
-        t.info[node] = make_int4(i, e, nx, parent);
-        t.depth_leaf[node] = d | (leaf ? 256 : 0);
-        t.cell[node] = pre;
-        if (parent >= 0) t.child8[(size_t)parent * 8 + (int)(pre & 7ull)] = node;
-        int* ctr = &t.count[leaf ? kMaxDepth + 1 : d];
-        const int slot = warp_inc(ctr);
-        if (leaf) t.leaf_list[slot] = node;
-        else t.twig_list[t.twig_off[d] + slot] = node;
-        parent = node;
-        ++node;
-        dmax = d;
+    } else if (i < n) {
+        int lo, hi;
+        segment_of(t, n, i, lo, hi);
+        c = count_by_search(K, lo, hi, i, leaf_cap);
     }
-    atomicMax(t.maxdepth, dmax);
+    const int before = block_excl_scan(c, &s_tot);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const unsigned int epoch = (*ctl.epoch + 15u) & 0x3fffffffu;
+        const unsigned long long tag = (unsigned long long)epoch << 34;
+        if (lane == 0 && tile > 0)
+            atomicExch(status + tile, tag | (1ull << 32) | (unsigned int)s_tot);
+        unsigned int prefix = 0;
+        int spins = 0;
+        for (int j = tile - 1; j >= 0;) {
+            // lane l reads the word of tile j - l (past the first tile: nothing, final)
+            const unsigned long long v = j - lane >= 0 ? __ldcv(status + (j - lane)) : tag | (2ull << 32);
+            const unsigned int flag = (v >> 34) == (unsigned long long)epoch
+                                          ? (unsigned int)(v >> 32) & 3u : 0u;
+            const unsigned int fin = __ballot_sync(0xffffffffu, flag == 2u);
+            const unsigned int none = __ballot_sync(0xffffffffu, flag == 0u);
+            // the lanes up to the first final word, all published?
+            const int last = fin ? __ffs(fin) - 1 : 31;
+            if (none & (0xffffffffu >> (31 - last))) {
+                if (++spins > kTopoSpinLimit) {
+                    if (lane == 0) atomicOr(err, 1);
+                    break;
+                }
+                __nanosleep(32);
+                continue;
+            }
+            unsigned int sum = lane <= last ? (unsigned int)v : 0u;
+            prefix += __reduce_add_sync(0xffffffffu, sum);
+            if (fin) break;
+            j -= 32;
+        }
+        if (lane == 0) {
+            atomicExch(status + tile, tag | (2ull << 32) | (prefix + (unsigned int)s_tot));
+            s_prefix = (int)prefix;
+        }
+    }
+    __syncthreads();
+    const int first = s_prefix, tot = s_tot;
+    if (i < n) {
+        cnt[i] = c;
+        off[i] = first + before;
+    }
+    // the capacity bounds the box count of sorted keys; clamp in case it ever did not
+    if (threadIdx.x == 0 && base + kTopoThreads >= n) *t.nnodes = min(first + tot, t.cap);
+    const int lim = min(first + tot, t.cap);
+    for (int b = first + threadIdx.x; b < lim; b += kTopoThreads) t.arrive[b] = 0;
+    int4* rows = reinterpret_cast<int4*>(t.child8);
+    for (int r = 2 * first + threadIdx.x; r < 2 * lim; r += kTopoThreads)
+        rows[r] = make_int4(-1, -1, -1, -1);
+}
+
+// The boxes that start at each position, with their parents.  The parent of the first
+// one, of depth d0 - 1, starts at the last earlier position whose first box is no
+// deeper: found in a table of minima of the first depths over 1, 2, 4, .. 256 positions
+// (nine steps in shared memory, 256 positions back), else by search.  A leaf ends where
+// the next box starts and skips to the next box; twigs take their end and skip from
+// their last child (the moments' bottom-up sweep).
+constexpr int kTopoLevels = 9;
+
+__global__ void __launch_bounds__(kTopoThreads)
+k_topo_emit(const unsigned long long* __restrict__ K, int n, const int* __restrict__ cnt,
+            const int* __restrict__ off, Tree t)
+{
+    __shared__ unsigned char mn[kTopoLevels][2 * kTopoThreads];
+    __shared__ unsigned int starts[kTopoThreads / 32];
+    __shared__ int s_depth;
+    const int base = blockIdx.x * kTopoThreads, i = base + threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int k = threadIdx.x; k < 2 * kTopoThreads; k += kTopoThreads)
+        mn[0][k] = (unsigned char)fd_at(K, t, n, base - kTopoThreads + k);
+    const int c = i < n ? cnt[i] : 0;
+    const unsigned int sb = __ballot_sync(0xffffffffu, c > 0);
+    if (lane == 0) starts[w] = sb;
+    if (threadIdx.x == 0) s_depth = 0;
+    for (int v = 1; v < kTopoLevels; ++v) {
+        __syncthreads();
+        const int h = 1 << (v - 1);
+        for (int k = threadIdx.x; k < 2 * kTopoThreads; k += kTopoThreads)
+            mn[v][k] = min(mn[v - 1][k], k >= h ? mn[v - 1][k - h] : (unsigned char)255);
+    }
+    __syncthreads();
+    if (c > 0) {
+        int lo, hi;
+        segment_of(t, n, i, lo, hi);
+        const int d0 = i == lo ? 0 : mn[0][kTopoThreads + threadIdx.x];
+        int parent = -1;
+        if (d0 > 0) {
+            int k = kTopoThreads + (int)threadIdx.x - 1;
+#pragma unroll
+            for (int v = kTopoLevels - 1; v >= 0; --v)
+                if (k - (1 << v) + 1 >= 0 && mn[v][k] >= d0) k -= 1 << v;
+            int pb, dp;
+            if (k >= 0) {
+                pb = base - kTopoThreads + k;
+                dp = pb == lo ? 0 : mn[0][k];
+            } else {
+                pb = box_begin(K, lo, i, d0 - 1);
+                dp = first_depth(K, lo, pb);
+            }
+            parent = off[pb] + (d0 - 1 - dp);
+        }
+        // the next start: in this warp, in a later warp of the block, or by search
+        int e = -1;
+        const unsigned int later = lane < 31 ? sb >> (lane + 1) : 0u;
+        if (later) e = i + __ffs(later);
+        for (int ww = w + 1; ww < kTopoThreads / 32 && e < 0; ++ww)
+            if (starts[ww]) e = base + ww * 32 + __ffs(starts[ww]) - 1;
+        if (e < 0) e = box_end(K, hi, i, d0 + c - 1);
+        int node = off[i];
+        for (int j = 0; j < c; ++j) {
+            if (node >= t.cap || parent >= t.cap) break;  // cannot happen: the capacity bounds the box count
+            const int d = d0 + j;
+            const bool leaf = j == c - 1;
+            const unsigned long long pre = prefix_at(K[i], d);
+            t.info[node] = make_int4(i, leaf ? e : -1, leaf ? node + 1 : -1, parent);
+            t.depth_leaf[node] = d | (leaf ? 256 : 0);
+            t.cell[node] = pre;
+            if (parent >= 0) t.child8[(size_t)parent * 8 + (int)(pre & 7ull)] = node;
+            parent = node;
+            ++node;
+        }
+        atomicMax(&s_depth, d0 + c - 1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_depth > 0) atomicMax(t.maxdepth, s_depth);
 }
 
 // ---------------------------------------------------------------- moments
@@ -541,63 +535,64 @@ __device__ __forceinline__ void finish_box(const double* a, const double z[3],
     m[MT] = -0.5 * (m[MQ] + m[MQ + 3] + m[MQ + 5]);
 }
 
-__global__ void k_clear_children(Tree t)
+// Sum over the eight lanes of a group by an xor butterfly, in every lane:
+// ((s0 + s4) + (s2 + s6)) + ((s1 + s5) + (s3 + s7)).
+template <class T>
+__device__ __forceinline__ T sum8(T v)
 {
-    const int nn = *t.nnodes;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x)
-        t.arrive[i] = 0;
-    const int total = nn * 8;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x)
-        t.child8[i] = -1;
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
 }
 
-// Moments of twig p (depth d) from its eight child slots in octant order, each
-// child's moments shifted to the twig's geometric centre.  The children were
-// written by other threads of the same launch: their records are read through
-// L2 (__ldcg) after the fence of the bottom-up sweep.
-__device__ void twig_combine_f64(const Cube* __restrict__ cube, const Tree& t, int p, int d)
+// Moments of twig p (depth d; p < 0: none) by a group of eight lanes, one child slot o
+// each (ch < 0: empty), the child's moments shifted to the twig's geometric centre.  The
+// children were written by other threads of the same launch: their records are read
+// through L2 (__ldcg) after the acquire of the bottom-up sweep.
+__device__ __forceinline__ void twig_combine_f64(const Cube* __restrict__ cube, const Tree& t,
+                                                 int p, int d, int o, int ch)
 {
-    const Cube cb = cube_of(cube, t, t.info[p].x);
-    double zp[3], ps;
-    box_centre(cb, t.cell[p], d, zp, &ps);
+    double zp[3] = {0, 0, 0}, ps;
+    if (p >= 0) box_centre(cube_of(cube, t, t.info[p].x), t.cell[p], d, zp, &ps);
     double a[14];
 #pragma unroll
     for (int k = 0; k < 14; ++k) a[k] = 0.0;
-#pragma unroll 1
-    for (int o = 0; o < 8; ++o) {
-        const int ch = t.child8[(size_t)p * 8 + o];
-        if (ch < 0) continue;
+    if (ch >= 0) {
         const double* cm = t.mom + (size_t)ch * kMom;
-        double S0k = __ldcg(cm + MS0), Mk = __ldcg(cm + MM);
+        const double S0k = __ldcg(cm + MS0), Mk = __ldcg(cm + MM);
         double e[3], dk[3], qk[6];
         for (int k = 0; k < 3; ++k) {
             e[k] = __ldcg(cm + MC + k) - zp[k];
             dk[k] = __ldcg(cm + MD + k);
         }
         for (int k = 0; k < 6; ++k) qk[k] = __ldcg(cm + MQ + k);
-        a[0] += S0k;
-        a[1] += Mk;
+        a[0] = S0k;
+        a[1] = Mk;
         for (int k = 0; k < 3; ++k) {
-            a[2 + k] += S0k * e[k];
-            a[5 + k] += dk[k] + Mk * e[k];
+            a[2 + k] = S0k * e[k];
+            a[5 + k] = dk[k] + Mk * e[k];
         }
         // Q_k + D_k e^T + e D_k^T + M_k e e^T
-        double me0 = Mk * e[0], me1 = Mk * e[1], me2 = Mk * e[2];
-        a[8] += qk[0] + (2.0 * dk[0] + me0) * e[0];
-        a[9] += qk[1] + dk[0] * e[1] + (dk[1] + me1) * e[0];
-        a[10] += qk[2] + dk[0] * e[2] + (dk[2] + me2) * e[0];
-        a[11] += qk[3] + (2.0 * dk[1] + me1) * e[1];
-        a[12] += qk[4] + dk[1] * e[2] + (dk[2] + me2) * e[1];
-        a[13] += qk[5] + (2.0 * dk[2] + me2) * e[2];
+        const double me0 = Mk * e[0], me1 = Mk * e[1], me2 = Mk * e[2];
+        a[8] = qk[0] + (2.0 * dk[0] + me0) * e[0];
+        a[9] = qk[1] + dk[0] * e[1] + (dk[1] + me1) * e[0];
+        a[10] = qk[2] + dk[0] * e[2] + (dk[2] + me2) * e[0];
+        a[11] = qk[3] + (2.0 * dk[1] + me1) * e[1];
+        a[12] = qk[4] + dk[1] * e[2] + (dk[2] + me2) * e[1];
+        a[13] = qk[5] + (2.0 * dk[2] + me2) * e[2];
     }
-    double rec[kMom];
-    finish_box(a, zp, rec, t.delta + p);
-    double* pm = t.mom + (size_t)p * kMom;
 #pragma unroll
-    for (int k = 0; k < kMom; ++k) pm[k] = rec[k];
+    for (int k = 0; k < 14; ++k) a[k] = sum8(a[k]);
+    if (p >= 0 && o == 0) {
+        double rec[kMom];
+        finish_box(a, zp, rec, t.delta + p);
+        double* pm = t.mom + (size_t)p * kMom;
+#pragma unroll
+        for (int k = 0; k < kMom; ++k)
+            if (k != MR2) pm[k] = rec[k];
+    }
 }
-
-constexpr int kMomThreads = 64;  // threads per block of the leaf kernels
 
 // atomicAdd with acquire-release semantics at device scope: the caller's
 // earlier writes are visible to whoever reads the counter after it (release),
@@ -612,101 +607,143 @@ __device__ __forceinline__ int atomic_add_acq_rel(int* ctr, int v)
     return old;
 }
 
-// Bottom-up sweep from a finished box: each box counts its finished children
-// (t.arrive, zeroed before the launch); the thread that finishes the last child
-// combines the parent and carries on upwards.  No thread waits for another, and
-// every twig is combined once, from all its children, whichever thread does it.
+// Bottom-up sweep from the finished boxes of a warp's lanes (node < 0: none): each box
+// counts its finished children (t.arrive, cleared with the topology); the lane that
+// finishes the last child has the parent combined, four parents at a time by groups of
+// eight lanes, and carries on upwards.  No thread waits for another, and every twig is
+// combined once, from all its children, whichever warp does it.
 template <class Combine>
 __device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combine)
 {
-    int p = t.info[node].w;
-    while (p >= 0) {
-        int nch = 0, last = -1;
+    const int lane = threadIdx.x & 31;
+    int p = node >= 0 ? t.info[node].w : -1;
+    while (__any_sync(0xffffffffu, p >= 0)) {
+        // this box's records (written by any lane of the warp) are published with its
+        // arrival; the last arrival sees every sibling's
+        __syncwarp();
+        bool ready = false;
+        if (p >= 0) {
+            const int4* row = reinterpret_cast<const int4*>(t.child8 + (size_t)p * 8);
+            const int4 r0 = row[0], r1 = row[1];
+            const int ch[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+            int nch = 0, last = -1;
 #pragma unroll
-        for (int o = 0; o < 8; ++o) {
-            const int ch = t.child8[(size_t)p * 8 + o];
-            nch += ch >= 0;
-            if (ch >= 0) last = ch;
+            for (int o = 0; o < 8; ++o) {
+                nch += ch[o] >= 0;
+                if (ch[o] >= 0) last = ch[o];
+            }
+            ready = atomic_add_acq_rel(&t.arrive[p], 1) + 1 >= nch;
+            if (ready) {
+                // a twig ends where its last child (in octant order, so last in
+                // pre-order) ends, and skips to where that child skips
+                const int4 lc = __ldcg(&t.info[last]);
+                int* ip = reinterpret_cast<int*>(&t.info[p]);
+                ip[1] = lc.y;
+                ip[2] = lc.z;
+            } else {
+                p = -1;
+            }
         }
-        // this box's records are published with its arrival; the last arrival
-        // sees every sibling's
-        if (atomic_add_acq_rel(&t.arrive[p], 1) + 1 < nch) return;
-        // a twig ends where its last child (in octant order, so last in pre-order)
-        // ends, and skips to where that child skips
-        const int4 lc = __ldcg(&t.info[last]);
-        int* ip = reinterpret_cast<int*>(&t.info[p]);
-        ip[1] = lc.y;
-        ip[2] = lc.z;
-        combine(p, t.depth_leaf[p] & 255);
-        p = t.info[p].w;
+        unsigned int todo = __ballot_sync(0xffffffffu, ready);
+        __syncwarp();   // what the acquiring lanes see, every lane sees
+        while (todo) {
+            // the (lane / 8)-th of the lanes that are left
+            unsigned int m = todo;
+            for (int g = 0; g < (lane >> 3) && m; ++g) m &= m - 1u;
+            const int src = m ? __ffs(m) - 1 : -1;
+            const int q = __shfl_sync(0xffffffffu, p, src < 0 ? 0 : src);
+            const int pp = src < 0 ? -1 : q;
+            const int o = lane & 7;
+            const int ch = pp >= 0 ? t.child8[(size_t)pp * 8 + o] : -1;
+            combine(pp, pp >= 0 ? t.depth_leaf[pp] & 255 : 0, o, ch);
+            for (int g = 0; g < 4 && todo; ++g) todo &= todo - 1u;
+        }
+        __syncwarp();
+        if (p >= 0) p = t.info[p].w;
     }
 }
 
-// Moments of every leaf from its particles, one thread per leaf, summed about
-// the leaf's geometric centre in key order.
-__global__ void __launch_bounds__(kMomThreads)
-k_moments_leaves(const double* __restrict__ x, const double* __restrict__ y,
-                 const double* __restrict__ z, const int8_t* __restrict__ sp,
-                 const double* __restrict__ qsp, const Cube* __restrict__ cube, Tree t,
-                 float4* __restrict__ src32, int want_f32)
+// A block's leaves: those that start among its kMomTile positions, compacted in
+// position order; returns their number.
+constexpr int kMomThreads = 128;
+constexpr int kMomTile = 256;      // positions per block
+constexpr int kMomHalo = 32;       // largest leaf that is summed from shared memory
+constexpr unsigned short kNoOwner = 0xffff;
+
+__device__ __forceinline__ int block_leaves(const int* __restrict__ cnt, int base, int n,
+                                            int* list)
 {
-    const int nl = t.count[kMaxDepth + 1];
+    __shared__ int s_tot;
+    int total = 0;
+    for (int part = 0; part < kMomTile; part += kMomThreads) {
+        const int i = base + part + threadIdx.x;
+        const bool start = i < n && cnt[i] > 0;
+        const int at = block_excl_scan(start ? 1 : 0, &s_tot);
+        if (start) list[total + at] = i;
+        total += s_tot;
+        __syncthreads();
+    }
+    return total;
+}
+
+// FP64 moments of every leaf from its particles, one thread per leaf, summed about
+// the leaf's geometric centre in key order, then the twigs (sweep_up).
+__global__ void __launch_bounds__(kMomThreads)
+k_moments(const double* __restrict__ x, const double* __restrict__ y,
+          const double* __restrict__ z, const int8_t* __restrict__ sp,
+          const double* __restrict__ qsp, int n, const int* __restrict__ cnt,
+          const int* __restrict__ off, const Cube* __restrict__ cube, Tree t)
+{
+    __shared__ int list[kMomTile];
+    const int nl = block_leaves(cnt, blockIdx.x * kMomTile, n, list);
     const double q0 = qsp[0], q1 = qsp[1];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nl; i += gridDim.x * blockDim.x) {
-        const int node = t.leaf_list[i];
-        const int dl = t.depth_leaf[node];
-        const int4 inf = t.info[node];
-        const Cube cb = cube_of(cube, t, inf.x);
-        double zc[3], side;
-        box_centre(cb, t.cell[node], dl & 255, zc, &side);
-        double a[14];
+    for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kMomThreads) {
+        const int l = l0 + (threadIdx.x & 31);
+        int node = -1;
+        if (l < nl) {
+            const int i = list[l];
+            node = min(off[i] + cnt[i] - 1, t.cap - 1);
+            const int4 inf = t.info[node];
+            double zc[3], side;
+            box_centre(cube_of(cube, t, inf.x), t.cell[node], t.depth_leaf[node] & 255, zc, &side);
+            double a[14];
 #pragma unroll
-        for (int k = 0; k < 14; ++k) a[k] = 0.0;
-        for (int j = inf.x; j < inf.y; ++j) {
-            double qj = sp[j] ? q1 : q0;
-            double aq = fabs(qj);
-            double yv[3] = {x[j] - zc[0], y[j] - zc[1], z[j] - zc[2]};
-            a[0] += aq;
-            a[1] += qj;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                a[2 + k] += aq * yv[k];
-                a[5 + k] += qj * yv[k];
-            }
-            double qy0 = qj * yv[0], qy1 = qj * yv[1];
-            a[8] += qy0 * yv[0];
-            a[9] += qy0 * yv[1];
-            a[10] += qy0 * yv[2];
-            a[11] += qy1 * yv[1];
-            a[12] += qy1 * yv[2];
-            a[13] += qj * yv[2] * yv[2];
-        }
-        double rec[kMom];
-        finish_box(a, zc, rec, t.delta + node);
-        double* m = t.mom + (size_t)node * kMom;
-#pragma unroll
-        for (int k = 0; k < kMom; ++k) m[k] = rec[k];
-        if (want_f32) {
-            // paired layout: src32[2p] = {nx_2p, nx_2p+1, ny_2p, ny_2p+1},
-            // src32[2p+1] = {nz_2p, nz_2p+1, q_2p, q_2p+1}, n = c_leaf - x
-            float* f = reinterpret_cast<float*>(src32);
+            for (int k = 0; k < 14; ++k) a[k] = 0.0;
             for (int j = inf.x; j < inf.y; ++j) {
                 double qj = sp[j] ? q1 : q0;
-                size_t b = (size_t)(j >> 1) * 8 + (j & 1);
-                f[b] = (float)(rec[MC] - x[j]);
-                f[b + 2] = (float)(rec[MC + 1] - y[j]);
-                f[b + 4] = (float)(rec[MC + 2] - z[j]);
-                f[b + 6] = (float)qj;
+                double aq = fabs(qj);
+                double yv[3] = {x[j] - zc[0], y[j] - zc[1], z[j] - zc[2]};
+                a[0] += aq;
+                a[1] += qj;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    a[2 + k] += aq * yv[k];
+                    a[5 + k] += qj * yv[k];
+                }
+                double qy0 = qj * yv[0], qy1 = qj * yv[1];
+                a[8] += qy0 * yv[0];
+                a[9] += qy0 * yv[1];
+                a[10] += qy0 * yv[2];
+                a[11] += qy1 * yv[1];
+                a[12] += qy1 * yv[2];
+                a[13] += qj * yv[2] * yv[2];
             }
+            double rec[kMom];
+            finish_box(a, zc, rec, t.delta + node);
+            double* m = t.mom + (size_t)node * kMom;
+#pragma unroll
+            for (int k = 0; k < kMom; ++k)
+                if (k != MR2) m[k] = rec[k];
         }
-        sweep_up(t, node, [&](int p, int d) { twig_combine_f64(cube, t, p, d); });
+        sweep_up(t, node, [&](int p, int d, int o, int ch) { twig_combine_f64(cube, t, p, d, o, ch); });
     }
 }
 
 // ---- FP32 moments (FP32C contexts).  Offsets from a box's geometric centre z
 // are at most one box side, so they are formed in FP64 once and summed in FP32;
 // the expansion centre is c = z + e exactly as stored (FP64), and D, Q are taken
-// about that same point.  Compact per-box record mom32 = {e xyz, S0, M, D xyz,
+// about that same point; the FP64 record of such a box holds its centre only.  Compact
+// per-box record mom32 = {e xyz, S0, M, D xyz,
 // Q xx xy xz yy yz zz, 0, 0} feeds the twig combine.
 __device__ __forceinline__ void finish_box_f32(const float* a, const double z[3], float* m32,
                                                double* __restrict__ m64,
@@ -732,23 +769,18 @@ __device__ __forceinline__ void finish_box_f32(const float* a, const double z[3]
     m32[14] = 0.f;
     m32[15] = 0.f;
     for (int k = 0; k < 3; ++k) m64[MC + k] = z[k] + (double)e[k];
-    m64[MM] = M;
-    for (int k = 0; k < 3; ++k) m64[MD + k] = d[k];
-    for (int k = 0; k < 6; ++k) m64[MQ + k] = q[k];
-    m64[MS0] = S0;
     *delta = sqrtf(fmaf(e[0], e[0], fmaf(e[1], e[1], e[2] * e[2])));
 }
 
-// Child slot o of twig p shifted to the twig's centre (zeros for an empty slot).
+// Child slot o of a twig shifted to the twig's centre (zeros for an empty slot).
 // The child's expansion centre lies at its own geometric centre plus its FP32
 // offset e_child (mom32), and its geometric centre at the twig's plus q = side/4
 // along each axis, signed by the octant bit (x bit 0, y bit 1, z bit 2): the shift
 // is q +/- e_child, formed in FP32 without touching the FP64 unit.
-__device__ __forceinline__ void twig_child_f32(const Tree& t, int p, int o, float q, float* a)
+__device__ __forceinline__ void twig_child_f32(const Tree& t, int ch, int o, float q, float* a)
 {
 #pragma unroll
     for (int k = 0; k < 14; ++k) a[k] = 0.f;
-    const int ch = t.child8[(size_t)p * 8 + o];
     if (ch < 0) return;
     const float4* r32 = reinterpret_cast<const float4*>(t.mom32 + (size_t)ch * 16);
     const float4 R0 = __ldcg(r32), R1 = __ldcg(r32 + 1), R2 = __ldcg(r32 + 2),
@@ -774,116 +806,184 @@ __device__ __forceinline__ void twig_child_f32(const Tree& t, int p, int o, floa
     a[13] = qk[5] + (2.f * dk[2] + me2) * e[2];
 }
 
-// FP32 moments of twig p (depth d) from its eight shifted child slots, summed as
-// ((s0 + s4) + (s2 + s6)) + ((s1 + s5) + (s3 + s7)): the order of an xor
-// butterfly over the slots.
-__device__ void twig_combine_f32(const Cube* __restrict__ cube, const Tree& t, int p, int d)
+// FP32 moments of twig p (depth d; p < 0: none) by a group of eight lanes, one child
+// slot each, summed by an xor butterfly over the slots.
+__device__ __forceinline__ void twig_combine_f32(const Cube* __restrict__ cube, const Tree& t,
+                                                 int p, int d, int o, int ch)
 {
-    const Cube cb = cube_of(cube, t, t.info[p].x);
-    double zp[3], ps;
-    box_centre(cb, t.cell[p], d, zp, &ps);
-    const float q = (float)(0.25 * ps);
-    float u[14], v[14], w[14];
-    const int order[4][2] = {{0, 4}, {2, 6}, {1, 5}, {3, 7}};
-#pragma unroll 1
-    for (int g = 0; g < 4; ++g) {
-        float b0[14], b1[14];
-        twig_child_f32(t, p, order[g][0], q, b0);
-        twig_child_f32(t, p, order[g][1], q, b1);
+    double zp[3] = {0, 0, 0}, ps = 0.0;
+    if (p >= 0) box_centre(cube_of(cube, t, t.info[p].x), t.cell[p], d, zp, &ps);
+    float a[14];
+    twig_child_f32(t, ch, o, (float)(0.25 * ps), a);
 #pragma unroll
-        for (int k = 0; k < 14; ++k) {
-            const float s = b0[k] + b1[k];
-            if (g == 0) u[k] = s;
-            else if (g == 1) u[k] = u[k] + s;
-            else if (g == 2) v[k] = s;
-            else v[k] = v[k] + s;
-        }
+    for (int k = 0; k < 14; ++k) a[k] = sum8(a[k]);
+    if (p >= 0 && o == 0) {
+        float m32[16];
+        finish_box_f32(a, zp, m32, t.mom + (size_t)p * kMom, t.delta + p);
+        float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)p * 16);
+        for (int k = 0; k < 4; ++k)
+            w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
     }
-#pragma unroll
-    for (int k = 0; k < 14; ++k) w[k] = u[k] + v[k];
-    float m32[16];
-    finish_box_f32(w, zp, m32, t.mom + (size_t)p * kMom, t.delta + p);
-    float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)p * 16);
-    for (int k = 0; k < 4; ++k)
-        w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
 }
 
-// Leaves, one thread per leaf (full lanes for the FP64 offsets), then the
-// bottom-up sweep over the twigs (sweep_up).
+// FP32C contexts: a block takes the leaves that start among its kMomTile positions.
+// kTile (leaves of up to kMomHalo particles): the particles' offsets from their leaf's
+// geometric centre are formed with one particle per lane (the FP64 pipe takes a warp
+// instruction for 16 cycles however many lanes are active) and kept in shared memory,
+// where each leaf's thread sums them in key order; the source records are written one
+// particle per lane again.  Larger leaves: one thread per leaf does all of it.  Then
+// the twigs (sweep_up).
+template <bool kTile>
 __global__ void __launch_bounds__(kMomThreads)
-k_moments_leaves_f32(const double* __restrict__ x, const double* __restrict__ y,
-                     const double* __restrict__ z, const int8_t* __restrict__ sp,
-                     const double* __restrict__ qsp, const Cube* __restrict__ cube, Tree t,
-                     float4* __restrict__ src32)
+k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
+              const double* __restrict__ z, const int8_t* __restrict__ sp,
+              const double* __restrict__ qsp, int n, const int* __restrict__ cnt,
+              const int* __restrict__ off, const Cube* __restrict__ cube, Tree t,
+              float4* __restrict__ src32)
 {
-    const int nl = t.count[kMaxDepth + 1];
+    __shared__ int list[kMomTile];
+    __shared__ double ctr[kTile ? kMomTile : 1][3];                  // geometric centre, then c
+    __shared__ float4 ys[kTile ? kMomTile + kMomHalo : 1];           // offset, charge
+    __shared__ unsigned short owner[kTile ? kMomTile + kMomHalo : 1];
+    const int base = blockIdx.x * kMomTile;
+    const int nl = block_leaves(cnt, base, n, list);
     const float q0 = (float)qsp[0], q1 = (float)qsp[1];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nl; i += gridDim.x * blockDim.x) {
-        const int node = t.leaf_list[i];
-        const int dl = t.depth_leaf[node];
-        const int4 inf = t.info[node];
-        const Cube cb = cube_of(cube, t, inf.x);
-        double zc[3], side;
-        box_centre(cb, t.cell[node], dl & 255, zc, &side);
-        float a[14];
-#pragma unroll
-        for (int k = 0; k < 14; ++k) a[k] = 0.f;
-#pragma unroll 4
-        for (int j = inf.x; j < inf.y; ++j) {
-            float qj = sp[j] ? q1 : q0;
-            float aq = fabsf(qj);
-            float yv[3] = {(float)(x[j] - zc[0]), (float)(y[j] - zc[1]), (float)(z[j] - zc[2])};
-            a[0] += aq;
-            a[1] += qj;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                a[2 + k] = fmaf(aq, yv[k], a[2 + k]);
-                a[5 + k] = fmaf(qj, yv[k], a[5 + k]);
-            }
-            float qy0 = qj * yv[0], qy1 = qj * yv[1];
-            a[8] = fmaf(qy0, yv[0], a[8]);
-            a[9] = fmaf(qy0, yv[1], a[9]);
-            a[10] = fmaf(qy0, yv[2], a[10]);
-            a[11] = fmaf(qy1, yv[1], a[11]);
-            a[12] = fmaf(qy1, yv[2], a[12]);
-            a[13] = fmaf(qj * yv[2], yv[2], a[13]);
+    float* f = reinterpret_cast<float*>(src32);
+    if (kTile) {
+        for (int l = threadIdx.x; l < nl; l += kMomThreads) {
+            const int i = list[l];
+            const int node = min(off[i] + cnt[i] - 1, t.cap - 1);
+            const int4 inf = t.info[node];
+            double side;
+            box_centre(cube_of(cube, t, inf.x), t.cell[node], t.depth_leaf[node] & 255, ctr[l], &side);
+            const int e = min(inf.y - base, kMomTile + kMomHalo);
+            const bool fat = inf.y - inf.x > kMomHalo;   // a depth-cap box: its thread does it all
+            for (int k = i - base; k < e; ++k) owner[k] = fat ? kNoOwner : (unsigned short)l;
         }
-        float m32[16];
-        double* m = t.mom + (size_t)node * kMom;
-        finish_box_f32(a, zc, m32, m, t.delta + node);
-        float4* r32 = reinterpret_cast<float4*>(t.mom32 + (size_t)node * 16);
-        for (int k = 0; k < 4; ++k)
-            r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
+        __syncthreads();
+        const int first = nl > 0 ? list[0] - base : kMomTile;
+        const int end = nl > 0 ? min(t.info[min(off[list[nl - 1]] + cnt[list[nl - 1]] - 1, t.cap - 1)].y - base,
+                                     kMomTile + kMomHalo) : 0;
+        for (int k = first + threadIdx.x; k < end; k += kMomThreads) {
+            const int j = base + k;
+            if (owner[k] == kNoOwner) continue;
+            const double* zc = ctr[owner[k]];
+            ys[k] = make_float4((float)(x[j] - zc[0]), (float)(y[j] - zc[1]), (float)(z[j] - zc[2]),
+                                sp[j] ? q1 : q0);
+        }
+        __syncthreads();
+        for (int l = threadIdx.x; l < nl; l += kMomThreads) {
+            const int i = list[l];
+            const int node = min(off[i] + cnt[i] - 1, t.cap - 1);
+            const int e = t.info[node].y - base;
+            if (e - (i - base) > kMomHalo) continue;
+            float a[14];
+#pragma unroll
+            for (int k = 0; k < 14; ++k) a[k] = 0.f;
+#pragma unroll 4
+            for (int k = i - base; k < e; ++k) {
+                const float4 v = ys[k];
+                const float qj = v.w, aq = fabsf(qj);
+                const float yv[3] = {v.x, v.y, v.z};
+                a[0] += aq;
+                a[1] += qj;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    a[2 + c] = fmaf(aq, yv[c], a[2 + c]);
+                    a[5 + c] = fmaf(qj, yv[c], a[5 + c]);
+                }
+                float qy0 = qj * yv[0], qy1 = qj * yv[1];
+                a[8] = fmaf(qy0, yv[0], a[8]);
+                a[9] = fmaf(qy0, yv[1], a[9]);
+                a[10] = fmaf(qy0, yv[2], a[10]);
+                a[11] = fmaf(qy1, yv[1], a[11]);
+                a[12] = fmaf(qy1, yv[2], a[12]);
+                a[13] = fmaf(qj * yv[2], yv[2], a[13]);
+            }
+            float m32[16];
+            double* m = t.mom + (size_t)node * kMom;
+            double zc[3] = {ctr[l][0], ctr[l][1], ctr[l][2]};
+            double c64[3];
+            finish_box_f32(a, zc, m32, c64, t.delta + node);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                m[MC + c] = c64[c];
+                ctr[l][c] = c64[c];
+            }
+            float4* r32 = reinterpret_cast<float4*>(t.mom32 + (size_t)node * 16);
+            for (int k = 0; k < 4; ++k)
+                r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
+        }
+        __syncthreads();
         // paired sources: src32[2p] = {nx_2p, nx_2p+1, ny_2p, ny_2p+1},
         // src32[2p+1] = {nz_2p, nz_2p+1, q_2p, q_2p+1}, n = c_leaf - x
-        const double cx = m[MC], cy = m[MC + 1], cz = m[MC + 2];
-        float* f = reinterpret_cast<float*>(src32);
-        for (int j = inf.x; j < inf.y; ++j) {
-            size_t b = (size_t)(j >> 1) * 8 + (j & 1);
-            f[b] = (float)(cx - x[j]);
-            f[b + 2] = (float)(cy - y[j]);
-            f[b + 4] = (float)(cz - z[j]);
-            f[b + 6] = sp[j] ? q1 : q0;
+        for (int k = first + threadIdx.x; k < end; k += kMomThreads) {
+            const int j = base + k;
+            if (owner[k] == kNoOwner) continue;
+            const double* c = ctr[owner[k]];
+            const size_t b = (size_t)(j >> 1) * 8 + (j & 1);
+            f[b] = (float)(c[0] - x[j]);
+            f[b + 2] = (float)(c[1] - y[j]);
+            f[b + 4] = (float)(c[2] - z[j]);
+            f[b + 6] = ys[k].w;
         }
-        sweep_up(t, node, [&](int p, int d) { twig_combine_f32(cube, t, p, d); });
+    }
+    for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kMomThreads) {
+        const int l = l0 + (threadIdx.x & 31);
+        int node = -1;
+        if (l < nl) {
+            const int i = list[l];
+            node = min(off[i] + cnt[i] - 1, t.cap - 1);
+            const int4 inf = t.info[node];
+            if (!kTile || inf.y - inf.x > kMomHalo) {
+                double zc[3], side;
+                box_centre(cube_of(cube, t, inf.x), t.cell[node], t.depth_leaf[node] & 255, zc, &side);
+                float a[14];
+#pragma unroll
+                for (int k = 0; k < 14; ++k) a[k] = 0.f;
+                for (int j = inf.x; j < inf.y; ++j) {
+                    float qj = sp[j] ? q1 : q0;
+                    float aq = fabsf(qj);
+                    float yv[3] = {(float)(x[j] - zc[0]), (float)(y[j] - zc[1]),
+                                   (float)(z[j] - zc[2])};
+                    a[0] += aq;
+                    a[1] += qj;
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        a[2 + k] = fmaf(aq, yv[k], a[2 + k]);
+                        a[5 + k] = fmaf(qj, yv[k], a[5 + k]);
+                    }
+                    float qy0 = qj * yv[0], qy1 = qj * yv[1];
+                    a[8] = fmaf(qy0, yv[0], a[8]);
+                    a[9] = fmaf(qy0, yv[1], a[9]);
+                    a[10] = fmaf(qy0, yv[2], a[10]);
+                    a[11] = fmaf(qy1, yv[1], a[11]);
+                    a[12] = fmaf(qy1, yv[2], a[12]);
+                    a[13] = fmaf(qj * yv[2], yv[2], a[13]);
+                }
+                float m32[16];
+                double* m = t.mom + (size_t)node * kMom;
+                finish_box_f32(a, zc, m32, m, t.delta + node);
+                float4* r32 = reinterpret_cast<float4*>(t.mom32 + (size_t)node * 16);
+                for (int k = 0; k < 4; ++k)
+                    r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
+                const double cx = m[MC], cy = m[MC + 1], cz = m[MC + 2];
+                for (int j = inf.x; j < inf.y; ++j) {
+                    size_t b = (size_t)(j >> 1) * 8 + (j & 1);
+                    f[b] = (float)(cx - x[j]);
+                    f[b + 2] = (float)(cy - y[j]);
+                    f[b + 4] = (float)(cz - z[j]);
+                    f[b + 6] = sp[j] ? q1 : q0;
+                }
+            }
+        }
+        sweep_up(t, node, [&](int p, int d, int o, int ch) { twig_combine_f32(cube, t, p, d, o, ch); });
     }
 }
 
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-size_t scan_partials_words(int n) { return (size_t)((n + kScanTile - 1) / kScanTile) + 1; }
-
-void launch_scan(const int* in, int* out, int n, int* partials, int* total, cudaStream_t s)
-{
-    count_launch(3);
-    int nb = (n + kScanTile - 1) / kScanTile;
-    if (nb < 1) nb = 1;
-    k_scan_reduce<<<nb, kScanThreads, 0, s>>>(in, n, partials);
-    k_scan_partials<<<1, kScanThreads, 0, s>>>(partials, nb, total);
-    k_scan_apply<<<nb, kScanThreads, 0, s>>>(in, out, n, partials);
-}
-
 void launch_bbox(const double* x, const double* y, const double* z, int n, double* partials,
                  int nblk, Cube* cubes, const int* cloud_start, int n_clouds, BuildCtl ctl,
                  cudaStream_t s)
@@ -904,35 +1004,39 @@ void launch_keys(const double* x, const double* y, const double* z, int n, const
 }
 
 void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* pos_cnt,
-                     int* pos_off, int* scan_part, Tree t, cudaStream_t s)
+                     int* pos_off, Tree t, BuildCtl ctl, unsigned long long* status, int* err,
+                     cudaStream_t s)
 {
-    count_launch(3);
+    count_launch(2);
     const int nb = (n + kTopoThreads - 1) / kTopoThreads;
-    const bool win = leaf_cap <= kTopoWin;
-    if (win) k_topo_count_win<<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, t);
-    else k_topo_count<<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, t);
-    launch_scan(pos_cnt, pos_off, n, scan_part, t.nnodes, s);
-    k_clear_children<<<2 * 152, 256, 0, s>>>(t);
-    if (win) k_topo_emit<true><<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, pos_off, t);
-    else k_topo_emit<false><<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, pos_off, t);
+    if (leaf_cap <= kTopoWin)
+        k_topo_scan<true><<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, pos_off, t, ctl,
+                                                      status, err);
+    else
+        k_topo_scan<false><<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, pos_off, t, ctl,
+                                                       status, err);
+    k_topo_emit<<<nb, kTopoThreads, 0, s>>>(key, n, pos_cnt, pos_off, t);
 }
 
+size_t topo_status_words(int n) { return (size_t)((n + kTopoThreads - 1) / kTopoThreads) + 1; }
+
 void launch_moments(const double* x, const double* y, const double* z, const int8_t* sp,
-                    const double* qsp, int n, const Cube* cube, Tree t, float4* src32,
-                    int want_f32, cudaStream_t s)
+                    const double* qsp, int n, int leaf_cap, const int* pos_cnt,
+                    const int* pos_off, const Cube* cube, Tree t, float4* src32, int want_f32,
+                    cudaStream_t s)
 {
     // leaves from their particles, then every twig as its last child finishes
     // (bottom-up sweep with arrival counters), in one launch
     count_launch(1);
-    // small blocks spread the leaf threads (about one per eight particles) evenly
-    // over the SMs
-    int blocks = (n + kMomThreads - 1) / kMomThreads;
-    if (blocks > 16 * 152) blocks = 16 * 152;
-    if (blocks < 1) blocks = 1;
-    if (want_f32)
-        k_moments_leaves_f32<<<blocks, kMomThreads, 0, s>>>(x, y, z, sp, qsp, cube, t, src32);
+    const int nb = (n + kMomTile - 1) / kMomTile;
+    if (!want_f32)
+        k_moments<<<nb, kMomThreads, 0, s>>>(x, y, z, sp, qsp, n, pos_cnt, pos_off, cube, t);
+    else if (leaf_cap <= kMomHalo)
+        k_moments_f32<true><<<nb, kMomThreads, 0, s>>>(x, y, z, sp, qsp, n, pos_cnt, pos_off, cube,
+                                                       t, src32);
     else
-        k_moments_leaves<<<blocks, kMomThreads, 0, s>>>(x, y, z, sp, qsp, cube, t, src32, 0);
+        k_moments_f32<false><<<nb, kMomThreads, 0, s>>>(x, y, z, sp, qsp, n, pos_cnt, pos_off,
+                                                        cube, t, src32);
 }
 
 }  // namespace ucp

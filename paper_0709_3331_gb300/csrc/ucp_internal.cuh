@@ -43,6 +43,7 @@ inline void count_launch(int k) { g_launches.fetch_add((unsigned long long)k, st
 
 // One FP64 box record, 16 doubles (128 B), read by the FP64 walk.
 // {c.x, c.y, c.z, rcrit2, M, D.x, D.y, D.z, Qxx, Qxy, Qxz, Qyy, Qyz, Qzz, S0, -tr(Q)/2}
+// (FP32C contexts: c and rcrit2 only, the rest in mom32)
 // rcrit2 = (s/theta + delta)^2 is filled per walk (it depends on theta).
 constexpr int kMom = 16;
 enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
@@ -72,10 +73,6 @@ struct Tree {
     float* mom32;            // FP32C contexts: 16 floats per box {e xyz, S0, M, D, Q, 0, 0}
     int* child8;             // 8 child slots per box (octant order), -1 = empty
     int* arrive;             // finished children per box (moments' bottom-up sweep)
-    int* leaf_list;          // the leaves, any order
-    int* twig_list;          // the twigs of depth d at twig_off[d] .. + count[d]
-    int* count;              // count[d] twigs of depth d (d <= 20), count[kMaxDepth + 1] leaves
-    int twig_off[kMaxDepth + 2];
     // clouds: cloud[i] = cloud of key-sorted position i, whose segment is
     // [cloud_start[c], cloud_start[c + 1]); NULL cloud = one cloud over [0, n)
     const unsigned char* cloud;
@@ -99,9 +96,9 @@ enum CtlIdx {
     kCtlTile = kCtlHist + kSortPassesMax * kRadix, // tile counters: passes, then the clouds' pass
     kCtlLong = kCtlTile + kSortPassesMax + 1,      // raised: a run too long for the run sort
     kCtlBarrier,                                   // arrivals at the full sort's barrier
+    kCtlTopoTile,                                  // tiles of the topology's scan
     kCtlMaxDepth,
-    kCtlCount,                                     // kMaxDepth + 2 list counters
-    kCtlWords = kCtlCount + kMaxDepth + 2
+    kCtlWords
 };
 struct BuildCtl {
     int* words;              // kCtlWords
@@ -140,12 +137,13 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
                 cudaStream_t s);
 int sort_selftest_timeout(const SortScratch& sc, cudaStream_t s);
 void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* pos_cnt,
-                     int* pos_off, int* scan_part, Tree t, cudaStream_t s);
+                     int* pos_off, Tree t, BuildCtl ctl, unsigned long long* status, int* err,
+                     cudaStream_t s);
+size_t topo_status_words(int n);
 void launch_moments(const double* x, const double* y, const double* z, const int8_t* sp,
-                    const double* qsp, int n, const Cube* cube, Tree t, float4* src32,
-                    int want_f32, cudaStream_t s);
-void launch_scan(const int* in, int* out, int n, int* partials, int* total, cudaStream_t s);
-size_t scan_partials_words(int n);
+                    const double* qsp, int n, int leaf_cap, const int* pos_cnt,
+                    const int* pos_off, const Cube* cube, Tree t, float4* src32, int want_f32,
+                    cudaStream_t s);
 
 // ---- walk (ucp_walk.cu) ----
 struct WalkArgs {

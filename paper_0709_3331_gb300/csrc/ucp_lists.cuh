@@ -206,6 +206,7 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const
         if ((lane >> 3) < pop) {
             const int2 e = W.stack[top - 1 - (lane >> 3)];
             box = __ldg(a.t.child8 + (size_t)e.x * 8 + (lane & 7));
+            if (box <= e.x) box = -1;   // a child comes after its parent: the walk ends
             mask = (unsigned int)e.y;
         }
         top -= pop;

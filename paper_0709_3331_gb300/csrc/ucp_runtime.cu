@@ -40,7 +40,7 @@ struct ucp_ctx {
     SortScratch sort = {};
     BuildCtl ctl = {};
     int passes = 3;          // of the sort over the key's top digits
-    int* scan_part = nullptr;
+    unsigned long long* topo_status = nullptr;
     int* sel_part = nullptr;
     int* pos_cnt = nullptr;
     int* pos_off = nullptr;
@@ -247,9 +247,10 @@ int build(ucp_ctx* c)
     c->sorted_buf = b;
     c->cur = k ^ 1;
     k = c->cur;
-    launch_topology(c->key[b], n, c->leaf_cap, c->pos_cnt, c->pos_off, c->scan_part, c->t, c->s);
-    launch_moments(c->st[k][0], c->st[k][1], c->st[k][2], c->sp[k], c->qsp, n, c->cube, c->t,
-                   c->src32, c->precision == UCP_FP32C, c->s);
+    launch_topology(c->key[b], n, c->leaf_cap, c->pos_cnt, c->pos_off, c->t, c->ctl,
+                    c->topo_status, c->sort.err, c->s);
+    launch_moments(c->st[k][0], c->st[k][1], c->st[k][2], c->sp[k], c->qsp, n, c->leaf_cap,
+                   c->pos_cnt, c->pos_off, c->cube, c->t, c->src32, c->precision == UCP_FP32C, c->s);
     c->tree_valid = true;
     c->acc_valid = false;
     c->phi_valid = false;
@@ -502,7 +503,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->sort.test_epoch, 1);
     dalloc(c, &c->sort.test_keys, sort_test_words());
     dalloc(c, &c->sort.test_vals, sort_test_words());
-    dalloc(c, &c->scan_part, scan_partials_words(c->n));
+    dalloc(c, &c->topo_status, topo_status_words(c->n));
     dalloc(c, &c->pos_cnt, n);
     dalloc(c, &c->pos_off, n);
     const size_t cz = (size_t)cap;
@@ -515,22 +516,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->t.delta, cz);
     dalloc(c, &c->t.hdr, cz);
     dalloc(c, &c->t.child8, cz * 8);
-    dalloc(c, &c->t.leaf_list, cz);
     dalloc(c, &c->t.arrive, cz);
-    {
-        // twigs of depth d: at most min(8^d, n / (leaf_cap + 1)); none at the depth cap
-        int64_t off = 0, pow8 = 1;
-        for (int d = 0; d <= kMaxDepth + 1; ++d) {
-            c->t.twig_off[d] = (int)off;
-            if (d < kMaxDepth)
-                for (int i = 0; i < n_clouds; ++i) {
-                    int64_t twigs = sizes[i] / (c->leaf_cap + 1);
-                    off += pow8 < twigs ? pow8 : twigs;
-                }
-            if (pow8 < ((int64_t)1 << 40)) pow8 *= 8;
-        }
-        dalloc(c, &c->t.twig_list, (size_t)(off > 0 ? off : 1));
-    }
     if (c->precision == UCP_FP32C) {
         dalloc(c, &c->t.lo, cz);
         dalloc(c, &c->t.rec, cz * kRec);
@@ -581,7 +567,6 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     if ((rc = commit(c))) return bail(rc);
 
     c->t.maxdepth = c->ctl.words + kCtlMaxDepth;
-    c->t.count = c->ctl.words + kCtlCount;
     c->t.cloud_start = c->cloud_start;
     c->t.cloud = c->cloud;
     std::vector<unsigned char> cl;
@@ -591,7 +576,11 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
             for (int j = c->cloud_start_h[i]; j < c->cloud_start_h[i + 1]; ++j)
                 cl[j] = (unsigned char)i;
     }
-    if (cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) ||
+    // box tables a build has not filled are read only after a wait that gave up: empty
+    if (cudaMemsetAsync(c->t.info, 0, sizeof(int4) * cz, c->s) ||
+        cudaMemsetAsync(c->t.child8, 0xff, 8 * sizeof(int) * cz, c->s) ||
+        cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) ||
+        cudaMemsetAsync(c->topo_status, 0, 8 * topo_status_words(c->n), c->s) ||
         cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) ||
         cudaMemsetAsync(c->ctl.epoch, 0, sizeof(unsigned int), c->s) ||
         // the pad slot of an odd count is read (masked) by the pair loop: keep it finite
@@ -1362,6 +1351,11 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
     std::vector<int> dl(nn);
     std::vector<unsigned long long> cell(nn);
     std::vector<double> mom((size_t)nn * kMom), delta(nn);
+    const bool f32 = c->precision == UCP_FP32C;
+    std::vector<float> mom32(f32 ? (size_t)nn * 16 : 0);
+    if (f32)
+        CK(cudaMemcpyAsync(mom32.data(), c->t.mom32, sizeof(float) * 16 * nn, cudaMemcpyDeviceToHost,
+                           c->s));
     CK(cudaMemcpyAsync(info.data(), c->t.info, sizeof(int4) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(dl.data(), c->t.depth_leaf, sizeof(int) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(cell.data(), c->t.cell, 8 * (size_t)nn, cudaMemcpyDeviceToHost, c->s));
@@ -1392,7 +1386,14 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
                 g[a] = lo + off;
             }
             g[3] = s;
-            const double* m = mom.data() + (size_t)i * kMom;
+            double* m = mom.data() + (size_t)i * kMom;
+            if (f32) {  // {e xyz, S0, M, D, Q}
+                const float* r = mom32.data() + (size_t)i * 16;
+                m[MS0] = r[3];
+                m[MM] = r[4];
+                for (int a = 0; a < 3; ++a) m[MD + a] = r[5 + a];
+                for (int a = 0; a < 6; ++a) m[MQ + a] = r[8 + a];
+            }
             g[4] = m[MS0];
             g[5] = m[MM];
             for (int a = 0; a < 3; ++a) g[6 + a] = m[MC + a];

@@ -200,8 +200,11 @@ k_walk_fp64(WalkArgs a)
             }
             const int pop = top > kPopWide ? 1 : min(top, 4);
             box = -1;
-            if ((lane >> 3) < pop)
-                box = __ldg(a.t.child8 + (size_t)stack[top - 1 - (lane >> 3)] * 8 + (lane & 7));
+            if ((lane >> 3) < pop) {
+                const int twig = stack[top - 1 - (lane >> 3)];
+                box = __ldg(a.t.child8 + (size_t)twig * 8 + (lane & 7));
+                if (box <= twig) box = -1;   // a child comes after its parent: the walk ends
+            }
             top -= pop;
             __syncwarp();
         }
@@ -737,15 +740,14 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
         if (want_f32) {
             t.lo[nd] = make_float4((float)((double)chx - ux), (float)((double)chy - uy),
                                    (float)((double)chz - uz), __int_as_float(t.info[nd].z));
-            const float qxx = (float)m[MQ], qyy = (float)m[MQ + 3], qzz = (float)m[MQ + 5];
-            const float M = (float)m[MM];
+            const float4* m32 = reinterpret_cast<const float4*>(t.mom32 + (size_t)nd * 16);
+            const float4 f1 = m32[1], f2 = m32[2], f3 = m32[3];   // {M, D}, {Q..}, {Q.., 0, 0}
+            const float M = f1.x, qxx = f2.x, qyy = f2.w, qzz = f3.y;
             float4* r = t.rec + (size_t)nd * kRec;
             r[0] = make_float4(-chx, -chy, -chz, M);
-            r[1] = make_float4((float)m[MD], (float)m[MD + 1], (float)m[MD + 2],
-                               -0.5f * ((qxx + qyy) + qzz));
-            r[2] = make_float4(0.5f * qxx, 0.5f * (float)m[MQ + 1], 0.5f * (float)m[MQ + 2],
-                               0.5f * qyy);
-            r[3] = make_float4(0.5f * (float)m[MQ + 4], 0.5f * qzz, -M, 0.f);
+            r[1] = make_float4(f1.y, f1.z, f1.w, -0.5f * ((qxx + qyy) + qzz));
+            r[2] = make_float4(0.5f * qxx, 0.5f * f2.y, 0.5f * f2.z, 0.5f * qyy);
+            r[3] = make_float4(0.5f * f3.x, 0.5f * qzz, -M, 0.f);
         }
     }
 }
