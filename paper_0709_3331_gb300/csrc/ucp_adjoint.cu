@@ -161,9 +161,9 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
         auto direct_pairs = [&](const int2* leaves, int cnt) {
             const LeafRun run(a, leaves, cnt);
             for (int base = 0; base < run.total; base += 32) {
-                int j, nd;
+                int j, nd, first;
                 unsigned int mask;
-                run.at(base + lane, j, nd, mask);
+                run.at(base + lane, j, nd, first, mask);
                 double xj = 0.0, yj = 0.0, zj = 0.0, qj = 0.0;
                 if (mask) {
                     xj = a.x[j];
@@ -427,16 +427,17 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
         auto direct_pairs = [&](const int2* leaves, int cnt) {
             const LeafRun run(a, leaves, cnt);
             for (int base = 0; base < run.total; base += 32) {
-                int j, nd;
+                int j, nd, first;
                 unsigned int mask;
-                run.at(base + lane, j, nd, mask);
+                run.at(base + lane, j, nd, first, mask);
                 float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A;
                 float nx = 0.f, ny = 0.f, nz = 0.f, qj = 0.f;
                 if (mask) {
                     // r = (x_t - c_leaf) + (c_leaf - x_j), the first from float pairs
                     A = __ldg(a.t.hdr + nd);
                     B = __ldg(a.t.lo + nd);
-                    const float4 P = __ldg(S + (j & ~1)), Q = __ldg(S + (j | 1));
+                    const int at = src_place(first, nd) + (j & ~1) - (first & ~1);
+                    const float4 P = __ldg(S + at), Q = __ldg(S + at + 1);
                     const bool odd = j & 1;
                     nx = odd ? P.y : P.x;
                     ny = odd ? P.w : P.z;

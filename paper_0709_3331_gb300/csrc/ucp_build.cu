@@ -826,6 +826,22 @@ __device__ __forceinline__ void twig_combine_f32(const Cube* __restrict__ cube, 
     }
 }
 
+// One particle's source record, and the empty halves of its leaf's pairs.
+__device__ __forceinline__ void put_source(float* f, int place, int begin, int j, float nx, float ny,
+                                           float nz, float q)
+{
+    float* d = f + (size_t)(place + (j & ~1) - (begin & ~1)) * 4 + (j & 1);
+    d[0] = nx;
+    d[2] = ny;
+    d[4] = nz;
+    d[6] = q;
+}
+__device__ __forceinline__ void put_empty_halves(float* f, int place, int begin, int end)
+{
+    if (begin & 1) put_source(f, place, begin, begin - 1, kFarAway, 0.f, 0.f, 0.f);
+    if (end & 1) put_source(f, place, begin, end, kFarAway, 0.f, 0.f, 0.f);
+}
+
 // FP32C contexts: a block takes the leaves that start among its kMomTile positions.
 // kTile (leaves of up to kMomHalo particles): the particles' offsets from their leaf's
 // geometric centre are formed with one particle per lane (the FP64 pipe takes a warp
@@ -845,6 +861,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
     __shared__ double ctr[kTile ? kMomTile : 1][3];                  // geometric centre, then c
     __shared__ float4 ys[kTile ? kMomTile + kMomHalo : 1];           // offset, charge
     __shared__ unsigned short owner[kTile ? kMomTile + kMomHalo : 1];
+    __shared__ int place[kTile ? kMomTile : 1];
     const int base = blockIdx.x * kMomTile;
     const int nl = block_leaves(cnt, base, n, list);
     const float q0 = (float)qsp[0], q1 = (float)qsp[1];
@@ -858,6 +875,8 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
             box_centre(cube_of(cube, t, inf.x), t.cell[node], t.depth_leaf[node] & 255, ctr[l], &side);
             const int e = min(inf.y - base, kMomTile + kMomHalo);
             const bool fat = inf.y - inf.x > kMomHalo;   // a depth-cap box: its thread does it all
+            place[l] = src_place(i, node);
+            if (!fat) put_empty_halves(f, place[l], i, inf.y);
             for (int k = i - base; k < e; ++k) owner[k] = fat ? kNoOwner : (unsigned short)l;
         }
         __syncthreads();
@@ -915,17 +934,12 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                 r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
         }
         __syncthreads();
-        // paired sources: src32[2p] = {nx_2p, nx_2p+1, ny_2p, ny_2p+1},
-        // src32[2p+1] = {nz_2p, nz_2p+1, q_2p, q_2p+1}, n = c_leaf - x
         for (int k = first + threadIdx.x; k < end; k += kMomThreads) {
-            const int j = base + k;
-            if (owner[k] == kNoOwner) continue;
-            const double* c = ctr[owner[k]];
-            const size_t b = (size_t)(j >> 1) * 8 + (j & 1);
-            f[b] = (float)(c[0] - x[j]);
-            f[b + 2] = (float)(c[1] - y[j]);
-            f[b + 4] = (float)(c[2] - z[j]);
-            f[b + 6] = ys[k].w;
+            const int j = base + k, l = owner[k];
+            if (l == kNoOwner) continue;
+            const double* c = ctr[l];
+            put_source(f, place[l], list[l], j, (float)(c[0] - x[j]), (float)(c[1] - y[j]),
+                       (float)(c[2] - z[j]), ys[k].w);
         }
     }
     for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kMomThreads) {
@@ -968,13 +982,11 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                 for (int k = 0; k < 4; ++k)
                     r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
                 const double cx = m[MC], cy = m[MC + 1], cz = m[MC + 2];
-                for (int j = inf.x; j < inf.y; ++j) {
-                    size_t b = (size_t)(j >> 1) * 8 + (j & 1);
-                    f[b] = (float)(cx - x[j]);
-                    f[b + 2] = (float)(cy - y[j]);
-                    f[b + 4] = (float)(cz - z[j]);
-                    f[b + 6] = sp[j] ? q1 : q0;
-                }
+                const int at = src_place(inf.x, node);
+                put_empty_halves(f, at, inf.x, inf.y);
+                for (int j = inf.x; j < inf.y; ++j)
+                    put_source(f, at, inf.x, j, (float)(cx - x[j]), (float)(cy - y[j]),
+                               (float)(cz - z[j]), sp[j] ? q1 : q0);
             }
         }
         sweep_up(t, node, [&](int p, int d, int o, int ch) { twig_combine_f32(cube, t, p, d, o, ch); });

@@ -57,6 +57,20 @@ enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
 //         {Qyz / 2, Qzz / 2, -M, 0}         64 B: four lanes load one box
 constexpr int kRec = 4;
 
+// FP32C sources: offsets n = c_leaf - x and charges in pairs of particles, two float4
+// per pair {nx0, nx1, ny0, ny1}, {nz0, nz1, q0, q1}, particle j in the half j & 1.
+// Every leaf starts at a place of its own, so that its pairs hold no other leaf's
+// particles: an empty half (before an odd first particle, after an odd last one) is far
+// away and has no charge.  src_place: float4 index of the first pair of the leaf `box`
+// whose first particle is `begin` (two leaves never overlap: a later one has a later
+// box, which moves it two places on).
+__host__ __device__ __forceinline__ int src_place(int begin, int box)
+{
+    return (begin & ~1) + 2 * box;
+}
+constexpr int kSrcSlack = 64;        // float4 read (not used) past the last leaf
+constexpr float kFarAway = 1e18f;
+
 // Box topology {begin, end, next, parent}; depth and leaf flag separately.
 struct Tree {
     int cap;                 // box capacity
@@ -151,8 +165,7 @@ struct WalkArgs {
     const int8_t* sp;
     const double* qsp;      // charge per species (device, 2)
     const double* msp;      // mass per species (device, 2)
-    const float4* src32;    // FP32C sources, pairs of particles: {nx0, nx1, ny0, ny1},
-                            // {nz0, nz1, q0, q1} with n = c_leaf - x (key order)
+    const float4* src32;    // FP32C sources (src_place)
     Tree t;
     const int* targets;     // key-order slots of the targets, or NULL = all
     int ntargets;

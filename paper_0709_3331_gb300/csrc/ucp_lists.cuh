@@ -94,7 +94,8 @@ struct ChunkTarget {
 // Walks a chunk's targets, one per lane, through their cloud's tree with the lanes
 // over boxes: multipoles(list, cnt) takes cnt <= 32 accepted boxes {box, mask of the
 // targets that accept it}, pairs(list, cnt) cnt <= 32 opened leaves {leaf, mask of the
-// targets that open it}; both are called by the whole warp and may use W.stage.
+// targets that open it}; both are called by the whole warp and may use W.stage and their
+// part of the list.
 template <class Boxes, class Pairs>
 __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const ChunkTarget& tg,
                                            int cloud, Boxes& multipoles,
@@ -217,6 +218,7 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const
 // The particles of up to 32 opened leaves {leaf, mask} as one run over the lanes.
 struct LeafRun {
     int total, end, first;       // end: of this lane's leaf in the run; first: begin - start
+    int begin;                   // of this lane's leaf
     int2 lm;
 
     __device__ __forceinline__ LeafRun(const WalkArgs& a, const int2* leaves, int cnt)
@@ -236,10 +238,13 @@ struct LeafRun {
         }
         total = __shfl_sync(0xffffffffu, end, 31);
         first = be.y - end;
+        begin = be.x;
     }
 
-    // particle f of the run: its slot, its leaf and that leaf's mask (0 past the end)
-    __device__ __forceinline__ void at(int f, int& j, int& leaf, unsigned int& mask) const
+    // particle f of the run: its slot, its leaf, that leaf's first slot and its mask (0
+    // past the end)
+    __device__ __forceinline__ void at(int f, int& j, int& leaf, int& leaf_begin,
+                                       unsigned int& mask) const
     {
         int owner = 0;           // leaves that end at or before f
 #pragma unroll
@@ -247,6 +252,7 @@ struct LeafRun {
             if (__shfl_sync(0xffffffffu, end, owner + o - 1) <= f) owner += o;
         j = __shfl_sync(0xffffffffu, first, owner) + f;
         leaf = __shfl_sync(0xffffffffu, lm.x, owner);
+        leaf_begin = __shfl_sync(0xffffffffu, begin, owner);
         mask = (unsigned int)__shfl_sync(0xffffffffu, lm.y, owner);
         if (f >= total) mask = 0u;
     }

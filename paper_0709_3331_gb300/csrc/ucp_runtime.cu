@@ -521,8 +521,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
         dalloc(c, &c->t.lo, cz);
         dalloc(c, &c->t.rec, cz * kRec);
         dalloc(c, &c->t.mom32, cz * 16);
-        // sources in pairs: 2 float4 per pair of particles (padded to an even count)
-        dalloc(c, &c->src32, n + 1);
+        dalloc(c, &c->src32, n + 2 * cz + kSrcSlack);
     }
     dalloc(c, &c->cube, (size_t)n_clouds);
     {
@@ -583,8 +582,6 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
         cudaMemsetAsync(c->topo_status, 0, 8 * topo_status_words(c->n), c->s) ||
         cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) ||
         cudaMemsetAsync(c->ctl.epoch, 0, sizeof(unsigned int), c->s) ||
-        // the pad slot of an odd count is read (masked) by the pair loop: keep it finite
-        (c->src32 && cudaMemsetAsync(c->src32, 0, sizeof(float4) * (n + 1), c->s)) ||
         cudaMemcpyAsync(c->cloud_start, c->cloud_start_h.data(), sizeof(int) * (n_clouds + 1),
                         cudaMemcpyHostToDevice, c->s) ||
         (c->cloud && cudaMemcpyAsync(c->cloud, cl.data(), n, cudaMemcpyHostToDevice, c->s)) ||

@@ -26,6 +26,16 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float v)
     s = t;
 }
 
+__device__ __forceinline__ void two_sum_acc2(float2& s, float2& c, float2 v)
+{
+    const float2 n = make_float2(-1.f, -1.f);
+    const float2 t = __fadd2_rn(s, v);
+    const float2 bp = __ffma2_rn(n, s, t);
+    const float2 ap = __ffma2_rn(n, bp, t);
+    c = __fadd2_rn(c, __fadd2_rn(__ffma2_rn(n, ap, s), __ffma2_rn(n, bp, v)));
+    s = t;
+}
+
 // ------------------------------------------------------------------ FP64
 // One warp walks one target; its lanes are boxes and sources.  A step of the
 // traversal pops up to four opened twigs from a stack and tests their children, one
@@ -235,24 +245,30 @@ k_walk_fp64(WalkArgs a)
 }
 
 // ------------------------------------------------------------------ FP32C
-// Kelbg pair factors in FP32 for u = r/lambda: p = (1 - e^-u)/u and
-// g = (1 - (1 + u) e^-u)/u^3, by their Taylor series below u = 1/2 (no
-// cancellation) and directly above.
-__device__ __forceinline__ void kelbg_pg(float u, float& p, float& g)
+// Kelbg factors of an unlike pair, 1 - e^-u of the potential and 1 - (1 + u) e^-u of the
+// field, u = r/lambda: directly from u = 1/2 on, below by their Taylor series (no
+// cancellation).  A coincident pair (r < 1e-18) takes the limit, potential 1/lambda and
+// no field: ri becomes 1/lambda with the factors 1 and 0.
+__device__ __forceinline__ void kelbg_factors(float d2, float& ri, float inv_lambda, float& fp,
+                                              float& fg)
 {
-    if (u < 0.5f) {
-        p = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5040.f, -1.f / 720.f),
-                                                    1.f / 120.f), -1.f / 24.f), 1.f / 6.f),
-                          -0.5f), 1.f);
-        float poly = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5760.f, -1.f / 840.f),
-                                                  1.f / 144.f), -1.f / 30.f), 0.125f),
-                          -1.f / 3.f);
-        g = 0.5f / u + poly;
+    const float u = d2 * ri * inv_lambda;
+    if (d2 < 1e-36f) {
+        ri = inv_lambda;
+        fp = 1.f;
+        fg = 0.f;
+    } else if (u >= 0.5f) {
+        const float e = __expf(-u);
+        fp = 1.f - e;
+        fg = 1.f - (1.f + u) * e;
     } else {
-        float e = __expf(-u);
-        float iu = 1.f / u;
-        p = (1.f - e) * iu;
-        g = (1.f - (1.f + u) * e) * iu * iu * iu;
+        fp = u * fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5040.f, -1.f / 720.f),
+                                                     1.f / 120.f), -1.f / 24.f), 1.f / 6.f),
+                              -0.5f), 1.f);
+        const float poly = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5760.f, -1.f / 840.f),
+                                                        1.f / 144.f), -1.f / 30.f), 0.125f),
+                                -1.f / 3.f);
+        fg = u * u * fmaf(u, poly, 0.5f);
     }
 }
 
@@ -316,10 +332,11 @@ k_walk_fp32c(WalkArgs a)
         const float xh = tg.xh, yh = tg.yh, zh = tg.zh, xl = tg.xl, yl = tg.yl, zl = tg.zl;
         const float qt = valid ? (a.sp[t] ? (float)q1 : (float)q0) : 0.f;
         const float inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
-        const float inv_lambda3 = inv_lambda * inv_lambda * inv_lambda;
         // compensated totals (sum, correction)
-        float sx = 0.f, sy = 0.f, sz = 0.f, sp = 0.f, cx = 0.f, cy = 0.f, cz = 0.f, cp = 0.f;
+        float2 sxy = splat(0.f), szp = sxy, cxy = sxy, czp = sxy;   // {x, y}, {z, potential}
         int np = 0, nm = 0;
+        // slots of the chunk's targets (ascending)
+        const int tmin = __shfl_sync(0xffffffffu, t, 0), tmax = __shfl_sync(0xffffffffu, t, ck.y - 1);
 
         // the last cnt <= 32 boxes of the list of accepted boxes
         auto multipoles = [&](const int2* boxes, int cnt) {
@@ -383,146 +400,101 @@ k_walk_fp32c(WalkArgs a)
                     bp = __ffma2_rn(g, __ffma2_rn(u, v, make_float2(f1.z, f1.w)), bp);
                 }
             }
-            two_sum_acc(sx, cx, -(bx.x + bx.y));
-            two_sum_acc(sy, cy, -(by.x + by.y));
-            two_sum_acc(sz, cz, -(bz.x + bz.y));
-            if (kPhi) two_sum_acc(sp, cp, bp.x + bp.y);
+            two_sum_acc2(sxy, cxy, make_float2(-(bx.x + bx.y), -(by.x + by.y)));
+            two_sum_acc2(szp, czp, make_float2(-(bz.x + bz.y), kPhi ? bp.x + bp.y : 0.f));
             __syncwarp();
         };
 
-        // the last cnt <= 32 leaves of the list of opened leaves, their sources brought
-        // into shared memory one leaf (32 float4: up to 32 sources) ahead
-        auto direct_pairs = [&](const int2* leaves, int cnt) {
-            float4* meta = reinterpret_cast<float4*>(W.stage);   // {-ch, begin}, {-cl, end}
+        // cnt <= 32 opened leaves, each one's sources brought into shared memory (up to
+        // 32 float4) while the leaf before it is summed
+        auto direct_pairs = [&](int2* leaves, int cnt) {
+            float4* meta = reinterpret_cast<float4*>(W.stage);   // {-ch, place}, {-cl, begin}
             float4* buf = meta + 64;                             // 2 x 32 float4
             if (lane < cnt) {
                 const int nd = leaves[lane].x;
                 float4 A = __ldg(H + nd), B = __ldg(a.t.lo + nd);
                 const int2 be = __ldg(reinterpret_cast<const int2*>(a.t.info + nd));
-                A.w = __int_as_float(be.x);
-                B.w = __int_as_float(be.y);
+                A.w = __int_as_float(src_place(be.x, nd));
+                B.w = __int_as_float(be.x);
                 meta[2 * lane] = A;
                 meta[2 * lane + 1] = B;
+                leaves[lane].x = be.y - be.x;                    // {particles, mask}
             }
             __syncwarp();
-            // float4 s + lane of a leaf's sources, which lie in pairs {x_2p, x_2p+1, y..,
-            // y..}, {z.., z.., q.., q..} as offsets c_leaf - x_j; a pair member outside
-            // [jb, je) is moved far away and takes no charge
-            auto fetch = [&](int jb, int je, int s) -> float4 {
-                const int i = s + lane;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (i < ((je + 1) & ~1)) v = __ldg(S + i);
-                if (lane & 1) {
-                    if (i <= jb) v.z = 0.f;
-                    if (i >= je) v.w = 0.f;
-                } else {
-                    if (i < jb) v.x = 1e18f;
-                    if (i + 1 >= je) v.y = 1e18f;
-                }
-                return v;
-            };
-            float2 px = splat(0.f), py = px, pz = px, pp = px;
-            int e = 0, b = 0;
-            int jb = __float_as_int(meta[0].w), je = __float_as_int(meta[1].w), s = jb & ~1;
-            float4 v = fetch(jb, je, s);
-            while (true) {
-                buf[b * 32 + lane] = v;
-                int e1 = e, jb1 = jb, je1 = je, s1 = s + 32;
-                if (s1 >= je) {
-                    ++e1;
-                    if (e1 < cnt) {
-                        jb1 = __float_as_int(meta[2 * e1].w);
-                        je1 = __float_as_int(meta[2 * e1 + 1].w);
-                        s1 = jb1 & ~1;
-                    }
-                }
-                if (e1 < cnt) v = fetch(jb1, je1, s1);
+            const float2 e2 = splat(eps2);
+            float4 v = __ldg(S + __float_as_int(meta[0].w) + lane);
+            for (int e = 0; e < cnt; ++e) {
+                float4* P = buf + (e & 1) * 32;
+                P[lane] = v;
+                if (e + 1 < cnt) v = __ldg(S + __float_as_int(meta[2 * e + 2].w) + lane);
                 __syncwarp();
-                if (leaves[e].y & me) {
-                    const float4 A = meta[2 * e], B = meta[2 * e + 1];
-                    const float rx = (xh + A.x) + (xl + B.x);
-                    const float ry = (yh + A.y) + (yl + B.y);
-                    const float rz = (zh + A.z) + (zl + B.z);
-                    const float4* P = buf + b * 32;
-                    const int pairs = (min(s + 32, je + 1) - s) >> 1;
-                    const int lo = max(jb, s), hi = min(je, s + 32);   // sources of this part
-                    const bool self = t >= lo && t < hi;
-                    np += hi - lo - (self ? 1 : 0);
+                const int2 nm1 = leaves[e];
+                if (!(nm1.y & me)) continue;
+                const float4 A = meta[2 * e], B = meta[2 * e + 1];
+                const float2 rx = splat((xh + A.x) + (xl + B.x));
+                const float2 ry = splat((yh + A.y) + (yl + B.y));
+                const float2 rz = splat((zh + A.z) + (zl + B.z));
+                const int begin = __float_as_int(B.w), num = nm1.x;
+                const int pairs = ((begin & 1) + num + 1) >> 1;
+                const bool self = (unsigned int)(t - begin) < (unsigned int)num;
+                np += num - (self ? 1 : 0);
+                // place of the target's own particle among the leaf's halves, or none
+                const int tp = self ? t - (begin & ~1) : -1;
+                float2 px = splat(0.f), py = px, pz = px, pp = px;
+                auto pair = [&](const float4 F, const float4 Q, bool ok0, bool ok1) {
+                    const float2 dx = __fadd2_rn(rx, make_float2(F.x, F.y));
+                    const float2 dy = __fadd2_rn(ry, make_float2(F.z, F.w));
+                    const float2 dz = __fadd2_rn(rz, make_float2(Q.x, Q.y));
+                    const float2 q = make_float2(Q.z, Q.w);
                     if (kKelbg) {
-                        // one source at a time: unlike charges (electron-ion) take the
-                        // Kelbg form, like charges the softened Coulomb law
-                        for (int j = lo; j < hi; ++j) {
-                            if (j == t) continue;
-                            const float4 F = P[(j & ~1) - s], Q = P[(j | 1) - s];
-                            const bool odd = j & 1;
-                            float dx = rx + (odd ? F.y : F.x);
-                            float dy = ry + (odd ? F.w : F.z);
-                            float dz = rz + (odd ? Q.y : Q.x);
-                            float qj = odd ? Q.w : Q.z;
-                            if (qj != qt) {
-                                float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                                if (r2 == 0.f) {
-                                    pp.x = fmaf(qj, inv_lambda, pp.x);
-                                    continue;
-                                }
-                                float r = sqrtf(r2);
-                                float pf, gf;
-                                kelbg_pg(r * inv_lambda, pf, gf);
-                                float fq = qj * gf * inv_lambda3;
-                                px.x = fmaf(fq, dx, px.x);
-                                py.x = fmaf(fq, dy, py.x);
-                                pz.x = fmaf(fq, dz, pz.x);
-                                pp.x = fmaf(qj * inv_lambda, pf, pp.x);
-                            } else {
-                                float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-                                float ri = rsqrt_ftz(r2);
-                                float qi = qj * ri;
-                                float qr3 = qi * ri * ri;
-                                px.x = fmaf(qr3, dx, px.x);
-                                py.x = fmaf(qr3, dy, py.x);
-                                pz.x = fmaf(qr3, dz, pz.x);
-                                pp.x += qi;
-                            }
-                        }
+                        // unlike charges (electron-ion) take the Kelbg form, unsoftened:
+                        // the Coulomb terms times 1 - e^-u and 1 - (1 + u) e^-u, u = r/lambda
+                        const bool un0 = q.x != qt, un1 = q.y != qt;
+                        const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                        const float2 r2 = __fadd2_rn(d2, make_float2(un0 ? 0.f : eps2,
+                                                                     un1 ? 0.f : eps2));
+                        float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                                ok1 ? rsqrt_ftz(r2.y) : 0.f);
+                        float2 fp = splat(1.f), fg = fp;
+                        if (un0 && ok0) kelbg_factors(d2.x, ri.x, inv_lambda, fp.x, fg.x);
+                        if (un1 && ok1) kelbg_factors(d2.y, ri.y, inv_lambda, fp.y, fg.y);
+                        const float2 qi = __fmul2_rn(q, ri);
+                        const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
+                        px = __ffma2_rn(qr3, dx, px);
+                        py = __ffma2_rn(qr3, dy, py);
+                        pz = __ffma2_rn(qr3, dz, pz);
+                        pp = __ffma2_rn(qi, fp, pp);
                     } else {
-                        const float2 rx2 = splat(rx), ry2 = splat(ry), rz2 = splat(rz),
-                                     e2 = splat(eps2);
-                        const int tp = self ? t - s : -1;  // the target's own place
-#pragma unroll 2
-                        for (int p = 0; p < pairs; ++p) {
-                            const float4 F = P[2 * p], Q = P[2 * p + 1];
-                            const float2 dx = __fadd2_rn(rx2, make_float2(F.x, F.y));
-                            const float2 dy = __fadd2_rn(ry2, make_float2(F.z, F.w));
-                            const float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
-                            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy,
-                                                         __ffma2_rn(dz, dz, e2)));
-                            const float2 ri = make_float2(
-                                2 * p != tp ? rsqrt_ftz(r2.x) : 0.f,
-                                2 * p + 1 != tp ? rsqrt_ftz(r2.y) : 0.f);
-                            const float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
-                            const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
-                            px = __ffma2_rn(qr3, dx, px);
-                            py = __ffma2_rn(qr3, dy, py);
-                            pz = __ffma2_rn(qr3, dz, pz);
-                            if (kPhi) pp = __fadd2_rn(pp, qi);
-                        }
+                        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+                        const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                                      ok1 ? rsqrt_ftz(r2.y) : 0.f);
+                        const float2 qi = __fmul2_rn(q, ri);
+                        const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
+                        px = __ffma2_rn(qr3, dx, px);
+                        py = __ffma2_rn(qr3, dy, py);
+                        pz = __ffma2_rn(qr3, dz, pz);
+                        if (kPhi) pp = __fadd2_rn(pp, qi);
                     }
+                };
+                if (pairs > 16) {
+                    // longer than the buffer: straight from memory
+                    const float4* F = S + __float_as_int(A.w);
+#pragma unroll 1
+                    for (int p = 0; p < pairs; ++p)
+                        pair(__ldg(F + 2 * p), __ldg(F + 2 * p + 1), 2 * p != tp, 2 * p + 1 != tp);
+                } else if (begin <= tmax && begin + num > tmin) {
+                    // may hold targets of the chunk
+#pragma unroll 1
+                    for (int p = 0; p < pairs; ++p)
+                        pair(P[2 * p], P[2 * p + 1], 2 * p != tp, 2 * p + 1 != tp);
+                } else {
+#pragma unroll 2
+                    for (int p = 0; p < pairs; ++p) pair(P[2 * p], P[2 * p + 1], true, true);
                 }
                 // a leaf's pairs are summed in FP32 and enter the total by a compensated
                 // add (folding every fourth leaf only is 1.5 % faster and 1 % less exact)
-                if (e1 != e) {
-                    two_sum_acc(sx, cx, px.x + px.y);
-                    two_sum_acc(sy, cy, py.x + py.y);
-                    two_sum_acc(sz, cz, pz.x + pz.y);
-                    if (kPhi) two_sum_acc(sp, cp, pp.x + pp.y);
-                    px = py = pz = pp = splat(0.f);
-                }
-                if (e1 >= cnt) break;
-                e = e1;
-                jb = jb1;
-                je = je1;
-                s = s1;
-                b ^= 1;
+                two_sum_acc2(sxy, cxy, make_float2(px.x + px.y, py.x + py.y));
+                two_sum_acc2(szp, czp, make_float2(pz.x + pz.y, kPhi ? pp.x + pp.y : 0.f));
             }
             __syncwarp();
         };
@@ -532,10 +504,10 @@ k_walk_fp32c(WalkArgs a)
         if (valid) {
             const int s = a.sp[t];
             const double qm = (s ? q1 : q0) / a.msp[s];
-            a.ax[t] = qm * ((double)sx + (double)cx);
-            a.ay[t] = qm * ((double)sy + (double)cy);
-            a.az[t] = qm * ((double)sz + (double)cz);
-            if (kPhi && a.phi) a.phi[t] = (double)sp + (double)cp;
+            a.ax[t] = qm * ((double)sxy.x + (double)cxy.x);
+            a.ay[t] = qm * ((double)sxy.y + (double)cxy.y);
+            a.az[t] = qm * ((double)szp.x + (double)czp.x);
+            if (kPhi && a.phi) a.phi[t] = (double)szp.y + (double)czp.y;
             a.cnt_p2p[t] = np;
             a.cnt_m2p[t] = nm;
         }
@@ -611,19 +583,18 @@ k_walk_fp32c_visits(WalkArgs a)
                 const float rx = (xh + A.x) + (xl + B.x), ry = (yh + A.y) + (yl + B.y),
                             rz = (zh + A.z) + (zl + B.z);
                 const int jb = __ldg(&a.t.info[nd].x), je = __ldg(&a.t.info[nd].y);
+                const float4* F = S + src_place(jb, nd);
                 const float2 rx2 = splat(rx), ry2 = splat(ry), rz2 = splat(rz), e2 = splat(eps2);
                 float2 px = splat(0.f), py = px, pz = px;
 #pragma unroll 2
-                for (int j = jb & ~1; j < je; j += 2) {
-                    const float4 P = __ldg(S + j), Q = __ldg(S + j + 1);
+                for (int j = jb & ~1; j < je; j += 2, F += 2) {
+                    const float4 P = __ldg(F), Q = __ldg(F + 1);
                     const float2 dx = __fadd2_rn(rx2, make_float2(P.x, P.y));
                     const float2 dy = __fadd2_rn(ry2, make_float2(P.z, P.w));
                     const float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
                     const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-                    const bool ok0 = j >= jb && j != t;
-                    const bool ok1 = j + 1 < je && j + 1 != t;
-                    const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
-                                                  ok1 ? rsqrt_ftz(r2.y) : 0.f);
+                    const float2 ri = make_float2(j != t ? rsqrt_ftz(r2.x) : 0.f,
+                                                  j + 1 != t ? rsqrt_ftz(r2.y) : 0.f);
                     const float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
                     const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
                     px = __ffma2_rn(qr3, dx, px);
