@@ -702,7 +702,6 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
                          int nsm, cudaStream_t s)
 {
     count_launch(3);
-    cudaMemsetAsync(a.work, 0, sizeof(int), s);
     cudaMemsetAsync(mu, 0, sizeof(double) * 3 * (size_t)n, s);
     if (a.src32) {
         int blocks = nsm * 16 < a.nchunks ? nsm * 16 : a.nchunks;

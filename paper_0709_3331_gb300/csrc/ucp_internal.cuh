@@ -159,7 +159,21 @@ void launch_moments(const double* x, const double* y, const double* z, const int
                     const int* pos_off, const Cube* cube, Tree t, float4* src32, int want_f32,
                     cudaStream_t s);
 
-// ---- walk (ucp_walk.cu) ----
+// ---- walk (ucp_walk.cu, ucp_schedule.cu) ----
+// Order in which a walk takes its chunks, and the costs it notes for the next order.
+constexpr int kCostBins = 256;
+struct WalkOrder {
+    int* order;             // chunk of every work item
+    float* cost;            // cycles per chunk of the last walk
+    int* bins;              // chunks per cost bin, then the rewrite's cursors (2 x kCostBins)
+};
+// bin of a cost, longest first: 16 bins per factor of two from 2^8 cycles up
+__device__ __forceinline__ int cost_bin(float c)
+{
+    const int b = (__float_as_int(c) >> 19) - ((127 + 8) << 4);
+    return kCostBins - 1 - (b < 0 ? 0 : (b > kCostBins - 1 ? kCostBins - 1 : b));
+}
+
 struct WalkArgs {
     const double* x; const double* y; const double* z;
     const int8_t* sp;
@@ -171,6 +185,7 @@ struct WalkArgs {
     int ntargets;
     const int4* chunks;     // {first target index, count <= 32, cloud, 0}, one cloud each
     int nchunks;
+    WalkOrder ord;          // FP32C forward walks only
     const int* pos_off;     // first box started at each sorted position (the roots)
     const Cube* cubes;      // per cloud: FP32C coordinates are taken relative to the centre
     double eps2;
@@ -182,15 +197,15 @@ struct WalkArgs {
     int* err;               // raised by a bounded wait that gave up
     unsigned long long* stats; // {p2p, m2p}
 };
-void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, cudaStream_t s);
+// per walk: box records, and the work counter and cost bins (may be NULL) cleared
+void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
+                        cudaStream_t s);
 void launch_walk_fp64(const WalkArgs& a, int nsm, cudaStream_t s);
 void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape);
 void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, cudaStream_t s);  // no potential
 int walk_shape_count();
-// Reorders a chunk list longest-first by the cost (20 per pair + 64 per multipole)
-// its targets had in the walk just finished; cost and tmp hold nchunks entries.
-void launch_chunk_order(int4* chunks, int nchunks, const int* targets, const int* cnt_p2p,
-                        const int* cnt_m2p, float* cost, int4* tmp, cudaStream_t s);
+// rewrites o.order longest-first by the costs of the walk just finished
+void launch_chunk_order(const WalkOrder& o, int nchunks, cudaStream_t s);
 
 // ---- adjoint (ucp_adjoint.cu) ----
 // mu (n particles, key order) = (d a / d x)^T lam over the targets of a (all
@@ -237,6 +252,6 @@ void launch_load_state(const double* pos, const double* vel, const int8_t* sp, i
 void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n,
                         const unsigned char* cloud, int* flags, cudaStream_t s);
 void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
-                   int4* chunks, cudaStream_t s);
+                   int4* chunks, int* order, cudaStream_t s);
 
 }  // namespace ucp

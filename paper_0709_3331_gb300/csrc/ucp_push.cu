@@ -196,9 +196,10 @@ __global__ void k_check_state(const double* __restrict__ pos, const double* __re
 }
 
 // Walk chunks of up to `width` consecutive targets, cloud by cloud: cloud c's run of
-// targets is [first[c], first[c + 1]), its chunks start at place[c].
+// targets is [first[c], first[c + 1]), its chunks start at place[c]; taken in list order.
 __global__ void k_chunks(const int* __restrict__ first, const int* __restrict__ place, int n_clouds,
-                         int width, int nchunks, int4* __restrict__ chunks)
+                         int width, int nchunks, int4* __restrict__ chunks,
+                         int* __restrict__ order)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nchunks) return;
@@ -210,6 +211,7 @@ __global__ void k_chunks(const int* __restrict__ first, const int* __restrict__ 
     }
     const int b = first[lo] + (i - place[lo]) * width;
     chunks[i] = make_int4(b, min(width, first[lo + 1] - b), lo, 0);
+    order[i] = i;
 }
 
 inline int nb(int n) { return (n + kT - 1) / kT > 0 ? (n + kT - 1) / kT : 1; }
@@ -284,11 +286,11 @@ void launch_check_state(const double* pos, const double* vel, const int8_t* sp, 
 }
 
 void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
-                   int4* chunks, cudaStream_t s)
+                   int4* chunks, int* order, cudaStream_t s)
 {
     if (nchunks < 1) return;
     count_launch(1);
-    k_chunks<<<nb(nchunks), kT, 0, s>>>(first, place, n_clouds, width, nchunks, chunks);
+    k_chunks<<<nb(nchunks), kT, 0, s>>>(first, place, n_clouds, width, nchunks, chunks, order);
 }
 
 }  // namespace ucp

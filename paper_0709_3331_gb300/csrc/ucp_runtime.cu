@@ -77,8 +77,10 @@ struct ucp_ctx {
     unsigned char* cloud = nullptr;    // cloud of each slot (batches only)
     int4* chunks_all = nullptr;        // walk chunks over all particles
     int4* chunks_e = nullptr;          // walk chunks over the compacted electrons
+    int* order_all = nullptr;          // order in which the walks take them
+    int* order_e = nullptr;
     float* chunk_cost = nullptr;       // per chunk, for the longest-first order
-    int4* chunk_tmp = nullptr;
+    int* cost_bins = nullptr;
     int n_chunks_all = 0, n_chunks_e = 0, n_chunks_all_cap = 0;
     int sorted_buf = 0;                // key[] / val[] buffer of the last sort
     std::vector<double> cloud_energy;  // per-cloud {KE_i, KE_e, PE, px, py, pz} of the last energy
@@ -265,8 +267,8 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
 {
     int k = c->cur;
     int f32 = c->precision == UCP_FP32C;
-    launch_mac_prepare(c->t, c->cube, theta, f32, c->s);
-    WalkArgs a;
+    launch_mac_prepare(c->t, c->cube, theta, f32, c->work, c->cost_bins, c->s);
+    WalkArgs a = {};
     a.x = c->st[k][0];
     a.y = c->st[k][1];
     a.z = c->st[k][2];
@@ -275,6 +277,7 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
     a.msp = c->msp;
     a.src32 = c->src32;
     a.t = c->t;
+    a.ord = {electrons_only ? c->order_e : c->order_all, c->chunk_cost, c->cost_bins};
     if (electrons_only) {
         launch_select(c->sp[k], UCP_ELECTRON, c->n, c->tlist, c->sel_part, c->cnt_p2p,
                       c->cnt_m2p, c->s);
@@ -310,9 +313,7 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
         prof_end(c);
         // the next walk over the same targets takes its chunks longest-first (the FP64
         // walk takes one target at a time: its end is as even without)
-        if (f32)
-            launch_chunk_order(electrons_only ? c->chunks_e : c->chunks_all, a.nchunks, a.targets,
-                               c->cnt_p2p, c->cnt_m2p, c->chunk_cost, c->chunk_tmp, c->s);
+        if (f32) launch_chunk_order(a.ord, a.nchunks, c->s);
         c->walk_targets += a.ntargets;
         c->walk_launches += 1;
     }
@@ -334,7 +335,7 @@ constexpr int kChunk = 32;
 // are the host's, the lists are written on the device.  table: room for 2 (n_clouds
 // + 1) ints on the host (its contents are uploaded) and on the device.
 int build_chunks(ucp_ctx* c, const int* first, int* host_table, int* table, int4* chunks,
-                 int* n_chunks)
+                 int* order, int* n_chunks)
 {
     const int nc = c->n_clouds;
     int* place = host_table + nc + 1;
@@ -348,7 +349,7 @@ int build_chunks(ucp_ctx* c, const int* first, int* host_table, int* table, int4
     place[nc] = total;
     if (total > c->n_chunks_all_cap) return fail(c, UCP_EINVAL, "internal: chunk capacity");
     CK(cudaMemcpyAsync(table, host_table, sizeof(int) * 2 * (nc + 1), cudaMemcpyHostToDevice, c->s));
-    launch_chunks(table, table + nc + 1, nc, kChunk, total, chunks, c->s);
+    launch_chunks(table, table + nc + 1, nc, kChunk, total, chunks, order, c->s);
     *n_chunks = total;
     return UCP_OK;
 }
@@ -548,7 +549,9 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->chunks_all, (size_t)nch);
     dalloc(c, &c->chunks_e, (size_t)nch);
     dalloc(c, &c->chunk_cost, (size_t)nch);
-    dalloc(c, &c->chunk_tmp, (size_t)nch);
+    dalloc(c, &c->order_all, (size_t)nch);
+    dalloc(c, &c->order_e, (size_t)nch);
+    dalloc(c, &c->cost_bins, 2 * kCostBins);
     dalloc(c, &c->qsp, 2);
     dalloc(c, &c->msp, 2);
     dalloc(c, &c->tlist, n);
@@ -596,7 +599,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     c->host_table = c->host_flags + 3 + 2 * UCP_MAX_CLOUDS;
     // the chunks over every particle follow from the sizes alone
     if ((rc = build_chunks(c, c->cloud_start_h.data(), c->host_table, c->chunk_table, c->chunks_all,
-                           &c->n_chunks_all)))
+                           c->order_all, &c->n_chunks_all)))
         return bail(rc);
     if (cudaStreamSynchronize(c->s) || check_launch(c, "create")) return bail(UCP_ECUDA);
     *out = c;
@@ -635,7 +638,8 @@ int ucp_set_state(ucp_ctx* c, const double* pos, const double* vel, const int8_t
     first[0] = 0;
     for (int cl = 0; cl < nc; ++cl) first[cl + 1] = first[cl] + fl[2 + cl];
     c->n_e = first[nc];
-    int rc = build_chunks(c, first, c->host_table, c->chunk_table, c->chunks_e, &c->n_chunks_e);
+    int rc = build_chunks(c, first, c->host_table, c->chunk_table, c->chunks_e, c->order_e,
+                          &c->n_chunks_e);
     if (rc) return rc;
     launch_load_state(dpos, dvel, dsp, c->n, c->st[k], c->sp[k], c->sp_caller, c->id[k], c->s);
     CK(cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s));
@@ -1052,7 +1056,7 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
     launch_ke_seed(ck + 2 * n3 * nseg + n3, c->sp_caller, c->n, c->m[UCP_ELECTRON], lv, dloss,
                    c->s);
     cudaMemsetAsync(lx, 0, sizeof(double) * n3, c->s);
-    WalkArgs a;
+    WalkArgs a = {};
     // reverse: for g = S .. 1: adjoint of the kicks at X_g, then of drift g; X_0 last
     for (int64_t sgi = nseg - 1; sgi >= 0 && !rc; --sgi) {
         const int64_t g0 = sgi * C, len = std::min(C, S - g0);
@@ -1073,7 +1077,7 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
             load_state(c, seg + n3 * (size_t)j, nullptr);
             if ((rc = build(c))) break;
             const int f32 = c->precision == UCP_FP32C;
-            launch_mac_prepare(c->t, c->cube, theta, f32, c->s);
+            launch_mac_prepare(c->t, c->cube, theta, f32, c->work, nullptr, c->s);
             int k = c->cur;
             launch_kick_lambda(lv, c->sp_caller, c->n, ce, ci, lam, c->s);
             launch_gather3(lam, c->id[k], c->n, lsorted, c->s);
@@ -1149,10 +1153,10 @@ int ucp_accel_vjp(ucp_ctx* c, double theta, double eps, const double* lam_in, do
         CK(cudaMemcpyAsync(c->stage, lam_in, sizeof(double) * n3, cudaMemcpyHostToDevice, c->s));
     if (!c->tree_valid && (rc = build(c))) return rc;
     const int f32 = c->precision == UCP_FP32C;
-    launch_mac_prepare(c->t, c->cube, theta, f32, c->s);
+    launch_mac_prepare(c->t, c->cube, theta, f32, c->work, nullptr, c->s);
     const int k = c->cur;
     launch_gather3(on_device ? lam_in : c->stage, c->id[k], c->n, lsorted, c->s);
-    WalkArgs a;
+    WalkArgs a = {};
     a.x = c->st[k][0];
     a.y = c->st[k][1];
     a.z = c->st[k][2];

@@ -322,8 +322,10 @@ k_walk_fp32c(WalkArgs a)
     const float4* __restrict__ S = a.src32;
     const float eps2 = (float)a.eps2;
 
-    for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
-         chunk = next_chunk(a.work, lane)) {
+    for (int item = next_chunk(a.work, lane); item < a.nchunks;
+         item = next_chunk(a.work, lane)) {
+        const long long began = clock64();
+        const int chunk = a.ord.order[item];
         const int4 ck = a.chunks[chunk];
         const int ti = ck.x + lane;
         const bool valid = lane < ck.y;
@@ -520,6 +522,9 @@ k_walk_fp32c(WalkArgs a)
         if (lane == 0) {
             atomicAdd(&a.stats[0], sp2);
             atomicAdd(&a.stats[1], sm2);
+            const float cost = (float)(clock64() - began);
+            a.ord.cost[chunk] = cost;
+            atomicAdd(&a.ord.bins[cost_bin(cost)], 1);
         }
     }
 }
@@ -547,8 +552,10 @@ k_walk_fp32c_visits(WalkArgs a)
     const float4* __restrict__ S = a.src32;
     const float eps2 = (float)a.eps2;
 
-    for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
-         chunk = next_chunk(a.work, lane)) {
+    for (int item = next_chunk(a.work, lane); item < a.nchunks;
+         item = next_chunk(a.work, lane)) {
+        const long long began = clock64();
+        const int chunk = a.ord.order[item];
         const int4 ck = a.chunks[chunk];
         const int t = lane < ck.y ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
         const bool valid = t >= 0;
@@ -678,14 +685,23 @@ k_walk_fp32c_visits(WalkArgs a)
         if (lane == 0) {
             atomicAdd(&a.stats[0], sp2);
             atomicAdd(&a.stats[1], sm2);
+            const float cost = (float)(clock64() - began);
+            a.ord.cost[chunk] = cost;
+            atomicAdd(&a.ord.bins[cost_bin(cost)], 1);
         }
     }
 }
 
 // Per walk: rcrit2 = (s/theta + delta)^2 of every box in FP64 (theta = 0:
 // +inf, nothing accepted), and the FP32C box records.
-__global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32)
+__global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32,
+                              int* work, int* bins)
 {
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) *work = 0;
+        if (bins)
+            for (int i = threadIdx.x; i < 2 * kCostBins; i += blockDim.x) bins[i] = 0;
+    }
     const int nn = *t.nnodes;
     for (int nd = blockIdx.x * blockDim.x + threadIdx.x; nd < nn; nd += gridDim.x * blockDim.x) {
         double* m = t.mom + (size_t)nd * kMom;
@@ -725,11 +741,12 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
 
 }  // namespace
 
-void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, cudaStream_t s)
+void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
+                        cudaStream_t s)
 {
     count_launch(1);
     int blocks = 4 * 152;
-    k_mac_prepare<<<blocks, 256, 0, s>>>(t, cube, theta, want_f32);
+    k_mac_prepare<<<blocks, 256, 0, s>>>(t, cube, theta, want_f32, work, bins);
 }
 
 // blocks of one warp: per_sm on every SM, or one per work item
@@ -743,7 +760,6 @@ void launch_walk_fp64(const WalkArgs& a, int nsm, cudaStream_t s)
 {
     count_launch(1);
     const int b = walk_blocks((int64_t)a.nchunks * 32, nsm, 16);
-    cudaMemsetAsync(a.work, 0, sizeof(int), s);
     // the potential is computed only when the caller reads it
     if (a.kelbg && a.phi) k_walk_fp64<true, true><<<b, 32, 0, s>>>(a);
     else if (a.kelbg) k_walk_fp64<true, false><<<b, 32, 0, s>>>(a);
@@ -780,7 +796,6 @@ static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, cudaStream_t 
 void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
 {
     count_launch(1);
-    cudaMemsetAsync(a.work, 0, sizeof(int), s);
     if (shape < 0 || shape >= walk_shape_count()) shape = 0;
     const int per_sm = kShapes[shape][1];
     const int b = walk_blocks(a.nchunks, nsm, per_sm);
@@ -794,7 +809,6 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
 void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, cudaStream_t s)
 {
     count_launch(1);
-    cudaMemsetAsync(a.work, 0, sizeof(int), s);
     const int wpb = kVisitThreads / 32;
     const int b = walk_blocks(((int64_t)a.nchunks + wpb - 1) / wpb, nsm, 7);
     k_walk_fp32c_visits<<<b, kVisitThreads, 0, s>>>(a);
