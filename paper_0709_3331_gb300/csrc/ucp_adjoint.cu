@@ -81,7 +81,7 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
         const ChunkTarget tg(a, t, ck.z);
         if (t >= 0) {
             const int s = a.sp[t];
-            const double qm = (s ? q1 : q0) / a.msp[s];
+            const double qm = a.msp[2 + s];
             W.tgt[lane][0] = a.x[t];
             W.tgt[lane][1] = a.y[t];
             W.tgt[lane][2] = a.z[t];
@@ -110,7 +110,7 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
                 if (!((mask >> g) & 1u)) continue;
                 const double R[3] = {W.tgt[g][0] - c[0], W.tgt[g][1] - c[1], W.tgt[g][2] - c[2]};
                 const double w[3] = {W.tgt[g][3], W.tgt[g][4], W.tgt[g][5]};
-                const double gi = rsqrt(dot3(R, R) + a.eps2);
+                const double gi = rsqrt_fp64(dot3(R, R) + a.eps2);
                 const double u = gi * gi, g3 = gi * u, g5 = g3 * u, g7 = g5 * u, g9 = g7 * u;
                 const double rw = dot3(R, w), rd = dot3(R, D), wd = dot3(w, D);
                 double q[3], qw[3];
@@ -177,7 +177,7 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
                     if (!((mask >> g) & 1u) || W.slot[g] == j) continue;
                     const double R[3] = {W.tgt[g][0] - xj, W.tgt[g][1] - yj, W.tgt[g][2] - zj};
                     const double w[3] = {W.tgt[g][3], W.tgt[g][4], W.tgt[g][5]};
-                    const double gi = rsqrt(dot3(R, R) + a.eps2);
+                    const double gi = rsqrt_fp64(dot3(R, R) + a.eps2);
                     const double u = gi * gi, cw = qj * (gi * u);
                     const double cr = -3.0 * (cw * u) * dot3(R, w);
 #pragma unroll
@@ -286,7 +286,6 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
     __shared__ AdjWarp shared;
     AdjWarp& W = shared;
     const int lane = threadIdx.x;
-    const double q0 = a.qsp[0], q1 = a.qsp[1];
     const float4* __restrict__ S = a.src32;
     const float2 e2 = splat((float)a.eps2);
 
@@ -299,7 +298,7 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
             float w[3] = {0.f, 0.f, 0.f};
             if (t >= 0) {
                 const int s = a.sp[t];
-                const double qm = (s ? q1 : q0) / a.msp[s];
+                const double qm = a.msp[2 + s];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) w[k] = (float)(qm * lam[3 * (size_t)t + k]);
             }

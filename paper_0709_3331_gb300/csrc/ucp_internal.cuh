@@ -178,7 +178,7 @@ struct WalkArgs {
     const double* x; const double* y; const double* z;
     const int8_t* sp;
     const double* qsp;      // charge per species (device, 2)
-    const double* msp;      // mass per species (device, 2)
+    const double* msp;      // mass, then charge over mass, per species (device, 4)
     const float4* src32;    // FP32C sources (src_place)
     Tree t;
     const int* targets;     // key-order slots of the targets, or NULL = all

@@ -553,7 +553,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->order_e, (size_t)nch);
     dalloc(c, &c->cost_bins, 2 * kCostBins);
     dalloc(c, &c->qsp, 2);
-    dalloc(c, &c->msp, 2);
+    dalloc(c, &c->msp, 4);
     dalloc(c, &c->tlist, n);
     dalloc(c, &c->sel_part, select_words(c->n));
     dalloc(c, &c->cnt_p2p, n);
@@ -578,6 +578,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
             for (int j = c->cloud_start_h[i]; j < c->cloud_start_h[i + 1]; ++j)
                 cl[j] = (unsigned char)i;
     }
+    const double mqm[4] = {c->m[0], c->m[1], c->q[0] / c->m[0], c->q[1] / c->m[1]};
     // box tables a build has not filled are read only after a wait that gave up: empty
     if (cudaMemsetAsync(c->t.info, 0, sizeof(int4) * cz, c->s) ||
         cudaMemsetAsync(c->t.child8, 0xff, 8 * sizeof(int) * cz, c->s) ||
@@ -589,7 +590,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
                         cudaMemcpyHostToDevice, c->s) ||
         (c->cloud && cudaMemcpyAsync(c->cloud, cl.data(), n, cudaMemcpyHostToDevice, c->s)) ||
         cudaMemcpyAsync(c->qsp, c->q, 2 * sizeof(double), cudaMemcpyHostToDevice, c->s) ||
-        cudaMemcpyAsync(c->msp, c->m, 2 * sizeof(double), cudaMemcpyHostToDevice, c->s) ||
+        cudaMemcpyAsync(c->msp, mqm, sizeof(mqm), cudaMemcpyHostToDevice, c->s) ||
         cudaMemsetAsync(c->stats, 0, 2 * sizeof(unsigned long long), c->s) ||
         cudaHostAlloc(&c->host_flags, sizeof(int) * (3 + 2 * UCP_MAX_CLOUDS + 2 * (UCP_MAX_CLOUDS + 1)),
                       0)) {

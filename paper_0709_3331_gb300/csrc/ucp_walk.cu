@@ -103,7 +103,7 @@ k_walk_fp64(WalkArgs a)
                 const double rx = xt - m0.x, ry = yt - m0.y, rz = zt - m1.x;
                 const double r2 = rx * rx + (ry * ry + (rz * rz + a.eps2));
                 const double M = m2.x;
-                const double g = rsqrt(r2);
+                const double g = rsqrt_fp64(r2);
                 const double u = g * g;
                 const double g3 = g * u;
                 const double qx = m4.x * rx + m4.y * ry + m5.x * rz;
@@ -144,7 +144,7 @@ k_walk_fp64(WalkArgs a)
                         ph += qj * ome / r;
                     }
                 } else {
-                    const double ri = rsqrt(dx * dx + (dy * dy + (dz * dz + a.eps2)));
+                    const double ri = rsqrt_fp64(dx * dx + (dy * dy + (dz * dz + a.eps2)));
                     const double qi = qj * ri;
                     const double qr3 = qi * (ri * ri);
                     ex += qr3 * dx;
@@ -219,19 +219,28 @@ k_walk_fp64(WalkArgs a)
             __syncwarp();
         }
         __syncwarp();
+        // sums over the lanes by halving exchanges (six additions for the four values):
+        // lanes 0, 8, 16 and 24 end with x, y, z and the potential
+        {
+            const bool hi = lane & 16;
+            const double k0 = hi ? ez : ex, k1 = hi ? ph : ey;
+            const double s0 = hi ? ex : ez, s1 = hi ? ey : ph;
+            const double v0 = k0 + __shfl_xor_sync(0xffffffffu, s0, 16);
+            const double v1 = k1 + __shfl_xor_sync(0xffffffffu, s1, 16);
+            const bool odd = lane & 8;
+            double v = (odd ? v1 : v0) + __shfl_xor_sync(0xffffffffu, odd ? v0 : v1, 8);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ex += __shfl_xor_sync(0xffffffffu, ex, o);
-            ey += __shfl_xor_sync(0xffffffffu, ey, o);
-            ez += __shfl_xor_sync(0xffffffffu, ez, o);
-            if (kPhi) ph += __shfl_xor_sync(0xffffffffu, ph, o);
+            for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if ((lane & 7) == 0) {
+                if (lane == 24) {
+                    if (kPhi && a.phi) a.phi[t] = v;
+                } else {
+                    double* out = lane == 0 ? a.ax : lane == 8 ? a.ay : a.az;
+                    out[t] = a.msp[2 + st] * v;
+                }
+            }
         }
         if (lane == 0) {
-            const double qm = (st ? q1 : q0) / a.msp[st];
-            a.ax[t] = qm * ex;
-            a.ay[t] = qm * ey;
-            a.az[t] = qm * ez;
-            if (kPhi && a.phi) a.phi[t] = ph;
             a.cnt_p2p[t] = np;
             a.cnt_m2p[t] = nm;
         }
@@ -505,7 +514,7 @@ k_walk_fp32c(WalkArgs a)
 
         if (valid) {
             const int s = a.sp[t];
-            const double qm = (s ? q1 : q0) / a.msp[s];
+            const double qm = a.msp[2 + s];
             a.ax[t] = qm * ((double)sxy.x + (double)cxy.x);
             a.ay[t] = qm * ((double)sxy.y + (double)cxy.y);
             a.az[t] = qm * ((double)szp.x + (double)czp.x);
@@ -546,7 +555,6 @@ k_walk_fp32c_visits(WalkArgs a)
     __shared__ int2 lists[kVisitThreads / 32][kVisitList];   // {opened leaf, mask}
     const int lane = threadIdx.x & 31;
     int2* lst = lists[threadIdx.x >> 5];
-    const double q0 = a.qsp[0], q1 = a.qsp[1];
     const float4* __restrict__ H = a.t.hdr;
     const float4* __restrict__ LO = a.t.lo;
     const float4* __restrict__ S = a.src32;
@@ -669,7 +677,7 @@ k_walk_fp32c_visits(WalkArgs a)
 
         if (valid) {
             const int s = a.sp[t];
-            const double qm = (s ? q1 : q0) / a.msp[s];
+            const double qm = a.msp[2 + s];
             a.ax[t] = qm * ((double)sx + (double)cx);
             a.ay[t] = qm * ((double)sy + (double)cy);
             a.az[t] = qm * ((double)sz + (double)cz);

@@ -57,3 +57,24 @@ def test_walk_lists(U, orc, prec, tol, n, leaf_cap, theta, fat):
     p_ref, _, _ = orc.run(pos, vel, sp, c.q, c.m, 1e-4, 2, 1, theta, eps, leaf_cap=leaf_cap,
                           nthreads=4)
     assert np.abs(p1 - p_ref).max() <= 1e-6 * np.abs(pos).max()
+
+
+def test_pair_potential_over_the_range(U):
+    """The FP64 walk's reciprocal square root at the ends of its own range and beyond: two
+    particles a known distance apart, 240 pairs as an ensemble.  r^2 is exact, so phi is
+    within an ulp of the charge over the distance, and the field three roundings more."""
+    rng = np.random.default_rng(3)
+    d = np.ldexp(rng.integers(1 << 19, 1 << 20, 240) / float(1 << 20), rng.integers(-60, 80, 240))
+    d[:8] = np.ldexp(1.0, [-31, -30, -29, 49, 50, 51, 0, 1])
+    m = len(d)
+    pos = np.zeros((2 * m, 3))
+    pos[1::2, 0] = d
+    sp = np.tile(np.array([0, 1], dtype=np.int8), m)
+    with U.Context(2 * m, (1.0, -1.0), (1.0, 1.0), leaf_cap=1, precision=0, sizes=[2] * m) as ctx:
+        ctx.set_state(pos, np.zeros_like(pos), sp)
+        acc, phi = ctx.tree_force(0.0, 0.0)
+    u = np.spacing(1.0 / d)
+    assert (np.abs(phi[0::2] + 1.0 / d) <= u).all() and (np.abs(phi[1::2] - 1.0 / d) <= u).all()
+    f = 1.0 / (d * d)
+    assert (np.abs(acc[0::2, 0] - f) <= 6 * np.spacing(f)).all()
+    assert (np.abs(acc[1::2, 0] + f) <= 6 * np.spacing(f)).all()
