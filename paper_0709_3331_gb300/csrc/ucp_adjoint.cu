@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(32, 12)
 k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __restrict__ mu,
                double* __restrict__ adj)
 {
+    follow();
     __shared__ AdjWarp64 shared;
     AdjWarp64& W = shared;
     const int lane = threadIdx.x;
@@ -283,6 +284,7 @@ __global__ void __launch_bounds__(32, 16)
 k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restrict__ mu,
                    float* __restrict__ adj)
 {
+    follow();
     __shared__ AdjWarp shared;
     AdjWarp& W = shared;
     const int lane = threadIdx.x;
@@ -518,6 +520,7 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
                                const double* __restrict__ qsp, Tree t,
                                const TA* __restrict__ adj, double* __restrict__ mu)
 {
+    follow();
     const int nn = *t.nnodes;
     for (int leaf = blockIdx.x * blockDim.x + threadIdx.x; leaf < nn;
          leaf += gridDim.x * blockDim.x) {
@@ -554,6 +557,7 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
 template <class TA>
 __global__ void k_zero_adj(const int* __restrict__ nnodes, TA* __restrict__ adj)
 {
+    follow();
     const size_t total = (size_t)*nnodes * 12;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
          i += (size_t)gridDim.x * blockDim.x)
@@ -564,6 +568,7 @@ __global__ void k_zero_adj(const int* __restrict__ nnodes, TA* __restrict__ adj)
 __global__ void k_gather3(const double* __restrict__ src, const unsigned int* __restrict__ id, int n,
                           double* __restrict__ dst)
 {
+    follow();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     size_t j = id[t];
@@ -576,6 +581,7 @@ __global__ void k_gather3(const double* __restrict__ src, const unsigned int* __
 __global__ void k_scatter_add3(const double* __restrict__ src, const unsigned int* __restrict__ id,
                                int n, double* __restrict__ dst)
 {
+    follow();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     size_t j = id[t];
@@ -588,6 +594,7 @@ __global__ void k_scatter_add3(const double* __restrict__ src, const unsigned in
 __global__ void k_kick_lambda(const double* __restrict__ lam_v, const int8_t* __restrict__ sp, int n,
                               double ce, double ci, double* __restrict__ out)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double f = sp[i] ? ce : ci;
@@ -597,6 +604,7 @@ __global__ void k_kick_lambda(const double* __restrict__ lam_v, const int8_t* __
 // y += a x over n x 3
 __global__ void k_axpy3(double* __restrict__ y, const double* __restrict__ x, double a, int n)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 3 * n) return;
     y[i] += a * x[i];
@@ -610,6 +618,7 @@ __global__ void __launch_bounds__(256)
 k_ke_seed(const double* __restrict__ v, const int8_t* __restrict__ sp, int n, double me,
           double* __restrict__ lam_v, double* __restrict__ part)
 {
+    follow();
     double acc = 0.0;
     for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
         const bool e = sp[i] != 0;
@@ -631,6 +640,7 @@ k_ke_seed(const double* __restrict__ v, const int8_t* __restrict__ sp, int n, do
 
 __global__ void k_ke_sum(const double* __restrict__ part, int nblk, double* __restrict__ loss)
 {
+    follow();
     const int lane = threadIdx.x;
     double acc = 0.0;
     for (int b = lane; b < nblk; b += 32) acc += part[b];
@@ -643,6 +653,7 @@ __global__ void k_ke_sum(const double* __restrict__ part, int nblk, double* __re
 __global__ void k_scatter_rows3(const double* __restrict__ src, const unsigned int* __restrict__ id,
                                 int n, double* __restrict__ dst)
 {
+    follow();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     const size_t j = id[t];
@@ -653,52 +664,52 @@ __global__ void k_scatter_rows3(const double* __restrict__ src, const unsigned i
 
 }  // namespace
 
-void launch_gather3(const double* src, const unsigned int* id, int n, double* dst, cudaStream_t s)
+void launch_gather3(const double* src, const unsigned int* id, int n, double* dst, Queue s)
 {
     count_launch(1);
-    k_gather3<<<(n + 255) / 256, 256, 0, s>>>(src, id, n, dst);
+    launch(k_gather3, (n + 255) / 256, 256, s, src, id, n, dst);
 }
 
 void launch_scatter_add3(const double* src, const unsigned int* id, int n, double* dst,
-                         cudaStream_t s)
+                         Queue s)
 {
     count_launch(1);
-    k_scatter_add3<<<(n + 255) / 256, 256, 0, s>>>(src, id, n, dst);
+    launch(k_scatter_add3, (n + 255) / 256, 256, s, src, id, n, dst);
 }
 
 void launch_kick_lambda(const double* lam_v, const int8_t* sp, int n, double ce, double ci,
-                        double* out, cudaStream_t s)
+                        double* out, Queue s)
 {
     count_launch(1);
-    k_kick_lambda<<<(n + 255) / 256, 256, 0, s>>>(lam_v, sp, n, ce, ci, out);
+    launch(k_kick_lambda, (n + 255) / 256, 256, s, lam_v, sp, n, ce, ci, out);
 }
 
-void launch_axpy3(double* y, const double* x, double a, int n, cudaStream_t s)
+void launch_axpy3(double* y, const double* x, double a, int n, Queue s)
 {
     count_launch(1);
-    k_axpy3<<<(3 * n + 255) / 256, 256, 0, s>>>(y, x, a, n);
+    launch(k_axpy3, (3 * n + 255) / 256, 256, s, y, x, a, n);
 }
 
 size_t ke_seed_words() { return 1 + kSeedBlocks; }
 
 void launch_ke_seed(const double* v, const int8_t* sp, int n, double me, double* lam_v,
-                    double* loss, cudaStream_t s)
+                    double* loss, Queue s)
 {
     count_launch(2);
     const int b = n < 256 * kSeedBlocks ? (n + 255) / 256 : kSeedBlocks;
-    k_ke_seed<<<b, 256, 0, s>>>(v, sp, n, me, lam_v, loss + 1);
-    k_ke_sum<<<1, 32, 0, s>>>(loss + 1, b, loss);
+    launch(k_ke_seed, b, 256, s, v, sp, n, me, lam_v, loss + 1);
+    launch(k_ke_sum, 1, 32, s, loss + 1, b, loss);
 }
 
 void launch_scatter_rows3(const double* src, const unsigned int* id, int n, double* dst,
-                          cudaStream_t s)
+                          Queue s)
 {
     count_launch(1);
-    k_scatter_rows3<<<(n + 255) / 256, 256, 0, s>>>(src, id, n, dst);
+    launch(k_scatter_rows3, (n + 255) / 256, 256, s, src, id, n, dst);
 }
 
 void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, double* adj, int n,
-                         int nsm, cudaStream_t s)
+                         int nsm, Queue s)
 {
     count_launch(3);
     cudaMemsetAsync(mu, 0, sizeof(double) * 3 * (size_t)n, s);
@@ -707,18 +718,18 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
         if (blocks < 1) blocks = 1;
         // FP32C context: FP32 walk, FP32 box accumulators (in the same buffer)
         float* adjf = reinterpret_cast<float*>(adj);
-        k_zero_adj<float><<<2 * 152, 256, 0, s>>>(a.t.nnodes, adjf);
-        k_walk_adjoint_f32<<<blocks, 32, 0, s>>>(a, lam, mu, adjf);
-        k_adjoint_push<float><<<4 * 152, 256, 0, s>>>(a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
+        launch(k_zero_adj<float>, 2 * 152, 256, s, a.t.nnodes, adjf);
+        launch(k_walk_adjoint_f32, blocks, 32, s, a, lam, mu, adjf);
+        launch(k_adjoint_push<float>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
     } else {
-        k_zero_adj<double><<<2 * 152, 256, 0, s>>>(a.t.nnodes, adj);
+        launch(k_zero_adj<double>, 2 * 152, 256, s, a.t.nnodes, adj);
         // eight targets per warp, fewer while that leaves an SM with under four warps
         int group = kAdjGroup;
         while (group > 1 && (int64_t)a.nchunks * (32 / group) < 4 * (int64_t)nsm) group /= 2;
         const int64_t items = (int64_t)a.nchunks * (32 / group);
         const int blocks = items < 1 ? 1 : items < 12 * nsm ? (int)items : 12 * nsm;
-        k_walk_adjoint<<<blocks, 32, 0, s>>>(a, group, lam, mu, adj);
-        k_adjoint_push<double><<<4 * 152, 256, 0, s>>>(a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
+        launch(k_walk_adjoint, blocks, 32, s, a, group, lam, mu, adj);
+        launch(k_adjoint_push<double>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
     }
 }
 

@@ -22,6 +22,7 @@ __global__ void k_bbox_partial(const double* __restrict__ x, const double* __res
                                const double* __restrict__ z, int n, double* __restrict__ part,
                                const int* __restrict__ cloud_start)
 {
+    follow();
     const int c = blockIdx.y;
     const int lo_i = cloud_start ? cloud_start[c] : 0, hi_i = cloud_start ? cloud_start[c + 1] : n;
     unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
@@ -70,6 +71,7 @@ __global__ void k_bbox_partial(const double* __restrict__ x, const double* __res
 // Block 0 also clears the build's counters and advances the tag of the published words.
 __global__ void k_bbox_final(const double* __restrict__ part, int nblk, Cube* cubes, BuildCtl ctl)
 {
+    follow();
     if (blockIdx.x == 0) {
         for (int i = threadIdx.x; i < kCtlWords; i += blockDim.x) ctl.words[i] = 0;
         // every build's published words carry a tag 16 above the previous build's, kept
@@ -154,6 +156,7 @@ k_keys(const double* __restrict__ x, const double* __restrict__ y, const double*
        int n, const Cube* __restrict__ cubes, const unsigned char* __restrict__ cloud,
        unsigned long long* __restrict__ key, int passes, int* __restrict__ hist)
 {
+    follow();
     __shared__ int h[kSortPassesMax][kRadix];
     for (int i = threadIdx.x; i < passes * kRadix; i += kKeyThreads) (&h[0][0])[i] = 0;
     __syncthreads();
@@ -323,6 +326,7 @@ __global__ void __launch_bounds__(kTopoThreads)
 k_topo_scan(const unsigned long long* __restrict__ K, int n, int leaf_cap, int* __restrict__ cnt,
             int* __restrict__ off, Tree t, BuildCtl ctl, unsigned long long* status, int* err)
 {
+    follow();
     __shared__ unsigned char fd[kWin ? kTopoThreads + 2 * kTopoWin : 1];
     __shared__ int s_tile, s_tot, s_prefix;
     if (threadIdx.x == 0) s_tile = atomicAdd(&ctl.words[kCtlTopoTile], 1);
@@ -407,6 +411,7 @@ __global__ void __launch_bounds__(kTopoThreads)
 k_topo_emit(const unsigned long long* __restrict__ K, int n, const int* __restrict__ cnt,
             const int* __restrict__ off, Tree t)
 {
+    follow();
     __shared__ unsigned char mn[kTopoLevels][2 * kTopoThreads];
     __shared__ unsigned int starts[kTopoThreads / 32];
     __shared__ int s_depth;
@@ -694,6 +699,7 @@ k_moments(const double* __restrict__ x, const double* __restrict__ y,
           const double* __restrict__ qsp, int n, const int* __restrict__ cnt,
           const int* __restrict__ off, const Cube* __restrict__ cube, Tree t)
 {
+    follow();
     __shared__ int list[kMomTile];
     const int nl = block_leaves(cnt, blockIdx.x * kMomTile, n, list);
     const double q0 = qsp[0], q1 = qsp[1];
@@ -857,6 +863,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
               const int* __restrict__ off, const Cube* __restrict__ cube, Tree t,
               float4* __restrict__ src32)
 {
+    follow();
     __shared__ int list[kMomTile];
     __shared__ double ctr[kTile ? kMomTile : 1][3];                  // geometric centre, then c
     __shared__ float4 ys[kTile ? kMomTile + kMomHalo : 1];           // offset, charge
@@ -998,36 +1005,36 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
 // ---------------------------------------------------------------- launchers
 void launch_bbox(const double* x, const double* y, const double* z, int n, double* partials,
                  int nblk, Cube* cubes, const int* cloud_start, int n_clouds, BuildCtl ctl,
-                 cudaStream_t s)
+                 Queue s)
 {
     count_launch(2);
-    k_bbox_partial<<<dim3(nblk, n_clouds), 256, 0, s>>>(x, y, z, n, partials, cloud_start);
-    k_bbox_final<<<n_clouds, 256, 0, s>>>(partials, nblk, cubes, ctl);
+    launch(k_bbox_partial, dim3(nblk, n_clouds), 256, s, x, y, z, n, partials, cloud_start);
+    launch(k_bbox_final, n_clouds, 256, s, partials, nblk, cubes, ctl);
 }
 
 void launch_keys(const double* x, const double* y, const double* z, int n, const Cube* cubes,
                  const unsigned char* cloud, unsigned long long* key, int passes, BuildCtl ctl,
-                 cudaStream_t s)
+                 Queue s)
 {
     count_launch(1);
     int nb = (n + kKeyThreads - 1) / kKeyThreads;
     if (nb > 8 * 152) nb = 8 * 152;
-    k_keys<<<nb, kKeyThreads, 0, s>>>(x, y, z, n, cubes, cloud, key, passes, ctl.words + kCtlHist);
+    launch(k_keys, nb, kKeyThreads, s, x, y, z, n, cubes, cloud, key, passes, ctl.words + kCtlHist);
 }
 
 void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* pos_cnt,
                      int* pos_off, Tree t, BuildCtl ctl, unsigned long long* status, int* err,
-                     cudaStream_t s)
+                     Queue s)
 {
     count_launch(2);
     const int nb = (n + kTopoThreads - 1) / kTopoThreads;
     if (leaf_cap <= kTopoWin)
-        k_topo_scan<true><<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, pos_off, t, ctl,
+        launch(k_topo_scan<true>, nb, kTopoThreads, s, key, n, leaf_cap, pos_cnt, pos_off, t, ctl,
                                                       status, err);
     else
-        k_topo_scan<false><<<nb, kTopoThreads, 0, s>>>(key, n, leaf_cap, pos_cnt, pos_off, t, ctl,
+        launch(k_topo_scan<false>, nb, kTopoThreads, s, key, n, leaf_cap, pos_cnt, pos_off, t, ctl,
                                                        status, err);
-    k_topo_emit<<<nb, kTopoThreads, 0, s>>>(key, n, pos_cnt, pos_off, t);
+    launch(k_topo_emit, nb, kTopoThreads, s, key, n, pos_cnt, pos_off, t);
 }
 
 size_t topo_status_words(int n) { return (size_t)((n + kTopoThreads - 1) / kTopoThreads) + 1; }
@@ -1035,19 +1042,19 @@ size_t topo_status_words(int n) { return (size_t)((n + kTopoThreads - 1) / kTopo
 void launch_moments(const double* x, const double* y, const double* z, const int8_t* sp,
                     const double* qsp, int n, int leaf_cap, const int* pos_cnt,
                     const int* pos_off, const Cube* cube, Tree t, float4* src32, int want_f32,
-                    cudaStream_t s)
+                    Queue s)
 {
     // leaves from their particles, then every twig as its last child finishes
     // (bottom-up sweep with arrival counters), in one launch
     count_launch(1);
     const int nb = (n + kMomTile - 1) / kMomTile;
     if (!want_f32)
-        k_moments<<<nb, kMomThreads, 0, s>>>(x, y, z, sp, qsp, n, pos_cnt, pos_off, cube, t);
+        launch(k_moments, nb, kMomThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off, cube, t);
     else if (leaf_cap <= kMomHalo)
-        k_moments_f32<true><<<nb, kMomThreads, 0, s>>>(x, y, z, sp, qsp, n, pos_cnt, pos_off, cube,
+        launch(k_moments_f32<true>, nb, kMomThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off, cube,
                                                        t, src32);
     else
-        k_moments_f32<false><<<nb, kMomThreads, 0, s>>>(x, y, z, sp, qsp, n, pos_cnt, pos_off,
+        launch(k_moments_f32<false>, nb, kMomThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off,
                                                         cube, t, src32);
 }
 

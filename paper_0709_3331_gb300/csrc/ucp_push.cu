@@ -15,6 +15,7 @@ __global__ void k_kick(double* __restrict__ vx, double* __restrict__ vy, double*
                        const double* __restrict__ az, const int8_t* __restrict__ sp, int species,
                        double h, int n, int times)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || sp[i] != species) return;
     double ux = vx[i], uy = vy[i], uz = vz[i];
@@ -36,6 +37,7 @@ __global__ void k_drift(double* __restrict__ x, double* __restrict__ y, double* 
                         const double* __restrict__ vx, const double* __restrict__ vy,
                         const double* __restrict__ vz, double dt, int n)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     x[i] = __fma_rn(dt, vx[i], x[i]);  // one rounding, as the kicks
@@ -51,6 +53,7 @@ __global__ void k_energy_partial(const double* __restrict__ vx, const double* __
                                  const int8_t* __restrict__ sp, const double* __restrict__ qsp,
                                  const double* __restrict__ msp, int n, double* __restrict__ part)
 {
+    follow();
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         int s = sp[i];
@@ -83,6 +86,7 @@ __global__ void k_energy_clouds(const double* __restrict__ vx, const double* __r
                                 const double* __restrict__ msp, const int* __restrict__ cloud_start,
                                 double* __restrict__ out)
 {
+    follow();
     const int c = blockIdx.x;
     double acc[6] = {0, 0, 0, 0, 0, 0};
     for (int i = cloud_start[c] + threadIdx.x; i < cloud_start[c + 1]; i += blockDim.x) {
@@ -111,6 +115,7 @@ __global__ void k_energy_clouds(const double* __restrict__ vx, const double* __r
 __global__ void __launch_bounds__(192)
 k_energy_final(const double* __restrict__ part, int nblk, double* __restrict__ out)
 {
+    follow();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double acc = 0.0;
     for (int b = lane; b < nblk; b += 32) acc += part[6 * b + k];
@@ -123,6 +128,7 @@ __global__ void k_scatter3(const double* __restrict__ ax, const double* __restri
                            const double* __restrict__ az, const unsigned int* __restrict__ id,
                            int n, double* __restrict__ out)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     unsigned int j = id[i];
@@ -134,6 +140,7 @@ __global__ void k_scatter3(const double* __restrict__ ax, const double* __restri
 __global__ void k_scatter1(const double* __restrict__ a, const unsigned int* __restrict__ id, int n,
                            double* __restrict__ out)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[id[i]] = a[i];
 }
@@ -141,6 +148,7 @@ __global__ void k_scatter1(const double* __restrict__ a, const unsigned int* __r
 __global__ void k_scatter_int(const int* __restrict__ a, const unsigned int* __restrict__ id, int n,
                               int* __restrict__ out)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[id[i]] = a[i];
 }
@@ -155,6 +163,7 @@ __global__ void k_load_state(const double* __restrict__ pos, const double* __res
                              double* __restrict__ vz, int8_t* __restrict__ sp_slot,
                              int8_t* __restrict__ sp_caller, unsigned int* __restrict__ id)
 {
+    follow();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const size_t b = 3 * (size_t)i;
@@ -176,6 +185,7 @@ __global__ void k_check_state(const double* __restrict__ pos, const double* __re
                               const int8_t* __restrict__ sp, int n,
                               const unsigned char* __restrict__ cloud, int* __restrict__ flags)
 {
+    follow();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     bool bad = false, wrong = false, electron = false;
@@ -201,6 +211,7 @@ __global__ void k_chunks(const int* __restrict__ first, const int* __restrict__ 
                          int width, int nchunks, int4* __restrict__ chunks,
                          int* __restrict__ order)
 {
+    follow();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nchunks) return;
     int lo = 0, hi = n_clouds;          // the cloud whose chunks hold i
@@ -220,77 +231,77 @@ inline int nb(int n) { return (n + kT - 1) / kT > 0 ? (n + kT - 1) / kT : 1; }
 
 void launch_kick(double* vx, double* vy, double* vz, const double* ax, const double* ay,
                  const double* az, const int8_t* sp, int species, double h, int n, int times,
-                 cudaStream_t s)
+                 Queue s)
 {
     count_launch(1);
-    k_kick<<<nb(n), kT, 0, s>>>(vx, vy, vz, ax, ay, az, sp, species, h, n, times);
+    launch(k_kick, nb(n), kT, s, vx, vy, vz, ax, ay, az, sp, species, h, n, times);
 }
 
 void launch_drift(double* x, double* y, double* z, const double* vx, const double* vy,
-                  const double* vz, double dt, int n, cudaStream_t s)
+                  const double* vz, double dt, int n, Queue s)
 {
     count_launch(1);
-    k_drift<<<nb(n), kT, 0, s>>>(x, y, z, vx, vy, vz, dt, n);
+    launch(k_drift, nb(n), kT, s, x, y, z, vx, vy, vz, dt, n);
 }
 
 void launch_energy(const double* vx, const double* vy, const double* vz, const double* phi,
                    const int8_t* sp, const double* qsp, const double* msp, int n,
-                   double* partials, int nblk, double* out6, cudaStream_t s)
+                   double* partials, int nblk, double* out6, Queue s)
 {
     count_launch(2);
-    k_energy_partial<<<nblk, kT, 0, s>>>(vx, vy, vz, phi, sp, qsp, msp, n, partials);
-    k_energy_final<<<1, 192, 0, s>>>(partials, nblk, out6);
+    launch(k_energy_partial, nblk, kT, s, vx, vy, vz, phi, sp, qsp, msp, n, partials);
+    launch(k_energy_final, 1, 192, s, partials, nblk, out6);
 }
 
 void launch_energy_clouds(const double* vx, const double* vy, const double* vz, const double* phi,
                           const int8_t* sp, const double* qsp, const double* msp,
-                          const int* cloud_start, int n_clouds, double* out, cudaStream_t s)
+                          const int* cloud_start, int n_clouds, double* out, Queue s)
 {
     count_launch(1);
-    k_energy_clouds<<<n_clouds, kT, 0, s>>>(vx, vy, vz, phi, sp, qsp, msp, cloud_start, out);
+    launch(k_energy_clouds, n_clouds, kT, s, vx, vy, vz, phi, sp, qsp, msp, cloud_start, out);
 }
 
 void launch_scatter3(const double* ax, const double* ay, const double* az, const unsigned int* id,
-                     int n, double* out, cudaStream_t s)
+                     int n, double* out, Queue s)
 {
     count_launch(1);
-    k_scatter3<<<nb(n), kT, 0, s>>>(ax, ay, az, id, n, out);
+    launch(k_scatter3, nb(n), kT, s, ax, ay, az, id, n, out);
 }
 
-void launch_scatter1(const double* a, const unsigned int* id, int n, double* out, cudaStream_t s)
+void launch_scatter1(const double* a, const unsigned int* id, int n, double* out, Queue s)
 {
     count_launch(1);
-    k_scatter1<<<nb(n), kT, 0, s>>>(a, id, n, out);
+    launch(k_scatter1, nb(n), kT, s, a, id, n, out);
 }
 
-void launch_scatter_int(const int* a, const unsigned int* id, int n, int* out, cudaStream_t s)
+void launch_scatter_int(const int* a, const unsigned int* id, int n, int* out, Queue s)
 {
     count_launch(1);
-    k_scatter_int<<<nb(n), kT, 0, s>>>(a, id, n, out);
+    launch(k_scatter_int, nb(n), kT, s, a, id, n, out);
 }
 
 void launch_load_state(const double* pos, const double* vel, const int8_t* sp, int n,
                        double* const* st6, int8_t* sp_slot, int8_t* sp_caller, unsigned int* id,
-                       cudaStream_t s)
+                       Queue s)
 {
     count_launch(1);
-    k_load_state<<<nb(n), kT, 0, s>>>(pos, vel, sp, n, st6[0], st6[1], st6[2], st6[3], st6[4],
+    launch(k_load_state, nb(n), kT, s, pos, vel, sp, n, st6[0], st6[1], st6[2], st6[3], st6[4],
                                       st6[5], sp_slot, sp_caller, id);
 }
 
 void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n,
-                        const unsigned char* cloud, int* flags, cudaStream_t s)
+                        const unsigned char* cloud, int* flags, Queue s)
 {
     count_launch(1);
-    k_check_state<<<nb(n), kT, 0, s>>>(pos, vel, sp, n, cloud, flags);
+    launch(k_check_state, nb(n), kT, s, pos, vel, sp, n, cloud, flags);
 }
 
 void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
-                   int4* chunks, int* order, cudaStream_t s)
+                   int4* chunks, int* order, Queue s)
 {
     if (nchunks < 1) return;
     count_launch(1);
-    k_chunks<<<nb(nchunks), kT, 0, s>>>(first, place, n_clouds, width, nchunks, chunks, order);
+    launch(k_chunks, nb(nchunks), kT, s, first, place, n_clouds, width, nchunks, chunks, order);
 }
 
 }  // namespace ucp

@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(kCostBins)
 k_chunk_order(const float* __restrict__ cost, int nchunks, const int* __restrict__ bins,
               int* __restrict__ cursor, int* __restrict__ order)
 {
+    follow();
     __shared__ int base[kCostBins];
     __shared__ int warp_sum[kCostBins / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -44,12 +45,12 @@ k_chunk_order(const float* __restrict__ cost, int nchunks, const int* __restrict
 
 }  // namespace
 
-void launch_chunk_order(const WalkOrder& o, int nchunks, cudaStream_t s)
+void launch_chunk_order(const WalkOrder& o, int nchunks, Queue s)
 {
     if (nchunks < 2) return;
     count_launch(1);
-    k_chunk_order<<<(nchunks + kCostBins - 1) / kCostBins, kCostBins, 0, s>>>(
-        o.cost, nchunks, o.bins, o.bins + kCostBins, o.order);
+    launch(k_chunk_order, (nchunks + kCostBins - 1) / kCostBins, kCostBins, s,
+           o.cost, nchunks, o.bins, o.bins + kCostBins, o.order);
 }
 
 }  // namespace ucp

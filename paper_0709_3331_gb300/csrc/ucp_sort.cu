@@ -65,6 +65,7 @@ k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __res
            unsigned int pass, int* err, int spin_limit,
            const unsigned char* __restrict__ digit_of_val)
 {
+    follow();
     const unsigned int epoch = (*epoch_dev + pass) & 0x3fffffffu;
     __shared__ int cnt[kSortWarps][kRadix];
     __shared__ int s_tile, s_fail, s_tot;
@@ -185,6 +186,7 @@ k_finish_sort(const unsigned long long* __restrict__ kin, const unsigned int* __
               unsigned long long* __restrict__ kout, int n, int low, StateRef in, StateRef out,
               const unsigned char* __restrict__ cloud, int* __restrict__ long_run)
 {
+    follow();
     __shared__ unsigned long long sk[kWindow + 1];   // place l - 1 of the window
     __shared__ unsigned int sv[kWindow + 1];
     __shared__ unsigned char sc[kWindow + 1];
@@ -245,6 +247,7 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
             int n, int n_clouds, int* ctl, int* counts,
             int* err, StateRef in, StateRef out, const unsigned char* __restrict__ cloud)
 {
+    follow();
     if (ctl[kCtlLong] == 0) return;
     __shared__ int cnt[kSortWarps][kRadix];
     __shared__ int s_base[kRadix];
@@ -401,7 +404,7 @@ size_t sort_status_words(int n)
 int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int passes,
                 const SortScratch& sc, BuildCtl ctl, const StateRef& in, const StateRef& out,
                 const unsigned char* cloud, const int* cloud_start, int n_clouds, int nsm,
-                cudaStream_t s)
+                Queue s)
 {
     const bool clouds = n_clouds > 1;
     count_launch(passes + 2 + (clouds ? 1 : 0));
@@ -409,8 +412,9 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
     const int low = kKeyBits - 8 * passes;
     int cur = 0;
     for (int p = 0; p < passes; ++p) {
-        k_onesweep<<<nb, kSortThreads, 0, s>>>(
-            key[cur], p == 0 ? nullptr : val[cur], key[cur ^ 1], val[cur ^ 1], n, low + 8 * p,
+        launch(k_onesweep, nb, kSortThreads, s, key[cur],
+               p == 0 ? static_cast<unsigned int*>(nullptr) : val[cur], key[cur ^ 1],
+               val[cur ^ 1], n, low + 8 * p,
             ctl.words + kCtlHist + p * kRadix, 1, kRadix, sc.status + (size_t)p * nb * kRadix,
             ctl.words + kCtlTile + p, ctl.epoch, (unsigned int)p, sc.err, kSortSpinLimit, nullptr);
         cur ^= 1;
@@ -418,15 +422,15 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
     if (clouds) {
         // a stable pass by cloud: (cloud, key) order, each cloud back in its fixed
         // segment; a cloud's first place is its segment's start
-        k_onesweep<<<nb, kSortThreads, 0, s>>>(
-            key[cur], val[cur], key[cur ^ 1], val[cur ^ 1], n, 0, cloud_start, 0, n_clouds,
+        launch(k_onesweep, nb, kSortThreads, s, key[cur], val[cur], key[cur ^ 1],
+               val[cur ^ 1], n, 0, cloud_start, 0, n_clouds,
             sc.status + (size_t)passes * nb * kRadix, ctl.words + kCtlTile + passes, ctl.epoch,
             (unsigned int)passes, sc.err, kSortSpinLimit, cloud);
         cur ^= 1;
     }
     const int fin = cur ^ 1;
-    k_finish_sort<<<(n + kFinish - 1) / kFinish, kFinish, 0, s>>>(
-        key[cur], val[cur], key[fin], n, low, in, out, cloud, ctl.words + kCtlLong);
+    launch(k_finish_sort, (n + kFinish - 1) / kFinish, kFinish, s, key[cur], val[cur],
+           key[fin], n, low, in, out, cloud, ctl.words + kCtlLong);
     unsigned long long *k0 = key[cur], *k1 = key[fin];
     unsigned int *v0 = val[cur], *v1 = val[fin];
     int* words = ctl.words;
@@ -440,7 +444,7 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
     return fin;
 }
 
-int sort_selftest_timeout(const SortScratch& sc, cudaStream_t s)
+int sort_selftest_timeout(const SortScratch& sc, Queue s)
 {
     // a lone block that takes tile 1 while tile 0 never publishes: its bounded
     // wait must run out, raise *err and leave the keys where they are
@@ -454,7 +458,7 @@ int sort_selftest_timeout(const SortScratch& sc, cudaStream_t s)
         cudaMemsetAsync(sc.test_vals, 0, sizeof(unsigned int) * 4 * kSortTile, s) != cudaSuccess)
         return -1;
     // input: tiles 0-1 of the test buffers; output: tiles 2-3
-    k_onesweep<<<1, kSortThreads, 0, s>>>(sc.test_keys, sc.test_vals, sc.test_keys + 2 * kSortTile,
+    launch(k_onesweep, 1, kSortThreads, s, sc.test_keys, sc.test_vals, sc.test_keys + 2 * kSortTile,
                                           sc.test_vals + 2 * kSortTile, 2 * kSortTile, 0,
                                           sc.test_ctl + 1, 1, kRadix, sc.status, sc.test_ctl,
                                           sc.test_epoch, 0u, sc.err, 2000, nullptr);
@@ -471,6 +475,7 @@ constexpr int kSelTile = kSelThreads * kSelItems;
 __global__ void __launch_bounds__(kSelThreads)
 k_select_count(const int8_t* __restrict__ sp, int species, int n, int* __restrict__ part)
 {
+    follow();
     const int base = blockIdx.x * kSelTile;
     int s = 0;
 #pragma unroll
@@ -489,6 +494,7 @@ __global__ void __launch_bounds__(kSelThreads)
 k_select_write(const int8_t* __restrict__ sp, int species, int n, const int* __restrict__ part,
                int* __restrict__ list, int* __restrict__ cnt0, int* __restrict__ cnt1)
 {
+    follow();
     __shared__ int tot, before;
     int b = 0;
     for (int i = threadIdx.x; i < (int)blockIdx.x; i += kSelThreads) b += part[i];
@@ -519,12 +525,12 @@ k_select_write(const int8_t* __restrict__ sp, int species, int n, const int* __r
 size_t select_words(int n) { return (size_t)((n + kSelTile - 1) / kSelTile) + 1; }
 
 void launch_select(const int8_t* sp, int species, int n, int* list, int* partials, int* cnt0,
-                   int* cnt1, cudaStream_t s)
+                   int* cnt1, Queue s)
 {
     count_launch(2);
     const int nb = (n + kSelTile - 1) / kSelTile;
-    k_select_count<<<nb, kSelThreads, 0, s>>>(sp, species, n, partials);
-    k_select_write<<<nb, kSelThreads, 0, s>>>(sp, species, n, partials, list, cnt0, cnt1);
+    launch(k_select_count, nb, kSelThreads, s, sp, species, n, partials);
+    launch(k_select_write, nb, kSelThreads, s, sp, species, n, partials, list, cnt0, cnt1);
 }
 
 }  // namespace ucp

@@ -64,6 +64,7 @@ template <bool kKelbg, bool kPhi>
 __global__ void __launch_bounds__(32, 16)
 k_walk_fp64(WalkArgs a)
 {
+    follow();
     __shared__ int stack[kStack], acc[64], src[64];
     const int lane = threadIdx.x;
     const unsigned int lt = (1u << lane) - 1u;
@@ -322,6 +323,7 @@ template <bool kKelbg, int kThreads, int kBlocks, bool kPhi>
 __global__ void __launch_bounds__(kThreads, kBlocks)
 k_walk_fp32c(WalkArgs a)
 {
+    follow();
     __shared__ WalkWarp shared[kThreads / 32];
     const int lane = threadIdx.x & 31;
     WalkWarp& W = shared[threadIdx.x >> 5];
@@ -552,6 +554,7 @@ constexpr int kVisitBatch = 32;     // visits summed in FP32 before a compensate
 __global__ void __launch_bounds__(kVisitThreads, 7)
 k_walk_fp32c_visits(WalkArgs a)
 {
+    follow();
     __shared__ int2 lists[kVisitThreads / 32][kVisitList];   // {opened leaf, mask}
     const int lane = threadIdx.x & 31;
     int2* lst = lists[threadIdx.x >> 5];
@@ -705,6 +708,7 @@ k_walk_fp32c_visits(WalkArgs a)
 __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32,
                               int* work, int* bins)
 {
+    follow();
     if (blockIdx.x == 0) {
         if (threadIdx.x == 0) *work = 0;
         if (bins)
@@ -750,11 +754,11 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
 }  // namespace
 
 void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
-                        cudaStream_t s)
+                        Queue s)
 {
     count_launch(1);
     int blocks = 4 * 152;
-    k_mac_prepare<<<blocks, 256, 0, s>>>(t, cube, theta, want_f32, work, bins);
+    launch(k_mac_prepare, blocks, 256, s, t, cube, theta, want_f32, work, bins);
 }
 
 // blocks of one warp: per_sm on every SM, or one per work item
@@ -764,15 +768,15 @@ static int walk_blocks(int64_t items, int nsm, int per_sm)
     return blocks < 1 ? 1 : blocks;
 }
 
-void launch_walk_fp64(const WalkArgs& a, int nsm, cudaStream_t s)
+void launch_walk_fp64(const WalkArgs& a, int nsm, Queue s)
 {
     count_launch(1);
     const int b = walk_blocks((int64_t)a.nchunks * 32, nsm, 16);
     // the potential is computed only when the caller reads it
-    if (a.kelbg && a.phi) k_walk_fp64<true, true><<<b, 32, 0, s>>>(a);
-    else if (a.kelbg) k_walk_fp64<true, false><<<b, 32, 0, s>>>(a);
-    else if (a.phi) k_walk_fp64<false, true><<<b, 32, 0, s>>>(a);
-    else k_walk_fp64<false, false><<<b, 32, 0, s>>>(a);
+    if (a.kelbg && a.phi) launch(k_walk_fp64<true, true>, b, 32, s, a);
+    else if (a.kelbg) launch(k_walk_fp64<true, false>, b, 32, s, a);
+    else if (a.phi) launch(k_walk_fp64<false, true>, b, 32, s, a);
+    else launch(k_walk_fp64<false, false>, b, 32, s, a);
 }
 
 // Launch shapes of the FP32C walk that the autotuner chooses from: blocks of one
@@ -785,23 +789,23 @@ static const int kShapes[][3] = {{32, 24, 0}, {32, 20, 0}, {32, 28, 0}, {32, 32,
 int walk_shape_count() { return (int)(sizeof(kShapes) / sizeof(kShapes[0])); }
 
 template <bool kKelbg, bool kPhi>
-static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, cudaStream_t s)
+static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, Queue s)
 {
     switch (per_sm) {
-    case 12: k_walk_fp32c<kKelbg, 32, 12, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 14: k_walk_fp32c<kKelbg, 32, 14, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 16: k_walk_fp32c<kKelbg, 32, 16, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 18: k_walk_fp32c<kKelbg, 32, 18, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 20: k_walk_fp32c<kKelbg, 32, 20, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 22: k_walk_fp32c<kKelbg, 32, 22, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 26: k_walk_fp32c<kKelbg, 32, 26, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 28: k_walk_fp32c<kKelbg, 32, 28, kPhi><<<b, 32, 0, s>>>(a); break;
-    case 32: k_walk_fp32c<kKelbg, 32, 32, kPhi><<<b, 32, 0, s>>>(a); break;
-    default: k_walk_fp32c<kKelbg, 32, 24, kPhi><<<b, 32, 0, s>>>(a); break;
+    case 12: launch(k_walk_fp32c<kKelbg, 32, 12, kPhi>, b, 32, s, a); break;
+    case 14: launch(k_walk_fp32c<kKelbg, 32, 14, kPhi>, b, 32, s, a); break;
+    case 16: launch(k_walk_fp32c<kKelbg, 32, 16, kPhi>, b, 32, s, a); break;
+    case 18: launch(k_walk_fp32c<kKelbg, 32, 18, kPhi>, b, 32, s, a); break;
+    case 20: launch(k_walk_fp32c<kKelbg, 32, 20, kPhi>, b, 32, s, a); break;
+    case 22: launch(k_walk_fp32c<kKelbg, 32, 22, kPhi>, b, 32, s, a); break;
+    case 26: launch(k_walk_fp32c<kKelbg, 32, 26, kPhi>, b, 32, s, a); break;
+    case 28: launch(k_walk_fp32c<kKelbg, 32, 28, kPhi>, b, 32, s, a); break;
+    case 32: launch(k_walk_fp32c<kKelbg, 32, 32, kPhi>, b, 32, s, a); break;
+    default: launch(k_walk_fp32c<kKelbg, 32, 24, kPhi>, b, 32, s, a); break;
     }
 }
 
-void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
+void launch_walk_fp32c(const WalkArgs& a, int nsm, Queue s, int shape)
 {
     count_launch(1);
     if (shape < 0 || shape >= walk_shape_count()) shape = 0;
@@ -814,12 +818,12 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, cudaStream_t s, int shape)
     else walk_fp32c_shape<false, false>(a, per_sm, b, s);
 }
 
-void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, cudaStream_t s)
+void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, Queue s)
 {
     count_launch(1);
     const int wpb = kVisitThreads / 32;
     const int b = walk_blocks(((int64_t)a.nchunks + wpb - 1) / wpb, nsm, 7);
-    k_walk_fp32c_visits<<<b, kVisitThreads, 0, s>>>(a);
+    launch(k_walk_fp32c_visits, b, kVisitThreads, s, a);
 }
 
 }  // namespace ucp
