@@ -719,7 +719,7 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
         // FP32C context: FP32 walk, FP32 box accumulators (in the same buffer)
         float* adjf = reinterpret_cast<float*>(adj);
         launch(k_zero_adj<float>, 2 * 152, 256, s, a.t.nnodes, adjf);
-        launch(k_walk_adjoint_f32, blocks, 32, s, a, lam, mu, adjf);
+        launch(k_walk_adjoint_f32, blocks, 32, s.whole(), a, lam, mu, adjf);
         launch(k_adjoint_push<float>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
     } else {
         launch(k_zero_adj<double>, 2 * 152, 256, s, a.t.nnodes, adj);
@@ -728,7 +728,7 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
         while (group > 1 && (int64_t)a.nchunks * (32 / group) < 4 * (int64_t)nsm) group /= 2;
         const int64_t items = (int64_t)a.nchunks * (32 / group);
         const int blocks = items < 1 ? 1 : items < 12 * nsm ? (int)items : 12 * nsm;
-        launch(k_walk_adjoint, blocks, 32, s, a, group, lam, mu, adj);
+        launch(k_walk_adjoint, blocks, 32, s.whole(), a, group, lam, mu, adj);
         launch(k_adjoint_push<double>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
     }
 }

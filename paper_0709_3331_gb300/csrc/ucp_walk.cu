@@ -773,10 +773,10 @@ void launch_walk_fp64(const WalkArgs& a, int nsm, Queue s)
     count_launch(1);
     const int b = walk_blocks((int64_t)a.nchunks * 32, nsm, 16);
     // the potential is computed only when the caller reads it
-    if (a.kelbg && a.phi) launch(k_walk_fp64<true, true>, b, 32, s, a);
-    else if (a.kelbg) launch(k_walk_fp64<true, false>, b, 32, s, a);
-    else if (a.phi) launch(k_walk_fp64<false, true>, b, 32, s, a);
-    else launch(k_walk_fp64<false, false>, b, 32, s, a);
+    if (a.kelbg && a.phi) launch(k_walk_fp64<true, true>, b, 32, s.whole(), a);
+    else if (a.kelbg) launch(k_walk_fp64<true, false>, b, 32, s.whole(), a);
+    else if (a.phi) launch(k_walk_fp64<false, true>, b, 32, s.whole(), a);
+    else launch(k_walk_fp64<false, false>, b, 32, s.whole(), a);
 }
 
 // Launch shapes of the FP32C walk that the autotuner chooses from: blocks of one
@@ -792,16 +792,16 @@ template <bool kKelbg, bool kPhi>
 static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, Queue s)
 {
     switch (per_sm) {
-    case 12: launch(k_walk_fp32c<kKelbg, 32, 12, kPhi>, b, 32, s, a); break;
-    case 14: launch(k_walk_fp32c<kKelbg, 32, 14, kPhi>, b, 32, s, a); break;
-    case 16: launch(k_walk_fp32c<kKelbg, 32, 16, kPhi>, b, 32, s, a); break;
-    case 18: launch(k_walk_fp32c<kKelbg, 32, 18, kPhi>, b, 32, s, a); break;
-    case 20: launch(k_walk_fp32c<kKelbg, 32, 20, kPhi>, b, 32, s, a); break;
-    case 22: launch(k_walk_fp32c<kKelbg, 32, 22, kPhi>, b, 32, s, a); break;
-    case 26: launch(k_walk_fp32c<kKelbg, 32, 26, kPhi>, b, 32, s, a); break;
-    case 28: launch(k_walk_fp32c<kKelbg, 32, 28, kPhi>, b, 32, s, a); break;
-    case 32: launch(k_walk_fp32c<kKelbg, 32, 32, kPhi>, b, 32, s, a); break;
-    default: launch(k_walk_fp32c<kKelbg, 32, 24, kPhi>, b, 32, s, a); break;
+    case 12: launch(k_walk_fp32c<kKelbg, 32, 12, kPhi>, b, 32, s.whole(), a); break;
+    case 14: launch(k_walk_fp32c<kKelbg, 32, 14, kPhi>, b, 32, s.whole(), a); break;
+    case 16: launch(k_walk_fp32c<kKelbg, 32, 16, kPhi>, b, 32, s.whole(), a); break;
+    case 18: launch(k_walk_fp32c<kKelbg, 32, 18, kPhi>, b, 32, s.whole(), a); break;
+    case 20: launch(k_walk_fp32c<kKelbg, 32, 20, kPhi>, b, 32, s.whole(), a); break;
+    case 22: launch(k_walk_fp32c<kKelbg, 32, 22, kPhi>, b, 32, s.whole(), a); break;
+    case 26: launch(k_walk_fp32c<kKelbg, 32, 26, kPhi>, b, 32, s.whole(), a); break;
+    case 28: launch(k_walk_fp32c<kKelbg, 32, 28, kPhi>, b, 32, s.whole(), a); break;
+    case 32: launch(k_walk_fp32c<kKelbg, 32, 32, kPhi>, b, 32, s.whole(), a); break;
+    default: launch(k_walk_fp32c<kKelbg, 32, 24, kPhi>, b, 32, s.whole(), a); break;
     }
 }
 
@@ -823,7 +823,7 @@ void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, Queue s)
     count_launch(1);
     const int wpb = kVisitThreads / 32;
     const int b = walk_blocks(((int64_t)a.nchunks + wpb - 1) / wpb, nsm, 7);
-    launch(k_walk_fp32c_visits, b, kVisitThreads, s, a);
+    launch(k_walk_fp32c_visits, b, kVisitThreads, s.whole(), a);
 }
 
 }  // namespace ucp
