@@ -5,6 +5,7 @@
 // Arithmetic that decides an integer (cube, cell coordinates, box centre) is
 // written with explicit round-to-nearest intrinsics in the order of the
 // definition, so that no multiply-add contraction changes a cell.
+#include "ucp_box.cuh"
 #include "ucp_scan.cuh"
 
 #include <math.h>
@@ -477,69 +478,6 @@ k_topo_emit(const unsigned long long* __restrict__ K, int n, const int* __restri
 }
 
 // ---------------------------------------------------------------- moments
-__device__ __forceinline__ unsigned int compact3(unsigned long long x)
-{
-    x &= 0x1249249249249249ull;
-    x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
-    x = (x | (x >> 4)) & 0x100f00f00f00f00full;
-    x = (x | (x >> 8)) & 0x001f0000ff0000ffull;
-    x = (x | (x >> 16)) & 0x001f00000000ffffull;
-    x = (x | (x >> 32)) & 0x1fffffull;
-    return (unsigned int)x;
-}
-
-// cube of the cloud that owns the box starting at sorted position i
-__device__ __forceinline__ Cube cube_of(const Cube* __restrict__ cubes, const Tree& t, int i)
-{
-    return cubes[t.cloud ? t.cloud[i] : 0];
-}
-
-// geometric box centre: lo + (cell + 1/2) * side, side = L 2^-depth
-__device__ __forceinline__ void box_centre(const Cube& cb, unsigned long long cell, int d,
-                                           double ctr[3], double* side)
-{
-    double s = ldexp(cb.L, -d);
-    *side = s;
-    unsigned int ic[3] = {compact3(cell), compact3(cell >> 1), compact3(cell >> 2)};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        double lo = __dsub_rn(cb.c[a], __dmul_rn(cb.L, 0.5));
-        ctr[a] = __dadd_rn(lo, __dmul_rn(__dadd_rn((double)ic[a], 0.5), s));
-    }
-}
-
-// Moments of one box from sums about its geometric centre z:
-//   a = {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)},  y = x - z.
-// The expansion centre is the |q|-weighted centroid c = z + e, e = sum|q|y / S0
-// (z when S0 = 0); shifting to c: D = sum q y - M e,
-// Q = sum q y y^T - (sum q y) e^T - e (sum q y)^T + M e e^T.  delta = |e|.
-__device__ __forceinline__ void finish_box(const double* a, const double z[3],
-                                           double* __restrict__ m, double* __restrict__ delta)
-{
-    double S0 = a[0], M = a[1];
-    double e[3];
-    const double inv = S0 > 0.0 ? 1.0 / S0 : 0.0;
-    for (int k = 0; k < 3; ++k) e[k] = a[2 + k] * inv;
-    double d[3];
-    for (int k = 0; k < 3; ++k) d[k] = a[5 + k];
-    m[MC + 0] = z[0] + e[0];
-    m[MC + 1] = z[1] + e[1];
-    m[MC + 2] = z[2] + e[2];
-    m[MM] = M;
-    for (int k = 0; k < 3; ++k) m[MD + k] = d[k] - M * e[k];
-    const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
-    for (int k = 0; k < 6; ++k)
-        m[MQ + k] = a[8 + k] - d[ia[k]] * e[ib[k]] - e[ia[k]] * d[ib[k]] + M * e[ia[k]] * e[ib[k]];
-    m[MS0] = S0;
-    // delta = |c - z| rounded like the definition: c is stored first, then differenced
-    double ex = __dsub_rn(m[MC + 0], z[0]);
-    double ey = __dsub_rn(m[MC + 1], z[1]);
-    double ez = __dsub_rn(m[MC + 2], z[2]);
-    *delta = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)),
-                                  __dmul_rn(ez, ez)));
-    m[MT] = -0.5 * (m[MQ] + m[MQ + 3] + m[MQ + 5]);
-}
-
 // Sum over the eight lanes of a group by an xor butterfly, in every lane:
 // ((s0 + s4) + (s2 + s6)) + ((s1 + s5) + (s3 + s7)).
 template <class T>
@@ -551,51 +489,98 @@ __device__ __forceinline__ T sum8(T v)
     return v;
 }
 
-// Moments of twig p (depth d; p < 0: none) by a group of eight lanes, one child slot o
-// each (ch < 0: empty), the child's moments shifted to the twig's geometric centre.  The
-// children were written by other threads of the same launch: their records are read
-// through L2 (__ldcg) after the acquire of the bottom-up sweep.
-__device__ __forceinline__ void twig_combine_f64(const Cube* __restrict__ cube, const Tree& t,
-                                                 int p, int d, int o, int ch)
+// A twig of the bottom-up sweep (id < 0: none).
+struct Twig {
+    int id, parent, first, depth;       // first: particle
+    unsigned long long cell;
+    int nch, last;                      // children, and the last of them
+};
+
+__device__ __forceinline__ Twig load_twig(const Tree& t, int p)
 {
-    double zp[3] = {0, 0, 0}, ps;
-    if (p >= 0) box_centre(cube_of(cube, t, t.info[p].x), t.cell[p], d, zp, &ps);
+    Twig w = {p, -1, 0, 0, 0ull, 0, -1};
+    if (p < 0) return w;
+    const int4* row = reinterpret_cast<const int4*>(t.child8 + (size_t)p * 8);
+    const int4 r0 = row[0], r1 = row[1];
+    w.first = t.info[p].x;
+    w.parent = t.info[p].w;
+    w.depth = t.depth_leaf[p] & 255;
+    w.cell = t.cell[p];
+    const int ch[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+        w.nch += ch[o] >= 0;
+        if (ch[o] >= 0) w.last = ch[o];
+    }
+    return w;
+}
+
+// One step of a sum by halving exchanges: lanes with the bit set keep b and send a, the
+// others keep a and send b.
+__device__ __forceinline__ double halve(bool bit, double a, double b, int mask)
+{
+    return (bit ? b : a) + __shfl_xor_sync(0xffffffffu, bit ? a : b, mask);
+}
+
+// Sums of a twig about its geometric centre by a group of eight lanes, one child slot o
+// each (ch < 0: empty): the child's sums shifted by the difference of the centres,
+// a quarter of the twig's side along each axis, signed by the octant bit.  The children
+// were written by other threads of the same launch: their records are read through L2
+// (__ldcg) after the acquire of the bottom-up sweep.  A level costs its latency and the
+// FP64 pipe's 16 cycles per warp instruction, so nothing but the sums goes up the tree
+// (moments follow from them with the walk's records, one box per lane), and they are
+// added by halving exchanges, 14 additions for 14 values instead of 42, which leave sums
+// o and 8 + o in lane o.  With the centroid, division and root of every level in the
+// chain, and 256 positions to a block, this kernel took 58 us at N = 2048 and 89 at
+// 131,072; now 30 and 62, and the moments 1.5 us of the walk's preparation.
+__device__ __forceinline__ void twig_sums_f64(const Cube* __restrict__ cube, const Tree& t,
+                                              const Twig& w, int o, int ch)
+{
     double a[14];
 #pragma unroll
     for (int k = 0; k < 14; ++k) a[k] = 0.0;
     if (ch >= 0) {
-        const double* cm = t.mom + (size_t)ch * kMom;
-        const double S0k = __ldcg(cm + MS0), Mk = __ldcg(cm + MM);
-        double e[3], dk[3], qk[6];
-        for (int k = 0; k < 3; ++k) {
-            e[k] = __ldcg(cm + MC + k) - zp[k];
-            dk[k] = __ldcg(cm + MD + k);
+        const double2* r = reinterpret_cast<const double2*>(t.mom + (size_t)ch * kMom);
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            const double2 v = __ldcg(r + k);
+            a[2 * k] = v.x;
+            a[2 * k + 1] = v.y;
         }
-        for (int k = 0; k < 6; ++k) qk[k] = __ldcg(cm + MQ + k);
-        a[0] = S0k;
-        a[1] = Mk;
+        const double h = ldexp(cube_of(cube, t, w.first).L, -(w.depth + 2));
+        const double e[3] = {o & 1 ? h : -h, o & 2 ? h : -h, o & 4 ? h : -h};
+        const double me[3] = {a[1] * e[0], a[1] * e[1], a[1] * e[2]};
+        // P + d e^T + e d^T + M e e^T
+        a[8] += (2.0 * a[5] + me[0]) * e[0];
+        a[9] += a[5] * e[1] + (a[6] + me[1]) * e[0];
+        a[10] += a[5] * e[2] + (a[7] + me[2]) * e[0];
+        a[11] += (2.0 * a[6] + me[1]) * e[1];
+        a[12] += a[6] * e[2] + (a[7] + me[2]) * e[1];
+        a[13] += (2.0 * a[7] + me[2]) * e[2];
+#pragma unroll
         for (int k = 0; k < 3; ++k) {
-            a[2 + k] = S0k * e[k];
-            a[5 + k] = dk[k] + Mk * e[k];
+            a[2 + k] += a[0] * e[k];
+            a[5 + k] += me[k];
         }
-        // Q_k + D_k e^T + e D_k^T + M_k e e^T
-        const double me0 = Mk * e[0], me1 = Mk * e[1], me2 = Mk * e[2];
-        a[8] = qk[0] + (2.0 * dk[0] + me0) * e[0];
-        a[9] = qk[1] + dk[0] * e[1] + (dk[1] + me1) * e[0];
-        a[10] = qk[2] + dk[0] * e[2] + (dk[2] + me2) * e[0];
-        a[11] = qk[3] + (2.0 * dk[1] + me1) * e[1];
-        a[12] = qk[4] + dk[1] * e[2] + (dk[2] + me2) * e[1];
-        a[13] = qk[5] + (2.0 * dk[2] + me2) * e[2];
+    }
+    // ((s0 + s4) + (s2 + s6)) + ((s1 + s5) + (s3 + s7)) of each value
+    const bool b4 = o & 4, b2 = o & 2, b1 = o & 1;
+    double u[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        u[k] = halve(b4, a[k], a[4 + k], 4);
+        u[4 + k] = halve(b4, a[8 + k], k < 2 ? a[12 + k] : 0.0, 4);
     }
 #pragma unroll
-    for (int k = 0; k < 14; ++k) a[k] = sum8(a[k]);
-    if (p >= 0 && o == 0) {
-        double rec[kMom];
-        finish_box(a, zp, rec, t.delta + p);
-        double* pm = t.mom + (size_t)p * kMom;
-#pragma unroll
-        for (int k = 0; k < kMom; ++k)
-            if (k != MR2) pm[k] = rec[k];
+    for (int k = 0; k < 2; ++k) {
+        u[k] = halve(b2, u[k], u[2 + k], 2);
+        u[4 + k] = halve(b2, u[4 + k], u[6 + k], 2);
+    }
+    const double lo = halve(b1, u[0], u[1], 1), hi = halve(b1, u[4], u[5], 1);
+    if (w.id >= 0) {
+        double* r = t.mom + (size_t)w.id * kMom;
+        r[o] = lo;
+        if (o < 6) r[8 + o] = hi;
     }
 }
 
@@ -621,66 +606,60 @@ template <class Combine>
 __device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combine)
 {
     const int lane = threadIdx.x & 31;
-    int p = node >= 0 ? t.info[node].w : -1;
-    while (__any_sync(0xffffffffu, p >= 0)) {
+    Twig w = load_twig(t, node >= 0 ? t.info[node].w : -1);
+    while (__any_sync(0xffffffffu, w.id >= 0)) {
         // this box's records (written by any lane of the warp) are published with its
         // arrival; the last arrival sees every sibling's
         __syncwarp();
-        bool ready = false;
-        if (p >= 0) {
-            const int4* row = reinterpret_cast<const int4*>(t.child8 + (size_t)p * 8);
-            const int4 r0 = row[0], r1 = row[1];
-            const int ch[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-            int nch = 0, last = -1;
-#pragma unroll
-            for (int o = 0; o < 8; ++o) {
-                nch += ch[o] >= 0;
-                if (ch[o] >= 0) last = ch[o];
-            }
-            ready = atomic_add_acq_rel(&t.arrive[p], 1) + 1 >= nch;
-            if (ready) {
-                // a twig ends where its last child (in octant order, so last in
-                // pre-order) ends, and skips to where that child skips
-                const int4 lc = __ldcg(&t.info[last]);
-                int* ip = reinterpret_cast<int*>(&t.info[p]);
-                ip[1] = lc.y;
-                ip[2] = lc.z;
-            } else {
-                p = -1;
-            }
-        }
+        const bool ready = w.id >= 0 && atomic_add_acq_rel(&t.arrive[w.id], 1) + 1 >= w.nch;
         unsigned int todo = __ballot_sync(0xffffffffu, ready);
-        __syncwarp();   // what the acquiring lanes see, every lane sees
+        // what the acquiring lanes see, every lane sees.  The next twig's records come in
+        // while this one is combined.
+        __syncwarp();
+        const Twig up = load_twig(t, ready ? w.parent : -1);
+        int4 lc;
+        if (ready) lc = __ldcg(&t.info[w.last]);
         while (todo) {
             // the (lane / 8)-th of the lanes that are left
             unsigned int m = todo;
             for (int g = 0; g < (lane >> 3) && m; ++g) m &= m - 1u;
-            const int src = m ? __ffs(m) - 1 : -1;
-            const int q = __shfl_sync(0xffffffffu, p, src < 0 ? 0 : src);
-            const int pp = src < 0 ? -1 : q;
+            const int src = m ? __ffs(m) - 1 : 0;
+            Twig q;
+            q.id = __shfl_sync(0xffffffffu, w.id, src);
+            q.first = __shfl_sync(0xffffffffu, w.first, src);
+            q.depth = __shfl_sync(0xffffffffu, w.depth, src);
+            q.cell = __shfl_sync(0xffffffffu, w.cell, src);
+            if (!m) q.id = -1;
             const int o = lane & 7;
-            const int ch = pp >= 0 ? t.child8[(size_t)pp * 8 + o] : -1;
-            combine(pp, pp >= 0 ? t.depth_leaf[pp] & 255 : 0, o, ch);
+            const int ch = q.id >= 0 ? t.child8[(size_t)q.id * 8 + o] : -1;
+            combine(q, o, ch);
             for (int g = 0; g < 4 && todo; ++g) todo &= todo - 1u;
         }
-        __syncwarp();
-        if (p >= 0) p = t.info[p].w;
+        if (ready) {
+            // a twig ends where its last child (in octant order, so last in pre-order)
+            // ends, and skips to where that child skips
+            int* ip = reinterpret_cast<int*>(&t.info[w.id]);
+            ip[1] = lc.y;
+            ip[2] = lc.z;
+        }
+        w = up;
     }
 }
 
-// A block's leaves: those that start among its kMomTile positions, compacted in
-// position order; returns their number.
-constexpr int kMomThreads = 128;
-constexpr int kMomTile = 256;      // positions per block
+// A block's leaves: those that start among its kPos positions, compacted in position
+// order; returns their number.
+constexpr int mom_threads(int pos) { return pos >= 256 ? 128 : 32; }
 constexpr int kMomHalo = 32;       // largest leaf that is summed from shared memory
 constexpr unsigned short kNoOwner = 0xffff;
 
+template <int kPos>
 __device__ __forceinline__ int block_leaves(const int* __restrict__ cnt, int base, int n,
                                             int* list)
 {
+    constexpr int kThreads = mom_threads(kPos);
     __shared__ int s_tot;
     int total = 0;
-    for (int part = 0; part < kMomTile; part += kMomThreads) {
+    for (int part = 0; part < kPos; part += kThreads) {
         const int i = base + part + threadIdx.x;
         const bool start = i < n && cnt[i] > 0;
         const int at = block_excl_scan(start ? 1 : 0, &s_tot);
@@ -691,19 +670,21 @@ __device__ __forceinline__ int block_leaves(const int* __restrict__ cnt, int bas
     return total;
 }
 
-// FP64 moments of every leaf from its particles, one thread per leaf, summed about
+// FP64 sums of every leaf from its particles, one thread per leaf, summed about
 // the leaf's geometric centre in key order, then the twigs (sweep_up).
-__global__ void __launch_bounds__(kMomThreads)
+template <int kPos>
+__global__ void __launch_bounds__(mom_threads(kPos))
 k_moments(const double* __restrict__ x, const double* __restrict__ y,
           const double* __restrict__ z, const int8_t* __restrict__ sp,
           const double* __restrict__ qsp, int n, const int* __restrict__ cnt,
           const int* __restrict__ off, const Cube* __restrict__ cube, Tree t)
 {
     follow();
-    __shared__ int list[kMomTile];
-    const int nl = block_leaves(cnt, blockIdx.x * kMomTile, n, list);
+    constexpr int kThreads = mom_threads(kPos);
+    __shared__ int list[kPos];
+    const int nl = block_leaves<kPos>(cnt, blockIdx.x * kPos, n, list);
     const double q0 = qsp[0], q1 = qsp[1];
-    for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kMomThreads) {
+    for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kThreads) {
         const int l = l0 + (threadIdx.x & 31);
         int node = -1;
         if (l < nl) {
@@ -715,6 +696,7 @@ k_moments(const double* __restrict__ x, const double* __restrict__ y,
             double a[14];
 #pragma unroll
             for (int k = 0; k < 14; ++k) a[k] = 0.0;
+#pragma unroll 4
             for (int j = inf.x; j < inf.y; ++j) {
                 double qj = sp[j] ? q1 : q0;
                 double aq = fabs(qj);
@@ -734,14 +716,12 @@ k_moments(const double* __restrict__ x, const double* __restrict__ y,
                 a[12] += qy1 * yv[2];
                 a[13] += qj * yv[2] * yv[2];
             }
-            double rec[kMom];
-            finish_box(a, zc, rec, t.delta + node);
-            double* m = t.mom + (size_t)node * kMom;
+            double2* r = reinterpret_cast<double2*>(t.mom + (size_t)node * kMom);
 #pragma unroll
-            for (int k = 0; k < kMom; ++k)
-                if (k != MR2) m[k] = rec[k];
+            for (int k = 0; k < 7; ++k) r[k] = make_double2(a[2 * k], a[2 * k + 1]);
         }
-        sweep_up(t, node, [&](int p, int d, int o, int ch) { twig_combine_f64(cube, t, p, d, o, ch); });
+        sweep_up(t, node,
+                 [&](const Twig& w, int o, int ch) { twig_sums_f64(cube, t, w, o, ch); });
     }
 }
 
@@ -812,21 +792,21 @@ __device__ __forceinline__ void twig_child_f32(const Tree& t, int ch, int o, flo
     a[13] = qk[5] + (2.f * dk[2] + me2) * e[2];
 }
 
-// FP32 moments of twig p (depth d; p < 0: none) by a group of eight lanes, one child
+// FP32 moments of a twig by a group of eight lanes, one child
 // slot each, summed by an xor butterfly over the slots.
 __device__ __forceinline__ void twig_combine_f32(const Cube* __restrict__ cube, const Tree& t,
-                                                 int p, int d, int o, int ch)
+                                                 const Twig& w, int o, int ch)
 {
     double zp[3] = {0, 0, 0}, ps = 0.0;
-    if (p >= 0) box_centre(cube_of(cube, t, t.info[p].x), t.cell[p], d, zp, &ps);
+    if (w.id >= 0) box_centre(cube_of(cube, t, w.first), w.cell, w.depth, zp, &ps);
     float a[14];
     twig_child_f32(t, ch, o, (float)(0.25 * ps), a);
 #pragma unroll
     for (int k = 0; k < 14; ++k) a[k] = sum8(a[k]);
-    if (p >= 0 && o == 0) {
+    if (w.id >= 0 && o == 0) {
         float m32[16];
-        finish_box_f32(a, zp, m32, t.mom + (size_t)p * kMom, t.delta + p);
-        float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)p * 16);
+        finish_box_f32(a, zp, m32, t.mom + (size_t)w.id * kMom, t.delta + w.id);
+        float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)w.id * 16);
         for (int k = 0; k < 4; ++k)
             w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
     }
@@ -848,15 +828,15 @@ __device__ __forceinline__ void put_empty_halves(float* f, int place, int begin,
     if (end & 1) put_source(f, place, begin, end, kFarAway, 0.f, 0.f, 0.f);
 }
 
-// FP32C contexts: a block takes the leaves that start among its kMomTile positions.
+// FP32C contexts: a block takes the leaves that start among its kPos positions.
 // kTile (leaves of up to kMomHalo particles): the particles' offsets from their leaf's
 // geometric centre are formed with one particle per lane (the FP64 pipe takes a warp
 // instruction for 16 cycles however many lanes are active) and kept in shared memory,
 // where each leaf's thread sums them in key order; the source records are written one
 // particle per lane again.  Larger leaves: one thread per leaf does all of it.  Then
 // the twigs (sweep_up).
-template <bool kTile>
-__global__ void __launch_bounds__(kMomThreads)
+template <bool kTile, int kPos>
+__global__ void __launch_bounds__(mom_threads(kPos))
 k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
               const double* __restrict__ z, const int8_t* __restrict__ sp,
               const double* __restrict__ qsp, int n, const int* __restrict__ cnt,
@@ -864,33 +844,34 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
               float4* __restrict__ src32)
 {
     follow();
-    __shared__ int list[kMomTile];
-    __shared__ double ctr[kTile ? kMomTile : 1][3];                  // geometric centre, then c
-    __shared__ float4 ys[kTile ? kMomTile + kMomHalo : 1];           // offset, charge
-    __shared__ unsigned short owner[kTile ? kMomTile + kMomHalo : 1];
-    __shared__ int place[kTile ? kMomTile : 1];
-    const int base = blockIdx.x * kMomTile;
-    const int nl = block_leaves(cnt, base, n, list);
+    constexpr int kThreads = mom_threads(kPos);
+    __shared__ int list[kPos];
+    __shared__ double ctr[kTile ? kPos : 1][3];                  // geometric centre, then c
+    __shared__ float4 ys[kTile ? kPos + kMomHalo : 1];           // offset, charge
+    __shared__ unsigned short owner[kTile ? kPos + kMomHalo : 1];
+    __shared__ int place[kTile ? kPos : 1];
+    const int base = blockIdx.x * kPos;
+    const int nl = block_leaves<kPos>(cnt, base, n, list);
     const float q0 = (float)qsp[0], q1 = (float)qsp[1];
     float* f = reinterpret_cast<float*>(src32);
     if (kTile) {
-        for (int l = threadIdx.x; l < nl; l += kMomThreads) {
+        for (int l = threadIdx.x; l < nl; l += kThreads) {
             const int i = list[l];
             const int node = min(off[i] + cnt[i] - 1, t.cap - 1);
             const int4 inf = t.info[node];
             double side;
             box_centre(cube_of(cube, t, inf.x), t.cell[node], t.depth_leaf[node] & 255, ctr[l], &side);
-            const int e = min(inf.y - base, kMomTile + kMomHalo);
+            const int e = min(inf.y - base, kPos + kMomHalo);
             const bool fat = inf.y - inf.x > kMomHalo;   // a depth-cap box: its thread does it all
             place[l] = src_place(i, node);
             if (!fat) put_empty_halves(f, place[l], i, inf.y);
             for (int k = i - base; k < e; ++k) owner[k] = fat ? kNoOwner : (unsigned short)l;
         }
         __syncthreads();
-        const int first = nl > 0 ? list[0] - base : kMomTile;
+        const int first = nl > 0 ? list[0] - base : kPos;
         const int end = nl > 0 ? min(t.info[min(off[list[nl - 1]] + cnt[list[nl - 1]] - 1, t.cap - 1)].y - base,
-                                     kMomTile + kMomHalo) : 0;
-        for (int k = first + threadIdx.x; k < end; k += kMomThreads) {
+                                     kPos + kMomHalo) : 0;
+        for (int k = first + threadIdx.x; k < end; k += kThreads) {
             const int j = base + k;
             if (owner[k] == kNoOwner) continue;
             const double* zc = ctr[owner[k]];
@@ -898,7 +879,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                                 sp[j] ? q1 : q0);
         }
         __syncthreads();
-        for (int l = threadIdx.x; l < nl; l += kMomThreads) {
+        for (int l = threadIdx.x; l < nl; l += kThreads) {
             const int i = list[l];
             const int node = min(off[i] + cnt[i] - 1, t.cap - 1);
             const int e = t.info[node].y - base;
@@ -941,7 +922,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                 r32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
         }
         __syncthreads();
-        for (int k = first + threadIdx.x; k < end; k += kMomThreads) {
+        for (int k = first + threadIdx.x; k < end; k += kThreads) {
             const int j = base + k, l = owner[k];
             if (l == kNoOwner) continue;
             const double* c = ctr[l];
@@ -949,7 +930,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                        (float)(c[2] - z[j]), ys[k].w);
         }
     }
-    for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kMomThreads) {
+    for (int l0 = threadIdx.x & ~31; l0 < nl; l0 += kThreads) {
         const int l = l0 + (threadIdx.x & 31);
         int node = -1;
         if (l < nl) {
@@ -996,7 +977,8 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                                (float)(cz - z[j]), sp[j] ? q1 : q0);
             }
         }
-        sweep_up(t, node, [&](int p, int d, int o, int ch) { twig_combine_f32(cube, t, p, d, o, ch); });
+        sweep_up(t, node,
+                 [&](const Twig& w, int o, int ch) { twig_combine_f32(cube, t, w, o, ch); });
     }
 }
 
@@ -1039,6 +1021,31 @@ void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* po
 
 size_t topo_status_words(int n) { return (size_t)((n + kTopoThreads - 1) / kTopoThreads) + 1; }
 
+template <int kPos>
+static void moments(const double* x, const double* y, const double* z, const int8_t* sp,
+                    const double* qsp, int n, int leaf_cap, const int* pos_cnt,
+                    const int* pos_off, const Cube* cube, Tree t, float4* src32, int want_f32,
+                    Queue s)
+{
+    constexpr int kThreads = mom_threads(kPos);
+    const int nb = (n + kPos - 1) / kPos;
+    if (!want_f32)
+        launch(k_moments<kPos>, nb, kThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off, cube, t);
+    else if (leaf_cap <= kMomHalo)
+        launch(k_moments_f32<true, kPos>, nb, kThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off,
+               cube, t, src32);
+    else
+        launch(k_moments_f32<false, kPos>, nb, kThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off,
+               cube, t, src32);
+}
+
+// Up to these sizes a block takes 32 positions instead of 256: the sweep is a chain of
+// levels whose FP64 (centres in FP32C contexts) then runs on more SMs at once.  Larger
+// systems fill the SMs either way, and the leaves of 256 positions fill a warp better.
+// FP64: 30 against 34 us at N = 2048, 45 against 51 at 16384, 59 against 56 at 32768;
+// FP32C: 22 against 27, 24 against 27, and at 65536 and 131072 31 against 32, 37 against 34.
+constexpr int kMomSmallF64 = 16384, kMomSmallF32 = 65536;
+
 void launch_moments(const double* x, const double* y, const double* z, const int8_t* sp,
                     const double* qsp, int n, int leaf_cap, const int* pos_cnt,
                     const int* pos_off, const Cube* cube, Tree t, float4* src32, int want_f32,
@@ -1047,15 +1054,10 @@ void launch_moments(const double* x, const double* y, const double* z, const int
     // leaves from their particles, then every twig as its last child finishes
     // (bottom-up sweep with arrival counters), in one launch
     count_launch(1);
-    const int nb = (n + kMomTile - 1) / kMomTile;
-    if (!want_f32)
-        launch(k_moments, nb, kMomThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off, cube, t);
-    else if (leaf_cap <= kMomHalo)
-        launch(k_moments_f32<true>, nb, kMomThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off, cube,
-                                                       t, src32);
+    if (n <= (want_f32 ? kMomSmallF32 : kMomSmallF64))
+        moments<32>(x, y, z, sp, qsp, n, leaf_cap, pos_cnt, pos_off, cube, t, src32, want_f32, s);
     else
-        launch(k_moments_f32<false>, nb, kMomThreads, s, x, y, z, sp, qsp, n, pos_cnt, pos_off,
-                                                        cube, t, src32);
+        moments<256>(x, y, z, sp, qsp, n, leaf_cap, pos_cnt, pos_off, cube, t, src32, want_f32, s);
 }
 
 }  // namespace ucp

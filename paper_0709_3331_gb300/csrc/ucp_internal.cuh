@@ -86,7 +86,9 @@ __device__ __forceinline__ void follow()
 // One FP64 box record, 16 doubles (128 B), read by the FP64 walk.
 // {c.x, c.y, c.z, rcrit2, M, D.x, D.y, D.z, Qxx, Qxy, Qxz, Qyy, Qyz, Qzz, S0, -tr(Q)/2}
 // (FP32C contexts: c and rcrit2 only, the rest in mom32)
-// rcrit2 = (s/theta + delta)^2 is filled per walk (it depends on theta).
+// rcrit2 = (s/theta + delta)^2 is filled per walk (it depends on theta).  Until its first
+// walk an FP64 tree holds in the same place each box's sums about its geometric centre,
+// {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)}.
 constexpr int kMom = 16;
 enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
 
@@ -239,8 +241,10 @@ struct WalkArgs {
     int* err;               // raised by a bounded wait that gave up
     unsigned long long* stats; // {p2p, m2p}
 };
-// per walk: box records, and the work counter and cost bins (may be NULL) cleared
-void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
+// per walk: box records, and the work counter and cost bins (may be NULL) cleared;
+// sums: t.mom still holds the sums launch_moments left in an FP64 context (moments now)
+void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int sums, int* work,
+                        int* bins,
                         Queue s);
 void launch_walk_fp64(const WalkArgs& a, int nsm, Queue s);
 void launch_walk_fp32c(const WalkArgs& a, int nsm, Queue s, int shape);

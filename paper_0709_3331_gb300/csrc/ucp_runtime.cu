@@ -85,6 +85,7 @@ struct ucp_ctx {
     int sorted_buf = 0;                // key[] / val[] buffer of the last sort
     std::vector<double> cloud_energy;  // per-cloud {KE_i, KE_e, PE, px, py, pz} of the last energy
     bool have_state = false, tree_valid = false, acc_valid = false;
+    bool sums = false;                // the tree's records hold sums, not moments yet (FP64)
     bool phi_valid = false;           // phi of every particle at the current positions
     double phi_theta = -1.0, phi_eps = -1.0;
     int64_t steps = 0, walk_targets = 0, walk_launches = 0;
@@ -253,10 +254,18 @@ int build(ucp_ctx* c)
                     c->topo_status, c->sort.err, c->s);
     launch_moments(c->st[k][0], c->st[k][1], c->st[k][2], c->sp[k], c->qsp, n, c->leaf_cap,
                    c->pos_cnt, c->pos_off, c->cube, c->t, c->src32, c->precision == UCP_FP32C, c->s);
+    c->sums = c->precision == UCP_FP64;
     c->tree_valid = true;
     c->acc_valid = false;
     c->phi_valid = false;
     return check_launch(c, "tree build");
+}
+
+// Per-walk box records (and, once per FP64 build, the moments).
+void prepare(ucp_ctx* c, double theta, int* bins)
+{
+    launch_mac_prepare(c->t, c->cube, theta, c->precision == UCP_FP32C, c->sums, c->work, bins, c->s);
+    c->sums = false;
 }
 
 // One walk over all particles (electrons_only = 0) or the electrons.  visits: in an
@@ -267,7 +276,7 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
 {
     int k = c->cur;
     int f32 = c->precision == UCP_FP32C;
-    launch_mac_prepare(c->t, c->cube, theta, f32, c->work, c->cost_bins, c->s);
+    prepare(c, theta, c->cost_bins);
     WalkArgs a = {};
     a.x = c->st[k][0];
     a.y = c->st[k][1];
@@ -876,6 +885,7 @@ static int run_block_graph(ucp_ctx* c, double dt_e, int kk, double theta, double
     c->cur = hit->cur_out;
     c->steps += kk;
     c->tree_valid = true;
+    c->sums = false;
     c->acc_valid = true;
     c->phi_valid = true;
     c->phi_theta = theta;
@@ -1091,7 +1101,7 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
             load_state(c, seg + n3 * (size_t)j, nullptr);
             if ((rc = build(c))) break;
             const int f32 = c->precision == UCP_FP32C;
-            launch_mac_prepare(c->t, c->cube, theta, f32, c->work, nullptr, c->s);
+            prepare(c, theta, nullptr);
             int k = c->cur;
             launch_kick_lambda(lv, c->sp_caller, c->n, ce, ci, lam, c->s);
             launch_gather3(lam, c->id[k], c->n, lsorted, c->s);
@@ -1167,7 +1177,7 @@ int ucp_accel_vjp(ucp_ctx* c, double theta, double eps, const double* lam_in, do
         CK(cudaMemcpyAsync(c->stage, lam_in, sizeof(double) * n3, cudaMemcpyHostToDevice, c->s));
     if (!c->tree_valid && (rc = build(c))) return rc;
     const int f32 = c->precision == UCP_FP32C;
-    launch_mac_prepare(c->t, c->cube, theta, f32, c->work, nullptr, c->s);
+    prepare(c, theta, nullptr);
     const int k = c->cur;
     launch_gather3(on_device ? lam_in : c->stage, c->id[k], c->n, lsorted, c->s);
     WalkArgs a = {};
@@ -1361,6 +1371,7 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
     CK(cudaStreamSynchronize(c->s));
     *nnodes = nn;
     if (!topo && !is_leaf && !geom) return UCP_OK;
+    if (c->sums) prepare(c, 1.0, nullptr);
     if (cap < nn) return fail(c, UCP_EINVAL, "capacity smaller than the box count");
     std::vector<int4> info(nn);
     std::vector<int> dl(nn);

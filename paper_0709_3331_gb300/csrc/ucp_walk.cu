@@ -8,6 +8,7 @@
 // key-consecutive targets per warp (k_walk_fp32c); each is described at its kernel.
 // In both, each target's sums are taken in a fixed order, so results do not depend
 // on scheduling.
+#include "ucp_box.cuh"
 #include "ucp_lists.cuh"
 
 #include <math.h>
@@ -704,9 +705,15 @@ k_walk_fp32c_visits(WalkArgs a)
 }
 
 // Per walk: rcrit2 = (s/theta + delta)^2 of every box in FP64 (theta = 0:
-// +inf, nothing accepted), and the FP32C box records.
-__global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32,
-                              int* work, int* bins)
+// +inf, nothing accepted), and the FP32C box records.  kSums: the first walk after an
+// FP64 build also makes the moments and delta from the sums that build left, one box per
+// lane: nearly all FP64 work, so its blocks are small and spread over the SMs.
+constexpr int prep_threads(bool sums) { return sums ? 64 : 256; }
+
+template <bool kSums>
+__global__ void __launch_bounds__(prep_threads(kSums))
+k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32, int* work,
+              int* bins)
 {
     follow();
     if (blockIdx.x == 0) {
@@ -721,6 +728,21 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
         const Cube& cb = cube[t.cloud ? t.cloud[t.info[nd].x] : 0];
         const double L = cb.L;
         double s = ldexp(L, -(dl & 255));
+        if (kSums) {
+            double a[14], z[3], side, rec[kMom];
+            const double2* r = reinterpret_cast<const double2*>(m);
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                const double2 v = r[k];
+                a[2 * k] = v.x;
+                a[2 * k + 1] = v.y;
+            }
+            box_centre(cb, t.cell[nd], dl & 255, z, &side);
+            finish_box(a, z, rec, t.delta + nd);
+#pragma unroll
+            for (int k = 0; k < kMom; ++k)
+                if (k != MR2) m[k] = rec[k];
+        }
         double r2;
         if (theta > 0.0) {
             double rc = __dadd_rn(__ddiv_rn(s, theta), t.delta[nd]);
@@ -753,12 +775,16 @@ __global__ void k_mac_prepare(Tree t, const Cube* __restrict__ cube, double thet
 
 }  // namespace
 
-void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
-                        Queue s)
+void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int sums, int* work,
+                        int* bins, Queue s)
 {
     count_launch(1);
-    int blocks = 4 * 152;
-    launch(k_mac_prepare, blocks, 256, s, t, cube, theta, want_f32, work, bins);
+    if (sums)
+        launch(k_mac_prepare<true>, 16 * 152, prep_threads(true), s, t, cube, theta, want_f32, work,
+               bins);
+    else
+        launch(k_mac_prepare<false>, 4 * 152, prep_threads(false), s, t, cube, theta, want_f32, work,
+               bins);
 }
 
 // blocks of one warp: per_sm on every SM, or one per work item
