@@ -59,7 +59,8 @@ struct Queue {
 };
 
 template <class... P, class... A>
-inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, const Queue& q, A... args)
+inline void launch_shared(void (*kernel)(P...), dim3 grid, dim3 block, int dynamic_bytes,
+                          const Queue& q, A... args)
 {
     cudaLaunchAttribute attr = {};
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -67,10 +68,17 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, const Queue& q, 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = dynamic_bytes;
     cfg.stream = q.s;
     cfg.attrs = &attr;
     cfg.numAttrs = q.chained ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, const Queue& q, A... args)
+{
+    launch_shared(kernel, grid, block, 0, q, args...);
 }
 
 // First statement of every kernel that launch() starts, by every thread: the next

@@ -283,6 +283,205 @@ __device__ __forceinline__ void kelbg_factors(float d2, float& ri, float inv_lam
     }
 }
 
+// A target of the FP32C walk as the sums see it.
+struct LaneTarget {
+    int t, tmin, tmax;              // slots: its own, the chunk's lowest and highest
+    float xh, yh, zh, xl, yl, zl, q, eps2, inv_lambda;
+};
+
+template <bool kKelbg>
+__device__ __forceinline__ LaneTarget lane_target(const WalkArgs& a, const ChunkTarget& tg, int n)
+{
+    LaneTarget g;
+    g.t = tg.t;
+    // slots of the chunk's targets are ascending
+    g.tmin = __shfl_sync(0xffffffffu, tg.t, 0);
+    g.tmax = __shfl_sync(0xffffffffu, tg.t, n - 1);
+    g.xh = tg.xh; g.yh = tg.yh; g.zh = tg.zh;
+    g.xl = tg.xl; g.yl = tg.yl; g.zl = tg.zl;
+    g.q = tg.t >= 0 ? (float)a.qsp[a.sp[tg.t] ? 1 : 0] : 0.f;
+    g.eps2 = (float)a.eps2;
+    g.inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
+    return g;
+}
+
+// Multipoles, lanes over targets: the sums {x, y}, {z, potential} of cnt <= 32 accepted
+// boxes (zeros outside their masks), staged two boxes side by side; nm counts them.
+template <bool kPhi>
+__device__ __forceinline__ void box_batch(const WalkArgs& a, float* stage, const int2* boxes, int cnt,
+                                          const LaneTarget& g_, int& nm, float2& fxy, float2& fzp)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned int me = 1u << lane;
+    const float xh = g_.xh, yh = g_.yh, zh = g_.zh, eps2 = g_.eps2;
+    const int part = lane & 3;
+#pragma unroll
+    for (int it = 0; it < kStage / 8; ++it) {
+        const int e = it * 8 + (lane >> 2);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (e < cnt) v = __ldg(a.t.rec + (size_t)boxes[e].x * kRec + part);
+        if (part == 3) v.w = __int_as_float(e < cnt ? boxes[e].y : 0);
+        float* d = stage + (e >> 1) * kStageStride + part * 8 + (e & 1);
+        d[0] = v.x;
+        d[2] = v.y;
+        d[4] = v.z;
+        d[6] = v.w;
+    }
+    __syncwarp();
+    // With g = (R.R + eps^2)^-1/2, u = g^2, q = Q R / 2, y = D + 5 u q:
+    //   E   = -g^3 [y + u q - (M + 3 u (T + y.R)) R]
+    //   phi = g (M + u (T + y.R - 2 u q.R)),   T = -tr(Q)/2
+    float2 bx = splat(0.f), by = bx, bz = bx, bp = bx;
+    const float2 x2 = splat(xh), y2 = splat(yh), z2 = splat(zh), e2 = splat(eps2);
+    const int pairs = (cnt + 1) >> 1;
+#pragma unroll 2
+    for (int p = 0; p < pairs; ++p) {
+        const float4* P = reinterpret_cast<const float4*>(stage + p * kStageStride);
+        const float4 f0 = P[0], f1 = P[1], f2 = P[2], f3 = P[3], f4 = P[4], f5 = P[5],
+                     f6 = P[6], f7 = P[7];
+        const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
+        const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
+        const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
+        const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __ffma2_rn(rz, rz, e2)));
+        const bool in0 = (__float_as_int(f7.z) & me) != 0;
+        const bool in1 = (__float_as_int(f7.w) & me) != 0;
+        const float2 g = make_float2(in0 ? rsqrt_ftz(r2.x) : 0.f,
+                                     in1 ? rsqrt_ftz(r2.y) : 0.f);
+        nm += in0;
+        nm += in1;
+        const float2 u = __fmul2_rn(g, g);
+        const float2 g3 = __fmul2_rn(g, u);
+        const float2 qxx = make_float2(f4.x, f4.y), qxy = make_float2(f4.z, f4.w),
+                     qxz = make_float2(f5.x, f5.y), qyy = make_float2(f5.z, f5.w),
+                     qyz = make_float2(f6.x, f6.y), qzz = make_float2(f6.z, f6.w);
+        const float2 qx = __ffma2_rn(qxx, rx, __ffma2_rn(qxy, ry, __fmul2_rn(qxz, rz)));
+        const float2 qy = __ffma2_rn(qxy, rx, __ffma2_rn(qyy, ry, __fmul2_rn(qyz, rz)));
+        const float2 qz = __ffma2_rn(qxz, rx, __ffma2_rn(qyz, ry, __fmul2_rn(qzz, rz)));
+        const float2 u5 = __fmul2_rn(splat(5.f), u);
+        const float2 yx = __ffma2_rn(u5, qx, make_float2(f2.x, f2.y));
+        const float2 yy = __ffma2_rn(u5, qy, make_float2(f2.z, f2.w));
+        const float2 yz = __ffma2_rn(u5, qz, make_float2(f3.x, f3.y));
+        const float2 w = __ffma2_rn(yx, rx, __ffma2_rn(yy, ry, __ffma2_rn(yz, rz,
+                                    make_float2(f3.z, f3.w))));
+        const float2 nk = __ffma2_rn(__fmul2_rn(splat(-3.f), u), w,
+                                     make_float2(f7.x, f7.y));
+        bx = __ffma2_rn(g3, __ffma2_rn(nk, rx, __ffma2_rn(u, qx, yx)), bx);
+        by = __ffma2_rn(g3, __ffma2_rn(nk, ry, __ffma2_rn(u, qy, yy)), by);
+        bz = __ffma2_rn(g3, __ffma2_rn(nk, rz, __ffma2_rn(u, qz, yz)), bz);
+        if (kPhi) {
+            const float2 qr = __ffma2_rn(qx, rx, __ffma2_rn(qy, ry, __fmul2_rn(qz, rz)));
+            const float2 v = __ffma2_rn(__fmul2_rn(splat(-2.f), u), qr, w);
+            bp = __ffma2_rn(g, __ffma2_rn(u, v, make_float2(f1.z, f1.w)), bp);
+        }
+    }
+    fxy = make_float2(-(bx.x + bx.y), -(by.x + by.y));
+    fzp = make_float2(-(bz.x + bz.y), kPhi ? bp.x + bp.y : 0.f);
+    __syncwarp();
+}
+
+// Direct pairs, lanes over targets: cnt <= 32 opened leaves, each one's sources brought
+// into shared memory (up to 32 float4) while the leaf before it is summed; add(e, {x, y},
+// {z, potential}) takes leaf e's sums in the lanes of its mask.
+template <bool kKelbg, bool kPhi, class Add>
+__device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2* leaves, int cnt,
+                                           const LaneTarget& g_, int& np, Add add)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned int me = 1u << lane;
+    const float4* __restrict__ H = a.t.hdr;
+    const float4* __restrict__ S = a.src32;
+    const float xh = g_.xh, yh = g_.yh, zh = g_.zh, xl = g_.xl, yl = g_.yl, zl = g_.zl;
+    const float qt = g_.q, eps2 = g_.eps2, inv_lambda = g_.inv_lambda;
+    const int t = g_.t, tmin = g_.tmin, tmax = g_.tmax;
+    float4* meta = reinterpret_cast<float4*>(stage);   // {-ch, place}, {-cl, begin}
+    float4* buf = meta + 64;                             // 2 x 32 float4
+    if (lane < cnt) {
+        const int nd = leaves[lane].x;
+        float4 A = __ldg(H + nd), B = __ldg(a.t.lo + nd);
+        const int2 be = __ldg(reinterpret_cast<const int2*>(a.t.info + nd));
+        A.w = __int_as_float(src_place(be.x, nd));
+        B.w = __int_as_float(be.x);
+        meta[2 * lane] = A;
+        meta[2 * lane + 1] = B;
+        leaves[lane].x = be.y - be.x;                    // {particles, mask}
+    }
+    __syncwarp();
+    const float2 e2 = splat(eps2);
+    float4 v = __ldg(S + __float_as_int(meta[0].w) + lane);
+    for (int e = 0; e < cnt; ++e) {
+        float4* P = buf + (e & 1) * 32;
+        P[lane] = v;
+        if (e + 1 < cnt) v = __ldg(S + __float_as_int(meta[2 * e + 2].w) + lane);
+        __syncwarp();
+        const int2 nm1 = leaves[e];
+        if (!(nm1.y & me)) continue;
+        const float4 A = meta[2 * e], B = meta[2 * e + 1];
+        const float2 rx = splat((xh + A.x) + (xl + B.x));
+        const float2 ry = splat((yh + A.y) + (yl + B.y));
+        const float2 rz = splat((zh + A.z) + (zl + B.z));
+        const int begin = __float_as_int(B.w), num = nm1.x;
+        const int pairs = ((begin & 1) + num + 1) >> 1;
+        const bool self = (unsigned int)(t - begin) < (unsigned int)num;
+        np += num - (self ? 1 : 0);
+        // place of the target's own particle among the leaf's halves, or none
+        const int tp = self ? t - (begin & ~1) : -1;
+        float2 px = splat(0.f), py = px, pz = px, pp = px;
+        auto pair = [&](const float4 F, const float4 Q, bool ok0, bool ok1) {
+            const float2 dx = __fadd2_rn(rx, make_float2(F.x, F.y));
+            const float2 dy = __fadd2_rn(ry, make_float2(F.z, F.w));
+            const float2 dz = __fadd2_rn(rz, make_float2(Q.x, Q.y));
+            const float2 q = make_float2(Q.z, Q.w);
+            if (kKelbg) {
+                // unlike charges (electron-ion) take the Kelbg form, unsoftened:
+                // the Coulomb terms times 1 - e^-u and 1 - (1 + u) e^-u, u = r/lambda
+                const bool un0 = q.x != qt, un1 = q.y != qt;
+                const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                const float2 r2 = __fadd2_rn(d2, make_float2(un0 ? 0.f : eps2,
+                                                             un1 ? 0.f : eps2));
+                float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                        ok1 ? rsqrt_ftz(r2.y) : 0.f);
+                float2 fp = splat(1.f), fg = fp;
+                if (un0 && ok0) kelbg_factors(d2.x, ri.x, inv_lambda, fp.x, fg.x);
+                if (un1 && ok1) kelbg_factors(d2.y, ri.y, inv_lambda, fp.y, fg.y);
+                const float2 qi = __fmul2_rn(q, ri);
+                const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
+                px = __ffma2_rn(qr3, dx, px);
+                py = __ffma2_rn(qr3, dy, py);
+                pz = __ffma2_rn(qr3, dz, pz);
+                pp = __ffma2_rn(qi, fp, pp);
+            } else {
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+                const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                              ok1 ? rsqrt_ftz(r2.y) : 0.f);
+                const float2 qi = __fmul2_rn(q, ri);
+                const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
+                px = __ffma2_rn(qr3, dx, px);
+                py = __ffma2_rn(qr3, dy, py);
+                pz = __ffma2_rn(qr3, dz, pz);
+                if (kPhi) pp = __fadd2_rn(pp, qi);
+            }
+        };
+        if (pairs > 16) {
+            // longer than the buffer: straight from memory
+            const float4* F = S + __float_as_int(A.w);
+#pragma unroll 1
+            for (int p = 0; p < pairs; ++p)
+                pair(__ldg(F + 2 * p), __ldg(F + 2 * p + 1), 2 * p != tp, 2 * p + 1 != tp);
+        } else if (begin <= tmax && begin + num > tmin) {
+            // may hold targets of the chunk
+#pragma unroll 1
+            for (int p = 0; p < pairs; ++p)
+                pair(P[2 * p], P[2 * p + 1], 2 * p != tp, 2 * p + 1 != tp);
+        } else {
+#pragma unroll 2
+            for (int p = 0; p < pairs; ++p) pair(P[2 * p], P[2 * p + 1], true, true);
+        }
+        add(e, make_float2(px.x + px.y, py.x + py.y),
+            make_float2(pz.x + pz.y, kPhi ? pp.x + pp.y : 0.f));
+    }
+    __syncwarp();
+}
+
 // One warp walks a chunk of up to 32 key-consecutive targets of one cloud, one per
 // lane, in three parts that alternate:
 //
@@ -319,6 +518,31 @@ __device__ __forceinline__ void kelbg_factors(float d2, float& ri, float inv_lam
 // per SM.  kPhi = false (walks whose potential nobody reads, e.g. the electron
 // substeps): the potential terms and their sums are left out; the field is computed
 // by the same operations in the same order, so accelerations are bit-identical.
+template <bool kPhi>
+__device__ __forceinline__ void write_target(const WalkArgs& a, int t, float2 sxy, float2 cxy,
+                                             float2 szp, float2 czp, int np, int nm)
+{
+    if (t >= 0) {
+        const int s = a.sp[t];
+        const double qm = a.msp[2 + s];
+        a.ax[t] = qm * ((double)sxy.x + (double)cxy.x);
+        a.ay[t] = qm * ((double)sxy.y + (double)cxy.y);
+        a.az[t] = qm * ((double)szp.x + (double)czp.x);
+        if (kPhi && a.phi) a.phi[t] = (double)szp.y + (double)czp.y;
+        a.cnt_p2p[t] = np;
+        a.cnt_m2p[t] = nm;
+    }
+    unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
+        sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&a.stats[0], sp2);
+        atomicAdd(&a.stats[1], sm2);
+    }
+}
 
 template <bool kKelbg, int kThreads, int kBlocks, bool kPhi>
 __global__ void __launch_bounds__(kThreads, kBlocks)
@@ -328,11 +552,6 @@ k_walk_fp32c(WalkArgs a)
     __shared__ WalkWarp shared[kThreads / 32];
     const int lane = threadIdx.x & 31;
     WalkWarp& W = shared[threadIdx.x >> 5];
-    const unsigned int me = 1u << lane;
-    const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const float4* __restrict__ H = a.t.hdr;
-    const float4* __restrict__ S = a.src32;
-    const float eps2 = (float)a.eps2;
 
     for (int item = next_chunk(a.work, lane); item < a.nchunks;
          item = next_chunk(a.work, lane)) {
@@ -340,200 +559,141 @@ k_walk_fp32c(WalkArgs a)
         const int chunk = a.ord.order[item];
         const int4 ck = a.chunks[chunk];
         const int ti = ck.x + lane;
-        const bool valid = lane < ck.y;
-        const int t = valid ? (a.targets ? a.targets[ti] : ti) : -1;
+        const int t = lane < ck.y ? (a.targets ? a.targets[ti] : ti) : -1;
         const ChunkTarget tg(a, t, ck.z);
-        const float xh = tg.xh, yh = tg.yh, zh = tg.zh, xl = tg.xl, yl = tg.yl, zl = tg.zl;
-        const float qt = valid ? (a.sp[t] ? (float)q1 : (float)q0) : 0.f;
-        const float inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
+        const LaneTarget lt = lane_target<kKelbg>(a, tg, ck.y);
         // compensated totals (sum, correction)
         float2 sxy = splat(0.f), szp = sxy, cxy = sxy, czp = sxy;   // {x, y}, {z, potential}
         int np = 0, nm = 0;
-        // slots of the chunk's targets (ascending)
-        const int tmin = __shfl_sync(0xffffffffu, t, 0), tmax = __shfl_sync(0xffffffffu, t, ck.y - 1);
-
-        // the last cnt <= 32 boxes of the list of accepted boxes
         auto multipoles = [&](const int2* boxes, int cnt) {
-            const int part = lane & 3;
-#pragma unroll
-            for (int it = 0; it < kStage / 8; ++it) {
-                const int e = it * 8 + (lane >> 2);
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (e < cnt) v = __ldg(a.t.rec + (size_t)boxes[e].x * kRec + part);
-                if (part == 3) v.w = __int_as_float(e < cnt ? boxes[e].y : 0);
-                float* d = W.stage + (e >> 1) * kStageStride + part * 8 + (e & 1);
-                d[0] = v.x;
-                d[2] = v.y;
-                d[4] = v.z;
-                d[6] = v.w;
-            }
-            __syncwarp();
-            // With g = (R.R + eps^2)^-1/2, u = g^2, q = Q R / 2, y = D + 5 u q:
-            //   E   = -g^3 [y + u q - (M + 3 u (T + y.R)) R]
-            //   phi = g (M + u (T + y.R - 2 u q.R)),   T = -tr(Q)/2
-            float2 bx = splat(0.f), by = bx, bz = bx, bp = bx;
-            const float2 x2 = splat(xh), y2 = splat(yh), z2 = splat(zh), e2 = splat(eps2);
-            const int pairs = (cnt + 1) >> 1;
-#pragma unroll 2
-            for (int p = 0; p < pairs; ++p) {
-                const float4* P = reinterpret_cast<const float4*>(W.stage + p * kStageStride);
-                const float4 f0 = P[0], f1 = P[1], f2 = P[2], f3 = P[3], f4 = P[4], f5 = P[5],
-                             f6 = P[6], f7 = P[7];
-                const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
-                const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
-                const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
-                const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __ffma2_rn(rz, rz, e2)));
-                const bool in0 = (__float_as_int(f7.z) & me) != 0;
-                const bool in1 = (__float_as_int(f7.w) & me) != 0;
-                const float2 g = make_float2(in0 ? rsqrt_ftz(r2.x) : 0.f,
-                                             in1 ? rsqrt_ftz(r2.y) : 0.f);
-                nm += in0;
-                nm += in1;
-                const float2 u = __fmul2_rn(g, g);
-                const float2 g3 = __fmul2_rn(g, u);
-                const float2 qxx = make_float2(f4.x, f4.y), qxy = make_float2(f4.z, f4.w),
-                             qxz = make_float2(f5.x, f5.y), qyy = make_float2(f5.z, f5.w),
-                             qyz = make_float2(f6.x, f6.y), qzz = make_float2(f6.z, f6.w);
-                const float2 qx = __ffma2_rn(qxx, rx, __ffma2_rn(qxy, ry, __fmul2_rn(qxz, rz)));
-                const float2 qy = __ffma2_rn(qxy, rx, __ffma2_rn(qyy, ry, __fmul2_rn(qyz, rz)));
-                const float2 qz = __ffma2_rn(qxz, rx, __ffma2_rn(qyz, ry, __fmul2_rn(qzz, rz)));
-                const float2 u5 = __fmul2_rn(splat(5.f), u);
-                const float2 yx = __ffma2_rn(u5, qx, make_float2(f2.x, f2.y));
-                const float2 yy = __ffma2_rn(u5, qy, make_float2(f2.z, f2.w));
-                const float2 yz = __ffma2_rn(u5, qz, make_float2(f3.x, f3.y));
-                const float2 w = __ffma2_rn(yx, rx, __ffma2_rn(yy, ry, __ffma2_rn(yz, rz,
-                                            make_float2(f3.z, f3.w))));
-                const float2 nk = __ffma2_rn(__fmul2_rn(splat(-3.f), u), w,
-                                             make_float2(f7.x, f7.y));
-                bx = __ffma2_rn(g3, __ffma2_rn(nk, rx, __ffma2_rn(u, qx, yx)), bx);
-                by = __ffma2_rn(g3, __ffma2_rn(nk, ry, __ffma2_rn(u, qy, yy)), by);
-                bz = __ffma2_rn(g3, __ffma2_rn(nk, rz, __ffma2_rn(u, qz, yz)), bz);
-                if (kPhi) {
-                    const float2 qr = __ffma2_rn(qx, rx, __ffma2_rn(qy, ry, __fmul2_rn(qz, rz)));
-                    const float2 v = __ffma2_rn(__fmul2_rn(splat(-2.f), u), qr, w);
-                    bp = __ffma2_rn(g, __ffma2_rn(u, v, make_float2(f1.z, f1.w)), bp);
-                }
-            }
-            two_sum_acc2(sxy, cxy, make_float2(-(bx.x + bx.y), -(by.x + by.y)));
-            two_sum_acc2(szp, czp, make_float2(-(bz.x + bz.y), kPhi ? bp.x + bp.y : 0.f));
-            __syncwarp();
+            float2 fxy, fzp;
+            box_batch<kPhi>(a, W.stage, boxes, cnt, lt, nm, fxy, fzp);
+            two_sum_acc2(sxy, cxy, fxy);
+            two_sum_acc2(szp, czp, fzp);
         };
-
-        // cnt <= 32 opened leaves, each one's sources brought into shared memory (up to
-        // 32 float4) while the leaf before it is summed
+        // a leaf's pairs are summed in FP32 and enter the total by a compensated add
+        // (folding every fourth leaf only is 1.5 % faster and 1 % less exact)
         auto direct_pairs = [&](int2* leaves, int cnt) {
-            float4* meta = reinterpret_cast<float4*>(W.stage);   // {-ch, place}, {-cl, begin}
-            float4* buf = meta + 64;                             // 2 x 32 float4
-            if (lane < cnt) {
-                const int nd = leaves[lane].x;
-                float4 A = __ldg(H + nd), B = __ldg(a.t.lo + nd);
-                const int2 be = __ldg(reinterpret_cast<const int2*>(a.t.info + nd));
-                A.w = __int_as_float(src_place(be.x, nd));
-                B.w = __int_as_float(be.x);
-                meta[2 * lane] = A;
-                meta[2 * lane + 1] = B;
-                leaves[lane].x = be.y - be.x;                    // {particles, mask}
-            }
-            __syncwarp();
-            const float2 e2 = splat(eps2);
-            float4 v = __ldg(S + __float_as_int(meta[0].w) + lane);
-            for (int e = 0; e < cnt; ++e) {
-                float4* P = buf + (e & 1) * 32;
-                P[lane] = v;
-                if (e + 1 < cnt) v = __ldg(S + __float_as_int(meta[2 * e + 2].w) + lane);
-                __syncwarp();
-                const int2 nm1 = leaves[e];
-                if (!(nm1.y & me)) continue;
-                const float4 A = meta[2 * e], B = meta[2 * e + 1];
-                const float2 rx = splat((xh + A.x) + (xl + B.x));
-                const float2 ry = splat((yh + A.y) + (yl + B.y));
-                const float2 rz = splat((zh + A.z) + (zl + B.z));
-                const int begin = __float_as_int(B.w), num = nm1.x;
-                const int pairs = ((begin & 1) + num + 1) >> 1;
-                const bool self = (unsigned int)(t - begin) < (unsigned int)num;
-                np += num - (self ? 1 : 0);
-                // place of the target's own particle among the leaf's halves, or none
-                const int tp = self ? t - (begin & ~1) : -1;
-                float2 px = splat(0.f), py = px, pz = px, pp = px;
-                auto pair = [&](const float4 F, const float4 Q, bool ok0, bool ok1) {
-                    const float2 dx = __fadd2_rn(rx, make_float2(F.x, F.y));
-                    const float2 dy = __fadd2_rn(ry, make_float2(F.z, F.w));
-                    const float2 dz = __fadd2_rn(rz, make_float2(Q.x, Q.y));
-                    const float2 q = make_float2(Q.z, Q.w);
-                    if (kKelbg) {
-                        // unlike charges (electron-ion) take the Kelbg form, unsoftened:
-                        // the Coulomb terms times 1 - e^-u and 1 - (1 + u) e^-u, u = r/lambda
-                        const bool un0 = q.x != qt, un1 = q.y != qt;
-                        const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-                        const float2 r2 = __fadd2_rn(d2, make_float2(un0 ? 0.f : eps2,
-                                                                     un1 ? 0.f : eps2));
-                        float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
-                                                ok1 ? rsqrt_ftz(r2.y) : 0.f);
-                        float2 fp = splat(1.f), fg = fp;
-                        if (un0 && ok0) kelbg_factors(d2.x, ri.x, inv_lambda, fp.x, fg.x);
-                        if (un1 && ok1) kelbg_factors(d2.y, ri.y, inv_lambda, fp.y, fg.y);
-                        const float2 qi = __fmul2_rn(q, ri);
-                        const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
-                        px = __ffma2_rn(qr3, dx, px);
-                        py = __ffma2_rn(qr3, dy, py);
-                        pz = __ffma2_rn(qr3, dz, pz);
-                        pp = __ffma2_rn(qi, fp, pp);
-                    } else {
-                        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-                        const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
-                                                      ok1 ? rsqrt_ftz(r2.y) : 0.f);
-                        const float2 qi = __fmul2_rn(q, ri);
-                        const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
-                        px = __ffma2_rn(qr3, dx, px);
-                        py = __ffma2_rn(qr3, dy, py);
-                        pz = __ffma2_rn(qr3, dz, pz);
-                        if (kPhi) pp = __fadd2_rn(pp, qi);
-                    }
-                };
-                if (pairs > 16) {
-                    // longer than the buffer: straight from memory
-                    const float4* F = S + __float_as_int(A.w);
-#pragma unroll 1
-                    for (int p = 0; p < pairs; ++p)
-                        pair(__ldg(F + 2 * p), __ldg(F + 2 * p + 1), 2 * p != tp, 2 * p + 1 != tp);
-                } else if (begin <= tmax && begin + num > tmin) {
-                    // may hold targets of the chunk
-#pragma unroll 1
-                    for (int p = 0; p < pairs; ++p)
-                        pair(P[2 * p], P[2 * p + 1], 2 * p != tp, 2 * p + 1 != tp);
-                } else {
-#pragma unroll 2
-                    for (int p = 0; p < pairs; ++p) pair(P[2 * p], P[2 * p + 1], true, true);
-                }
-                // a leaf's pairs are summed in FP32 and enter the total by a compensated
-                // add (folding every fourth leaf only is 1.5 % faster and 1 % less exact)
-                two_sum_acc2(sxy, cxy, make_float2(px.x + px.y, py.x + py.y));
-                two_sum_acc2(szp, czp, make_float2(pz.x + pz.y, kPhi ? pp.x + pp.y : 0.f));
-            }
-            __syncwarp();
+            leaf_batch<kKelbg, kPhi>(a, W.stage, leaves, cnt, lt, np,
+                                     [&](int, const float2 fxy, const float2 fzp) {
+                                         two_sum_acc2(sxy, cxy, fxy);
+                                         two_sum_acc2(szp, czp, fzp);
+                                     });
         };
 
         walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
 
-        if (valid) {
-            const int s = a.sp[t];
-            const double qm = a.msp[2 + s];
-            a.ax[t] = qm * ((double)sxy.x + (double)cxy.x);
-            a.ay[t] = qm * ((double)sxy.y + (double)cxy.y);
-            a.az[t] = qm * ((double)szp.x + (double)czp.x);
-            if (kPhi && a.phi) a.phi[t] = (double)szp.y + (double)czp.y;
-            a.cnt_p2p[t] = np;
-            a.cnt_m2p[t] = nm;
-        }
-        unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
-            sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
-        }
+        write_target<kPhi>(a, t, sxy, cxy, szp, czp, np, nm);
         if (lane == 0) {
-            atomicAdd(&a.stats[0], sp2);
-            atomicAdd(&a.stats[1], sm2);
+            const float cost = (float)(clock64() - began);
+            a.ord.cost[chunk] = cost;
+            atomicAdd(&a.ord.bins[cost_bin(cost)], 1);
+        }
+    }
+}
+
+// The same walk with kWays warps to a chunk, for systems too small to fill the SMs with a
+// warp per chunk, whose walks take as long as one chunk does (its chain of box records,
+// and one warp's rate of issue).  Every warp runs the whole traversal (they agree on it,
+// reading the same boxes), and warp w evaluates every kWays-th batch of multipoles or of
+// kSplitLeaves leaves into a slot of shared memory; one more warp adds the slots to the
+// totals in the order in which k_walk_fp32c adds them, a round of kWays slots behind, so
+// that the results are those of k_walk_fp32c bit for bit, whatever splits them.  N = 4099:
+// 187 -> 88 us (Kelbg law 321 -> 118); 16384: 242 -> 143 us; 50,000: 399 -> 383 us; one
+// warp per chunk again from 1520 chunks on (split_shape).
+constexpr int kSplitLeaves = 4;
+
+struct SplitSlot {
+    float4 v[kSplitLeaves][32];          // {x, y, z, potential} of a batch or leaf, per lane
+    unsigned int mask[kSplitLeaves];     // lanes that add it; 0 ends the slot
+};
+
+template <int kWays>
+struct SplitShared {
+    WalkWarp warp[kWays];
+    SplitSlot slot[2][kWays];
+    int2 counts[kWays][32];              // {pairs, boxes} per lane
+    int filled[2];                       // slots of a round; ~slots: the last round
+};
+
+template <bool kKelbg, bool kPhi, int kWays, int kBlocks>
+__global__ void __launch_bounds__((kWays + 1) * 32, kBlocks)
+k_walk_fp32c_split(WalkArgs a)
+{
+    follow();
+    extern __shared__ __align__(16) unsigned char split_bytes[];
+    SplitShared<kWays>& sh = *reinterpret_cast<SplitShared<kWays>*>(split_bytes);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long began = clock64();
+    const int chunk = a.ord.order[blockIdx.x];
+    const int4 ck = a.chunks[chunk];
+    const int t = lane < ck.y ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
+    // all warps meet once per round
+    auto meet = [] { asm volatile("bar.sync 1, %0;" ::"n"((kWays + 1) * 32) : "memory"); };
+    if (w < kWays) {
+        WalkWarp& W = sh.warp[w];
+        const ChunkTarget tg(a, t, ck.z);
+        const LaneTarget lt = lane_target<kKelbg>(a, tg, ck.y);
+        int np = 0, nm = 0, task = 0, round = 0;
+        auto turn = [&](auto fill) {
+            if ((task & (kWays - 1)) == w) fill(sh.slot[round & 1][w]);
+            if ((++task & (kWays - 1)) == 0) {
+                if (threadIdx.x == 0) sh.filled[round & 1] = kWays;
+                meet();
+                ++round;
+            }
+        };
+        auto multipoles = [&](const int2* boxes, int cnt) {
+            turn([&](SplitSlot& s) {
+                float2 fxy, fzp;
+                box_batch<kPhi>(a, W.stage, boxes, cnt, lt, nm, fxy, fzp);
+                s.v[0][lane] = make_float4(fxy.x, fxy.y, fzp.x, fzp.y);
+                if (lane < kSplitLeaves) s.mask[lane] = lane == 0 ? 0xffffffffu : 0u;
+            });
+        };
+        auto direct_pairs = [&](int2* leaves, int cnt) {
+            for (int e0 = 0; e0 < cnt; e0 += kSplitLeaves)
+                turn([&](SplitSlot& s) {
+                    const int c = min(kSplitLeaves, cnt - e0);
+                    if (lane < kSplitLeaves)
+                        s.mask[lane] = lane < c ? (unsigned int)leaves[e0 + lane].y : 0u;
+                    leaf_batch<kKelbg, kPhi>(a, W.stage, leaves + e0, c, lt, np,
+                                             [&](int e, const float2 fxy, const float2 fzp) {
+                                                 s.v[e][lane] = make_float4(fxy.x, fxy.y, fzp.x, fzp.y);
+                                             });
+                });
+        };
+        walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
+        sh.counts[w][lane] = make_int2(np, nm);
+        if (threadIdx.x == 0) sh.filled[round & 1] = ~(task & (kWays - 1));
+        meet();
+    } else {
+        float2 sxy = splat(0.f), szp = sxy, cxy = sxy, czp = sxy;
+        int filled = 0;
+        for (int round = 0; filled >= 0; ++round) {
+            meet();
+            filled = sh.filled[round & 1];
+            const int slots = filled < 0 ? ~filled : filled;
+            for (int k = 0; k < slots; ++k) {
+                const SplitSlot& s = sh.slot[round & 1][k];
+#pragma unroll
+                for (int e = 0; e < kSplitLeaves; ++e) {
+                    const unsigned int mask = s.mask[e];
+                    if (!mask) break;
+                    if (!(mask >> lane & 1u)) continue;
+                    const float4 v = s.v[e][lane];
+                    two_sum_acc2(sxy, cxy, make_float2(v.x, v.y));
+                    two_sum_acc2(szp, czp, make_float2(v.z, v.w));
+                }
+            }
+        }
+        int np = 0, nm = 0;
+        for (int k = 0; k < kWays; ++k) {
+            np += sh.counts[k][lane].x;
+            nm += sh.counts[k][lane].y;
+        }
+        write_target<kPhi>(a, t, sxy, cxy, szp, czp, np, nm);
+        if (lane == 0) {
             const float cost = (float)(clock64() - began);
             a.ord.cost[chunk] = cost;
             atomicAdd(&a.ord.bins[cost_bin(cost)], 1);
@@ -808,7 +968,8 @@ void launch_walk_fp64(const WalkArgs& a, int nsm, Queue s)
 // Launch shapes of the FP32C walk that the autotuner chooses from: blocks of one
 // warp, and how many of them are resident per SM, which sets the register budget,
 // {threads, blocks, 0}.  The persistent grid takes 32-target chunks from a counter,
-// so the shape changes the schedule, never a result.
+// so the shape changes the schedule, never a result.  (Of walks with more than 10 chunks
+// per SM; smaller ones take the block that suits their size, see walk_fp32c_few.)
 static const int kShapes[][3] = {{32, 24, 0}, {32, 20, 0}, {32, 28, 0}, {32, 32, 0},
                                  {32, 16, 0}, {32, 18, 0}, {32, 22, 0}, {32, 26, 0},
                                  {32, 14, 0}, {32, 12, 0}};
@@ -831,9 +992,41 @@ static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, Queue s)
     }
 }
 
+template <bool kKelbg, bool kPhi, int kWays, int kBlocks>
+static void walk_fp32c_split(const WalkArgs& a, Queue s)
+{
+    const int bytes = (int)sizeof(SplitShared<kWays>);
+    cudaFuncSetAttribute(k_walk_fp32c_split<kKelbg, kPhi, kWays, kBlocks>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    launch_shared(k_walk_fp32c_split<kKelbg, kPhi, kWays, kBlocks>, a.nchunks, (kWays + 1) * 32,
+                  bytes, s.whole(), a);
+}
+
+// Walks whose chunks are few enough for several warps each: a block per chunk, all of them
+// resident at once (the last rule: nearly), with the register budget that this number of
+// blocks per SM leaves.  The lines lie where the next rule is as fast, in us for 8, 4 (3
+// blocks per SM), 4 (5 blocks), 2 warps and 1 warp to a chunk, theta 0.5, with potential:
+//   256 chunks 116 126 140 188 225     512 chunks 170 143 163 207 242
+//   750 chunks 244 206 177 226 281    1024 chunks 335 280 256 256 310
+//  1563 chunks 537 433 378 383 399    2048 chunks 697 567 482 461 444
+template <bool kKelbg, bool kPhi>
+static bool walk_fp32c_few(const WalkArgs& a, int nsm, Queue s)
+{
+    if (a.nchunks <= 2 * nsm) walk_fp32c_split<kKelbg, kPhi, 8, 2>(a, s);
+    else if (a.nchunks <= 4 * nsm) walk_fp32c_split<kKelbg, kPhi, 4, 3>(a, s);
+    else if (a.nchunks <= 5 * nsm) walk_fp32c_split<kKelbg, kPhi, 4, 5>(a, s);
+    else if (a.nchunks <= 10 * nsm) walk_fp32c_split<kKelbg, kPhi, 2, 8>(a, s);
+    else return false;
+    return true;
+}
+
 void launch_walk_fp32c(const WalkArgs& a, int nsm, Queue s, int shape)
 {
     count_launch(1);
+    if (a.kelbg ? walk_fp32c_few<true, true>(a, nsm, s)
+                : a.phi ? walk_fp32c_few<false, true>(a, nsm, s)
+                        : walk_fp32c_few<false, false>(a, nsm, s))
+        return;
     if (shape < 0 || shape >= walk_shape_count()) shape = 0;
     const int per_sm = kShapes[shape][1];
     const int b = walk_blocks(a.nchunks, nsm, per_sm);
