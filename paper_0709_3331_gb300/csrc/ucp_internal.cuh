@@ -170,6 +170,10 @@ struct BuildCtl {
     int* words;              // kCtlWords
     unsigned int* epoch;     // tag of the published words, advanced every build
 };
+// One cloud of up to this many particles is sorted by one block (ucp_sort.cu).
+constexpr int kBlockSort = 6144, kBlockThreads = 1024;
+inline bool block_sorted(int n, int n_clouds) { return n_clouds == 1 && n <= kBlockSort; }
+
 void launch_bbox(const double* x, const double* y, const double* z, int n, double* partials,
                  int nblk, Cube* cubes, const int* cloud_start, int n_clouds, BuildCtl ctl,
                  Queue s);
@@ -195,8 +199,19 @@ struct StateRef {
     int8_t* sp;
     unsigned int* id;
 };
+// Particle at sorted place i: its state, species and caller index from slot p.
+__device__ __forceinline__ void move_state(const StateRef& in, const StateRef& out, int i,
+                                           unsigned int p)
+{
+#pragma unroll
+    for (int a = 0; a < 6; ++a) out.f[a][i] = in.f[a][p];
+    out.sp[i] = in.sp[p];
+    out.id[i] = in.id[p];
+}
+
 // Sorts key[0] (unsorted keys of the slots of `in`) and moves the state into key order
-// (`out`); returns the buffer (0 or 1) that holds the sorted keys.
+// (`out`), or leaves that to launch_topology (block_sorted), with the slots in order in
+// val[1]; returns the buffer (0 or 1) that holds the sorted keys.
 int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int passes,
                 const SortScratch& sc, BuildCtl ctl, const StateRef& in, const StateRef& out,
                 const unsigned char* cloud, const int* cloud_start, int n_clouds, int nsm,
@@ -204,7 +219,8 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
 int sort_selftest_timeout(const SortScratch& sc, Queue s);
 void launch_topology(const unsigned long long* key, int n, int leaf_cap, int* pos_cnt,
                      int* pos_off, Tree t, BuildCtl ctl, unsigned long long* status, int* err,
-                     Queue s);
+                     const StateRef& in,
+                     const StateRef& out, const unsigned int* from, Queue s);
 size_t topo_status_words(int n);
 void launch_moments(const double* x, const double* y, const double* z, const int8_t* sp,
                     const double* qsp, int n, int leaf_cap, const int* pos_cnt,

@@ -235,7 +235,7 @@ int build(ucp_ctx* c)
     launch_bbox(c->st[k][0], c->st[k][1], c->st[k][2], n, c->bbox_part, c->bbox_nblk, c->cube,
                 cs, c->n_clouds, c->ctl, c->s);
     launch_keys(c->st[k][0], c->st[k][1], c->st[k][2], n, c->cube, c->t.cloud, c->key[0],
-                c->passes, c->ctl, c->s);
+                block_sorted(n, c->n_clouds) ? 0 : c->passes, c->ctl, c->s);
     StateRef in, out;
     for (int a = 0; a < 6; ++a) {
         in.f[a] = c->st[k][a];
@@ -251,7 +251,8 @@ int build(ucp_ctx* c)
     c->cur = k ^ 1;
     k = c->cur;
     launch_topology(c->key[b], n, c->leaf_cap, c->pos_cnt, c->pos_off, c->t, c->ctl,
-                    c->topo_status, c->sort.err, c->s);
+                    c->topo_status, c->sort.err, in, out,
+                    block_sorted(n, c->n_clouds) ? c->val[1] : nullptr, c->s);
     launch_moments(c->st[k][0], c->st[k][1], c->st[k][2], c->sp[k], c->qsp, n, c->leaf_cap,
                    c->pos_cnt, c->pos_off, c->cube, c->t, c->src32, c->precision == UCP_FP32C, c->s);
     c->sums = c->precision == UCP_FP64;

@@ -7,8 +7,8 @@
 // part of a Gaussian cloud of 524,288 with three passes), and the kernel that moves
 // the state orders each run of its tile by the rest of the key in shared memory.  A
 // run longer than kRun raises a flag on the device, on which one further kernel,
-// otherwise empty, sorts the whole key.  Three passes of eight: 62 of 165 us at
-// N = 524,288.
+// otherwise empty, sorts the whole key.  Three passes take 53 us at N = 524,288, eight
+// took 165.
 #include "ucp_scan.cuh"
 
 namespace ucp {
@@ -163,16 +163,6 @@ k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __res
     }
 }
 
-// Particle at sorted place i: its state, species and caller index from slot p.
-__device__ __forceinline__ void move_state(const StateRef& in, const StateRef& out, int i,
-                                           unsigned int p)
-{
-#pragma unroll
-    for (int a = 0; a < 6; ++a) out.f[a][i] = in.f[a][p];
-    out.sp[i] = in.sp[p];
-    out.id[i] = in.id[p];
-}
-
 // Orders the runs of equal top digits by (key, caller index) and moves the state.  A
 // block owns kFinish places and also sees the kRun places on either side, so that
 // every run that touches its places and is no longer than kRun lies in its window;
@@ -234,6 +224,158 @@ k_finish_sort(const unsigned long long* __restrict__ kin, const unsigned int* __
         const int l = 1 + kRun + threadIdx.x;
         kout[i] = sk[l];
         move_state(in, out, i, sv[l]);
+    }
+}
+
+// One cloud of up to kBlockSort particles by one block of 32 warps, all in shared
+// memory: the same passes over the top digits and the same ordering of runs, or, when a
+// run is too long, passes over the caller index and the whole key.  The state is moved by
+// the topology's blocks (one SM would take longer for its traffic than for the sort).
+// A chain of barriers and shared-memory latencies, about 3 us for every 1024 particles:
+// in place of two or three passes of one to four blocks, the run kernel and the empty
+// full sort it takes 11.5 for 27 us at N = 2048 and 22 for 40 at 4099 (a build of such a
+// cloud 111 -> 96 and 128 -> 112 us, with the extents also by one block); at 6000 a build
+// still gains 8 us, at 8192 it would lose 2.
+constexpr int kBlockItems = kBlockSort / kBlockThreads;
+constexpr int kBlockWarps = kBlockThreads / 32;
+
+struct BlockSortShared {
+    unsigned long long key[kBlockSort];
+    unsigned short val[kBlockSort];
+    int cnt[kBlockWarps][kRadix];    // keys of a digit in warp w before, then its first place
+    int part[4][kRadix];             // the same for each eight warps
+    int sums[kRadix / 32];
+};
+
+__global__ void __launch_bounds__(kBlockThreads)
+k_sort_block(const unsigned long long* __restrict__ kin, unsigned long long* __restrict__ kout,
+             unsigned int* __restrict__ vout, int n, const unsigned int* __restrict__ id)
+{
+    follow();
+    extern __shared__ __align__(16) unsigned char sort_bytes[];
+    BlockSortShared& sh = *reinterpret_cast<BlockSortShared*>(sort_bytes);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int items = (n + kBlockThreads - 1) / kBlockThreads;
+    const int first = w * 32 * items + lane;        // a warp owns a contiguous part
+    unsigned long long kk[kBlockItems];
+    unsigned int vv[kBlockItems];
+#pragma unroll
+    for (int j = 0; j < kBlockItems; ++j) {
+        const int i = first + 32 * j;
+        const bool ok = j < items && i < n;
+        kk[j] = ok ? kin[i] : 0ull;
+        vv[j] = ok ? (unsigned int)i : 0u;
+    }
+    // one stable pass by digit(key, slot) < kRadix
+    auto pass = [&](auto digit) {
+        for (int i = threadIdx.x; i < kBlockWarps * kRadix; i += kBlockThreads) (&sh.cnt[0][0])[i] = 0;
+        __syncthreads();
+        unsigned int place[kBlockItems];            // digit << 16 | rank in the warp
+#pragma unroll
+        for (int j = 0; j < kBlockItems; ++j) {
+            if (j >= items) break;
+            const bool ok = first + 32 * j < n;
+            const int d = ok ? (int)digit(kk[j], vv[j]) : kRadix + lane;   // invalid lanes unique
+            const unsigned int peers = __match_any_sync(0xffffffffu, d);
+            const int leader = __ffs(peers) - 1;
+            int before = 0;
+            if (ok && lane == leader) {
+                before = sh.cnt[w][d];
+                sh.cnt[w][d] = before + __popc(peers);
+            }
+            before = __shfl_sync(0xffffffffu, before, leader);
+            place[j] = (unsigned int)d << 16 | (unsigned int)(before + __popc(peers & ((1u << lane) - 1u)));
+            __syncwarp();
+        }
+        __syncthreads();
+        const int d = threadIdx.x & (kRadix - 1), q = threadIdx.x / kRadix;
+        int sum = 0;
+#pragma unroll
+        for (int k = 0; k < kBlockWarps / 4; ++k) {
+            const int c = sh.cnt[q * (kBlockWarps / 4) + k][d];
+            sh.cnt[q * (kBlockWarps / 4) + k][d] = sum;
+            sum += c;
+        }
+        sh.part[q][d] = sum;
+        __syncthreads();
+        int total = 0, upto = 0;
+        if (w < kRadix / 32) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) total += sh.part[k][d];
+            upto = warp_incl_scan(total, lane);
+            if (lane == 31) sh.sums[w] = upto;
+        }
+        __syncthreads();
+        if (w < kRadix / 32) {
+            int at = upto - total;
+            for (int k = 0; k < w; ++k) at += sh.sums[k];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int c = sh.part[k][d];
+                sh.part[k][d] = at;
+                at += c;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kBlockItems; ++j) {
+            if (j >= items || first + 32 * j >= n) break;
+            const int dj = place[j] >> 16;
+            const int p = sh.part[w / (kBlockWarps / 4)][dj] + sh.cnt[w][dj] + (int)(place[j] & 0xffffu);
+            sh.key[p] = kk[j];
+            sh.val[p] = (unsigned short)vv[j];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kBlockItems; ++j) {
+            const int i = first + 32 * j;
+            if (j >= items || i >= n) break;
+            kk[j] = sh.key[i];
+            vv[j] = sh.val[i];
+        }
+    };
+    auto by_key = [&](int shift) {
+        pass([&](unsigned long long k, unsigned int) { return (unsigned int)(k >> shift) & 0xffu; });
+    };
+    constexpr int low = kKeyBits - 16;      // two passes: runs of 4 in the densest part at 6144
+    by_key(low);
+    by_key(low + 8);
+    // each particle's place in its run of equal top digits, by (key, caller index)
+    int place[kBlockItems];
+    bool too_long = false;
+#pragma unroll
+    for (int j = 0; j < kBlockItems; ++j) {
+        const int i = first + 32 * j;
+        place[j] = i;
+        if (j >= items || i >= n) break;
+        const unsigned long long k = kk[j], top = k >> low;
+        int b = i, e = i + 1;
+        while (b > 0 && i - b <= kRun && sh.key[b - 1] >> low == top) --b;
+        while (e < n && e - b <= kRun && sh.key[e] >> low == top) ++e;
+        if (e - b > kRun) {
+            too_long = true;
+            continue;
+        }
+        int at = b;
+        for (int o = b; o < e; ++o) {
+            const unsigned long long ko = sh.key[o];
+            at += ko < k || (ko == k && o != i && id[sh.val[o]] < id[vv[j]]);
+        }
+        place[j] = at;
+    }
+    if (__syncthreads_or(too_long)) {
+        static_assert(kBlockSort <= kRadix * kRadix, "two digits of the caller index");
+        pass([&](unsigned long long, unsigned int v) { return id[v] & 0xffu; });
+        pass([&](unsigned long long, unsigned int v) { return id[v] >> 8; });
+        for (int shift = 0; shift < kKeyBits; shift += 8) by_key(shift);
+#pragma unroll
+        for (int j = 0; j < kBlockItems; ++j) place[j] = first + 32 * j;
+    }
+#pragma unroll
+    for (int j = 0; j < kBlockItems; ++j) {
+        if (j >= items || first + 32 * j >= n) break;
+        kout[place[j]] = kk[j];
+        vout[place[j]] = vv[j];
     }
 }
 
@@ -407,6 +549,14 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
                 Queue s)
 {
     const bool clouds = n_clouds > 1;
+    if (block_sorted(n, n_clouds)) {
+        count_launch(1);
+        const int bytes = (int)sizeof(BlockSortShared);
+        cudaFuncSetAttribute(k_sort_block, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        launch_shared(k_sort_block, 1, kBlockThreads, bytes, s, key[0], key[1], val[1], n,
+                      in.id);
+        return 1;
+    }
     count_launch(passes + 2 + (clouds ? 1 : 0));
     const int nb = (n + kSortTile - 1) / kSortTile;
     const int low = kKeyBits - 8 * passes;
