@@ -127,6 +127,83 @@ struct ChunkTarget {
     }
 };
 
+// The targets of `mask` that accept this lane's box (box < 0: none), h its record; called
+// by the whole warp.
+__device__ __forceinline__ unsigned int accept_mask(const WalkArgs& a, float* stage,
+                                                    const ChunkTarget& tg, int box,
+                                                    unsigned int mask, const float4 h)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned int lt = (1u << lane) - 1u, me = 1u << lane;
+    const bool has = box >= 0;
+    const float rc2 = fabsf(h.w);
+    const float dx = fabsf(tg.gx + h.x), dy = fabsf(tg.gy + h.y), dz = fabsf(tg.gz + h.z);
+    const float nx = fmaxf(dx - tg.ex, 0.f), ny = fmaxf(dy - tg.ey, 0.f), nz = fmaxf(dz - tg.ez, 0.f);
+    const float fx = dx + tg.ex, fy = dy + tg.ey, fz = dz + tg.ez;
+    const float near2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
+    const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+    const bool all_acc = near2 - rc2 > fmaf(tg.gwa, near2, tg.gwb);
+    const bool all_opn = rc2 - far2 > fmaf(tg.gwa, far2, tg.gwb);
+    unsigned int am = has && all_acc ? mask : 0u;   // targets that accept the box
+    const bool some = has && !all_acc && !all_opn;
+    const unsigned int between = __ballot_sync(0xffffffffu, some);
+    if (between) {
+        // decided target by target, two boxes per packed operation: pairs of
+        // {-c} x, y, z, {-rcrit2}, {box, mask}, side by side
+        const int slot = some ? __popc(between & lt) : -1;
+        const int cnt = __popc(between);
+        if (some) {
+            float* d = stage + (slot >> 1) * 12 + (slot & 1);
+            d[0] = h.x;
+            d[2] = h.y;
+            d[4] = h.z;
+            d[6] = -rc2;
+            d[8] = __int_as_float(box);
+            d[10] = __int_as_float((int)mask);
+        }
+        if (lane == 0 && (cnt & 1)) {
+            float* d = stage + (cnt >> 1) * 12 + 1;
+            d[0] = d[2] = d[4] = d[6] = d[8] = d[10] = 0.f;
+        }
+        __syncwarp();
+        const float2 x2 = splat(tg.xh), y2 = splat(tg.yh), z2 = splat(tg.zh);
+        for (int p = 0; 2 * p < cnt; ++p) {
+            const float4* P = reinterpret_cast<const float4*>(stage + p * 12);
+            const float4 f0 = P[0], f1 = P[1], f2 = P[2];
+            const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
+            const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
+            const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
+            const float2 d2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+            const float2 dm = __fadd2_rn(d2, make_float2(f1.z, f1.w));
+            const float2 win = __ffma2_rn(splat(tg.wa), d2, splat(tg.wb));
+            const bool in0 = (__float_as_int(f2.z) & me) != 0;
+            const bool in1 = (__float_as_int(f2.w) & me) != 0;
+            bool acc0 = in0 && dm.x > 0.f, acc1 = in1 && dm.y > 0.f;
+            // Within the FP32 error of d2 - rcrit2 the decision is taken again in
+            // FP64 exactly as the FP64 walk takes it, so both precisions open the
+            // same boxes.  Per axis R is off by at most 2^-23 (|x_t| + |R|), so
+            // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
+            // included) with X_t the target's largest coordinate; with
+            // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
+            // a million at the bench size).
+            const bool again0 = in0 && fabsf(dm.x) <= win.x;
+            const bool again1 = in1 && fabsf(dm.y) <= win.y;
+            if (again0)
+                acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + tg.t,
+                                    a.y + tg.t, a.z + tg.t);
+            if (again1)
+                acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kMom, a.x + tg.t,
+                                    a.y + tg.t, a.z + tg.t);
+            const unsigned int am0 = __ballot_sync(0xffffffffu, acc0);
+            const unsigned int am1 = __ballot_sync(0xffffffffu, acc1);
+            if (slot == 2 * p) am = am0;
+            if (slot == 2 * p + 1) am = am1;
+        }
+        __syncwarp();
+    }
+    return am;
+}
+
 // Walks a chunk's targets, one per lane, through their cloud's tree with the lanes
 // over boxes: multipoles(list, cnt) takes cnt <= 32 accepted boxes {box, mask of the
 // targets that accept it}, pairs(list, cnt) cnt <= 32 opened leaves {leaf, mask of the
@@ -138,7 +215,7 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const
                                            Pairs& direct_pairs)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned int lt = (1u << lane) - 1u, me = 1u << lane;
+    const unsigned int lt = (1u << lane) - 1u;
     int top = 0, na = 0, nl = 0;
     // the first step tests the root for every target
     int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[cloud] : 0] : -1;
@@ -147,71 +224,8 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const
         const bool has = box >= 0;
         const float4 h = has ? __ldg(a.t.hdr + box) : make_float4(0.f, 0.f, 0.f, 0.f);
         const bool leaf = __float_as_int(h.w) < 0;
-        const float rc2 = fabsf(h.w);
-        const float dx = fabsf(tg.gx + h.x), dy = fabsf(tg.gy + h.y), dz = fabsf(tg.gz + h.z);
-        const float nx = fmaxf(dx - tg.ex, 0.f), ny = fmaxf(dy - tg.ey, 0.f), nz = fmaxf(dz - tg.ez, 0.f);
-        const float fx = dx + tg.ex, fy = dy + tg.ey, fz = dz + tg.ez;
-        const float near2 = fmaf(nx, nx, fmaf(ny, ny, nz * nz));
-        const float far2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
-        const bool all_acc = near2 - rc2 > fmaf(tg.gwa, near2, tg.gwb);
-        const bool all_opn = rc2 - far2 > fmaf(tg.gwa, far2, tg.gwb);
-        unsigned int am = has && all_acc ? mask : 0u;   // targets that accept the box
-        const bool some = has && !all_acc && !all_opn;
-        const unsigned int between = __ballot_sync(0xffffffffu, some);
-        if (between) {
-            // decided target by target, two boxes per packed operation: pairs of
-            // {-c} x, y, z, {-rcrit2}, {box, mask}, side by side
-            const int slot = some ? __popc(between & lt) : -1;
-            const int cnt = __popc(between);
-            if (some) {
-                float* d = W.stage + (slot >> 1) * 12 + (slot & 1);
-                d[0] = h.x;
-                d[2] = h.y;
-                d[4] = h.z;
-                d[6] = -rc2;
-                d[8] = __int_as_float(box);
-                d[10] = __int_as_float((int)mask);
-            }
-            if (lane == 0 && (cnt & 1)) {
-                float* d = W.stage + (cnt >> 1) * 12 + 1;
-                d[0] = d[2] = d[4] = d[6] = d[8] = d[10] = 0.f;
-            }
-            __syncwarp();
-            const float2 x2 = splat(tg.xh), y2 = splat(tg.yh), z2 = splat(tg.zh);
-            for (int p = 0; 2 * p < cnt; ++p) {
-                const float4* P = reinterpret_cast<const float4*>(W.stage + p * 12);
-                const float4 f0 = P[0], f1 = P[1], f2 = P[2];
-                const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
-                const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
-                const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
-                const float2 d2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
-                const float2 dm = __fadd2_rn(d2, make_float2(f1.z, f1.w));
-                const float2 win = __ffma2_rn(splat(tg.wa), d2, splat(tg.wb));
-                const bool in0 = (__float_as_int(f2.z) & me) != 0;
-                const bool in1 = (__float_as_int(f2.w) & me) != 0;
-                bool acc0 = in0 && dm.x > 0.f, acc1 = in1 && dm.y > 0.f;
-                // Within the FP32 error of d2 - rcrit2 the decision is taken again in
-                // FP64 exactly as the FP64 walk takes it, so both precisions open the
-                // same boxes.  Per axis R is off by at most 2^-23 (|x_t| + |R|), so
-                // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
-                // included) with X_t the target's largest coordinate; with
-                // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
-                // a million at the bench size).
-                const bool again0 = in0 && fabsf(dm.x) <= win.x;
-                const bool again1 = in1 && fabsf(dm.y) <= win.y;
-                if (again0)
-                    acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + tg.t,
-                                        a.y + tg.t, a.z + tg.t);
-                if (again1)
-                    acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kMom, a.x + tg.t,
-                                        a.y + tg.t, a.z + tg.t);
-                const unsigned int am0 = __ballot_sync(0xffffffffu, acc0);
-                const unsigned int am1 = __ballot_sync(0xffffffffu, acc1);
-                if (slot == 2 * p) am = am0;
-                if (slot == 2 * p + 1) am = am1;
-            }
-            __syncwarp();
-        }
+        // targets that accept the box
+        const unsigned int am = accept_mask(a, W.stage, tg, box, mask, h);
         const unsigned int om = has ? mask & ~am : 0u;  // targets that open it
         const unsigned int A = __ballot_sync(0xffffffffu, am != 0u);
         const unsigned int OL = __ballot_sync(0xffffffffu, om != 0u && leaf);

@@ -18,15 +18,6 @@ namespace ucp {
 namespace {
 
 // Error-free sum (Knuth's TwoSum) folded into a running correction.
-__device__ __forceinline__ void two_sum_acc(float& s, float& c, float v)
-{
-    float t = s + v;
-    float bp = t - s;
-    float ap = t - bp;
-    c += (s - ap) + (v - bp);
-    s = t;
-}
-
 __device__ __forceinline__ void two_sum_acc2(float2& s, float2& c, float2 v)
 {
     const float2 n = make_float2(-1.f, -1.f);
@@ -305,15 +296,12 @@ __device__ __forceinline__ LaneTarget lane_target(const WalkArgs& a, const Chunk
     return g;
 }
 
-// Multipoles, lanes over targets: the sums {x, y}, {z, potential} of cnt <= 32 accepted
-// boxes (zeros outside their masks), staged two boxes side by side; nm counts them.
-template <bool kPhi>
-__device__ __forceinline__ void box_batch(const WalkArgs& a, float* stage, const int2* boxes, int cnt,
-                                          const LaneTarget& g_, int& nm, float2& fxy, float2& fzp)
+// The records of cnt <= 32 boxes into shared memory, the fields of two side by side, the
+// last of them the box's mask (0 past the end).
+__device__ __forceinline__ void stage_boxes(const WalkArgs& a, float* stage, const int2* boxes,
+                                            int cnt)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned int me = 1u << lane;
-    const float xh = g_.xh, yh = g_.yh, zh = g_.zh, eps2 = g_.eps2;
     const int part = lane & 3;
 #pragma unroll
     for (int it = 0; it < kStage / 8; ++it) {
@@ -327,6 +315,17 @@ __device__ __forceinline__ void box_batch(const WalkArgs& a, float* stage, const
         d[4] = v.z;
         d[6] = v.w;
     }
+}
+
+// Multipoles, lanes over targets: the sums {x, y}, {z, potential} of cnt <= 32 accepted
+// boxes (zeros outside their masks), staged two boxes side by side; nm counts them.
+template <bool kPhi>
+__device__ __forceinline__ void box_batch(const WalkArgs& a, float* stage, const int2* boxes, int cnt,
+                                          const LaneTarget& g_, int& nm, float2& fxy, float2& fzp)
+{
+    const unsigned int me = 1u << (threadIdx.x & 31);
+    const float xh = g_.xh, yh = g_.yh, zh = g_.zh, eps2 = g_.eps2;
+    stage_boxes(a, stage, boxes, cnt);
     __syncwarp();
     // With g = (R.R + eps^2)^-1/2, u = g^2, q = Q R / 2, y = D + 5 u q:
     //   E   = -g^3 [y + u q - (M + 3 u (T + y.R)) R]
@@ -703,164 +702,244 @@ k_walk_fp32c_split(WalkArgs a)
 
 // ---- The FP32C walk of ucp_grad_ke_electrons' forward runs: a chunk's targets visit
 // boxes in pre-order, one box per step in all lanes, and multipoles are summed box by
-// box, 32 visits to a compensated add.  Its forces agree with k_walk_fp32c's to about
-// 2e-8, but the gradient of an unresolved run amplifies such a difference to 1e-3 of
-// single components within 20 electron steps (close electron-ion encounters), and this
-// order of sums is the one whose gradients the library has always returned.  1.4
-// against 0.95 ms per walk over the electrons at N = 262,144, a tenth of a gradient.
-constexpr int kVisitThreads = 128;
-constexpr int kVisitList = 64;      // opened leaves buffered per warp
+// box, 32 visits to a compensated add; opened leaves wait in lists of 64.  Its forces
+// agree with k_walk_fp32c's to about 2e-8, but the gradient of an unresolved run
+// amplifies such a difference to 1e-3 of single components within 20 electron steps
+// (close electron-ion encounters), and this order of sums is the one whose gradients the
+// library has always returned.
+//
+// The traversal has its lanes over boxes, as walk_lists has, but opens one twig at a time:
+// a stack holds the boxes to come, tested when their parent was opened, first on top; a
+// step lists the visits up to the next opened twig and tests that twig's children.  After
+// every 32 visits the round's leaves are summed as in k_walk_fp32c, then its accepted
+// boxes, two to a packed operation but added one after the other.  With one box tested
+// and evaluated per visit in all lanes the walk took 1.60 ms over the electrons at N =
+// 262,144; this one takes 1.1 ms, a gradient of 20 steps 98.6 ms for 114.1.
+//
+// kTwo: a second warp does the sums, a round behind the first.  Where chunks are few it
+// shortens the chain that such a walk waits for (20,000 particles: gradient 28.4 for
+// 30.6 ms); from 60,000 on (938 chunks) the warps are better used on chunks.
+constexpr int kVisitList = 64;      // opened leaves to a list
 constexpr int kVisitBatch = 32;     // visits summed in FP32 before a compensated add
+constexpr int kVisitRing = 256;     // leaves listed and not yet summed: < 64 + 2 (64 + 32)
+constexpr int visit_blocks(bool two) { return two ? 12 : 24; }   // per SM
+constexpr int kVisitStack = 7 * kMaxDepth + 8;
 
-__global__ void __launch_bounds__(kVisitThreads, 7)
+struct __align__(16) VisitShared {
+    float stage[kStage / 2 * kStageStride];
+    int2 box[2][kVisitBatch];       // {accepted box, mask} of a round
+    int2 ring[kVisitRing];          // {opened leaf, mask}
+    int2 leaf[32];
+    int4 stack[kVisitStack];        // visits to come
+    float test[16 * 12];            // of accept_mask, when stage is the other warp's
+    int boxes[2], leaves[2];        // of a round: its boxes, the end of its leaves
+    int last[2];
+    int item;
+};
+
+// The accepted boxes of a round, added to b in order: cnt <= 32 as box_batch stages them.
+// q is Q R / 2 and s6 = 6 u, exact doubles or halves of the terms of
+//   E = -g^3 (3 u Q R + D) + g^3 (3 u (5/2 u R.Q R + D.R - tr(Q)/2) + M) R.
+__device__ __forceinline__ void box_batch_in_order(const WalkArgs& a, float* stage,
+                                                   const int2* boxes, int cnt,
+                                                   const ChunkTarget& tg, float eps2, int& nm,
+                                                   float& bx, float& by, float& bz)
+{
+    const unsigned int me = 1u << (threadIdx.x & 31);
+    stage_boxes(a, stage, boxes, cnt);
+    __syncwarp();
+    const float2 x2 = splat(tg.xh), y2 = splat(tg.yh), z2 = splat(tg.zh), e2 = splat(eps2);
+    const int pairs = (cnt + 1) >> 1;
+#pragma unroll 2
+    for (int p = 0; p < pairs; ++p) {
+        const float4* P = reinterpret_cast<const float4*>(stage + p * kStageStride);
+        const float4 f0 = P[0], f1 = P[1], f2 = P[2], f3 = P[3], f4 = P[4], f5 = P[5], f6 = P[6],
+                     f7 = P[7];
+        const float2 rx = __fadd2_rn(x2, make_float2(f0.x, f0.y));
+        const float2 ry = __fadd2_rn(y2, make_float2(f0.z, f0.w));
+        const float2 rz = __fadd2_rn(z2, make_float2(f1.x, f1.y));
+        const float2 d2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+        const float2 r2 = __fadd2_rn(d2, e2);
+        const bool in0 = (__float_as_int(f7.z) & me) != 0;
+        const bool in1 = (__float_as_int(f7.w) & me) != 0;
+        const float2 g = make_float2(in0 ? rsqrt_ftz(r2.x) : 0.f, in1 ? rsqrt_ftz(r2.y) : 0.f);
+        nm += in0;
+        nm += in1;
+        const float2 u = __fmul2_rn(g, g);
+        const float2 g3 = __fmul2_rn(g, u);
+        const float2 qxx = make_float2(f4.x, f4.y), qxy = make_float2(f4.z, f4.w),
+                     qxz = make_float2(f5.x, f5.y), qyy = make_float2(f5.z, f5.w),
+                     qyz = make_float2(f6.x, f6.y), qzz = make_float2(f6.z, f6.w);
+        const float2 qx = __ffma2_rn(qxx, rx, __ffma2_rn(qxy, ry, __fmul2_rn(qxz, rz)));
+        const float2 qy = __ffma2_rn(qxy, rx, __ffma2_rn(qyy, ry, __fmul2_rn(qyz, rz)));
+        const float2 qz = __ffma2_rn(qxz, rx, __ffma2_rn(qyz, ry, __fmul2_rn(qzz, rz)));
+        const float2 rqr = __ffma2_rn(rx, qx, __ffma2_rn(ry, qy, __fmul2_rn(rz, qz)));
+        const float2 dx = make_float2(f2.x, f2.y), dy = make_float2(f2.z, f2.w),
+                     dz = make_float2(f3.x, f3.y);
+        const float2 w = __ffma2_rn(dx, rx, __ffma2_rn(dy, ry, __ffma2_rn(dz, rz,
+                                    make_float2(f3.z, f3.w))));
+        const float2 s3 = __fmul2_rn(splat(3.f), u), s6 = __fadd2_rn(s3, s3);
+        const float2 aa = __fmul2_rn(g3, __ffma2_rn(s3, __ffma2_rn(splat(5.f), __fmul2_rn(u, rqr), w),
+                                                    make_float2(f1.z, f1.w)));
+        const float2 ex = __ffma2_rn(s6, qx, dx), ey = __ffma2_rn(s6, qy, dy),
+                     ez = __ffma2_rn(s6, qz, dz);
+        bx = fmaf(-g3.x, ex.x, fmaf(aa.x, rx.x, bx));
+        by = fmaf(-g3.x, ey.x, fmaf(aa.x, ry.x, by));
+        bz = fmaf(-g3.x, ez.x, fmaf(aa.x, rz.x, bz));
+        bx = fmaf(-g3.y, ex.y, fmaf(aa.y, rx.y, bx));
+        by = fmaf(-g3.y, ey.y, fmaf(aa.y, ry.y, by));
+        bz = fmaf(-g3.y, ez.y, fmaf(aa.y, rz.y, bz));
+    }
+    __syncwarp();
+}
+
+template <bool kTwo>
+__global__ void __launch_bounds__(kTwo ? 64 : 32, visit_blocks(kTwo))
 k_walk_fp32c_visits(WalkArgs a)
 {
     follow();
-    __shared__ int2 lists[kVisitThreads / 32][kVisitList];   // {opened leaf, mask}
+    __shared__ __align__(16) VisitShared sh;
     const int lane = threadIdx.x & 31;
-    int2* lst = lists[threadIdx.x >> 5];
+    const unsigned int lt = (1u << lane) - 1u;
+    const bool traverses = threadIdx.x < 32, sums = !kTwo || threadIdx.x >= 32;
     const float4* __restrict__ H = a.t.hdr;
-    const float4* __restrict__ LO = a.t.lo;
-    const float4* __restrict__ S = a.src32;
     const float eps2 = (float)a.eps2;
 
-    for (int item = next_chunk(a.work, lane); item < a.nchunks;
-         item = next_chunk(a.work, lane)) {
+    while (true) {
+        if (threadIdx.x == 0) sh.item = atomicAdd(a.work, 1);
+        __syncthreads();
+        const int item = sh.item;
+        if (item >= a.nchunks) break;
         const long long began = clock64();
         const int chunk = a.ord.order[item];
         const int4 ck = a.chunks[chunk];
         const int t = lane < ck.y ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
-        const bool valid = t >= 0;
-        const int root = a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0];
-        const int end = __float_as_int(LO[root].w);
-        float xh = 0.f, yh = 0.f, zh = 0.f, xl = 0.f, yl = 0.f, zl = 0.f;
-        if (valid) {
-            const double* cc = a.cubes[ck.z].c;
-            const double X = a.x[t] - cc[0], Y = a.y[t] - cc[1], Z = a.z[t] - cc[2];
-            xh = (float)X; yh = (float)Y; zh = (float)Z;
-            xl = (float)(X - (double)xh); yl = (float)(Y - (double)yh); zl = (float)(Z - (double)zh);
-        }
-        const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
-        const float wa = fmaf(0.5f, bt, 4e-6f), wb = 0.5f * bt;   // see walk_lists
-        float sx = 0.f, sy = 0.f, sz = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
-        float bx = 0.f, by = 0.f, bz = 0.f;
-        int np = 0, nm = 0, vis = 0, npl = 0;
-        int skip = valid ? 0 : 0x7fffffff;
-
-        auto fold = [&]() {
-            two_sum_acc(sx, cx, bx);
-            two_sum_acc(sy, cy, by);
-            two_sum_acc(sz, cz, bz);
-            bx = by = bz = 0.f;
-        };
-        auto flush = [&]() {
-            __syncwarp();
-            for (int e = 0; e < npl; ++e) {
-                if (!(((unsigned int)lst[e].y >> lane) & 1u)) continue;
-                const int nd = lst[e].x;
-                const float4 A = H[nd], B = LO[nd];
-                const float rx = (xh + A.x) + (xl + B.x), ry = (yh + A.y) + (yl + B.y),
-                            rz = (zh + A.z) + (zl + B.z);
-                const int jb = __ldg(&a.t.info[nd].x), je = __ldg(&a.t.info[nd].y);
-                const float4* F = S + src_place(jb, nd);
-                const float2 rx2 = splat(rx), ry2 = splat(ry), rz2 = splat(rz), e2 = splat(eps2);
-                float2 px = splat(0.f), py = px, pz = px;
-#pragma unroll 2
-                for (int j = jb & ~1; j < je; j += 2, F += 2) {
-                    const float4 P = __ldg(F), Q = __ldg(F + 1);
-                    const float2 dx = __fadd2_rn(rx2, make_float2(P.x, P.y));
-                    const float2 dy = __fadd2_rn(ry2, make_float2(P.z, P.w));
-                    const float2 dz = __fadd2_rn(rz2, make_float2(Q.x, Q.y));
-                    const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-                    const float2 ri = make_float2(j != t ? rsqrt_ftz(r2.x) : 0.f,
-                                                  j + 1 != t ? rsqrt_ftz(r2.y) : 0.f);
-                    const float2 qi = __fmul2_rn(make_float2(Q.z, Q.w), ri);
-                    const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
-                    px = __ffma2_rn(qr3, dx, px);
-                    py = __ffma2_rn(qr3, dy, py);
-                    pz = __ffma2_rn(qr3, dz, pz);
+        const ChunkTarget tg(a, t, ck.z);
+        float2 sxy = splat(0.f), sz0 = sxy, cxy = sxy, cz0 = sxy;
+        int np = 0, nm = 0, done = 0;
+        // a round: its leaves, then its boxes
+        auto sum_round = [&](int r) {
+            const int cnt = sh.boxes[r], upto = sh.leaves[r];
+            if (done < upto) {
+                LaneTarget lt;
+                lt.t = t;
+                lt.tmin = __shfl_sync(0xffffffffu, t, 0);
+                lt.tmax = __shfl_sync(0xffffffffu, t, ck.y - 1);
+                lt.xh = tg.xh; lt.yh = tg.yh; lt.zh = tg.zh;
+                lt.xl = tg.xl; lt.yl = tg.yl; lt.zl = tg.zl;
+                lt.q = lt.inv_lambda = 0.f;
+                lt.eps2 = eps2;
+                while (done < upto) {
+                    const int m = min(32, upto - done);
+                    if (lane < m) sh.leaf[lane] = sh.ring[(done + lane) & (kVisitRing - 1)];
+                    __syncwarp();
+                    leaf_batch<false, false>(a, sh.stage, sh.leaf, m, lt, np,
+                                             [&](int, const float2 fxy, const float2 fzp) {
+                                                 two_sum_acc2(sxy, cxy, fxy);
+                                                 two_sum_acc2(sz0, cz0, fzp);
+                                             });
+                    done += m;
                 }
-                np += (je - jb) - ((t >= jb && t < je) ? 1 : 0);
-                two_sum_acc(sx, cx, px.x + px.y);
-                two_sum_acc(sy, cy, py.x + py.y);
-                two_sum_acc(sz, cz, pz.x + pz.y);
             }
-            npl = 0;
-            __syncwarp();
+            float bx = 0.f, by = 0.f, bz = 0.f;
+            if (cnt) box_batch_in_order(a, sh.stage, sh.box[r], cnt, tg, eps2, nm, bx, by, bz);
+            two_sum_acc2(sxy, cxy, make_float2(bx, by));
+            two_sum_acc2(sz0, cz0, make_float2(bz, 0.f));
         };
-
-        int node = root;
-        while (node < end) {
-            const float4 A = H[node], B = LO[node];
-            const float4* r = a.t.rec + (size_t)node * kRec;
-            const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
-            const int nxt = __float_as_int(B.w);
-            const bool leaf = __float_as_int(A.w) < 0;
-            const bool active = node >= skip;
-            const float rx = xh + A.x, ry = yh + A.y, rz = zh + A.z;
-            const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            const float dm = d2 - fabsf(A.w);
-            bool acc = active && dm > 0.f;
-            if (active && fabsf(dm) <= fmaf(wa, d2, wb))
-                acc = accepts_fp64(a.t.mom + (size_t)node * kMom, a.x + t, a.y + t, a.z + t);
-            const unsigned int om = __ballot_sync(0xffffffffu, active && !acc);
-            int next = nxt;
-            if (om) {
-                if (leaf) {
-                    if (lane == 0) lst[npl] = make_int2(node, (int)om);
-                    ++npl;
+        // the two warps meet once per round
+        auto meet = [] { asm volatile("bar.sync 1, 64;" ::: "memory"); };
+        if (traverses) {
+            int vis = 0, r = 0, nb = 0, listed = 0, given = 0;   // leaves listed, given on
+            auto close = [&](bool last) {
+                if (lane == 0) {
+                    sh.boxes[r] = nb;
+                    sh.leaves[r] = given;
+                    sh.last[r] = last;
+                }
+                nb = 0;
+                if (kTwo) {
+                    meet();
+                    r ^= 1;
                 } else {
-                    if (acc) skip = nxt;
-                    next = node + 1;
+                    __syncwarp();
+                    sum_round(0);
+                    __syncwarp();
                 }
+            };
+            // lists the visits of lanes [from, to) of a window, in order; ends: the last of
+            // them is the last of its round
+            auto list = [&](const int4 e, int from, int to, bool ends) {
+                const bool mine = lane >= from && lane < to;
+                const unsigned int am = __ballot_sync(0xffffffffu, mine && e.y != 0);
+                if (mine && e.y) sh.box[r][nb + __popc(am & lt)] = make_int2(e.x, e.y);
+                nb += __popc(am);
+                const unsigned int ol = __ballot_sync(0xffffffffu, mine && e.z != 0 && e.w != 0);
+                if (mine && e.z && e.w)
+                    sh.ring[(listed + __popc(ol & lt)) & (kVisitRing - 1)] = make_int2(e.x, e.z);
+                listed += __popc(ol);
+                // a full list is summed before the boxes of the visit after its last leaf
+                const bool full = listed - given >= kVisitList;
+                const bool late = full && ends && listed - given == kVisitList && (ol >> (to - 1) & 1u);
+                if (full && !late) given += kVisitList;
+                if (ends) close(false);
+                if (late) given += kVisitList;
+            };
+            int top = 0;
+            int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0] : -1;
+            unsigned int mask = __ballot_sync(0xffffffffu, t >= 0);
+            while (true) {
+                // the boxes that follow, first on top: {box, accepting, opening targets, leaf}
+                const float4 h = box >= 0 ? __ldg(H + box) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const unsigned int am = accept_mask(a, sh.test, tg, box, mask, h);
+                const unsigned int follow_up = __ballot_sync(0xffffffffu, box >= 0);
+                if (box >= 0)
+                    sh.stack[top + __popc(follow_up & ~lt) - 1] =
+                        make_int4(box, (int)am, (int)(mask & ~am), __float_as_int(h.w) < 0);
+                top += __popc(follow_up);
+                __syncwarp();
+                // visits up to the next opened twig
+                int4 e;
+                unsigned int twigs;
+                int n;
+                do {
+                    const int cnt = min(top, 32);
+                    e = lane < cnt ? sh.stack[top - 1 - lane] : make_int4(-1, 0, 0, 0);
+                    twigs = __ballot_sync(0xffffffffu, e.z != 0 && e.w == 0);
+                    n = twigs ? __ffs(twigs) : cnt;
+                    const int room = kVisitBatch - (vis & (kVisitBatch - 1));
+                    list(e, 0, min(n, room), n >= room);
+                    if (n > room) list(e, room, n, false);
+                    vis += n;
+                    top -= n;
+                } while (!twigs && top > 0);
+                if (!twigs) break;
+                const int twig = __shfl_sync(0xffffffffu, e.x, n - 1);
+                mask = (unsigned int)__shfl_sync(0xffffffffu, e.z, n - 1);
+                __syncwarp();
+                box = lane < 8 ? __ldg(a.t.child8 + (size_t)twig * 8 + lane) : -1;
+                if (box <= twig) box = -1;      // a child comes after its parent: the walk ends
             }
-            if (acc) {
-                const float g = rsqrt_ftz(d2 + eps2);
-                const float u = g * g, g3 = g * u;
-                const float Qxx = 2.f * r2.x, Qxy = 2.f * r2.y, Qxz = 2.f * r2.z, Qyy = 2.f * r2.w,
-                            Qyz = 2.f * r3.x, Qzz = 2.f * r3.y;
-                const float QRx = fmaf(Qxx, rx, fmaf(Qxy, ry, Qxz * rz));
-                const float QRy = fmaf(Qxy, rx, fmaf(Qyy, ry, Qyz * rz));
-                const float QRz = fmaf(Qxz, rx, fmaf(Qyz, ry, Qzz * rz));
-                const float RQR = fmaf(rx, QRx, fmaf(ry, QRy, rz * QRz));
-                const float w = fmaf(r1.x, rx, fmaf(r1.y, ry, fmaf(r1.z, rz, r1.w)));
-                const float h = u * RQR, s3 = 3.f * u;
-                const float aa = g3 * fmaf(s3, fmaf(2.5f, h, w), r0.w);
-                const float mg3 = -g3;
-                bx = fmaf(mg3, fmaf(s3, QRx, r1.x), fmaf(aa, rx, bx));
-                by = fmaf(mg3, fmaf(s3, QRy, r1.y), fmaf(aa, ry, by));
-                bz = fmaf(mg3, fmaf(s3, QRz, r1.z), fmaf(aa, rz, bz));
-                ++nm;
+            given = listed;
+            close(true);
+        } else {
+            int r = 0;
+            bool last = false;
+            while (!last) {
+                meet();
+                last = sh.last[r];
+                sum_round(r);
+                r ^= 1;
             }
-            if ((++vis & (kVisitBatch - 1)) == 0) fold();
-            node = next;
-            if (npl == kVisitList) flush();
         }
-        flush();
-        fold();
-
-        if (valid) {
-            const int s = a.sp[t];
-            const double qm = a.msp[2 + s];
-            a.ax[t] = qm * ((double)sx + (double)cx);
-            a.ay[t] = qm * ((double)sy + (double)cy);
-            a.az[t] = qm * ((double)sz + (double)cz);
-            a.cnt_p2p[t] = np;
-            a.cnt_m2p[t] = nm;
+        if (sums) {
+            write_target<false>(a, t, sxy, cxy, sz0, cz0, np, nm);
+            if (lane == 0) {
+                const float cost = (float)(clock64() - began);
+                a.ord.cost[chunk] = cost;
+                atomicAdd(&a.ord.bins[cost_bin(cost)], 1);
+            }
         }
-        unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
-            sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
-        }
-        if (lane == 0) {
-            atomicAdd(&a.stats[0], sp2);
-            atomicAdd(&a.stats[1], sm2);
-            const float cost = (float)(clock64() - began);
-            a.ord.cost[chunk] = cost;
-            atomicAdd(&a.ord.bins[cost_bin(cost)], 1);
-        }
+        __syncthreads();
     }
 }
 
@@ -1040,9 +1119,12 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, Queue s, int shape)
 void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, Queue s)
 {
     count_launch(1);
-    const int wpb = kVisitThreads / 32;
-    const int b = walk_blocks(((int64_t)a.nchunks + wpb - 1) / wpb, nsm, 7);
-    launch(k_walk_fp32c_visits, b, kVisitThreads, s.whole(), a);
+    if (a.nchunks <= 4 * nsm)
+        launch(k_walk_fp32c_visits<true>, walk_blocks(a.nchunks, nsm, visit_blocks(true)), 64,
+               s.whole(), a);
+    else
+        launch(k_walk_fp32c_visits<false>, walk_blocks(a.nchunks, nsm, visit_blocks(false)), 32,
+               s.whole(), a);
 }
 
 }  // namespace ucp
