@@ -208,16 +208,18 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
     }
 }
 
-// ---- FP32 form (FP32C contexts): one warp per chunk of up to 32 targets, the
+// ---- FP32 form (FP32C contexts): one warp per group of up to 16 targets, the
 // traversal of the FP32C walk (the same decisions).  Both parts of the derivative
 // run with the lanes over the sources: 32 accepted boxes, or 32 particles of opened
-// leaves, one per lane, against the chunk's targets two at a time in packed FP32x2.
+// leaves, one per lane, against the group's targets two at a time in packed FP32x2.
 // A lane then holds its source's own sums (12 box terms, or 3 components) in
 // registers and adds them to memory once per batch; the targets' sums are three
 // values per target summed over the lanes by halving exchanges, four targets at a
 // time.  All terms are linear in the target's weight w = (q/m) lambda.  A pair's
 // separation is formed from the leaf's centroid and the particle's offset, as in the
 // forward walks.
+//
+// Groups are taken longest chunk first, by the costs that the forward walks noted.
 //
 // What bounds it: the FP32 pipe (63 % busy), by the box part's 113 packed operations
 // per box and pair of targets.  The form before took the lanes over targets and summed
@@ -271,18 +273,20 @@ __device__ __forceinline__ void red_add4(float* p, float x, float y, float z, fl
                  :: "l"(p), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
 }
 
+constexpr int kTargets = 16;
+
 struct __align__(16) AdjWarp {
     WalkWarp walk;
     // two targets: relative to the chunk's centre and weights {x, y}, {z, wx}, {wy, wz};
     // relative to the cube's centre as float pairs {xh, yh}, {zh, xl}, {yl, zl}
-    float4 tgt[16][6];
-    float mt[8][32];         // four targets' sums: lane L holds value L / 2
-    int slot[32];            // the targets' slots
+    float4 tgt[kTargets / 2][6];
+    float mt[kTargets / 4][32];         // four targets' sums: lane L holds value L / 2
+    int slot[kTargets];      // the targets' slots
 };
 
 __global__ void __launch_bounds__(32, 16)
-k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restrict__ mu,
-                   float* __restrict__ adj)
+k_walk_adjoint_f32(WalkArgs a, int group, const double* __restrict__ lam,
+                   double* __restrict__ mu, float* __restrict__ adj)
 {
     follow();
     __shared__ AdjWarp shared;
@@ -291,9 +295,14 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
     const float4* __restrict__ S = a.src32;
     const float2 e2 = splat((float)a.eps2);
 
-    for (int chunk = next_chunk(a.work, lane); chunk < a.nchunks;
-         chunk = next_chunk(a.work, lane)) {
-        const int4 ck = a.chunks[chunk];
+    const int per = 32 / group;
+    while (true) {
+        const unsigned int item = (unsigned int)next_chunk(a.work, lane);
+        if (item >= (unsigned int)a.nchunks * per) break;
+        int4 ck = a.chunks[a.ord.order[item / per]];
+        ck.x += (int)(item % per) * group;
+        ck.y = min(group, ck.y - (int)(item % per) * group);
+        if (ck.y <= 0) continue;
         const int t = lane < ck.y ? (a.targets ? a.targets[ck.x + lane] : ck.x + lane) : -1;
         const ChunkTarget tg(a, t, ck.z);
         {
@@ -304,22 +313,24 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
 #pragma unroll
                 for (int k = 0; k < 3; ++k) w[k] = (float)(qm * lam[3 * (size_t)t + k]);
             }
-            float* d = reinterpret_cast<float*>(W.tgt[lane >> 1]) + (lane & 1);
-            d[0] = (tg.xh - tg.gx) + tg.xl;
-            d[2] = (tg.yh - tg.gy) + tg.yl;
-            d[4] = (tg.zh - tg.gz) + tg.zl;
-            d[6] = w[0];
-            d[8] = w[1];
-            d[10] = w[2];
-            d[12] = tg.xh;
-            d[14] = tg.yh;
-            d[16] = tg.zh;
-            d[18] = tg.xl;
-            d[20] = tg.yl;
-            d[22] = tg.zl;
-            W.slot[lane] = t >= 0 ? t : 0x7fffffff;
+            if (lane < kTargets) {
+                float* d = reinterpret_cast<float*>(W.tgt[lane >> 1]) + (lane & 1);
+                d[0] = (tg.xh - tg.gx) + tg.xl;
+                d[2] = (tg.yh - tg.gy) + tg.yl;
+                d[4] = (tg.zh - tg.gz) + tg.zl;
+                d[6] = w[0];
+                d[8] = w[1];
+                d[10] = w[2];
+                d[12] = tg.xh;
+                d[14] = tg.yh;
+                d[16] = tg.zh;
+                d[18] = tg.xl;
+                d[20] = tg.yl;
+                d[22] = tg.zl;
+                W.slot[lane] = t >= 0 ? t : 0x7fffffff;
+            }
 #pragma unroll
-            for (int g = 0; g < 8; ++g) W.mt[g][lane] = 0.f;
+            for (int g = 0; g < kTargets / 4; ++g) W.mt[g][lane] = 0.f;
             __syncwarp();
         }
         const int groups = (ck.y + 3) >> 2;
@@ -447,7 +458,7 @@ k_walk_adjoint_f32(WalkArgs a, const double* __restrict__ lam, double* __restric
                     // the particle's own place among the targets, if it has one
                     int pos = 0;
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1)
+                    for (int o = kTargets / 2; o > 0; o >>= 1)
                         if (W.slot[pos + o - 1] < j) pos += o;
                     if (W.slot[pos] == j) mask &= ~(1u << pos);
                 }
@@ -714,12 +725,16 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
     count_launch(3);
     cudaMemsetAsync(mu, 0, sizeof(double) * 3 * (size_t)n, s);
     if (a.src32) {
-        int blocks = nsm * 16 < a.nchunks ? nsm * 16 : a.nchunks;
-        if (blocks < 1) blocks = 1;
+        // 16 targets to a warp, fewer where chunks are few.  A gradient of 20 steps with 4,
+        // 8 and 16: 13.4 14.0 15.2 ms at 4000 particles (63 and 125 chunks), 33.4 (8) 34.5
+        // at 40,000, 52.5 51.8 at 120,000 (1875 and 3750)
+        const int group = a.nchunks < nsm ? 4 : a.nchunks < 10 * nsm ? 8 : kTargets;
+        const int64_t items = (int64_t)a.nchunks * (32 / group);
+        const int blocks = items < 1 ? 1 : items < 16 * nsm ? (int)items : 16 * nsm;
         // FP32C context: FP32 walk, FP32 box accumulators (in the same buffer)
         float* adjf = reinterpret_cast<float*>(adj);
         launch(k_zero_adj<float>, 2 * 152, 256, s, a.t.nnodes, adjf);
-        launch(k_walk_adjoint_f32, blocks, 32, s.whole(), a, lam, mu, adjf);
+        launch(k_walk_adjoint_f32, blocks, 32, s.whole(), a, group, lam, mu, adjf);
         launch(k_adjoint_push<float>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
     } else {
         launch(k_zero_adj<double>, 2 * 152, 256, s, a.t.nnodes, adj);

@@ -1123,11 +1123,13 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
                 a.ntargets = c->n_e;
                 a.chunks = c->chunks_e;
                 a.nchunks = c->n_chunks_e;
+                a.ord.order = c->order_e;
             } else {
                 a.targets = nullptr;
                 a.ntargets = c->n;
                 a.chunks = c->chunks_all;
                 a.nchunks = c->n_chunks_all;
+                a.ord.order = c->order_all;
             }
             a.pos_off = c->pos_off;
             a.cubes = c->cube;
@@ -1194,6 +1196,7 @@ int ucp_accel_vjp(ucp_ctx* c, double theta, double eps, const double* lam_in, do
     a.ntargets = c->n;
     a.chunks = c->chunks_all;
     a.nchunks = c->n_chunks_all;
+    a.ord.order = c->order_all;
     a.pos_off = c->pos_off;
     a.cubes = c->cube;
     a.eps2 = eps * eps;
