@@ -305,12 +305,12 @@ void launch_select(const int8_t* sp, int species, int n, int* list, int* partial
                    int* cnt1, Queue s);
 void launch_drift(double* x, double* y, double* z, const double* vx, const double* vy,
                   const double* vz, double dt, int n, Queue s);
+// out[6 c ..]: observables of cloud c (cloud_start NULL: one cloud over [0, n)); partials
+// holds 6 n_clouds nblk doubles
 void launch_energy(const double* vx, const double* vy, const double* vz, const double* phi,
                    const int8_t* sp, const double* qsp, const double* msp, int n,
-                   double* partials, int nblk, double* out6, Queue s);
-void launch_energy_clouds(const double* vx, const double* vy, const double* vz, const double* phi,
-                          const int8_t* sp, const double* qsp, const double* msp,
-                          const int* cloud_start, int n_clouds, double* out, Queue s);
+                   const int* cloud_start, int n_clouds, double* partials, int nblk, double* out,
+                   Queue s);
 void launch_scatter3(const double* ax, const double* ay, const double* az, const unsigned int* id,
                      int n, double* out, Queue s);
 void launch_scatter1(const double* a, const unsigned int* id, int n, double* out, Queue s);

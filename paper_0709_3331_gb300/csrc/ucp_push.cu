@@ -47,15 +47,20 @@ __global__ void k_drift(double* __restrict__ x, double* __restrict__ y, double* 
 
 // Deterministic two-level reduction: fixed per-thread strides, fixed tree in
 // the block, partials summed in block order by one thread.
-// out6 = {KE_ion, KE_electron, PE, px, py, pz}
+// out[6 c ..] = {KE_ion, KE_electron, PE, px, py, pz} of cloud c = blockIdx.y (cloud_start
+// NULL: of everything).
 __global__ void k_energy_partial(const double* __restrict__ vx, const double* __restrict__ vy,
                                  const double* __restrict__ vz, const double* __restrict__ phi,
                                  const int8_t* __restrict__ sp, const double* __restrict__ qsp,
-                                 const double* __restrict__ msp, int n, double* __restrict__ part)
+                                 const double* __restrict__ msp, int n,
+                                 const int* __restrict__ cloud_start, double* __restrict__ part)
 {
     follow();
+    const int c = blockIdx.y, end = cloud_start ? cloud_start[c + 1] : n;
+    part += (size_t)c * gridDim.x * 6;
     double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = (cloud_start ? cloud_start[c] : 0) + blockIdx.x * blockDim.x + threadIdx.x; i < end;
+         i += gridDim.x * blockDim.x) {
         int s = sp[i];
         double m = msp[s];
         double ux = vx[i], uy = vy[i], uz = vz[i];
@@ -78,38 +83,6 @@ __global__ void k_energy_partial(const double* __restrict__ vx, const double* __
         for (int k = 0; k < 6; ++k) part[blockIdx.x * 6 + k] = sh[0][k];
 }
 
-// Per-cloud observables, one block per cloud over its segment (fixed order):
-// out[6 c ..] = {KE_ion, KE_electron, PE, px, py, pz}
-__global__ void k_energy_clouds(const double* __restrict__ vx, const double* __restrict__ vy,
-                                const double* __restrict__ vz, const double* __restrict__ phi,
-                                const int8_t* __restrict__ sp, const double* __restrict__ qsp,
-                                const double* __restrict__ msp, const int* __restrict__ cloud_start,
-                                double* __restrict__ out)
-{
-    follow();
-    const int c = blockIdx.x;
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int i = cloud_start[c] + threadIdx.x; i < cloud_start[c + 1]; i += blockDim.x) {
-        int s = sp[i];
-        double m = msp[s];
-        double ux = vx[i], uy = vy[i], uz = vz[i];
-        acc[s] += 0.5 * m * (ux * ux + uy * uy + uz * uz);
-        acc[2] += 0.5 * qsp[s] * phi[i];
-        acc[3] += m * ux;
-        acc[4] += m * uy;
-        acc[5] += m * uz;
-    }
-    __shared__ double sh[kT][6];
-    for (int k = 0; k < 6; ++k) sh[threadIdx.x][k] = acc[k];
-    __syncthreads();
-    for (int st = kT / 2; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st)
-            for (int k = 0; k < 6; ++k) sh[threadIdx.x][k] += sh[threadIdx.x + st][k];
-        __syncthreads();
-    }
-    if (threadIdx.x < 6) out[6 * c + threadIdx.x] = sh[0][threadIdx.x];
-}
-
 // Six warps, one per observable: lane l adds partials l, l + 32, ..., then the
 // lanes are added by a fixed butterfly (a deterministic order).
 __global__ void __launch_bounds__(192)
@@ -117,11 +90,12 @@ k_energy_final(const double* __restrict__ part, int nblk, double* __restrict__ o
 {
     follow();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    part += (size_t)blockIdx.x * nblk * 6;
     double acc = 0.0;
     for (int b = lane; b < nblk; b += 32) acc += part[6 * b + k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) out[k] = acc;
+    if (lane == 0) out[6 * blockIdx.x + k] = acc;
 }
 
 __global__ void k_scatter3(const double* __restrict__ ax, const double* __restrict__ ay,
@@ -246,19 +220,13 @@ void launch_drift(double* x, double* y, double* z, const double* vx, const doubl
 
 void launch_energy(const double* vx, const double* vy, const double* vz, const double* phi,
                    const int8_t* sp, const double* qsp, const double* msp, int n,
-                   double* partials, int nblk, double* out6, Queue s)
+                   const int* cloud_start, int n_clouds, double* partials, int nblk, double* out,
+                   Queue s)
 {
     count_launch(2);
-    launch(k_energy_partial, nblk, kT, s, vx, vy, vz, phi, sp, qsp, msp, n, partials);
-    launch(k_energy_final, 1, 192, s, partials, nblk, out6);
-}
-
-void launch_energy_clouds(const double* vx, const double* vy, const double* vz, const double* phi,
-                          const int8_t* sp, const double* qsp, const double* msp,
-                          const int* cloud_start, int n_clouds, double* out, Queue s)
-{
-    count_launch(1);
-    launch(k_energy_clouds, n_clouds, kT, s, vx, vy, vz, phi, sp, qsp, msp, cloud_start, out);
+    launch(k_energy_partial, dim3(nblk, n_clouds), kT, s, vx, vy, vz, phi, sp, qsp, msp, n,
+           cloud_start, partials);
+    launch(k_energy_final, n_clouds, 192, s, partials, nblk, out);
 }
 
 void launch_scatter3(const double* ax, const double* ay, const double* az, const unsigned int* id,

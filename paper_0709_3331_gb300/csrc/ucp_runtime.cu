@@ -544,11 +544,14 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
         if (c->bbox_nblk > lim) c->bbox_nblk = lim;
         if (c->bbox_nblk < 1) c->bbox_nblk = 1;
     }
-    c->en_nblk = (int)((n + 2047) / 2048);
-    if (c->en_nblk > 4 * c->nsm) c->en_nblk = 4 * c->nsm;
+    // per cloud: a block for every 2048 particles of the largest (an ensemble's 65,536: 32;
+    // with one block to a cloud its energy took 319 us)
+    c->en_nblk = (int)((*std::max_element(sizes, sizes + n_clouds) + 2047) / 2048);
+    const int en_lim = n_clouds > 1 ? 32 : 4 * c->nsm;
+    if (c->en_nblk > en_lim) c->en_nblk = en_lim;
     if (c->en_nblk < 1) c->en_nblk = 1;
     dalloc(c, &c->bbox_part, (size_t)n_clouds * c->bbox_nblk * 6);
-    dalloc(c, &c->en_part, (size_t)c->en_nblk * 6);
+    dalloc(c, &c->en_part, (size_t)n_clouds * c->en_nblk * 6);
     dalloc(c, &c->en_out, (size_t)6 * n_clouds);
     // clouds: segment starts, the (static) cloud of every slot, walk chunk capacity
     dalloc(c, &c->cloud_start, (size_t)n_clouds + 1);
@@ -1228,14 +1231,13 @@ int ucp_energy(ucp_ctx* c, double theta, double eps, double out[6])
         return rc;
     int k = c->cur;
     double r[6] = {0, 0, 0, 0, 0, 0};
+    launch_energy(c->st[k][3], c->st[k][4], c->st[k][5], c->phi, c->sp[k], c->qsp, c->msp, c->n,
+                  c->n_clouds > 1 ? c->cloud_start : nullptr, c->n_clouds, c->en_part, c->en_nblk,
+                  c->en_out, c->s);
     if (c->n_clouds == 1) {
-        launch_energy(c->st[k][3], c->st[k][4], c->st[k][5], c->phi, c->sp[k], c->qsp, c->msp,
-                      c->n, c->en_part, c->en_nblk, c->en_out, c->s);
         CK(cudaMemcpyAsync(r, c->en_out, sizeof(r), cudaMemcpyDeviceToHost, c->s));
         CK(cudaStreamSynchronize(c->s));
     } else {
-        launch_energy_clouds(c->st[k][3], c->st[k][4], c->st[k][5], c->phi, c->sp[k], c->qsp,
-                             c->msp, c->cloud_start, c->n_clouds, c->en_out, c->s);
         std::vector<double> per(6 * (size_t)c->n_clouds);
         CK(cudaMemcpyAsync(per.data(), c->en_out, sizeof(double) * per.size(),
                            cudaMemcpyDeviceToHost, c->s));
