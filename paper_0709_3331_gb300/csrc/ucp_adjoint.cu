@@ -49,7 +49,7 @@ __device__ __forceinline__ double dot3(const double* a, const double* b)
 // 68 %); groups get smaller when eight would leave SMs without work.  The form
 // before summed each box's 12 values and each pair's three over the warp in FP64
 // (75 and 15 additions): accelerations and their vector-Jacobian product at N = 4,096
-// took 15.9 ms against 2.0.
+// took 15.9 ms, now 1.55.
 constexpr int kAdjGroup = 8;
 
 struct __align__(16) AdjWarp64 {
@@ -221,11 +221,11 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
 //
 // Groups are taken longest chunk first, by the costs that the forward walks noted.
 //
-// What bounds it: the FP32 pipe (63 % busy), by the box part's 113 packed operations
+// What bounds it: the FP32 pipe (61 % busy), by the box part's 113 packed operations
 // per box and pair of targets.  The form before took the lanes over targets and summed
 // each box's 12 values over the warp (70 instructions beside 110 of arithmetic,
 // unpacked) and each pair's three: 6.1 ms over every particle at N = 262,144 against
-// 3.1, over the electrons 4.1 against 1.95.
+// 2.9, over the electrons 4.1 against 1.65 (whole chunks in list order: 3.1 and 1.95).
 
 // Warp sums of 16 values by halving exchanges: at each xor step a lane keeps half of
 // its values and adds the partner's copy of that half, so 16 values take 16

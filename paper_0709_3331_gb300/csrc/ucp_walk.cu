@@ -40,9 +40,9 @@ __device__ __forceinline__ void two_sum_acc2(float2& s, float2& c, float2 v)
 // however many of its lanes are active (2 multiply-adds per clock and SM).  One
 // target per warp keeps all lanes at work in both lists (of 32 targets in a warp
 // 65 % took part in a multipole and 35 % in a direct pair) and the FP32 criterion
-// leaves the pipe to the interactions: a walk over N = 131,072 particles takes 13.8 ms
-// (31.0 with 32 targets per warp and the criterion in FP64), over 2,048 0.10 ms
-// (1.85).  A target's sums
+// leaves the pipe to the interactions: a walk over N = 131,072 particles takes 12.7 ms
+// (31.0 with 32 targets per warp, the criterion in FP64 and the library's root), over
+// 2,048 0.10 ms (1.85).  A target's sums
 // are over its own boxes and sources in an order set by the tree alone, so they do
 // not depend on the launch.
 //
@@ -505,12 +505,12 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
 // What bounds it (N = 524,288, theta 0.5, leaves of 32, no potential): per chunk
 // 1,950 children tested in about 70 steps, 1,775 boxes evaluated (68 % of the lanes
 // take part, the others accepted an ancestor) and 162 leaves of 11 sources summed
-// (44 %); of the 2.5 ms of a walk over every particle the multipoles take 1.45 (the
-// FP32 pipe: an FFMA2 holds it for two cycles), the pairs 0.8 and the traversal
-// 0.4.  The form before, a depth-first walk that tested one box per visit in all
-// lanes and evaluated it one box at a time, took 3.75 ms (1.27e5 against 1.81e5 warp
-// instructions per chunk); with the potential 2.7 against 4.1 ms, over the electrons
-// 1.5 against 2.25 ms.  Blocks of one warp keep the shared arrays at constant
+// (44 %); of the 2.28 ms of a walk over every particle the multipoles take 1.1 (the
+// FP32 pipe: an FFMA2 holds it for two cycles; 61 % busy over the whole walk), the pairs
+// 0.7 and the traversal 0.4.  A depth-first walk that tested one box per visit in all
+// lanes and evaluated it one box at a time took 3.75 ms (1.81e5 against 1.12e5 warp
+// instructions per chunk); with the potential 4.1 against 2.45 ms, over the electrons
+// 2.25 against 1.38.  Blocks of one warp keep the shared arrays at constant
 // addresses: 8 % faster than blocks of two to eight warps at the same occupancy.
 //
 // kThreads threads per block (one warp), register budget for kBlocks resident blocks
