@@ -49,7 +49,7 @@ __device__ __forceinline__ double dot3(const double* a, const double* b)
 // 68 %); groups get smaller when eight would leave SMs without work.  The form
 // before summed each box's 12 values and each pair's three over the warp in FP64
 // (75 and 15 additions): accelerations and their vector-Jacobian product at N = 4,096
-// took 15.9 ms, now 1.55.
+// took 15.9 ms, now 1.47.
 constexpr int kAdjGroup = 8;
 
 struct __align__(16) AdjWarp64 {
@@ -525,6 +525,9 @@ k_walk_adjoint_f32(WalkArgs a, int group, const double* __restrict__ lam,
 
 // Every particle of a leaf receives the source-side terms of the leaf and of
 // all its ancestors: q_s (sum alpha - sum Gamma (x_s - c)) + |q_s| sum kappa / S0.
+// One thread per leaf, in blocks of one warp: the FP64 pipe bounds it (55 operations per
+// leaf and ancestor, 25 per particle), and so its few warps spread evenly over the SMs (a
+// gradient of 20 steps at 20,000 particles 22.7 -> 22.0 ms against blocks of eight warps).
 template <class TA>
 __global__ void k_adjoint_push(const double* __restrict__ x, const double* __restrict__ y,
                                const double* __restrict__ z, const int8_t* __restrict__ sp,
@@ -537,7 +540,8 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
          leaf += gridDim.x * blockDim.x) {
         if (!(t.depth_leaf[leaf] & 256)) continue;
         double A[3] = {0, 0, 0}, G[6] = {0, 0, 0, 0, 0, 0}, Cc[3] = {0, 0, 0}, K[3] = {0, 0, 0};
-        for (int nd = leaf; nd >= 0; nd = t.info[nd].w) {
+        for (int nd = leaf, up; nd >= 0; nd = up) {
+            up = t.info[nd].w;
             double r[12];
             for (int k = 0; k < 12; ++k) r[k] = (double)adj[(size_t)nd * 12 + k];
             const double* m = t.mom + (size_t)nd * kMom;
@@ -735,7 +739,7 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
         float* adjf = reinterpret_cast<float*>(adj);
         launch(k_zero_adj<float>, 2 * 152, 256, s, a.t.nnodes, adjf);
         launch(k_walk_adjoint_f32, blocks, 32, s.whole(), a, group, lam, mu, adjf);
-        launch(k_adjoint_push<float>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
+        launch(k_adjoint_push<float>, 32 * 152, 32, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
     } else {
         launch(k_zero_adj<double>, 2 * 152, 256, s, a.t.nnodes, adj);
         // eight targets per warp, fewer while that leaves an SM with under four warps
@@ -744,7 +748,7 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
         const int64_t items = (int64_t)a.nchunks * (32 / group);
         const int blocks = items < 1 ? 1 : items < 12 * nsm ? (int)items : 12 * nsm;
         launch(k_walk_adjoint, blocks, 32, s.whole(), a, group, lam, mu, adj);
-        launch(k_adjoint_push<double>, 4 * 152, 256, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
+        launch(k_adjoint_push<double>, 32 * 152, 32, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
     }
 }
 

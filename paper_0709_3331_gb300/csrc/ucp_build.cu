@@ -675,7 +675,7 @@ __device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combin
         __syncwarp();
         const Twig up = load_twig(t, ready ? w.parent : -1);
         int4 lc;
-        if (ready) lc = __ldcg(&t.info[w.last]);
+        if (ready) lc = __ldcg(&t.info[max(w.last, 0)]);
         while (todo) {
             // the (lane / 8)-th of the lanes that are left
             unsigned int m = todo;

@@ -41,20 +41,18 @@ __device__ __forceinline__ float rsqrt_ftz(float x)
 extern std::atomic<unsigned long long> g_launches;
 inline void count_launch(int k) { g_launches.fetch_add((unsigned long long)k, std::memory_order_relaxed); }
 
-// The stream of a context's launches.  chained: each kernel is launched as a
-// programmatic dependent of the one before it, so that its blocks are placed while
-// that one drains (they wait in follow() until it has finished).  That takes 2-3 us
-// off each of the ~25 kernels of a substep, but costs the host about 3 us more per
-// launch: set where the host runs ahead of the GPU or is not involved (runs of several
-// substeps, the gradient, captured blocks), not for a single build and walk.
-// 11 substeps at N = 2048, FP64: 2.28 -> 2.05 ms; one chained force call at 4101
-// particles, FP32C, would take 0.41 ms for 0.35.
+// The stream of a context's launches.  chained: a kernel is launched as a programmatic
+// dependent of the one before it, so that its blocks are placed while that one drains
+// (they wait in follow() until it has finished): 1-2 us off each of the ~25 kernels of a
+// substep.  Force call at 8192 particles, FP32C, 244 -> 227 us; 11 substeps at N = 2048,
+// FP64, 2.28 -> 2.04 ms.
 struct Queue {
     cudaStream_t s = nullptr;
-    bool chained = false;
+    bool chained = true;
     operator cudaStream_t() const { return s; }
     // for the walks: their blocks, a few to every SM, would be dealt out unevenly around
-    // those of the kernel ahead (FP64 walk at N = 131,072: 7.2 -> 8.3 ms)
+    // those of the kernel ahead (FP64 walk at N = 131,072: 7.2 -> 8.3 ms; force call at
+    // 4099 particles, FP32C: 0.35 -> 0.41 ms)
     Queue whole() const { return {s, false}; }
 };
 

@@ -731,17 +731,6 @@ int ucp_tree_force(ucp_ctx* c, double theta, double eps, double* acc, double* ph
     return UCP_OK;
 }
 
-// Kernels launched while this lives are chained (Queue).
-struct Chained {
-    Queue& q;
-    const bool was;
-    Chained(Queue& queue, bool on) : q(queue), was(queue.chained) { q.chained = was || on; }
-    ~Chained() { q.chained = was; }
-};
-
-// From this many substeps in one call the host runs ahead of the GPU (Queue).
-constexpr int64_t kChainSubsteps = 4;
-
 // The split-step push; with store != NULL the positions after every electron
 // substep are written there in caller order (n x 3 doubles per substep).  gradient:
 // a forward run of the gradient, whose potential nobody reads.
@@ -749,7 +738,6 @@ static int run_blocks(ucp_ctx* c, double dt_e, int kk, int64_t nblocks, double t
                       double* store, bool gradient = false)
 {
     int rc;
-    const Chained chained(c->s, nblocks * kk >= kChainSubsteps);
     if (!c->acc_valid) {
         if (!c->tree_valid && (rc = build(c))) return rc;
         if ((rc = force(c, theta, eps, 0, false, gradient))) return rc;
@@ -810,7 +798,7 @@ static int run_block_graph(ucp_ctx* c, double dt_e, int kk, double theta, double
         const int cur0 = c->cur;
         const int64_t steps0 = c->steps, wt0 = c->walk_targets, wl0 = c->walk_launches;
         const Queue orig = c->s;
-        c->s = {c->cap_stream, true};
+        c->s.s = c->cap_stream;
         const unsigned long long l0 = g_launches.load();
         cudaGraph_t graph = nullptr;
         int rc = UCP_OK;
@@ -1060,7 +1048,6 @@ int ucp_grad_ke_electrons(ucp_ctx* c, double dt_e, int kk, int64_t n_steps, doub
         launch_scatter3(c->st[k][0], c->st[k][1], c->st[k][2], c->id[k], c->n, dst, c->s);
         launch_scatter3(c->st[k][3], c->st[k][4], c->st[k][5], c->id[k], c->n, dst + n3, c->s);
     };
-    const Chained chained(c->s, true);
     const double h_e = 0.5 * dt_e, h_i = 0.5 * (double)kk * dt_e;
     int64_t steps0 = c->steps;
     // forward, checkpoints at g = 0, C, 2C, ...; the last segment's positions are

@@ -1,6 +1,6 @@
-"""Runs of several substeps, whose kernels are launched as dependents of one another,
-against the same substeps one call at a time, whose kernels are not, and against captured
-blocks: the same state bit for bit, from one particle to several waves of blocks."""
+"""Runs of several substeps, whose kernels are launched as dependents of one another, against
+the same substeps one call at a time and against captured blocks: the same state bit for
+bit, from one particle to several waves of blocks."""
 import numpy as np
 import pytest
 
