@@ -36,81 +36,53 @@ __device__ __forceinline__ double dot3(const double* a, const double* b)
     return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// ---- FP64 form: one warp per group of up to kAdjGroup targets, the traversal of
-// the FP32C walk on the FP64 contexts' records (FP32 criterion, again in FP64 within
-// its window: the FP64 walk's decisions).  The lanes are the sources, 32 accepted
-// boxes or 32 particles of opened leaves, and every lane goes through the group's
-// targets, so a source's own sums stay in its registers and a target's partial sums
-// in shared memory, one per lane, until the end.  All terms are linear in the
+// ---- FP64 form: one warp per target, the traversal of the FP32C walk on the FP64
+// contexts' records (FP32 criterion, again in FP64 within its window: the FP64 walk's
+// decisions).  The lanes are the sources, 32 accepted boxes or 32 particles of opened
+// leaves.  A box's or source's own terms are added to memory as they come; the target's
+// partial sums stay in the lanes' registers until the end.  All terms are linear in the
 // target's weight w = (q/m) lambda.
 //
-// What bounds it: the FP64 pipe (about 120 operations per box and target, 16 cycles
-// per warp instruction).  Eight targets per warp keep 85 % of the lanes at work (32:
-// 68 %); groups get smaller when eight would leave SMs without work.  The form
-// before summed each box's 12 values and each pair's three over the warp in FP64
-// (75 and 15 additions): accelerations and their vector-Jacobian product at N = 4,096
-// took 15.9 ms, now 1.47.
-constexpr int kAdjGroup = 8;
-
-struct __align__(16) AdjWarp64 {
-    WalkWarp walk;
-    double mt[kAdjGroup][3][32];      // partial sums of the targets, per lane
-    double tgt[kAdjGroup][6];         // position and weight
-    int slot[kAdjGroup];
-};
-
-__global__ void __launch_bounds__(32, 12)
-k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __restrict__ mu,
+// What bounds it: the FP64 pipe (about 120 operations per box, 16 cycles per warp
+// instruction however many lanes are active) and the box terms' additions in memory.  One
+// target per warp keeps every lane at work and fills the SMs from a few hundred targets
+// on; eight targets per warp, with their sums in shared memory and a quarter of the
+// additions, left 15 % of the lanes idle: a vector-Jacobian product 870 against 543 us at
+// N = 4,096, 43.9 against 33.8 ms at 131,072.  Eight warps per SM are as fast as twelve and
+// 2 % faster at the smallest sizes.
+__global__ void __launch_bounds__(32, 8)
+k_walk_adjoint(WalkArgs a, const double* __restrict__ lam, double* __restrict__ mu,
                double* __restrict__ adj)
 {
     follow();
-    __shared__ AdjWarp64 shared;
-    AdjWarp64& W = shared;
+    __shared__ WalkWarp W;
     const int lane = threadIdx.x;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
-    const int per = 32 / group;       // groups per chunk
 
     while (true) {
         const unsigned int item = (unsigned int)next_chunk(a.work, lane);
-        if (item / per >= (unsigned int)a.nchunks) break;
-        const int4 ck = a.chunks[item / per];
-        const int skip = (int)(item % per) * group;
-        const int nt = min(group, ck.y - skip);
-        if (nt <= 0) continue;
-        const int ti = ck.x + skip + lane;
-        const int t = lane < nt ? (a.targets ? a.targets[ti] : ti) : -1;
-        const ChunkTarget tg(a, t, ck.z);
-        if (t >= 0) {
-            const int s = a.sp[t];
-            const double qm = a.msp[2 + s];
-            W.tgt[lane][0] = a.x[t];
-            W.tgt[lane][1] = a.y[t];
-            W.tgt[lane][2] = a.z[t];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) W.tgt[lane][3 + k] = qm * lam[3 * (size_t)t + k];
-            W.slot[lane] = t;
-        }
-        for (int g = 0; g < nt; ++g)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) W.mt[g][k][lane] = 0.0;
-        __syncwarp();
+        if (item / 32 >= (unsigned int)a.nchunks) break;
+        const int4 ck = a.chunks[item / 32];
+        if ((int)(item % 32) >= ck.y) continue;
+        const int ti = ck.x + (int)(item % 32);
+        const int t = a.targets ? a.targets[ti] : ti;
+        const ChunkTarget tg(a, lane == 0 ? t : -1, ck.z);
+        const double X[3] = {a.x[t], a.y[t], a.z[t]};
+        const double qm = a.msp[2 + a.sp[t]];
+        const double w[3] = {qm * lam[3 * (size_t)t], qm * lam[3 * (size_t)t + 1],
+                             qm * lam[3 * (size_t)t + 2]};
+        double mt[3] = {0.0, 0.0, 0.0};
 
         // The same terms as the FP32 form below: the target takes -H, the box alpha,
         // Gamma and kappa.
         auto multipoles = [&](const int2* boxes, int cnt) {
-            const int2 bm = lane < cnt ? boxes[lane] : make_int2(0, 0);
-            const unsigned int mask = (unsigned int)bm.y;
-            const double* m = a.t.mom + (size_t)bm.x * kMom;
-            const double c[3] = {m[MC], m[MC + 1], m[MC + 2]};
-            const double M = m[MM], D[3] = {m[MD], m[MD + 1], m[MD + 2]};
-            const double Q[6] = {m[MQ], m[MQ + 1], m[MQ + 2], m[MQ + 3], m[MQ + 4], m[MQ + 5]};
-            const double T = m[MT];                       // -tr(Q)/2
-            double al[3] = {0, 0, 0}, ga[6] = {0, 0, 0, 0, 0, 0}, ka[3] = {0, 0, 0}, tr = 0.0;
-#pragma unroll 1
-            for (int g = 0; g < nt; ++g) {
-                if (!((mask >> g) & 1u)) continue;
-                const double R[3] = {W.tgt[g][0] - c[0], W.tgt[g][1] - c[1], W.tgt[g][2] - c[2]};
-                const double w[3] = {W.tgt[g][3], W.tgt[g][4], W.tgt[g][5]};
+            if (lane < cnt) {
+                const int box = boxes[lane].x;
+                const double* m = a.t.mom + (size_t)box * kMom;
+                const double R[3] = {X[0] - m[MC], X[1] - m[MC + 1], X[2] - m[MC + 2]};
+                const double M = m[MM], D[3] = {m[MD], m[MD + 1], m[MD + 2]};
+                const double Q[6] = {m[MQ], m[MQ + 1], m[MQ + 2], m[MQ + 3], m[MQ + 4], m[MQ + 5]};
+                const double T = m[MT];                       // -tr(Q)/2
                 const double gi = rsqrt_fp64(dot3(R, R) + a.eps2);
                 const double u = gi * gi, g3 = gi * u, g5 = g3 * u, g7 = g5 * u, g9 = g7 * u;
                 const double rw = dot3(R, w), rd = dot3(R, D), wd = dot3(w, D);
@@ -125,36 +97,22 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
                 const double aR = g53 * (M * rw - wd) + p7 * rd;
                 const double aw = -(M * g3 + g53 * rd);
                 const double h7 = 0.5 * p7;
+                double* d = adj + (size_t)box * 12;
                 double b[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const double kk = kr * R[k] + (kw * w[k] + (g53 * qw[k] - p7 * q[k]));
-                    ka[k] += kk;
-                    W.mt[g][k][lane] -= aR * R[k] + (aw * w[k] + (kk - p5 * D[k]));
-                    al[k] += p5 * R[k] - g3 * w[k];
+                    atomicAdd(d + 9 + k, kk);
+                    mt[k] -= aR * R[k] + (aw * w[k] + (kk - p5 * D[k]));
+                    atomicAdd(d + k, p5 * R[k] - g3 * w[k]);
                     b[k] = g53 * w[k] - h7 * R[k];
                 }
-                tr += p5;
-                ga[0] += b[0] * R[0];
-                ga[1] += b[0] * R[1] + b[1] * R[0];
-                ga[2] += b[0] * R[2] + b[2] * R[0];
-                ga[3] += b[1] * R[1];
-                ga[4] += b[1] * R[2] + b[2] * R[1];
-                ga[5] += b[2] * R[2];
-            }
-            if (mask) {
-                double* d = adj + (size_t)bm.x * 12;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    atomicAdd(d + k, al[k]);
-                    atomicAdd(d + 9 + k, ka[k]);
-                }
-                atomicAdd(d + 3, 2.0 * ga[0] + tr);
-                atomicAdd(d + 4, ga[1]);
-                atomicAdd(d + 5, ga[2]);
-                atomicAdd(d + 6, 2.0 * ga[3] + tr);
-                atomicAdd(d + 7, ga[4]);
-                atomicAdd(d + 8, 2.0 * ga[5] + tr);
+                atomicAdd(d + 3, 2.0 * (b[0] * R[0]) + p5);
+                atomicAdd(d + 4, b[0] * R[1] + b[1] * R[0]);
+                atomicAdd(d + 5, b[0] * R[2] + b[2] * R[0]);
+                atomicAdd(d + 6, 2.0 * (b[1] * R[1]) + p5);
+                atomicAdd(d + 7, b[1] * R[2] + b[2] * R[1]);
+                atomicAdd(d + 8, 2.0 * (b[2] * R[2]) + p5);
             }
             __syncwarp();
         };
@@ -165,44 +123,29 @@ k_walk_adjoint(WalkArgs a, int group, const double* __restrict__ lam, double* __
                 int j, nd, first;
                 unsigned int mask;
                 run.at(base + lane, j, nd, first, mask);
-                double xj = 0.0, yj = 0.0, zj = 0.0, qj = 0.0;
-                if (mask) {
-                    xj = a.x[j];
-                    yj = a.y[j];
-                    zj = a.z[j];
-                    qj = a.sp[j] ? q1 : q0;
-                }
-                double s[3] = {0.0, 0.0, 0.0};
-#pragma unroll 1
-                for (int g = 0; g < nt; ++g) {
-                    if (!((mask >> g) & 1u) || W.slot[g] == j) continue;
-                    const double R[3] = {W.tgt[g][0] - xj, W.tgt[g][1] - yj, W.tgt[g][2] - zj};
-                    const double w[3] = {W.tgt[g][3], W.tgt[g][4], W.tgt[g][5]};
-                    const double gi = rsqrt_fp64(dot3(R, R) + a.eps2);
-                    const double u = gi * gi, cw = qj * (gi * u);
-                    const double cr = -3.0 * (cw * u) * dot3(R, w);
+                if (!mask || j == t) continue;
+                const double R[3] = {X[0] - a.x[j], X[1] - a.y[j], X[2] - a.z[j]};
+                const double qj = a.sp[j] ? q1 : q0;
+                const double gi = rsqrt_fp64(dot3(R, R) + a.eps2);
+                const double u = gi * gi, cw = qj * (gi * u);
+                const double cr = -3.0 * (cw * u) * dot3(R, w);
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const double tv = cr * R[k] + cw * w[k];
-                        s[k] -= tv;
-                        W.mt[g][k][lane] += tv;
-                    }
+                for (int k = 0; k < 3; ++k) {
+                    const double tv = cr * R[k] + cw * w[k];
+                    mt[k] += tv;
+                    atomicAdd(&mu[3 * (size_t)j + k], -tv);
                 }
-                if (mask)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) atomicAdd(&mu[3 * (size_t)j + k], s[k]);
             }
             __syncwarp();
         };
 
-        walk_lists(a, W.walk, tg, ck.z, multipoles, direct_pairs);
+        walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
 
-        for (int v = lane; v < 3 * nt; v += 32) {
-            // the lanes' partial sums of one component, in lane order
-            const double* p = W.mt[v / 3][v % 3];
-            double sum = 0.0;
-            for (int k = 0; k < 32; ++k) sum += p[(k + lane) & 31];
-            atomicAdd(&mu[3 * (size_t)W.slot[v / 3] + v % 3], sum);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) mt[k] += __shfl_xor_sync(0xffffffffu, mt[k], o);
+            if (lane == k) atomicAdd(&mu[3 * (size_t)t + k], mt[k]);
         }
         __syncwarp();
     }
@@ -742,12 +685,9 @@ void launch_walk_adjoint(const WalkArgs& a, const double* lam, double* mu, doubl
         launch(k_adjoint_push<float>, 32 * 152, 32, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adjf, mu);
     } else {
         launch(k_zero_adj<double>, 2 * 152, 256, s, a.t.nnodes, adj);
-        // eight targets per warp, fewer while that leaves an SM with under four warps
-        int group = kAdjGroup;
-        while (group > 1 && (int64_t)a.nchunks * (32 / group) < 4 * (int64_t)nsm) group /= 2;
-        const int64_t items = (int64_t)a.nchunks * (32 / group);
-        const int blocks = items < 1 ? 1 : items < 12 * nsm ? (int)items : 12 * nsm;
-        launch(k_walk_adjoint, blocks, 32, s.whole(), a, group, lam, mu, adj);
+        const int64_t items = (int64_t)a.nchunks * 32;
+        const int blocks = items < 1 ? 1 : items < 8 * nsm ? (int)items : 8 * nsm;
+        launch(k_walk_adjoint, blocks, 32, s.whole(), a, lam, mu, adj);
         launch(k_adjoint_push<double>, 32 * 152, 32, s, a.x, a.y, a.z, a.sp, a.qsp, a.t, adj, mu);
     }
 }
