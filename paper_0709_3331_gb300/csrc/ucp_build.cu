@@ -638,6 +638,7 @@ __device__ __forceinline__ void twig_sums_f64(const Cube* __restrict__ cube, con
         double* r = t.mom + (size_t)w.id * kMom;
         r[o] = lo;
         if (o < 6) r[8 + o] = hi;
+        if (o == 7) t.delta[w.id] = kSumsDelta;
     }
 }
 
@@ -776,6 +777,7 @@ k_moments(const double* __restrict__ x, const double* __restrict__ y,
             double2* r = reinterpret_cast<double2*>(t.mom + (size_t)node * kMom);
 #pragma unroll
             for (int k = 0; k < 7; ++k) r[k] = make_double2(a[2 * k], a[2 * k + 1]);
+            t.delta[node] = kSumsDelta;
         }
         sweep_up(t, node,
                  [&](const Twig& w, int o, int ch) { twig_sums_f64(cube, t, w, o, ch); });

@@ -94,8 +94,11 @@ __device__ __forceinline__ void follow()
 // (FP32C contexts: c and rcrit2 only, the rest in mom32)
 // rcrit2 = (s/theta + delta)^2 is filled per walk (it depends on theta).  Until its first
 // walk an FP64 tree holds in the same place each box's sums about its geometric centre,
-// {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)}.
+// {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)}, and kSumsDelta as the box's delta.
+// The mark is the record's own, on the device, so that a captured sequence of launches
+// finds the records as they are whenever it is replayed.
 constexpr int kMom = 16;
+constexpr double kSumsDelta = -1.0;
 enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
 
 // FP32 box records, written per walk (they hold rcrit2, which depends on theta):
@@ -263,10 +266,9 @@ struct WalkArgs {
     int* err;               // raised by a bounded wait that gave up
     unsigned long long* stats; // {p2p, m2p}
 };
-// per walk: box records, and the work counter and cost bins (may be NULL) cleared;
-// sums: t.mom still holds the sums launch_moments left in an FP64 context (moments now)
-void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int sums, int* work,
-                        int* bins,
+// per walk: box records (in an FP64 context also the moments, where they are still the sums
+// launch_moments left), and the work counter and cost bins (may be NULL) cleared
+void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
                         Queue s);
 void launch_walk_fp64(const WalkArgs& a, int nsm, Queue s);
 void launch_walk_fp32c(const WalkArgs& a, int nsm, Queue s, int shape);

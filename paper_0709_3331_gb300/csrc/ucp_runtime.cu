@@ -85,7 +85,6 @@ struct ucp_ctx {
     int sorted_buf = 0;                // key[] / val[] buffer of the last sort
     std::vector<double> cloud_energy;  // per-cloud {KE_i, KE_e, PE, px, py, pz} of the last energy
     bool have_state = false, tree_valid = false, acc_valid = false;
-    bool sums = false;                // the tree's records hold sums, not moments yet (FP64)
     bool phi_valid = false;           // phi of every particle at the current positions
     double phi_theta = -1.0, phi_eps = -1.0;
     int64_t steps = 0, walk_targets = 0, walk_launches = 0;
@@ -255,18 +254,16 @@ int build(ucp_ctx* c)
                     block_sorted(n, c->n_clouds) ? c->val[1] : nullptr, c->s);
     launch_moments(c->st[k][0], c->st[k][1], c->st[k][2], c->sp[k], c->qsp, n, c->leaf_cap,
                    c->pos_cnt, c->pos_off, c->cube, c->t, c->src32, c->precision == UCP_FP32C, c->s);
-    c->sums = c->precision == UCP_FP64;
     c->tree_valid = true;
     c->acc_valid = false;
     c->phi_valid = false;
     return check_launch(c, "tree build");
 }
 
-// Per-walk box records (and, once per FP64 build, the moments).
+// Per-walk box records (and, at the first walk after an FP64 build, the moments).
 void prepare(ucp_ctx* c, double theta, int* bins)
 {
-    launch_mac_prepare(c->t, c->cube, theta, c->precision == UCP_FP32C, c->sums, c->work, bins, c->s);
-    c->sums = false;
+    launch_mac_prepare(c->t, c->cube, theta, c->precision == UCP_FP32C, c->work, bins, c->s);
 }
 
 // One walk over all particles (electrons_only = 0) or the electrons.  visits: in an
@@ -877,7 +874,6 @@ static int run_block_graph(ucp_ctx* c, double dt_e, int kk, double theta, double
     c->cur = hit->cur_out;
     c->steps += kk;
     c->tree_valid = true;
-    c->sums = false;
     c->acc_valid = true;
     c->phi_valid = true;
     c->phi_theta = theta;
@@ -1364,7 +1360,7 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
     CK(cudaStreamSynchronize(c->s));
     *nnodes = nn;
     if (!topo && !is_leaf && !geom) return UCP_OK;
-    if (c->sums) prepare(c, 1.0, nullptr);
+    if (c->precision == UCP_FP64) prepare(c, 1.0, nullptr);  // moments, if no walk made them
     if (cap < nn) return fail(c, UCP_EINVAL, "capacity smaller than the box count");
     std::vector<int4> info(nn);
     std::vector<int> dl(nn);

@@ -944,15 +944,15 @@ k_walk_fp32c_visits(WalkArgs a)
 }
 
 // Per walk: rcrit2 = (s/theta + delta)^2 of every box in FP64 (theta = 0:
-// +inf, nothing accepted), and the FP32C box records.  kSums: the first walk after an
-// FP64 build also makes the moments and delta from the sums that build left, one box per
-// lane: nearly all FP64 work, so its blocks are small and spread over the SMs.
-constexpr int prep_threads(bool sums) { return sums ? 64 : 256; }
+// +inf, nothing accepted), and the FP32C box records.  In an FP64 context (kFp64) the
+// moments and delta of every box that still holds the sums its build left are made from
+// them first, one box per lane: nearly all FP64 work, so its blocks are small and spread
+// over the SMs.
+constexpr int prep_threads(bool fp64) { return fp64 ? 64 : 256; }
 
-template <bool kSums>
-__global__ void __launch_bounds__(prep_threads(kSums))
-k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32, int* work,
-              int* bins)
+template <bool kFp64>
+__global__ void __launch_bounds__(prep_threads(kFp64))
+k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, int* bins)
 {
     follow();
     if (blockIdx.x == 0) {
@@ -967,7 +967,7 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32,
         const Cube& cb = cube[t.cloud ? t.cloud[t.info[nd].x] : 0];
         const double L = cb.L;
         double s = ldexp(L, -(dl & 255));
-        if (kSums) {
+        if (kFp64 && t.delta[nd] == kSumsDelta) {
             double a[14], z[3], side, rec[kMom];
             const double2* r = reinterpret_cast<const double2*>(m);
 #pragma unroll
@@ -997,7 +997,7 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32,
         const float chx = (float)ux, chy = (float)uy, chz = (float)uz;
         const float rc2 = (float)r2;
         t.hdr[nd] = make_float4(-chx, -chy, -chz, (dl & 256) ? -rc2 : rc2);
-        if (want_f32) {
+        if (!kFp64) {
             t.lo[nd] = make_float4((float)((double)chx - ux), (float)((double)chy - uy),
                                    (float)((double)chz - uz), __int_as_float(t.info[nd].z));
             const float4* m32 = reinterpret_cast<const float4*>(t.mom32 + (size_t)nd * 16);
@@ -1014,16 +1014,14 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int want_f32,
 
 }  // namespace
 
-void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int sums, int* work,
-                        int* bins, Queue s)
+void launch_mac_prepare(Tree t, const Cube* cube, double theta, int want_f32, int* work, int* bins,
+                        Queue s)
 {
     count_launch(1);
-    if (sums)
-        launch(k_mac_prepare<true>, 16 * 152, prep_threads(true), s, t, cube, theta, want_f32, work,
-               bins);
+    if (want_f32)
+        launch(k_mac_prepare<false>, 4 * 152, prep_threads(false), s, t, cube, theta, work, bins);
     else
-        launch(k_mac_prepare<false>, 4 * 152, prep_threads(false), s, t, cube, theta, want_f32, work,
-               bins);
+        launch(k_mac_prepare<true>, 16 * 152, prep_threads(true), s, t, cube, theta, work, bins);
 }
 
 // blocks of one warp: per_sm on every SM, or one per work item
