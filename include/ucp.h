@@ -125,8 +125,10 @@ int ucp_step(ucp_ctx* ctx, double dt_e, int ion_substep_ratio, int64_t n_electro
              double theta, double eps);
 
 /* Gradient of the electron kinetic energy after a run.  From the current state
- * (x0, v0), advances n_steps electron substeps exactly as ucp_step(dt_e, k,
- * n_steps, theta, eps) and returns *loss = L = sum over electrons of m v^2 / 2 at
+ * (x0, v0), advances n_steps electron substeps as ucp_step(dt_e, k, n_steps, theta,
+ * eps) does (FP32C contexts: with the same boxes and pairs, but sums in an order of their
+ * own, so that forces agree to about 2e-8; the run is then the same whichever calls came
+ * before it) and returns *loss = L = sum over electrons of m v^2 / 2 at
  * the end, grad_x = dL/dx0 and grad_v = dL/dv0 (N x 3, caller order; either may
  * be NULL).  Reverse mode: the discrete adjoint of every kick and drift, and at
  * every substep the adjoint of the TREE force with the tree held fixed (the same

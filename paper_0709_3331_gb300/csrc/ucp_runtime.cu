@@ -85,6 +85,7 @@ struct ucp_ctx {
     int sorted_buf = 0;                // key[] / val[] buffer of the last sort
     std::vector<double> cloud_energy;  // per-cloud {KE_i, KE_e, PE, px, py, pz} of the last energy
     bool have_state = false, tree_valid = false, acc_valid = false;
+    bool acc_visits = false;          // the stored accelerations are the visits walk's
     bool phi_valid = false;           // phi of every particle at the current positions
     double phi_theta = -1.0, phi_eps = -1.0;
     int64_t steps = 0, walk_targets = 0, walk_launches = 0;
@@ -324,7 +325,10 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
         c->walk_targets += a.ntargets;
         c->walk_launches += 1;
     }
-    if (!electrons_only) c->acc_valid = true;
+    if (!electrons_only) {
+        c->acc_valid = true;
+        c->acc_visits = f32 && visits;
+    }
     if (!electrons_only && want_phi) {
         c->phi_valid = true;
         c->phi_theta = theta;
@@ -730,12 +734,14 @@ int ucp_tree_force(ucp_ctx* c, double theta, double eps, double* acc, double* ph
 
 // The split-step push; with store != NULL the positions after every electron
 // substep are written there in caller order (n x 3 doubles per substep).  gradient:
-// a forward run of the gradient, whose potential nobody reads.
+// a forward run of the gradient, whose potential nobody reads; it starts from stored
+// accelerations only if its own walk left them, so that the recomputation of its first
+// stretch, which starts from a loaded state, is that run bit for bit.
 static int run_blocks(ucp_ctx* c, double dt_e, int kk, int64_t nblocks, double theta, double eps,
                       double* store, bool gradient = false)
 {
     int rc;
-    if (!c->acc_valid) {
+    if (!c->acc_valid || c->acc_visits != (gradient && c->precision == UCP_FP32C)) {
         if (!c->tree_valid && (rc = build(c))) return rc;
         if ((rc = force(c, theta, eps, 0, false, gradient))) return rc;
     }
@@ -987,7 +993,7 @@ int ucp_step(ucp_ctx* c, double dt_e, int kk, int64_t n_electron_steps, double t
     int rc = valid_walk_args(c, theta, eps);
     if (rc) return rc;
     if (!c->use_graphs) return run_blocks(c, dt_e, kk, n_electron_steps / kk, theta, eps, nullptr);
-    if (!c->acc_valid) {
+    if (!c->acc_valid || c->acc_visits) {
         if (!c->tree_valid && (rc = build(c))) return rc;
         if ((rc = force(c, theta, eps, 0, false))) return rc;
     }
