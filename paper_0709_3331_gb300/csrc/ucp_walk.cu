@@ -247,37 +247,46 @@ k_walk_fp64(WalkArgs a)
 }
 
 // ------------------------------------------------------------------ FP32C
-// Kelbg factors of an unlike pair, 1 - e^-u of the potential and 1 - (1 + u) e^-u of the
-// field, u = r/lambda: directly from u = 1/2 on, below by their Taylor series (no
-// cancellation).  A coincident pair (r < 1e-18) takes the limit, potential 1/lambda and
-// no field: ri becomes 1/lambda with the factors 1 and 0.
-__device__ __forceinline__ void kelbg_factors(float d2, float& ri, float inv_lambda, float& fp,
-                                              float& fg)
+// Kelbg factors of an unlike pair, u = r/lambda: its potential is q ri fp and its field
+// q ri^3 fg r_vec, with fp = 1 - e^-u and fg = 1 - (1 + u) e^-u from u = 1/2 on.  Below, ri
+// becomes 1/lambda and the factors fp / u and fg / u^3 follow from Taylor series (no
+// cancellation, and no power of 1/r: the field of a close pair tends to q / (2 lambda^2),
+// where r^-3 overflows from r = 1.5e-13 down).  ri comes in as rsqrt_ftz of d2 and is taken
+// again where that flushed d2.  A pair at r = 0 takes the limits, potential 1/lambda and no
+// field.
+__device__ __forceinline__ void kelbg_factors(float d2, float& ri, float lambda, float inv_lambda,
+                                              float& fp, float& fg)
 {
+    if (d2 < 1.17549435e-38f) {      // the smallest normal float
+        if (d2 == 0.f) {
+            ri = inv_lambda;
+            fp = 1.f;
+            fg = 0.f;
+            return;
+        }
+        ri = rsqrtf(d2);
+    }
     const float u = d2 * ri * inv_lambda;
-    if (d2 < 1e-36f) {
-        ri = inv_lambda;
-        fp = 1.f;
-        fg = 0.f;
-    } else if (u >= 0.5f) {
+    if (u >= 0.5f) {
         const float e = __expf(-u);
         fp = 1.f - e;
         fg = 1.f - (1.f + u) * e;
     } else {
-        fp = u * fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5040.f, -1.f / 720.f),
-                                                     1.f / 120.f), -1.f / 24.f), 1.f / 6.f),
-                              -0.5f), 1.f);
+        fp = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5040.f, -1.f / 720.f),
+                                                 1.f / 120.f), -1.f / 24.f), 1.f / 6.f),
+                          -0.5f), 1.f);
         const float poly = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5760.f, -1.f / 840.f),
                                                         1.f / 144.f), -1.f / 30.f), 0.125f),
                                 -1.f / 3.f);
-        fg = u * u * fmaf(u, poly, 0.5f);
+        fg = fmaf(0.5f, ri * lambda, poly);
+        ri = inv_lambda;
     }
 }
 
 // A target of the FP32C walk as the sums see it.
 struct LaneTarget {
     int t, tmin, tmax;              // slots: its own, the chunk's lowest and highest
-    float xh, yh, zh, xl, yl, zl, q, eps2, inv_lambda;
+    float xh, yh, zh, xl, yl, zl, q, eps2, lambda, inv_lambda;
 };
 
 template <bool kKelbg>
@@ -292,6 +301,7 @@ __device__ __forceinline__ LaneTarget lane_target(const WalkArgs& a, const Chunk
     g.xl = tg.xl; g.yl = tg.yl; g.zl = tg.zl;
     g.q = tg.t >= 0 ? (float)a.qsp[a.sp[tg.t] ? 1 : 0] : 0.f;
     g.eps2 = (float)a.eps2;
+    g.lambda = kKelbg ? (float)a.lambda : 0.f;
     g.inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
     return g;
 }
@@ -390,7 +400,7 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
     const float4* __restrict__ H = a.t.hdr;
     const float4* __restrict__ S = a.src32;
     const float xh = g_.xh, yh = g_.yh, zh = g_.zh, xl = g_.xl, yl = g_.yl, zl = g_.zl;
-    const float qt = g_.q, eps2 = g_.eps2, inv_lambda = g_.inv_lambda;
+    const float qt = g_.q, eps2 = g_.eps2;
     const int t = g_.t, tmin = g_.tmin, tmax = g_.tmax;
     float4* meta = reinterpret_cast<float4*>(stage);   // {-ch, place}, {-cl, begin}
     float4* buf = meta + 64;                             // 2 x 32 float4
@@ -431,8 +441,7 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
             const float2 dz = __fadd2_rn(rz, make_float2(Q.x, Q.y));
             const float2 q = make_float2(Q.z, Q.w);
             if (kKelbg) {
-                // unlike charges (electron-ion) take the Kelbg form, unsoftened:
-                // the Coulomb terms times 1 - e^-u and 1 - (1 + u) e^-u, u = r/lambda
+                // unlike charges (electron-ion) take the Kelbg form, unsoftened
                 const bool un0 = q.x != qt, un1 = q.y != qt;
                 const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
                 const float2 r2 = __fadd2_rn(d2, make_float2(un0 ? 0.f : eps2,
@@ -440,8 +449,8 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
                 float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
                                         ok1 ? rsqrt_ftz(r2.y) : 0.f);
                 float2 fp = splat(1.f), fg = fp;
-                if (un0 && ok0) kelbg_factors(d2.x, ri.x, inv_lambda, fp.x, fg.x);
-                if (un1 && ok1) kelbg_factors(d2.y, ri.y, inv_lambda, fp.y, fg.y);
+                if (un0 && ok0) kelbg_factors(d2.x, ri.x, g_.lambda, g_.inv_lambda, fp.x, fg.x);
+                if (un1 && ok1) kelbg_factors(d2.y, ri.y, g_.lambda, g_.inv_lambda, fp.y, fg.y);
                 const float2 qi = __fmul2_rn(q, ri);
                 const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
                 px = __ffma2_rn(qr3, dx, px);
@@ -827,7 +836,7 @@ k_walk_fp32c_visits(WalkArgs a)
                 lt.tmax = __shfl_sync(0xffffffffu, t, ck.y - 1);
                 lt.xh = tg.xh; lt.yh = tg.yh; lt.zh = tg.zh;
                 lt.xl = tg.xl; lt.yl = tg.yl; lt.zl = tg.zl;
-                lt.q = lt.inv_lambda = 0.f;
+                lt.q = lt.lambda = lt.inv_lambda = 0.f;
                 lt.eps2 = eps2;
                 while (done < upto) {
                     const int m = min(32, upto - done);
