@@ -185,9 +185,9 @@ __device__ __forceinline__ unsigned int accept_mask(const WalkArgs& a, float* st
             // |error| <= 2^-22 sqrt(3) X_t d + 2^-21 d2 (rcrit2's rounding
             // included) with X_t the target's largest coordinate; with
             // d <= (d2 + 1) / 2 that lies inside wa d2 + wb (rare: a few tests in
-            // a million at the bench size).
-            const bool again0 = in0 && fabsf(dm.x) <= win.x;
-            const bool again1 = in1 && fabsf(dm.y) <= win.y;
+            // a million at the bench size).  Where d2 overflows it is taken there too.
+            const bool again0 = in0 && !(fabsf(dm.x) > win.x);
+            const bool again1 = in1 && !(fabsf(dm.y) > win.y);
             if (again0)
                 acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + tg.t,
                                     a.y + tg.t, a.z + tg.t);

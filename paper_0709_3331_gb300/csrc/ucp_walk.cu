@@ -158,7 +158,7 @@ k_walk_fp64(WalkArgs a)
             const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
             const float dm = d2 - fabsf(h.w);
             bool ok = has && dm > 0.f;
-            if (has && fabsf(dm) <= fmaf(wa, d2, wb))
+            if (has && !(fabsf(dm) > fmaf(wa, d2, wb)))   // also where FP32 overflows
                 ok = accepts_fp64(a.t.mom + (size_t)box * kMom, X + t, Y + t, Z + t);
             const unsigned int A = __ballot_sync(0xffffffffu, ok);
             const unsigned int OL = __ballot_sync(0xffffffffu, has && !ok && leaf);
@@ -1004,7 +1004,9 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
         // one value
         const double ux = m[0] - cb.c[0], uy = m[1] - cb.c[1], uz = m[2] - cb.c[2];
         const float chx = (float)ux, chy = (float)uy, chz = (float)uz;
-        const float rc2 = (float)r2;
+        // finite as r2 is: past the range of FP32 it stands for "larger", and a box as far
+        // away is decided in FP64
+        const float rc2 = theta > 0.0 ? fminf((float)r2, 3.40282347e38f) : (float)r2;
         t.hdr[nd] = make_float4(-chx, -chy, -chz, (dl & 256) ? -rc2 : rc2);
         if (!kFp64) {
             t.lo[nd] = make_float4((float)((double)chx - ux), (float)((double)chy - uy),
