@@ -254,8 +254,8 @@ k_walk_fp64(WalkArgs a)
 // where r^-3 overflows from r = 1.5e-13 down).  ri comes in as rsqrt_ftz of d2 and is taken
 // again where that flushed d2.  A pair at r = 0 takes the limits, potential 1/lambda and no
 // field.
-__device__ __forceinline__ void kelbg_factors(float d2, float& ri, float lambda, float inv_lambda,
-                                              float& fp, float& fg)
+__device__ __forceinline__ void kelbg_factors(float d2, float& ri, float inv_lambda, float& fp,
+                                              float& fg)
 {
     if (d2 < 1.17549435e-38f) {      // the smallest normal float
         if (d2 == 0.f) {
@@ -278,7 +278,7 @@ __device__ __forceinline__ void kelbg_factors(float d2, float& ri, float lambda,
         const float poly = fmaf(u, fmaf(u, fmaf(u, fmaf(u, fmaf(u, 1.f / 5760.f, -1.f / 840.f),
                                                         1.f / 144.f), -1.f / 30.f), 0.125f),
                                 -1.f / 3.f);
-        fg = fmaf(0.5f, ri * lambda, poly);
+        fg = __fdividef(0.5f, u) + poly;
         ri = inv_lambda;
     }
 }
@@ -286,7 +286,7 @@ __device__ __forceinline__ void kelbg_factors(float d2, float& ri, float lambda,
 // A target of the FP32C walk as the sums see it.
 struct LaneTarget {
     int t, tmin, tmax;              // slots: its own, the chunk's lowest and highest
-    float xh, yh, zh, xl, yl, zl, q, eps2, lambda, inv_lambda;
+    float xh, yh, zh, xl, yl, zl, q, eps2, inv_lambda;
 };
 
 template <bool kKelbg>
@@ -301,7 +301,6 @@ __device__ __forceinline__ LaneTarget lane_target(const WalkArgs& a, const Chunk
     g.xl = tg.xl; g.yl = tg.yl; g.zl = tg.zl;
     g.q = tg.t >= 0 ? (float)a.qsp[a.sp[tg.t] ? 1 : 0] : 0.f;
     g.eps2 = (float)a.eps2;
-    g.lambda = kKelbg ? (float)a.lambda : 0.f;
     g.inv_lambda = kKelbg ? (float)(1.0 / a.lambda) : 0.f;
     return g;
 }
@@ -400,7 +399,7 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
     const float4* __restrict__ H = a.t.hdr;
     const float4* __restrict__ S = a.src32;
     const float xh = g_.xh, yh = g_.yh, zh = g_.zh, xl = g_.xl, yl = g_.yl, zl = g_.zl;
-    const float qt = g_.q, eps2 = g_.eps2;
+    const float qt = g_.q, eps2 = g_.eps2, inv_lambda = g_.inv_lambda;
     const int t = g_.t, tmin = g_.tmin, tmax = g_.tmax;
     float4* meta = reinterpret_cast<float4*>(stage);   // {-ch, place}, {-cl, begin}
     float4* buf = meta + 64;                             // 2 x 32 float4
@@ -449,8 +448,8 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
                 float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
                                         ok1 ? rsqrt_ftz(r2.y) : 0.f);
                 float2 fp = splat(1.f), fg = fp;
-                if (un0 && ok0) kelbg_factors(d2.x, ri.x, g_.lambda, g_.inv_lambda, fp.x, fg.x);
-                if (un1 && ok1) kelbg_factors(d2.y, ri.y, g_.lambda, g_.inv_lambda, fp.y, fg.y);
+                if (un0 && ok0) kelbg_factors(d2.x, ri.x, inv_lambda, fp.x, fg.x);
+                if (un1 && ok1) kelbg_factors(d2.y, ri.y, inv_lambda, fp.y, fg.y);
                 const float2 qi = __fmul2_rn(q, ri);
                 const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
                 px = __ffma2_rn(qr3, dx, px);
@@ -836,7 +835,7 @@ k_walk_fp32c_visits(WalkArgs a)
                 lt.tmax = __shfl_sync(0xffffffffu, t, ck.y - 1);
                 lt.xh = tg.xh; lt.yh = tg.yh; lt.zh = tg.zh;
                 lt.xl = tg.xl; lt.yl = tg.yl; lt.zl = tg.zl;
-                lt.q = lt.lambda = lt.inv_lambda = 0.f;
+                lt.q = lt.inv_lambda = 0.f;
                 lt.eps2 = eps2;
                 while (done < upto) {
                     const int m = min(32, upto - done);
@@ -976,8 +975,9 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
         const Cube& cb = cube[t.cloud ? t.cloud[t.info[nd].x] : 0];
         const double L = cb.L;
         double s = ldexp(L, -(dl & 255));
-        if (kFp64 && t.delta[nd] == kSumsDelta) {
-            double a[14], z[3], side, rec[kMom];
+        // (everything loaded before the test, so that no load waits for another)
+        double a[14], delta = t.delta[nd], c[3] = {m[MC], m[MC + 1], m[MC + 2]};
+        if (kFp64) {
             const double2* r = reinterpret_cast<const double2*>(m);
 #pragma unroll
             for (int k = 0; k < 7; ++k) {
@@ -985,15 +985,21 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
                 a[2 * k] = v.x;
                 a[2 * k + 1] = v.y;
             }
+        }
+        if (kFp64 && delta == kSumsDelta) {
+            double z[3], side, rec[kMom];
             box_centre(cb, t.cell[nd], dl & 255, z, &side);
-            finish_box(a, z, rec, t.delta + nd);
+            finish_box(a, z, rec, &delta);
+            t.delta[nd] = delta;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) c[k] = rec[MC + k];
 #pragma unroll
             for (int k = 0; k < kMom; ++k)
                 if (k != MR2) m[k] = rec[k];
         }
         double r2;
         if (theta > 0.0) {
-            double rc = __dadd_rn(__ddiv_rn(s, theta), t.delta[nd]);
+            double rc = __dadd_rn(__ddiv_rn(s, theta), delta);
             r2 = __dmul_rn(rc, rc);
         } else {
             r2 = INFINITY;
@@ -1002,7 +1008,7 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
         // the centroid, relative to the cube's centre as the walk's targets are,
         // enters negated (x_t - c as a sum); the trace term of the expansion as
         // one value
-        const double ux = m[0] - cb.c[0], uy = m[1] - cb.c[1], uz = m[2] - cb.c[2];
+        const double ux = c[0] - cb.c[0], uy = c[1] - cb.c[1], uz = c[2] - cb.c[2];
         const float chx = (float)ux, chy = (float)uy, chz = (float)uz;
         // finite as r2 is: past the range of FP32 it stands for "larger", and a box as far
         // away is decided in FP64
