@@ -36,9 +36,8 @@ __device__ __forceinline__ double dot3(const double* a, const double* b)
     return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// ---- FP64 form: one warp per target, the traversal of the FP32C walk on the FP64
-// contexts' records (FP32 criterion, again in FP64 within its window: the FP64 walk's
-// decisions).  The lanes are the sources, 32 accepted boxes or 32 particles of opened
+// ---- FP64 form: one warp per target, the traversal of the FP32C walk with the FP64 walk's
+// decisions.  The lanes are the sources, 32 accepted boxes or 32 particles of opened
 // leaves.  A box's or source's own terms are added to memory as they come; the target's
 // partial sums stay in the lanes' registers until the end.  All terms are linear in the
 // target's weight w = (q/m) lambda.
@@ -66,7 +65,7 @@ k_walk_adjoint(WalkArgs a, const double* __restrict__ lam, double* __restrict__ 
         if ((int)(item % 32) >= ck.y) continue;
         const int ti = ck.x + (int)(item % 32);
         const int t = a.targets ? a.targets[ti] : ti;
-        const ChunkTarget tg(a, lane == 0 ? t : -1, ck.z);
+        const OneTarget tg(a, t, ck.z);
         const double X[3] = {a.x[t], a.y[t], a.z[t]};
         const double qm = a.msp[2 + a.sp[t]];
         const double w[3] = {qm * lam[3 * (size_t)t], qm * lam[3 * (size_t)t + 1],
@@ -139,7 +138,11 @@ k_walk_adjoint(WalkArgs a, const double* __restrict__ lam, double* __restrict__ 
             __syncwarp();
         };
 
-        walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
+        walk_lists(a, W, 1u, ck.z,
+                   [&](int box, unsigned int, const float4 h) {
+                       return box >= 0 && tg.accepts(a, box, h) ? 1u : 0u;
+                   },
+                   multipoles, direct_pairs);
 
 #pragma unroll
         for (int k = 0; k < 3; ++k) {

@@ -66,6 +66,42 @@ static __device__ __noinline__ bool accepts_fp64(const double* m, const double* 
     return m[MR2] < __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
+// A target of an FP64 context: its decisions are taken in FP32 on the traversal records and
+// again in FP64 within the rounding of d2 - rcrit2.  Per axis R is off by at most 2^-23
+// (|x_t| + |R|), so |error| <= 2^-22 sqrt(3) X d + 2^-21 d2 (rcrit2's rounding included),
+// X the target's largest coordinate.  With d <= (d2 / u + u) / 2 that lies inside wa d2 + wb;
+// u = side / 32 makes the window the same in every unit of length (u was 1: coordinates
+// from 4e6 up or 1e-7 down were all decided twice) and keeps it narrow down to the smallest
+// boxes.  1e-37 covers what underflows; where FP32's range ends, the window is infinite or
+// not a number and FP64 decides.  At N = 20,000 and units of 2^-40, 2^20 and 2^40 a force
+// call took 1.68, 1.52 and 1.59 ms, now 1.33 (r^2 past rsqrt_fp64's range), 1.24 and 1.24,
+// as at 1; a vector-Jacobian product 13.4, 5.5 and 13.3 ms, now 3.6 to 3.7.
+struct OneTarget {
+    int t;
+    float x, y, z, wa, wb;   // relative to the centre of the cloud's cube; the window
+
+    __device__ __forceinline__ OneTarget(const WalkArgs& a, int t_, int cloud) : t(t_)
+    {
+        const Cube& cube = a.cubes[cloud];
+        x = (float)(a.x[t] - cube.c[0]);
+        y = (float)(a.y[t] - cube.c[1]);
+        z = (float)(a.z[t] - cube.c[2]);
+        const float b = 5e-7f * fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z)));
+        wa = fmaf(b, (float)(16.0 / 2097152.0 * cube.kscale), 4e-6f);   // kscale = 2^21 / side
+        wb = fmaf(b, (float)cube.L * (1.f / 64.f), 1e-37f);
+    }
+
+    // does it accept the box of record h?
+    __device__ __forceinline__ bool accepts(const WalkArgs& a, int box, const float4 h) const
+    {
+        const float rx = x + h.x, ry = y + h.y, rz = z + h.z;
+        const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+        const float dm = d2 - fabsf(h.w);
+        if (fabsf(dm) > fmaf(wa, d2, wb)) return dm > 0.f;
+        return accepts_fp64(a.t.mom + (size_t)box * kMom, a.x + t, a.y + t, a.z + t);
+    }
+};
+
 constexpr int kStage = 32;           // accepted boxes evaluated per batch
 constexpr int kStageStride = 36;     // floats per staged pair of boxes (32 used; 16-byte aligned)
 
@@ -204,14 +240,15 @@ __device__ __forceinline__ unsigned int accept_mask(const WalkArgs& a, float* st
     return am;
 }
 
-// Walks a chunk's targets, one per lane, through their cloud's tree with the lanes
-// over boxes: multipoles(list, cnt) takes cnt <= 32 accepted boxes {box, mask of the
+// Walks targets, a bit each of `targets`, through their cloud's tree with the lanes over
+// boxes: accept(box, mask, h) gives the targets of mask that accept a lane's box (< 0: none)
+// of record h; multipoles(list, cnt) takes cnt <= 32 accepted boxes {box, mask of the
 // targets that accept it}, pairs(list, cnt) cnt <= 32 opened leaves {leaf, mask of the
-// targets that open it}; both are called by the whole warp and may use W.stage and their
-// part of the list.
-template <class Boxes, class Pairs>
-__device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const ChunkTarget& tg,
-                                           int cloud, Boxes& multipoles,
+// targets that open it}; all are called by the whole warp and may use W.stage, the last two
+// their part of the list.
+template <class Accept, class Boxes, class Pairs>
+__device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, unsigned int targets,
+                                           int cloud, Accept accept, Boxes& multipoles,
                                            Pairs& direct_pairs)
 {
     const int lane = threadIdx.x & 31;
@@ -219,13 +256,13 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const
     int top = 0, na = 0, nl = 0;
     // the first step tests the root for every target
     int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[cloud] : 0] : -1;
-    unsigned int mask = __ballot_sync(0xffffffffu, tg.t >= 0);
+    unsigned int mask = targets;
     while (true) {
         const bool has = box >= 0;
         const float4 h = has ? __ldg(a.t.hdr + box) : make_float4(0.f, 0.f, 0.f, 0.f);
         const bool leaf = __float_as_int(h.w) < 0;
         // targets that accept the box
-        const unsigned int am = accept_mask(a, W.stage, tg, box, mask, h);
+        const unsigned int am = accept(box, mask, h);
         const unsigned int om = has ? mask & ~am : 0u;  // targets that open it
         const unsigned int A = __ballot_sync(0xffffffffu, am != 0u);
         const unsigned int OL = __ballot_sync(0xffffffffu, om != 0u && leaf);
@@ -263,6 +300,18 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const
         top -= pop;
         __syncwarp();
     }
+}
+
+// The same for a chunk's targets, one per lane.
+template <class Boxes, class Pairs>
+__device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const ChunkTarget& tg,
+                                           int cloud, Boxes& multipoles, Pairs& direct_pairs)
+{
+    walk_lists(a, W, __ballot_sync(0xffffffffu, tg.t >= 0), cloud,
+               [&](int box, unsigned int mask, const float4 h) {
+                   return accept_mask(a, W.stage, tg, box, mask, h);
+               },
+               multipoles, direct_pairs);
 }
 
 // The particles of up to 32 opened leaves {leaf, mask} as one run over the lanes.

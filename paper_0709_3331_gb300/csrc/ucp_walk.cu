@@ -78,10 +78,7 @@ k_walk_fp64(WalkArgs a)
         const int t = a.targets ? a.targets[ti] : ti;
         const double xt = X[t], yt = Y[t], zt = Z[t];
         const int8_t st = SP[t];
-        const double* cc = a.cubes[ck.z].c;
-        const float xh = (float)(xt - cc[0]), yh = (float)(yt - cc[1]), zh = (float)(zt - cc[2]);
-        const float bt = 5e-7f * fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
-        const float wa = fmaf(0.5f, bt, 4e-6f), wb = 0.5f * bt;
+        const OneTarget tg(a, t, ck.z);
         double ex = 0.0, ey = 0.0, ez = 0.0, ph = 0.0;
         int top = 0, na = 0, nq = 0, np = 0, nm = 0;
 
@@ -154,12 +151,7 @@ k_walk_fp64(WalkArgs a)
             const bool has = box >= 0;
             const float4 h = has ? __ldg(H + box) : make_float4(0.f, 0.f, 0.f, 0.f);
             const bool leaf = __float_as_int(h.w) < 0;
-            const float rx = xh + h.x, ry = yh + h.y, rz = zh + h.z;
-            const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            const float dm = d2 - fabsf(h.w);
-            bool ok = has && dm > 0.f;
-            if (has && !(fabsf(dm) > fmaf(wa, d2, wb)))   // also where FP32 overflows
-                ok = accepts_fp64(a.t.mom + (size_t)box * kMom, X + t, Y + t, Z + t);
+            const bool ok = has && tg.accepts(a, box, h);
             const unsigned int A = __ballot_sync(0xffffffffu, ok);
             const unsigned int OL = __ballot_sync(0xffffffffu, has && !ok && leaf);
             const unsigned int OT = __ballot_sync(0xffffffffu, has && !ok && !leaf);
