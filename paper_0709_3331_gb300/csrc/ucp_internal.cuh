@@ -229,7 +229,8 @@ void launch_moments(const double* x, const double* y, const double* z, const int
                     Queue s);
 
 // ---- walk (ucp_walk.cu, ucp_schedule.cu) ----
-// Order in which a walk takes its chunks, and the costs it notes for the next order.
+// Order in which a walk takes its chunks, and the costs it notes for the next order (of the
+// same state's next substep or walk: a new state starts from list order).
 constexpr int kCostBins = 256;
 struct WalkOrder {
     int* order;             // chunk of every work item
@@ -322,6 +323,6 @@ void launch_load_state(const double* pos, const double* vel, const int8_t* sp, i
 void launch_check_state(const double* pos, const double* vel, const int8_t* sp, int n,
                         const unsigned char* cloud, int* flags, Queue s);
 void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
-                   int4* chunks, int* order, Queue s);
+                   int4* chunks, int* order, int n_other, int* other, Queue s);
 
 }  // namespace ucp

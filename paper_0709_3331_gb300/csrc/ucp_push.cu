@@ -180,13 +180,15 @@ __global__ void k_check_state(const double* __restrict__ pos, const double* __re
 }
 
 // Walk chunks of up to `width` consecutive targets, cloud by cloud: cloud c's run of
-// targets is [first[c], first[c + 1]), its chunks start at place[c]; taken in list order.
+// targets is [first[c], first[c + 1]), its chunks start at place[c]; taken in list order, as
+// are the first n_other of another list (whose chunks stay).
 __global__ void k_chunks(const int* __restrict__ first, const int* __restrict__ place, int n_clouds,
                          int width, int nchunks, int4* __restrict__ chunks,
-                         int* __restrict__ order)
+                         int* __restrict__ order, int n_other, int* __restrict__ other)
 {
     follow();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n_other) other[i] = i;
     if (i >= nchunks) return;
     int lo = 0, hi = n_clouds;          // the cloud whose chunks hold i
     while (hi - lo > 1) {
@@ -265,11 +267,13 @@ void launch_check_state(const double* pos, const double* vel, const int8_t* sp, 
 }
 
 void launch_chunks(const int* first, const int* place, int n_clouds, int width, int nchunks,
-                   int4* chunks, int* order, Queue s)
+                   int4* chunks, int* order, int n_other, int* other, Queue s)
 {
-    if (nchunks < 1) return;
+    const int most = nchunks > n_other ? nchunks : n_other;
+    if (most < 1) return;
     count_launch(1);
-    launch(k_chunks, nb(nchunks), kT, s, first, place, n_clouds, width, nchunks, chunks, order);
+    launch(k_chunks, nb(most), kT, s, first, place, n_clouds, width, nchunks, chunks, order, n_other,
+           other);
 }
 
 }  // namespace ucp

@@ -344,9 +344,10 @@ constexpr int kChunk = 32;
 
 // Chunk lists from the first target of every cloud (n_clouds + 1 values): the counts
 // are the host's, the lists are written on the device.  table: room for 2 (n_clouds
-// + 1) ints on the host (its contents are uploaded) and on the device.
+// + 1) ints on the host (its contents are uploaded) and on the device.  other: the order of
+// another list's n_other chunks, back to list order with this one's (NULL: none).
 int build_chunks(ucp_ctx* c, const int* first, int* host_table, int* table, int4* chunks,
-                 int* order, int* n_chunks)
+                 int* order, int* n_chunks, int* other, int n_other)
 {
     const int nc = c->n_clouds;
     int* place = host_table + nc + 1;
@@ -360,7 +361,7 @@ int build_chunks(ucp_ctx* c, const int* first, int* host_table, int* table, int4
     place[nc] = total;
     if (total > c->n_chunks_all_cap) return fail(c, UCP_EINVAL, "internal: chunk capacity");
     CK(cudaMemcpyAsync(table, host_table, sizeof(int) * 2 * (nc + 1), cudaMemcpyHostToDevice, c->s));
-    launch_chunks(table, table + nc + 1, nc, kChunk, total, chunks, order, c->s);
+    launch_chunks(table, table + nc + 1, nc, kChunk, total, chunks, order, n_other, other, c->s);
     *n_chunks = total;
     return UCP_OK;
 }
@@ -614,7 +615,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     c->host_table = c->host_flags + 3 + 2 * UCP_MAX_CLOUDS;
     // the chunks over every particle follow from the sizes alone
     if ((rc = build_chunks(c, c->cloud_start_h.data(), c->host_table, c->chunk_table, c->chunks_all,
-                           c->order_all, &c->n_chunks_all)))
+                           c->order_all, &c->n_chunks_all, nullptr, 0)))
         return bail(rc);
     if (cudaStreamSynchronize(c->s) || check_launch(c, "create")) return bail(UCP_ECUDA);
     *out = c;
@@ -654,7 +655,7 @@ int ucp_set_state(ucp_ctx* c, const double* pos, const double* vel, const int8_t
     for (int cl = 0; cl < nc; ++cl) first[cl + 1] = first[cl] + fl[2 + cl];
     c->n_e = first[nc];
     int rc = build_chunks(c, first, c->host_table, c->chunk_table, c->chunks_e, c->order_e,
-                          &c->n_chunks_e);
+                          &c->n_chunks_e, c->order_all, c->n_chunks_all);
     if (rc) return rc;
     launch_load_state(dpos, dvel, dsp, c->n, c->st[k], c->sp[k], c->sp_caller, c->id[k], c->s);
     CK(cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s));
