@@ -379,9 +379,10 @@ k_sort_block(const unsigned long long* __restrict__ kin, unsigned long long* __r
     }
 }
 
-// The whole key, when a run was too long: eight LSD passes (a ninth by cloud), runs of
-// equal keys by caller index, and the state, by blocks that meet at a barrier (a
-// cooperative launch; its waits are bounded).  Returns at once when no run was.
+// The whole key, when a run was too long, by blocks that meet at a barrier (a cooperative
+// launch; its waits are bounded): every particle at the place of its caller index first, so
+// that equal keys, however many, come out in that order of the stable passes; then eight
+// LSD passes (a ninth by cloud), and the state.  Returns at once when no run was.
 constexpr int kFullBlocks = 304;
 
 __global__ void __launch_bounds__(kSortThreads)
@@ -424,10 +425,16 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
     const int t0 = (int)((long long)tiles * blockIdx.x / nb), t1 = (int)((long long)tiles * (blockIdx.x + 1) / nb);
     const int lo = t0 * kSortTile, hi = min(n, t1 * kSortTile);
 
-    // the passes' result (k0, v0) is the input; any order would do, ties end by caller
-    // index
-    unsigned long long *ka = k0, *kb = k1;
-    unsigned int *va = v0, *vb = v1;
+    // caller indices are a permutation (after a wait that gave up they may repeat, and leave
+    // a place as it was)
+    for (int i = lo + threadIdx.x; i < hi; i += kSortThreads) {
+        const unsigned int v = v0[i], d = in.id[v];
+        __stcg(k1 + d, k0[i]);
+        __stcg(v1 + d, v);
+    }
+    barrier();
+    unsigned long long *ka = k1, *kb = k0;
+    unsigned int *va = v1, *vb = v0;
     const int passes = 8 + (n_clouds > 1 ? 1 : 0);
     for (int p = 0; p < passes && !lost; ++p) {
         int* cn = counts + (size_t)(p & 1) * kFullBlocks * kRadix;
@@ -494,28 +501,6 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
         va = vb;
         vb = tv;
     }
-    if (lost) return;
-    // equal keys by caller index: the thread at a run's first place sorts it
-    for (int i = lo + threadIdx.x; i < hi && i < n - 1; i += kSortThreads) {
-        const unsigned long long k = __ldcg(ka + i);
-        const auto joins = [&](int j) {
-            return j > 0 && j < n && __ldcg(ka + j) == k && __ldcg(ka + j - 1) == k &&
-                   (!cloud || cloud[j] == cloud[j - 1]);
-        };
-        if (joins(i) || !joins(i + 1)) continue;
-        int e = i + 1;
-        while (joins(e)) ++e;
-        for (int a = i + 1; a < e; ++a) {
-            const unsigned int pv = __ldcg(va + a), idv = in.id[pv];
-            int b = a - 1;
-            while (b >= i && in.id[__ldcg(va + b)] > idv) {
-                __stcg(va + b + 1, __ldcg(va + b));
-                --b;
-            }
-            __stcg(va + b + 1, pv);
-        }
-    }
-    barrier();
     if (lost) return;
     // the sorted keys end in k1 whatever the number of passes
     for (int i = lo + threadIdx.x; i < hi; i += kSortThreads) {
