@@ -184,7 +184,7 @@ void launch_keys(const double* x, const double* y, const double* z, int n, const
 struct SortScratch {
     unsigned long long* status;    // passes x tiles x 256 published words
     int* err;                      // raised by a wait that gave up
-    int* full_counts;              // full sort: 2 x blocks x 256 digit counts
+    int* full_counts;              // full sort: digit counts of its eight passes
     unsigned int* test_epoch;      // tag used by the bounded-wait self-test (1)
     int* test_ctl;                 // its tile counter and 256 zero offsets
     unsigned long long* test_keys; // 4 tiles, for the bounded-wait self-test

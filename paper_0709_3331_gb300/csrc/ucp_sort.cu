@@ -48,61 +48,40 @@ __device__ __forceinline__ void rank_chunk(TileRanks& r, int c, bool ok, int dig
     __syncwarp();
 }
 
-// One stable LSD pass in a single kernel (decoupled look-back).  A block takes
-// the next tile from a counter, ranks its keys stably, and publishes its per-digit
-// count; the digit offset of the tile is the sum of the counts of all earlier tiles,
-// read back through their published words {epoch, flag (1 = count of the tile, 2 =
-// inclusive prefix), value}, on top of the digit's first place: the scan of the digit
-// counts `digits`, or (scan = 0) `digits` itself, its first ndigits valid.  A block
-// waits only on tiles taken before its own, whose blocks are running, and
-// every wait is bounded: past spin_limit polls it raises *err, keeps its keys
-// where they are and leaves (the host reports UCP_ETIMEOUT).
-__global__ void __launch_bounds__(kSortThreads)
-k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __restrict__ vin,
-           unsigned long long* __restrict__ kout, unsigned int* __restrict__ vout, int n,
-           int shift, const int* __restrict__ digits, int scan, int ndigits,
-           unsigned long long* status, int* tile_ctr, const unsigned int* __restrict__ epoch_dev,
-           unsigned int pass, int* err, int spin_limit,
-           const unsigned char* __restrict__ digit_of_val)
+// Shared memory of a pass: keys of a digit in each warp, and whether a wait gave up.
+struct PassShared {
+    int cnt[kSortWarps][kRadix];
+    int fail;
+};
+
+// A tile of one stable LSD pass (decoupled look-back): ranks the tile's keys r stably and
+// publishes the per-digit count; the digit offset of the tile is the sum of the counts of
+// all earlier tiles, read back through their published words {epoch, flag (1 = count of the
+// tile, 2 = inclusive prefix), value}, on top of the digit's first place (thread d: digit
+// d's).  A block waits only on earlier tiles, whose blocks are running, and every wait is
+// bounded: past spin_limit polls it raises *err and leaves its keys where they are (the host
+// reports UCP_ETIMEOUT).  sh.cnt is zero at the start.  kL2: another block of the same launch
+// reads what this one writes.
+template <bool kL2, class Digit>
+__device__ __forceinline__ void place_tile(TileRanks& r, int n, int tile, Digit digit, int first,
+                                           unsigned long long* status, unsigned int epoch, int* err,
+                                           int spin_limit, PassShared& sh,
+                                           unsigned long long* kout, unsigned int* vout)
 {
-    follow();
-    const unsigned int epoch = (*epoch_dev + pass) & 0x3fffffffu;
-    __shared__ int cnt[kSortWarps][kRadix];
-    __shared__ int s_tile, s_fail, s_tot;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        s_tile = atomicAdd(tile_ctr, 1);
-        s_fail = 0;
-    }
-    for (int d = lane; d < kRadix; d += 32) cnt[w][d] = 0;
-    const int dv = (int)threadIdx.x < ndigits ? digits[threadIdx.x] : 0;  // kSortThreads == kRadix
-    __syncthreads();
-    const int tile = s_tile;
     const int base = tile * kSortTile + w * (kSortTile / kSortWarps);
-    TileRanks r;
-#pragma unroll
-    for (int c = 0; c < kSortChunks; ++c) {
-        const int i = base + c * 32 + lane;
-        const bool ok = i < n;
-        r.kk[c] = ok ? kin[i] : 0ull;
-        r.vv[c] = ok ? (vin ? vin[i] : (unsigned int)i) : 0u;
-    }
-    const int first = scan ? block_excl_scan(dv, &s_tot) : dv;
 #pragma unroll
     for (int c = 0; c < kSortChunks; ++c) {
         const bool ok = base + c * 32 + lane < n;
-        // digit: 8 key bits, or (cloud pass) the cloud of the element's previous slot
-        const int d = !ok ? 0 : digit_of_val ? (int)digit_of_val[r.vv[c]]
-                                             : (int)((r.kk[c] >> shift) & 0xffu);
-        rank_chunk(r, c, ok, d, cnt[w], lane);
+        rank_chunk(r, c, ok, ok ? digit(r.kk[c], r.vv[c]) : 0, sh.cnt[w], lane);
     }
     __syncthreads();
     {
         const int d = threadIdx.x;
         int total = 0;
         for (int ww = 0; ww < kSortWarps; ++ww) {
-            int t = cnt[ww][d];
-            cnt[ww][d] = total;
+            int t = sh.cnt[ww][d];
+            sh.cnt[ww][d] = total;
             total += t;
         }
         const unsigned long long tag = (unsigned long long)epoch << 34;
@@ -139,7 +118,7 @@ k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __res
                 if (blocked) {
                     if (++spins > spin_limit) {
                         atomicOr(err, 1);
-                        s_fail = 1;
+                        sh.fail = 1;
                         break;
                     }
                     __nanosleep(64);
@@ -148,19 +127,65 @@ k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __res
         }
         atomicExch(mine, tag | (2ull << 32) | (prefix + (unsigned int)total));
         const int off = first + (int)prefix;
-        for (int ww = 0; ww < kSortWarps; ++ww) cnt[ww][d] += off;
+        for (int ww = 0; ww < kSortWarps; ++ww) sh.cnt[ww][d] += off;
     }
     __syncthreads();
-    const bool fail = s_fail != 0;
+    const bool fail = sh.fail != 0;
 #pragma unroll
     for (int c = 0; c < kSortChunks; ++c) {
         const int i = base + c * 32 + lane;
         if (i < n) {
-            const int p = fail ? i : cnt[w][r.dig[c]] + r.rank[c];
-            kout[p] = r.kk[c];
-            vout[p] = r.vv[c];
+            const int p = fail ? i : sh.cnt[w][r.dig[c]] + r.rank[c];
+            if (kL2) {
+                __stcg(kout + p, r.kk[c]);
+                __stcg(vout + p, r.vv[c]);
+            } else {
+                kout[p] = r.kk[c];
+                vout[p] = r.vv[c];
+            }
         }
     }
+}
+
+// One pass: a block takes the next tile from a counter.  A digit's first place is the scan of
+// the digit counts `digits`, or (scan = 0) `digits` itself, its first ndigits valid.
+__global__ void __launch_bounds__(kSortThreads)
+k_onesweep(const unsigned long long* __restrict__ kin, const unsigned int* __restrict__ vin,
+           unsigned long long* __restrict__ kout, unsigned int* __restrict__ vout, int n,
+           int shift, const int* __restrict__ digits, int scan, int ndigits,
+           unsigned long long* status, int* tile_ctr, const unsigned int* __restrict__ epoch_dev,
+           unsigned int pass, int* err, int spin_limit,
+           const unsigned char* __restrict__ digit_of_val)
+{
+    follow();
+    const unsigned int epoch = (*epoch_dev + pass) & 0x3fffffffu;
+    __shared__ PassShared sh;
+    __shared__ int s_tile, s_tot;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        s_tile = atomicAdd(tile_ctr, 1);
+        sh.fail = 0;
+    }
+    for (int d = lane; d < kRadix; d += 32) sh.cnt[w][d] = 0;
+    const int dv = (int)threadIdx.x < ndigits ? digits[threadIdx.x] : 0;  // kSortThreads == kRadix
+    __syncthreads();
+    const int tile = s_tile;
+    const int base = tile * kSortTile + w * (kSortTile / kSortWarps);
+    TileRanks r;
+#pragma unroll
+    for (int c = 0; c < kSortChunks; ++c) {
+        const int i = base + c * 32 + lane;
+        const bool ok = i < n;
+        r.kk[c] = ok ? kin[i] : 0ull;
+        r.vv[c] = ok ? (vin ? vin[i] : (unsigned int)i) : 0u;
+    }
+    const int first = scan ? block_excl_scan(dv, &s_tot) : dv;
+    // digit: 8 key bits, or (cloud pass) the cloud of the element's previous slot
+    place_tile<false>(r, n, tile,
+                      [&](unsigned long long k, unsigned int v) {
+                          return digit_of_val ? (int)digit_of_val[v] : (int)((k >> shift) & 0xffu);
+                      },
+                      first, status, epoch, err, spin_limit, sh, kout, vout);
 }
 
 // Orders the runs of equal top digits by (key, caller index) and moves the state.  A
@@ -379,24 +404,32 @@ k_sort_block(const unsigned long long* __restrict__ kin, unsigned long long* __r
     }
 }
 
-// The whole key, when a run was too long, by blocks that meet at a barrier (a cooperative
-// launch; its waits are bounded): every particle at the place of its caller index first, so
-// that equal keys, however many, come out in that order of the stable passes; then eight
-// LSD passes (a ninth by cloud), and the state.  Returns at once when no run was.
-constexpr int kFullBlocks = 304;
+// The whole key, when a run was too long, by resident blocks that meet at a barrier after
+// every pass (a cooperative launch; its waits are bounded).  Every particle goes to the place
+// of its caller index first, so that equal keys, however many, come out in that order of the
+// stable passes, and all passes' digits are counted on the way; then eight LSD passes (a
+// ninth by cloud) as in k_onesweep, a block taking every gridDim-th tile, and the state.
+// Returns at once when no run was.  A build with a particle at 100, 1000 and 1e5 sigma takes
+// 385, 348 and 342 us at N = 524,288 and 2.58, 2.45 and 2.08 ms at 4,194,304 (204 us and 1.41
+// ms without it); with a block per SM, a pass over the keys for each digit's counts and runs
+// of equal keys ordered by one thread each it took 433, 391 and 575 us, 3.15, 3.07 and 5.13
+// ms, and sorting every key by eight passes in each build 410, 430 and 447 us, 2.27, 2.50
+// and 2.33 ms (396 us and 2.42 ms without the particle).
+constexpr int kFullPasses = 8;
+constexpr int kFullPerSM = 2;        // resident blocks, which the register budget allows
 
-__global__ void __launch_bounds__(kSortThreads)
+__global__ void __launch_bounds__(kSortThreads, kFullPerSM)
 k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, unsigned int* v1,
-            int n, int n_clouds, int* ctl, int* counts,
-            int* err, StateRef in, StateRef out, const unsigned char* __restrict__ cloud)
+            int n, int n_clouds, int* ctl, const unsigned int* __restrict__ epoch_dev, int* counts,
+            unsigned long long* status, int* err, StateRef in, StateRef out,
+            const unsigned char* __restrict__ cloud, const int* __restrict__ cloud_start)
 {
     follow();
     if (ctl[kCtlLong] == 0) return;
-    __shared__ int cnt[kSortWarps][kRadix];
-    __shared__ int s_base[kRadix];
+    __shared__ PassShared sh;
     __shared__ int s_tot;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nb = gridDim.x;
+    const int stride = gridDim.x * kSortThreads, at = blockIdx.x * kSortThreads + threadIdx.x;
     int met = 0;
     bool lost = false;
     auto barrier = [&]() {
@@ -406,7 +439,7 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
             atomicAdd(&ctl[kCtlBarrier], 1);
             ++met;
             int spins = 0;
-            while (*(volatile int*)&ctl[kCtlBarrier] < met * nb) {
+            while (*(volatile int*)&ctl[kCtlBarrier] < met * (int)gridDim.x) {
                 if (++spins > (kSortSpinLimit << 3)) {
                     atomicOr(err, 1);
                     break;
@@ -420,49 +453,41 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
         lost = s_tot != 0;
         __syncthreads();
     };
-    // a block's contiguous part, in whole tiles
-    const int tiles = (n + kSortTile - 1) / kSortTile;
-    const int t0 = (int)((long long)tiles * blockIdx.x / nb), t1 = (int)((long long)tiles * (blockIdx.x + 1) / nb);
-    const int lo = t0 * kSortTile, hi = min(n, t1 * kSortTile);
-
+    if (threadIdx.x == 0) sh.fail = 0;
+    for (int i = at; i < kFullPasses * kRadix; i += stride) __stcg(counts + i, 0);
+    barrier();
+    if (lost) return;
     // caller indices are a permutation (after a wait that gave up they may repeat, and leave
     // a place as it was)
-    for (int i = lo + threadIdx.x; i < hi; i += kSortThreads) {
+    static_assert(kFullPasses == kSortWarps, "sh.cnt holds the counts of every pass");
+    for (int d = lane; d < kRadix; d += 32) sh.cnt[w][d] = 0;
+    __syncthreads();
+    for (int i = at; i < n; i += stride) {
+        const unsigned long long k = k0[i];
         const unsigned int v = v0[i], d = in.id[v];
-        __stcg(k1 + d, k0[i]);
+        __stcg(k1 + d, k);
         __stcg(v1 + d, v);
+#pragma unroll
+        for (int p = 0; p < kFullPasses; ++p) atomicAdd(&sh.cnt[p][(unsigned int)(k >> (8 * p)) & 0xffu], 1);
+    }
+    __syncthreads();
+    for (int p = 0; p < kFullPasses; ++p) {
+        const int c = sh.cnt[p][threadIdx.x];
+        if (c) atomicAdd(counts + p * kRadix + threadIdx.x, c);
     }
     barrier();
     unsigned long long *ka = k1, *kb = k0;
     unsigned int *va = v1, *vb = v0;
-    const int passes = 8 + (n_clouds > 1 ? 1 : 0);
+    const int tiles = (n + kSortTile - 1) / kSortTile;
+    const int passes = kFullPasses + (n_clouds > 1 ? 1 : 0);
     for (int p = 0; p < passes && !lost; ++p) {
-        int* cn = counts + (size_t)(p & 1) * kFullBlocks * kRadix;
-        for (int d = threadIdx.x; d < kRadix; d += kSortThreads) s_base[d] = 0;
-        __syncthreads();
-        auto digit = [&](unsigned long long k, unsigned int v) {
-            return p == 8 ? (int)cloud[v] : (int)((k >> (8 * p)) & 0xffu);
-        };
-        for (int i = lo + threadIdx.x; i < hi; i += kSortThreads)
-            atomicAdd(&s_base[digit(__ldcg(ka + i), __ldcg(va + i))], 1);
-        __syncthreads();
-        __stcg(cn + (size_t)blockIdx.x * kRadix + threadIdx.x, s_base[threadIdx.x]);
-        barrier();
-        if (lost) break;
-        {
-            int tot = 0, mine = 0;
-            for (int b = 0; b < nb; ++b) {
-                const int c = __ldcg(cn + (size_t)b * kRadix + threadIdx.x);
-                if (b < (int)blockIdx.x) mine += c;
-                tot += c;
-            }
-            const int first = block_excl_scan(tot, &s_tot);
-            s_base[threadIdx.x] = first + mine;
-        }
-        for (int tile = t0; tile < t1; ++tile) {
-            __syncthreads();
-            for (int d = lane; d < kRadix; d += 32) cnt[w][d] = 0;
-            __syncwarp();
+        // tags of their own, after those of the passes over the top digits
+        const unsigned int epoch = (*epoch_dev + kSortPassesMax + 1 + p) & 0x3fffffffu;
+        const int first = p < kFullPasses
+                              ? block_excl_scan(__ldcg(counts + p * kRadix + threadIdx.x), &s_tot)
+                              : (int)threadIdx.x < n_clouds ? cloud_start[threadIdx.x] : 0;
+        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+            for (int d = lane; d < kRadix; d += 32) sh.cnt[w][d] = 0;
             const int base = tile * kSortTile + w * (kSortTile / kSortWarps);
             TileRanks r;
 #pragma unroll
@@ -471,27 +496,15 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
                 const bool ok = i < n;
                 r.kk[c] = ok ? __ldcg(ka + i) : 0ull;
                 r.vv[c] = ok ? __ldcg(va + i) : 0u;
-                rank_chunk(r, c, ok, ok ? digit(r.kk[c], r.vv[c]) : 0, cnt[w], lane);
             }
+            __syncwarp();
+            place_tile<true>(r, n, tile,
+                             [&](unsigned long long k, unsigned int v) {
+                                 return p == kFullPasses ? (int)cloud[v]
+                                                         : (int)((k >> (8 * p)) & 0xffu);
+                             },
+                             first, status, epoch, err, kSortSpinLimit, sh, kb, vb);
             __syncthreads();
-            {
-                int run = s_base[threadIdx.x];
-                for (int ww = 0; ww < kSortWarps; ++ww) {
-                    const int c = cnt[ww][threadIdx.x];
-                    cnt[ww][threadIdx.x] = run;
-                    run += c;
-                }
-                s_base[threadIdx.x] = run;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int c = 0; c < kSortChunks; ++c) {
-                if (base + c * 32 + lane < n) {
-                    const int q = cnt[w][r.dig[c]] + r.rank[c];
-                    __stcg(kb + q, r.kk[c]);
-                    __stcg(vb + q, r.vv[c]);
-                }
-            }
         }
         barrier();
         unsigned long long* tk = ka;
@@ -503,7 +516,7 @@ k_sort_full(unsigned long long* k0, unsigned long long* k1, unsigned int* v0, un
     }
     if (lost) return;
     // the sorted keys end in k1 whatever the number of passes
-    for (int i = lo + threadIdx.x; i < hi; i += kSortThreads) {
+    for (int i = at; i < n; i += stride) {
         if (ka != k1) k1[i] = __ldcg(ka + i);
         move_state(in, out, i, __ldcg(va + i));
     }
@@ -520,7 +533,7 @@ int sort_passes(int64_t largest_cloud)
 }
 
 size_t sort_test_words() { return 4 * (size_t)kSortTile; }
-size_t sort_full_words() { return 2 * (size_t)kFullBlocks * kRadix; }
+size_t sort_full_words() { return (size_t)kFullPasses * kRadix; }
 
 size_t sort_status_words(int n)
 {
@@ -566,14 +579,14 @@ int launch_sort(unsigned long long* key[2], unsigned int* val[2], int n, int pas
     const int fin = cur ^ 1;
     launch(k_finish_sort, (n + kFinish - 1) / kFinish, kFinish, s, key[cur], val[cur],
            key[fin], n, low, in, out, cloud, ctl.words + kCtlLong);
-    unsigned long long *k0 = key[cur], *k1 = key[fin];
-    unsigned int *v0 = val[cur], *v1 = val[fin];
+    unsigned long long *k0 = key[cur], *k1 = key[fin], *status = sc.status;
+    unsigned int *v0 = val[cur], *v1 = val[fin], *epoch = ctl.epoch;
     int* words = ctl.words;
     int *counts = sc.full_counts, *err = sc.err;
     StateRef si = in, so = out;
-    void* args[] = {&k0, &k1, &v0, &v1, &n, &n_clouds, &words, &counts, &err, &si, &so, &cloud};
-    int blocks = nb < kFullBlocks ? nb : kFullBlocks;
-    if (blocks > nsm) blocks = nsm;
+    void* args[] = {&k0, &k1, &v0, &v1, &n, &n_clouds, &words, &epoch, &counts,
+                    &status, &err, &si, &so, &cloud, &cloud_start};
+    const int blocks = nb < kFullPerSM * nsm ? nb : kFullPerSM * nsm;
     cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_sort_full), dim3(blocks),
                                 dim3(kSortThreads), args, 0, s);
     return fin;
