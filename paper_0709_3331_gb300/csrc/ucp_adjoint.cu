@@ -57,6 +57,7 @@ k_walk_adjoint(WalkArgs a, const double* __restrict__ lam, double* __restrict__ 
     __shared__ WalkWarp W;
     const int lane = threadIdx.x;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
+    const int gave_up = *a.err;
 
     while (true) {
         const unsigned int item = (unsigned int)next_chunk(a.work, lane);
@@ -138,7 +139,7 @@ k_walk_adjoint(WalkArgs a, const double* __restrict__ lam, double* __restrict__ 
             __syncwarp();
         };
 
-        walk_lists(a, W, 1u, ck.z,
+        walk_lists(a, gave_up, W, 1u, ck.z,
                    [&](int box, unsigned int, const float4 h) {
                        return box >= 0 && tg.accepts(a, box, h) ? 1u : 0u;
                    },
@@ -242,6 +243,7 @@ k_walk_adjoint_f32(WalkArgs a, int group, const double* __restrict__ lam,
     const float2 e2 = splat((float)a.eps2);
 
     const int per = 32 / group;
+    const int gave_up = *a.err;
     while (true) {
         const unsigned int item = (unsigned int)next_chunk(a.work, lane);
         if (item >= (unsigned int)a.nchunks * per) break;
@@ -455,7 +457,7 @@ k_walk_adjoint_f32(WalkArgs a, int group, const double* __restrict__ lam,
             __syncwarp();
         };
 
-        walk_lists(a, W.walk, tg, ck.z, multipoles, direct_pairs);
+        walk_lists(a, gave_up, W.walk, tg, ck.z, multipoles, direct_pairs);
 
         // value L / 2 of a group: components of target (L / 2) / 3 of its four
         const int term = lane >> 1;
@@ -488,6 +490,7 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
         double A[3] = {0, 0, 0}, G[6] = {0, 0, 0, 0, 0, 0}, Cc[3] = {0, 0, 0}, K[3] = {0, 0, 0};
         for (int nd = leaf, up; nd >= 0; nd = up) {
             up = t.info[nd].w;
+            if (up >= nd) up = -1;      // a parent comes before its child: the loop ends
             double r[12];
             for (int k = 0; k < 12; ++k) r[k] = (double)adj[(size_t)nd * 12 + k];
             const double* m = t.mom + (size_t)nd * kMom;

@@ -664,7 +664,10 @@ template <class Combine>
 __device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combine)
 {
     const int lane = threadIdx.x & 31;
-    Twig w = load_twig(t, node >= 0 ? t.info[node].w : -1);
+    // (a parent comes before its child: the sweep ends, also in tables that are no tree since
+    // a wait gave up)
+    int p = node >= 0 ? t.info[node].w : -1;
+    Twig w = load_twig(t, p < node ? p : -1);
     while (__any_sync(0xffffffffu, w.id >= 0)) {
         // this box's records (written by any lane of the warp) are published with its
         // arrival; the last arrival sees every sibling's
@@ -674,7 +677,7 @@ __device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combin
         // what the acquiring lanes see, every lane sees.  The next twig's records come in
         // while this one is combined.
         __syncwarp();
-        const Twig up = load_twig(t, ready ? w.parent : -1);
+        const Twig up = load_twig(t, ready && w.parent < w.id ? w.parent : -1);
         int4 lc;
         if (ready) lc = __ldcg(&t.info[max(w.last, 0)]);
         while (todo) {
@@ -932,7 +935,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                                      kPos + kMomHalo) : 0;
         for (int k = first + threadIdx.x; k < end; k += kThreads) {
             const int j = base + k;
-            if (owner[k] == kNoOwner) continue;
+            if (owner[k] >= nl) continue;    // none, or a place that no leaf of the block covers
             const double* zc = ctr[owner[k]];
             ys[k] = make_float4((float)(x[j] - zc[0]), (float)(y[j] - zc[1]), (float)(z[j] - zc[2]),
                                 sp[j] ? q1 : q0);
@@ -983,7 +986,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
         __syncthreads();
         for (int k = first + threadIdx.x; k < end; k += kThreads) {
             const int j = base + k, l = owner[k];
-            if (l == kNoOwner) continue;
+            if (l >= nl) continue;
             const double* c = ctr[l];
             put_source(f, place[l], list[l], j, (float)(c[0] - x[j]), (float)(c[1] - y[j]),
                        (float)(c[2] - z[j]), ys[k].w);

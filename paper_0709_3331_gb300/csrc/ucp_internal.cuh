@@ -264,7 +264,7 @@ struct WalkArgs {
     double* ax; double* ay; double* az; double* phi;  // key order; phi may be NULL
     int* cnt_p2p; int* cnt_m2p;                        // key order
     int* work;              // dynamic work counter (zeroed before launch)
-    int* err;               // raised by a bounded wait that gave up
+    const int* err;         // raised by a bounded wait that gave up: the tree is not walked
     unsigned long long* stats; // {p2p, m2p}
 };
 // per walk: box records (in an FP64 context also the moments, where they are still the sums

@@ -15,6 +15,15 @@ __device__ __forceinline__ int next_chunk(int* work, int lane)
     return __shfl_sync(0xffffffffu, c, 0);
 }
 
+// The first box of a walk, in lane 0 (-1 elsewhere): the root of the targets' cloud, or
+// none once a wait of the build gave up.  The tables are then no tree (children of several
+// parents, leaves that end before they begin), and the walks' stacks hold only a tree's.
+// gave_up: *a.err, which a kernel reads once at its start.
+__device__ __forceinline__ int first_box(const WalkArgs& a, int gave_up, int cloud, int lane)
+{
+    return lane == 0 && !gave_up ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[cloud] : 0] : -1;
+}
+
 // Twigs on the stack: up to kPopWide + 28 while four are popped per step; above
 // kPopWide one is popped per step, which adds at most 7 per level below it.
 constexpr int kPopWide = 64;
@@ -247,15 +256,15 @@ __device__ __forceinline__ unsigned int accept_mask(const WalkArgs& a, float* st
 // targets that open it}; all are called by the whole warp and may use W.stage, the last two
 // their part of the list.
 template <class Accept, class Boxes, class Pairs>
-__device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, unsigned int targets,
-                                           int cloud, Accept accept, Boxes& multipoles,
+__device__ __forceinline__ void walk_lists(const WalkArgs& a, int gave_up, WalkWarp& W,
+                                           unsigned int targets, int cloud, Accept accept, Boxes& multipoles,
                                            Pairs& direct_pairs)
 {
     const int lane = threadIdx.x & 31;
     const unsigned int lt = (1u << lane) - 1u;
     int top = 0, na = 0, nl = 0;
     // the first step tests the root for every target
-    int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[cloud] : 0] : -1;
+    int box = first_box(a, gave_up, cloud, lane);
     unsigned int mask = targets;
     while (true) {
         const bool has = box >= 0;
@@ -304,10 +313,11 @@ __device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, unsig
 
 // The same for a chunk's targets, one per lane.
 template <class Boxes, class Pairs>
-__device__ __forceinline__ void walk_lists(const WalkArgs& a, WalkWarp& W, const ChunkTarget& tg,
-                                           int cloud, Boxes& multipoles, Pairs& direct_pairs)
+__device__ __forceinline__ void walk_lists(const WalkArgs& a, int gave_up, WalkWarp& W,
+                                           const ChunkTarget& tg, int cloud, Boxes& multipoles,
+                                           Pairs& direct_pairs)
 {
-    walk_lists(a, W, __ballot_sync(0xffffffffu, tg.t >= 0), cloud,
+    walk_lists(a, gave_up, W, __ballot_sync(0xffffffffu, tg.t >= 0), cloud,
                [&](int box, unsigned int mask, const float4 h) {
                    return accept_mask(a, W.stage, tg, box, mask, h);
                },

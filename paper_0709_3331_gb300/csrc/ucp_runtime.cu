@@ -594,9 +594,13 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
                 cl[j] = (unsigned char)i;
     }
     const double mqm[4] = {c->m[0], c->m[1], c->q[0] / c->m[0], c->q[1] / c->m[1]};
-    // box tables a build has not filled are read only after a wait that gave up: empty
+    // box tables and slots a build has not filled are read only after a wait that gave up:
+    // empty
     if (cudaMemsetAsync(c->t.info, 0, sizeof(int4) * cz, c->s) ||
         cudaMemsetAsync(c->t.child8, 0xff, 8 * sizeof(int) * cz, c->s) ||
+        cudaMemsetAsync(c->val[0], 0, sizeof(unsigned int) * n, c->s) ||
+        cudaMemsetAsync(c->val[1], 0, sizeof(unsigned int) * n, c->s) ||
+        cudaMemsetAsync(c->t.depth_leaf, 0, sizeof(int) * cz, c->s) ||
         cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) ||
         cudaMemsetAsync(c->topo_status, 0, 8 * topo_status_words(c->n), c->s) ||
         cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) ||

@@ -61,6 +61,7 @@ k_walk_fp64(WalkArgs a)
     const int lane = threadIdx.x;
     const unsigned int lt = (1u << lane) - 1u;
     const double q0 = a.qsp[0], q1 = a.qsp[1];
+    const int gave_up = *a.err;
     const float4* __restrict__ H = a.t.hdr;
     const double* __restrict__ X = a.x;
     const double* __restrict__ Y = a.y;
@@ -146,7 +147,7 @@ k_walk_fp64(WalkArgs a)
             np += __popc(__ballot_sync(0xffffffffu, j != t));
         };
 
-        int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0] : -1;
+        int box = first_box(a, gave_up, ck.z, lane);
         while (true) {
             const bool has = box >= 0;
             const float4 h = has ? __ldg(H + box) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -551,6 +552,7 @@ k_walk_fp32c(WalkArgs a)
     __shared__ WalkWarp shared[kThreads / 32];
     const int lane = threadIdx.x & 31;
     WalkWarp& W = shared[threadIdx.x >> 5];
+    const int gave_up = *a.err;
 
     for (int item = next_chunk(a.work, lane); item < a.nchunks;
          item = next_chunk(a.work, lane)) {
@@ -580,7 +582,7 @@ k_walk_fp32c(WalkArgs a)
                                      });
         };
 
-        walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
+        walk_lists(a, gave_up, W, tg, ck.z, multipoles, direct_pairs);
 
         write_target<kPhi>(a, t, sxy, cxy, szp, czp, np, nm);
         if (lane == 0) {
@@ -623,6 +625,7 @@ k_walk_fp32c_split(WalkArgs a)
     extern __shared__ __align__(16) unsigned char split_bytes[];
     SplitShared<kWays>& sh = *reinterpret_cast<SplitShared<kWays>*>(split_bytes);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int gave_up = *a.err;
     const long long began = clock64();
     const int chunk = a.ord.order[blockIdx.x];
     const int4 ck = a.chunks[chunk];
@@ -662,7 +665,7 @@ k_walk_fp32c_split(WalkArgs a)
                                              });
                 });
         };
-        walk_lists(a, W, tg, ck.z, multipoles, direct_pairs);
+        walk_lists(a, gave_up, W, tg, ck.z, multipoles, direct_pairs);
         sh.counts[w][lane] = make_int2(np, nm);
         if (threadIdx.x == 0) sh.filled[round & 1] = ~(task & (kWays - 1));
         meet();
@@ -804,6 +807,7 @@ k_walk_fp32c_visits(WalkArgs a)
     const bool traverses = threadIdx.x < 32, sums = !kTwo || threadIdx.x >= 32;
     const float4* __restrict__ H = a.t.hdr;
     const float eps2 = (float)a.eps2;
+    const int gave_up = *a.err;
 
     while (true) {
         if (threadIdx.x == 0) sh.item = atomicAdd(a.work, 1);
@@ -885,7 +889,7 @@ k_walk_fp32c_visits(WalkArgs a)
                 if (late) given += kVisitList;
             };
             int top = 0;
-            int box = lane == 0 ? a.pos_off[a.t.cloud_start ? a.t.cloud_start[ck.z] : 0] : -1;
+            int box = first_box(a, gave_up, ck.z, lane);
             unsigned int mask = __ballot_sync(0xffffffffu, t >= 0);
             while (true) {
                 // the boxes that follow, first on top: {box, accepting, opening targets, leaf}
