@@ -483,6 +483,7 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
                                const TA* __restrict__ adj, double* __restrict__ mu)
 {
     follow();
+    constexpr bool kFp32 = sizeof(TA) == sizeof(float);     // FP32C contexts
     const int nn = *t.nnodes;
     for (int leaf = blockIdx.x * blockDim.x + threadIdx.x; leaf < nn;
          leaf += gridDim.x * blockDim.x) {
@@ -493,11 +494,11 @@ __global__ void k_adjoint_push(const double* __restrict__ x, const double* __res
             if (up >= nd) up = -1;      // a parent comes before its child: the loop ends
             double r[12];
             for (int k = 0; k < 12; ++k) r[k] = (double)adj[(size_t)nd * 12 + k];
-            const double* m = t.mom + (size_t)nd * kMom;
+            const double* m = t.mom + (size_t)nd * (kFp32 ? kCentre : kMom);
             double c[3] = {m[MC], m[MC + 1], m[MC + 2]};
             double Gc[3];
             qmul(r + 3, c, Gc);
-            const double S0 = t.mom32 ? (double)t.mom32[(size_t)nd * 16 + 3] : m[MS0];
+            const double S0 = kFp32 ? (double)t.mom32[(size_t)nd * 16 + 3] : m[MS0];
             const double inv = S0 > 0.0 ? 1.0 / S0 : 0.0;
             for (int k = 0; k < 3; ++k) {
                 A[k] += r[k];

@@ -867,7 +867,7 @@ __device__ __forceinline__ void twig_combine_f32(const Cube* __restrict__ cube, 
     for (int k = 0; k < 14; ++k) a[k] = sum8(a[k]);
     if (w.id >= 0 && o == 0) {
         float m32[16];
-        finish_box_f32(a, zp, m32, t.mom + (size_t)w.id * kMom, t.delta + w.id);
+        finish_box_f32(a, zp, m32, t.mom + (size_t)w.id * kCentre, t.delta + w.id);
         float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)w.id * 16);
         for (int k = 0; k < 4; ++k)
             w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
@@ -970,7 +970,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                 a[13] = fmaf(qj * yv[2], yv[2], a[13]);
             }
             float m32[16];
-            double* m = t.mom + (size_t)node * kMom;
+            double* m = t.mom + (size_t)node * kCentre;
             double zc[3] = {ctr[l][0], ctr[l][1], ctr[l][2]};
             double c64[3];
             finish_box_f32(a, zc, m32, c64, t.delta + node);
@@ -1026,7 +1026,7 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                     a[13] = fmaf(qj * yv[2], yv[2], a[13]);
                 }
                 float m32[16];
-                double* m = t.mom + (size_t)node * kMom;
+                double* m = t.mom + (size_t)node * kCentre;
                 finish_box_f32(a, zc, m32, m, t.delta + node);
                 float4* r32 = reinterpret_cast<float4*>(t.mom32 + (size_t)node * 16);
                 for (int k = 0; k < 4; ++k)

@@ -91,13 +91,13 @@ __device__ __forceinline__ void follow()
 
 // One FP64 box record, 16 doubles (128 B), read by the FP64 walk.
 // {c.x, c.y, c.z, rcrit2, M, D.x, D.y, D.z, Qxx, Qxy, Qxz, Qyy, Qyz, Qzz, S0, -tr(Q)/2}
-// (FP32C contexts: c and rcrit2 only, the rest in mom32)
+// FP32C contexts: the first kCentre of them, c and rcrit2 (the rest is in mom32).
 // rcrit2 = (s/theta + delta)^2 is filled per walk (it depends on theta).  Until its first
 // walk an FP64 tree holds in the same place each box's sums about its geometric centre,
 // {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)}, and kSumsDelta as the box's delta.
 // The mark is the record's own, on the device, so that a captured sequence of launches
 // finds the records as they are whenever it is replayed.
-constexpr int kMom = 16;
+constexpr int kMom = 16, kCentre = 4;
 constexpr double kSumsDelta = -1.0;
 enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
 
@@ -132,7 +132,7 @@ struct Tree {
     int4* info;              // {begin, end, next, parent}
     int* depth_leaf;         // depth | leaf << 8
     unsigned long long* cell;// key prefix of the box at its depth
-    double* mom;             // kMom doubles per box
+    double* mom;             // kMom doubles per box (FP32C contexts: kCentre)
     double* delta;           // |centroid - geometric centre| per box
     float4* hdr;             // traversal record per box
     float4* lo;              // FP32C contexts: low part of the centroid, next

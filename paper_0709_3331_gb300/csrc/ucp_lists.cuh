@@ -234,10 +234,10 @@ __device__ __forceinline__ unsigned int accept_mask(const WalkArgs& a, float* st
             const bool again0 = in0 && !(fabsf(dm.x) > win.x);
             const bool again1 = in1 && !(fabsf(dm.y) > win.y);
             if (again0)
-                acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kMom, a.x + tg.t,
+                acc0 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.x) * kCentre, a.x + tg.t,
                                     a.y + tg.t, a.z + tg.t);
             if (again1)
-                acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kMom, a.x + tg.t,
+                acc1 = accepts_fp64(a.t.mom + (size_t)__float_as_int(f2.y) * kCentre, a.x + tg.t,
                                     a.y + tg.t, a.z + tg.t);
             const unsigned int am0 = __ballot_sync(0xffffffffu, acc0);
             const unsigned int am1 = __ballot_sync(0xffffffffu, acc1);

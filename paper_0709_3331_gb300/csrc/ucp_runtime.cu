@@ -525,7 +525,7 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->t.info, cz);
     dalloc(c, &c->t.depth_leaf, cz);
     dalloc(c, &c->t.cell, cz);
-    dalloc(c, &c->t.mom, cz * kMom);
+    dalloc(c, &c->t.mom, cz * (c->precision == UCP_FP32C ? kCentre : kMom));
     dalloc(c, &c->t.delta, cz);
     dalloc(c, &c->t.hdr, cz);
     dalloc(c, &c->t.child8, cz * 8);
@@ -1376,8 +1376,9 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
     std::vector<int4> info(nn);
     std::vector<int> dl(nn);
     std::vector<unsigned long long> cell(nn);
-    std::vector<double> mom((size_t)nn * kMom), delta(nn);
     const bool f32 = c->precision == UCP_FP32C;
+    const int stride = f32 ? kCentre : kMom;
+    std::vector<double> mom((size_t)nn * stride), delta(nn);
     std::vector<float> mom32(f32 ? (size_t)nn * 16 : 0);
     if (f32)
         CK(cudaMemcpyAsync(mom32.data(), c->t.mom32, sizeof(float) * 16 * nn, cudaMemcpyDeviceToHost,
@@ -1385,7 +1386,7 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
     CK(cudaMemcpyAsync(info.data(), c->t.info, sizeof(int4) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(dl.data(), c->t.depth_leaf, sizeof(int) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaMemcpyAsync(cell.data(), c->t.cell, 8 * (size_t)nn, cudaMemcpyDeviceToHost, c->s));
-    CK(cudaMemcpyAsync(mom.data(), c->t.mom, sizeof(double) * kMom * nn, cudaMemcpyDeviceToHost,
+    CK(cudaMemcpyAsync(mom.data(), c->t.mom, sizeof(double) * stride * nn, cudaMemcpyDeviceToHost,
                        c->s));
     CK(cudaMemcpyAsync(delta.data(), c->t.delta, sizeof(double) * nn, cudaMemcpyDeviceToHost, c->s));
     CK(cudaStreamSynchronize(c->s));
@@ -1412,7 +1413,8 @@ int ucp_get_tree(ucp_ctx* c, int64_t* nnodes, int64_t cap, int32_t* topo, int8_t
                 g[a] = lo + off;
             }
             g[3] = s;
-            double* m = mom.data() + (size_t)i * kMom;
+            double m[kMom];
+            std::copy_n(mom.data() + (size_t)i * stride, stride, m);
             if (f32) {  // {e xyz, S0, M, D, Q}
                 const float* r = mom32.data() + (size_t)i * 16;
                 m[MS0] = r[3];

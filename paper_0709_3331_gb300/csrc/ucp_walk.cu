@@ -966,7 +966,7 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
     }
     const int nn = *t.nnodes;
     for (int nd = blockIdx.x * blockDim.x + threadIdx.x; nd < nn; nd += gridDim.x * blockDim.x) {
-        double* m = t.mom + (size_t)nd * kMom;
+        double* m = t.mom + (size_t)nd * (kFp64 ? kMom : kCentre);
         int dl = t.depth_leaf[nd];
         const Cube& cb = cube[t.cloud ? t.cloud[t.info[nd].x] : 0];
         const double L = cb.L;
