@@ -105,7 +105,7 @@ enum MomIdx { MC = 0, MR2 = 3, MM = 4, MD = 5, MQ = 8, MS0 = 14, MT = 15 };
 //   hdr = {-ch.x, -ch.y, -ch.z, +-rcrit2}   ch = fp32(c) relative to the cube's centre;
 //                                           the sign bit of rcrit2 marks a leaf
 // and, in FP32C contexts, read only for boxes that act or are opened,
-//   lo  = {-cl.x, -cl.y, -cl.z, bits(next)} cl = fp32(c - ch)
+//   lo  = {-cl.x, -cl.y, -cl.z, 0}          cl = fp32(c - ch)
 //   rec = {-ch.x, -ch.y, -ch.z, M}, {D.x, D.y, D.z, -tr(Q)/2}, {Qxx, Qxy, Qxz, Qyy} / 2,
 //         {Qyz / 2, Qzz / 2, -M, 0}         64 B: four lanes load one box
 constexpr int kRec = 4;
@@ -135,7 +135,7 @@ struct Tree {
     double* mom;             // kMom doubles per box (FP32C contexts: kCentre)
     double* delta;           // |centroid - geometric centre| per box
     float4* hdr;             // traversal record per box
-    float4* lo;              // FP32C contexts: low part of the centroid, next
+    float4* lo;              // FP32C contexts: low part of the centroid
     float4* rec;             // FP32C contexts: kRec float4 per box
     float* mom32;            // FP32C contexts: 16 floats per box {e xyz, S0, M, D, Q, 0, 0}
     int* child8;             // 8 child slots per box (octant order), -1 = empty

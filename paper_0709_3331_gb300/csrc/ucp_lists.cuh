@@ -37,8 +37,7 @@ constexpr int kStack = kPopWide + 28 + 7 * (kMaxDepth - 1) + 8;
 // rounded to 26 bits so that its square is exact, starts the second step, whose factor
 // 1/2 + 3/8 e follows from the rounding's remainder (e = 2 rem / y).  Close to
 // correctly rounded (at most 1.0 x 2^-53 off, rms as the library's); 8 % of a walk
-// against the library's rsqrt and its six (block of 10 steps at N = 131,072: 86.9 -> 79.5
-// ms).  Arguments outside [2^-60, 2^100) go to the library.
+// against rsqrt() (block of 10 steps at N = 131,072: 86.9 -> 79.5 ms).  Arguments outside [2^-60, 2^100) go to the library.
 __device__ __forceinline__ double rsqrt_fp64(double x)
 {
     const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);

@@ -482,6 +482,33 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
     __syncwarp();
 }
 
+// A target's results from its compensated sums, and the chunk's interaction counts.
+template <bool kPhi>
+__device__ __forceinline__ void write_target(const WalkArgs& a, int t, float2 sxy, float2 cxy,
+                                             float2 szp, float2 czp, int np, int nm)
+{
+    if (t >= 0) {
+        const int s = a.sp[t];
+        const double qm = a.msp[2 + s];
+        a.ax[t] = qm * ((double)sxy.x + (double)cxy.x);
+        a.ay[t] = qm * ((double)sxy.y + (double)cxy.y);
+        a.az[t] = qm * ((double)szp.x + (double)czp.x);
+        if (kPhi && a.phi) a.phi[t] = (double)szp.y + (double)czp.y;
+        a.cnt_p2p[t] = np;
+        a.cnt_m2p[t] = nm;
+    }
+    unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
+        sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&a.stats[0], sp2);
+        atomicAdd(&a.stats[1], sm2);
+    }
+}
+
 // One warp walks a chunk of up to 32 key-consecutive targets of one cloud, one per
 // lane, in three parts that alternate:
 //
@@ -514,44 +541,16 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
 // 2.25 against 1.38.  Blocks of one warp keep the shared arrays at constant
 // addresses: 8 % faster than blocks of two to eight warps at the same occupancy.
 //
-// kThreads threads per block (one warp), register budget for kBlocks resident blocks
-// per SM.  kPhi = false (walks whose potential nobody reads, e.g. the electron
+// Register budget for kBlocks resident blocks (of one warp) per SM.  kPhi = false (walks whose potential nobody reads, e.g. the electron
 // substeps): the potential terms and their sums are left out; the field is computed
 // by the same operations in the same order, so accelerations are bit-identical.
-template <bool kPhi>
-__device__ __forceinline__ void write_target(const WalkArgs& a, int t, float2 sxy, float2 cxy,
-                                             float2 szp, float2 czp, int np, int nm)
-{
-    if (t >= 0) {
-        const int s = a.sp[t];
-        const double qm = a.msp[2 + s];
-        a.ax[t] = qm * ((double)sxy.x + (double)cxy.x);
-        a.ay[t] = qm * ((double)sxy.y + (double)cxy.y);
-        a.az[t] = qm * ((double)szp.x + (double)czp.x);
-        if (kPhi && a.phi) a.phi[t] = (double)szp.y + (double)czp.y;
-        a.cnt_p2p[t] = np;
-        a.cnt_m2p[t] = nm;
-    }
-    unsigned long long sp2 = (unsigned long long)np, sm2 = (unsigned long long)nm;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        sp2 += __shfl_xor_sync(0xffffffffu, sp2, o);
-        sm2 += __shfl_xor_sync(0xffffffffu, sm2, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&a.stats[0], sp2);
-        atomicAdd(&a.stats[1], sm2);
-    }
-}
-
-template <bool kKelbg, int kThreads, int kBlocks, bool kPhi>
-__global__ void __launch_bounds__(kThreads, kBlocks)
+template <bool kKelbg, int kBlocks, bool kPhi>
+__global__ void __launch_bounds__(32, kBlocks)
 k_walk_fp32c(WalkArgs a)
 {
     follow();
-    __shared__ WalkWarp shared[kThreads / 32];
-    const int lane = threadIdx.x & 31;
-    WalkWarp& W = shared[threadIdx.x >> 5];
+    __shared__ WalkWarp W;
+    const int lane = threadIdx.x;
     const int gave_up = *a.err;
 
     for (int item = next_chunk(a.work, lane); item < a.nchunks;
@@ -601,7 +600,7 @@ k_walk_fp32c(WalkArgs a)
 // totals in the order in which k_walk_fp32c adds them, a round of kWays slots behind, so
 // that the results are those of k_walk_fp32c bit for bit, whatever splits them.  N = 4099:
 // 187 -> 88 us (Kelbg law 321 -> 118); 16384: 242 -> 143 us; 50,000: 399 -> 383 us; one
-// warp per chunk again from 1520 chunks on (split_shape).
+// warp per chunk again from 1520 chunks on (walk_fp32c_few).
 constexpr int kSplitLeaves = 4;
 
 struct SplitSlot {
@@ -1012,7 +1011,7 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
         t.hdr[nd] = make_float4(-chx, -chy, -chz, (dl & 256) ? -rc2 : rc2);
         if (!kFp64) {
             t.lo[nd] = make_float4((float)((double)chx - ux), (float)((double)chy - uy),
-                                   (float)((double)chz - uz), __int_as_float(t.info[nd].z));
+                                   (float)((double)chz - uz), 0.f);
             const float4* m32 = reinterpret_cast<const float4*>(t.mom32 + (size_t)nd * 16);
             const float4 f1 = m32[1], f2 = m32[2], f3 = m32[3];   // {M, D}, {Q..}, {Q.., 0, 0}
             const float M = f1.x, qxx = f2.x, qyy = f2.w, qzz = f3.y;
@@ -1069,16 +1068,16 @@ template <bool kKelbg, bool kPhi>
 static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, Queue s)
 {
     switch (per_sm) {
-    case 12: launch(k_walk_fp32c<kKelbg, 32, 12, kPhi>, b, 32, s.whole(), a); break;
-    case 14: launch(k_walk_fp32c<kKelbg, 32, 14, kPhi>, b, 32, s.whole(), a); break;
-    case 16: launch(k_walk_fp32c<kKelbg, 32, 16, kPhi>, b, 32, s.whole(), a); break;
-    case 18: launch(k_walk_fp32c<kKelbg, 32, 18, kPhi>, b, 32, s.whole(), a); break;
-    case 20: launch(k_walk_fp32c<kKelbg, 32, 20, kPhi>, b, 32, s.whole(), a); break;
-    case 22: launch(k_walk_fp32c<kKelbg, 32, 22, kPhi>, b, 32, s.whole(), a); break;
-    case 26: launch(k_walk_fp32c<kKelbg, 32, 26, kPhi>, b, 32, s.whole(), a); break;
-    case 28: launch(k_walk_fp32c<kKelbg, 32, 28, kPhi>, b, 32, s.whole(), a); break;
-    case 32: launch(k_walk_fp32c<kKelbg, 32, 32, kPhi>, b, 32, s.whole(), a); break;
-    default: launch(k_walk_fp32c<kKelbg, 32, 24, kPhi>, b, 32, s.whole(), a); break;
+    case 12: launch(k_walk_fp32c<kKelbg, 12, kPhi>, b, 32, s.whole(), a); break;
+    case 14: launch(k_walk_fp32c<kKelbg, 14, kPhi>, b, 32, s.whole(), a); break;
+    case 16: launch(k_walk_fp32c<kKelbg, 16, kPhi>, b, 32, s.whole(), a); break;
+    case 18: launch(k_walk_fp32c<kKelbg, 18, kPhi>, b, 32, s.whole(), a); break;
+    case 20: launch(k_walk_fp32c<kKelbg, 20, kPhi>, b, 32, s.whole(), a); break;
+    case 22: launch(k_walk_fp32c<kKelbg, 22, kPhi>, b, 32, s.whole(), a); break;
+    case 26: launch(k_walk_fp32c<kKelbg, 26, kPhi>, b, 32, s.whole(), a); break;
+    case 28: launch(k_walk_fp32c<kKelbg, 28, kPhi>, b, 32, s.whole(), a); break;
+    case 32: launch(k_walk_fp32c<kKelbg, 32, kPhi>, b, 32, s.whole(), a); break;
+    default: launch(k_walk_fp32c<kKelbg, 24, kPhi>, b, 32, s.whole(), a); break;
     }
 }
 
