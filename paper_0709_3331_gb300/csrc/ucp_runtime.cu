@@ -496,34 +496,39 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     if (cudaGetDevice(&c->device) != cudaSuccess) return bail(UCP_ECUDA);
     cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device);
     const size_t n = (size_t)c->n;
+    const size_t cz = (size_t)cap;
+    c->t.cap = (int)cap;
+    // what starts cleared, side by side.  Box tables and slots that a build has not filled
+    // are read only after a wait that gave up: empty
+    dalloc(c, &c->t.info, cz);
+    dalloc(c, &c->t.depth_leaf, cz);
+    dalloc(c, &c->val[0], n);
+    dalloc(c, &c->val[1], n);
+    dalloc(c, &c->sort.status, sort_status_words(c->n));
+    dalloc(c, &c->topo_status, topo_status_words(c->n));
+    dalloc(c, &c->sort.err, 1);
+    dalloc(c, &c->ctl.epoch, 1);
+    dalloc(c, &c->stats, 2);
+    const size_t cleared = c->slab_bytes;
     for (int b = 0; b < 2; ++b) {
         for (int a = 0; a < 6; ++a) dalloc(c, &c->st[b][a], n);
         dalloc(c, &c->sp[b], n);
         dalloc(c, &c->id[b], n);
         dalloc(c, &c->key[b], n);
-        dalloc(c, &c->val[b], n);
     }
     dalloc(c, &c->ax, n);
     dalloc(c, &c->ay, n);
     dalloc(c, &c->az, n);
     dalloc(c, &c->phi, n);
     dalloc(c, &c->ctl.words, kCtlWords);
-    dalloc(c, &c->ctl.epoch, 1);
-    dalloc(c, &c->sort.status, sort_status_words(c->n));
-    dalloc(c, &c->sort.err, 1);
     dalloc(c, &c->sort.full_counts, sort_full_words());
     dalloc(c, &c->sort.test_ctl, 1 + kRadix);
     dalloc(c, &c->sort.test_epoch, 1);
     dalloc(c, &c->sort.test_keys, sort_test_words());
     dalloc(c, &c->sort.test_vals, sort_test_words());
-    dalloc(c, &c->topo_status, topo_status_words(c->n));
     dalloc(c, &c->pos_cnt, n);
     dalloc(c, &c->pos_off, n);
-    const size_t cz = (size_t)cap;
-    c->t.cap = (int)cap;
     dalloc(c, &c->t.nnodes, 1);
-    dalloc(c, &c->t.info, cz);
-    dalloc(c, &c->t.depth_leaf, cz);
     dalloc(c, &c->t.cell, cz);
     dalloc(c, &c->t.mom, cz * (c->precision == UCP_FP32C ? kCentre : kMom));
     dalloc(c, &c->t.delta, cz);
@@ -574,7 +579,6 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
     dalloc(c, &c->cnt_p2p, n);
     dalloc(c, &c->cnt_m2p, n);
     dalloc(c, &c->work, 1);
-    dalloc(c, &c->stats, 2);
     dalloc(c, &c->flags, 2 + (size_t)n_clouds);
     dalloc(c, &c->chunk_table, 2 * ((size_t)n_clouds + 1));
     dalloc(c, &c->stage, 6 * n);
@@ -594,23 +598,13 @@ int ucp_create_batch(ucp_ctx** out, const ucp_params* p, int32_t n_clouds, const
                 cl[j] = (unsigned char)i;
     }
     const double mqm[4] = {c->m[0], c->m[1], c->q[0] / c->m[0], c->q[1] / c->m[1]};
-    // box tables and slots a build has not filled are read only after a wait that gave up:
-    // empty
-    if (cudaMemsetAsync(c->t.info, 0, sizeof(int4) * cz, c->s) ||
+    if (cudaMemsetAsync(c->slab, 0, cleared, c->s) ||
         cudaMemsetAsync(c->t.child8, 0xff, 8 * sizeof(int) * cz, c->s) ||
-        cudaMemsetAsync(c->val[0], 0, sizeof(unsigned int) * n, c->s) ||
-        cudaMemsetAsync(c->val[1], 0, sizeof(unsigned int) * n, c->s) ||
-        cudaMemsetAsync(c->t.depth_leaf, 0, sizeof(int) * cz, c->s) ||
-        cudaMemsetAsync(c->sort.status, 0, 8 * sort_status_words(c->n), c->s) ||
-        cudaMemsetAsync(c->topo_status, 0, 8 * topo_status_words(c->n), c->s) ||
-        cudaMemsetAsync(c->sort.err, 0, sizeof(int), c->s) ||
-        cudaMemsetAsync(c->ctl.epoch, 0, sizeof(unsigned int), c->s) ||
         cudaMemcpyAsync(c->cloud_start, c->cloud_start_h.data(), sizeof(int) * (n_clouds + 1),
                         cudaMemcpyHostToDevice, c->s) ||
         (c->cloud && cudaMemcpyAsync(c->cloud, cl.data(), n, cudaMemcpyHostToDevice, c->s)) ||
         cudaMemcpyAsync(c->qsp, c->q, 2 * sizeof(double), cudaMemcpyHostToDevice, c->s) ||
         cudaMemcpyAsync(c->msp, mqm, sizeof(mqm), cudaMemcpyHostToDevice, c->s) ||
-        cudaMemsetAsync(c->stats, 0, 2 * sizeof(unsigned long long), c->s) ||
         cudaHostAlloc(&c->host_flags, sizeof(int) * (3 + 2 * UCP_MAX_CLOUDS + 2 * (UCP_MAX_CLOUDS + 1)),
                       0)) {
         c->err = "initial copies failed";
