@@ -799,6 +799,8 @@ static int run_block_graph(ucp_ctx* c, double dt_e, int kk, double theta, double
             return fail(c, UCP_ECUDA, "capture stream");
         const int cur0 = c->cur;
         const int64_t steps0 = c->steps, wt0 = c->walk_targets, wl0 = c->walk_launches;
+        const bool phi0 = c->phi_valid;
+        const double theta0 = c->phi_theta, eps0 = c->phi_eps;
         const Queue orig = c->s;
         c->s.s = c->cap_stream;
         const unsigned long long l0 = g_launches.load();
@@ -821,6 +823,11 @@ static int run_block_graph(ucp_ctx* c, double dt_e, int kk, double theta, double
         c->steps = steps0;
         c->walk_targets = wt0;
         c->walk_launches = wl0;
+        // nothing has run: the forces and potentials stay those of the state as it is
+        c->acc_valid = true;
+        c->phi_valid = phi0;
+        c->phi_theta = theta0;
+        c->phi_eps = eps0;
         if (rc || ec != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
             cudaGetLastError();
