@@ -170,7 +170,8 @@ int ucp_set_graphs(ucp_ctx* ctx, int enable);
  * state (one walk over every particle and nine over the electrons; best of three
  * after a warm-up) and keeps the fastest shape for this context (returned in
  * *best_shape, that block's walk time in ms in *best_ms; either may be NULL).
- * Results do not depend on the shape.  FP64 contexts keep their single shape. */
+ * Results do not depend on the shape.  FP64 contexts keep their single shape, and walks of
+ * up to 10 chunks of 32 targets per SM take a form of their own whatever the shape. */
 int ucp_autotune(ucp_ctx* ctx, double theta, double eps, int* best_shape, float* best_ms);
 
 /* Number of FP32C walk launch shapes, and a call that sets one directly

@@ -2,7 +2,7 @@
 // targets took and counts the chunks by that cost in logarithmic bins; afterwards the
 // order in which the next walk over the same targets (the next substep) takes its chunks
 // is rewritten longest-first, so that the persistent grid does not end on a few long
-// ones.  The order of chunks changes no result: every warp walks whole chunks.
+// ones.  A new state starts from list order: another cloud's order is up to 7 % worse.  The order of chunks changes no result: every warp walks whole chunks.
 //
 // Measured cycles order the chunks better than their interaction counts (a chunk also
 // pays for the boxes and leaves that only some of its targets take), and with the counts
