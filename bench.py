@@ -609,7 +609,7 @@ def run_extras(c, W, ws, pos_d, vel_d, sp_d, Context, UCP_FP32C, UCP_FP64, timed
         "lambda_ei": 0.05, "ms_per_step": mk / 2,
         "interactions_per_s": float(stk[0] + stk[1]) / (mk / 1e3),
         "walk_ms_per_launch": wmk / max(wnk, 1),
-        "note": "electron-ion direct pairs take the Kelbg form one source at a time"}
+        "note": "electron-ion direct pairs take the Kelbg form, two sources to a packed operation"}
     ck.close()
 
     # ensemble of 64 independent clouds (sizes log-uniform 4096..65536, sigma_c =
