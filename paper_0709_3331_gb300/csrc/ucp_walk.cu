@@ -380,9 +380,53 @@ __device__ __forceinline__ void box_batch(const WalkArgs& a, float* stage, const
     __syncwarp();
 }
 
+// One pair of sources {nx0, nx1, ny0, ny1}, {nz0, nz1, q0, q1} on a target at r from their
+// leaf's centroid, added to p (two sums side by side); ok: not the target itself.
+struct PairSums {
+    float2 x = splat(0.f), y = x, z = x, p = x;
+};
+
+template <bool kKelbg, bool kPhi>
+__device__ __forceinline__ void add_pair(const float4 F, const float4 Q, float2 rx, float2 ry, float2 rz,
+                                         const LaneTarget& g, bool ok0, bool ok1, PairSums& s)
+{
+    const float2 dx = __fadd2_rn(rx, make_float2(F.x, F.y));
+    const float2 dy = __fadd2_rn(ry, make_float2(F.z, F.w));
+    const float2 dz = __fadd2_rn(rz, make_float2(Q.x, Q.y));
+    const float2 q = make_float2(Q.z, Q.w);
+    if (kKelbg) {
+        // unlike charges (electron-ion) take the Kelbg form, unsoftened
+        const bool un0 = q.x != g.q, un1 = q.y != g.q;
+        const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+        const float2 r2 = __fadd2_rn(d2, make_float2(un0 ? 0.f : g.eps2,
+                                                     un1 ? 0.f : g.eps2));
+        float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                ok1 ? rsqrt_ftz(r2.y) : 0.f);
+        float2 fp = splat(1.f), fg = fp;
+        if (un0 && ok0) kelbg_factors(d2.x, ri.x, g.inv_lambda, fp.x, fg.x);
+        if (un1 && ok1) kelbg_factors(d2.y, ri.y, g.inv_lambda, fp.y, fg.y);
+        const float2 qi = __fmul2_rn(q, ri);
+        const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
+        s.x = __ffma2_rn(qr3, dx, s.x);
+        s.y = __ffma2_rn(qr3, dy, s.y);
+        s.z = __ffma2_rn(qr3, dz, s.z);
+        s.p = __ffma2_rn(qi, fp, s.p);
+    } else {
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, splat(g.eps2))));
+        const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
+                                      ok1 ? rsqrt_ftz(r2.y) : 0.f);
+        const float2 qi = __fmul2_rn(q, ri);
+        const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
+        s.x = __ffma2_rn(qr3, dx, s.x);
+        s.y = __ffma2_rn(qr3, dy, s.y);
+        s.z = __ffma2_rn(qr3, dz, s.z);
+        if (kPhi) s.p = __fadd2_rn(s.p, qi);
+    }
+}
+
 // Direct pairs, lanes over targets: cnt <= 32 opened leaves, each one's sources brought
-// into shared memory (up to 32 float4) while the leaf before it is summed; add(e, {x, y},
-// {z, potential}) takes leaf e's sums in the lanes of its mask.
+// into shared memory (32 float4 at a time) while the leaf or the part before is summed;
+// add(e, {x, y}, {z, potential}) takes leaf e's sums in the lanes of its mask.
 template <bool kKelbg, bool kPhi, class Add>
 __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2* leaves, int cnt,
                                            const LaneTarget& g_, int& np, Add add)
@@ -415,6 +459,41 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
         if (e + 1 < cnt) v = __ldg(S + __float_as_int(meta[2 * e + 2].w) + lane);
         __syncwarp();
         const int2 nm1 = leaves[e];
+        if (nm1.x > 32) {
+            // part by part, 16 pairs at a time through the buffer, by the whole warp
+            const float4 A = meta[2 * e], B = meta[2 * e + 1];
+            const float2 rx = splat((xh + A.x) + (xl + B.x));
+            const float2 ry = splat((yh + A.y) + (yl + B.y));
+            const float2 rz = splat((zh + A.z) + (zl + B.z));
+            const int begin = __float_as_int(B.w), num = nm1.x;
+            const int pairs = ((begin & 1) + num + 1) >> 1;
+            const bool mine = (nm1.y & me) != 0;
+            const bool self = (unsigned int)(t - begin) < (unsigned int)num;
+            const int tp = self ? t - (begin & ~1) : -1;
+            const float4* F = S + __float_as_int(A.w);
+            PairSums sum;
+#pragma unroll 1
+            for (int p0 = 0; p0 < pairs; p0 += 16) {
+                float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (p0 + 16 < pairs) u = __ldg(F + 2 * (p0 + 16) + lane);
+                if (mine) {
+                    const int last = min(16, pairs - p0);
+#pragma unroll 2
+                    for (int p = 0; p < last; ++p)
+                        add_pair<kKelbg, kPhi>(P[2 * p], P[2 * p + 1], rx, ry, rz, g_,
+                                               2 * (p0 + p) != tp, 2 * (p0 + p) + 1 != tp, sum);
+                }
+                __syncwarp();
+                P[lane] = u;
+                __syncwarp();
+            }
+            if (mine) {
+                np += num - (self ? 1 : 0);
+                add(e, make_float2(sum.x.x + sum.x.y, sum.y.x + sum.y.y),
+                    make_float2(sum.z.x + sum.z.y, kPhi ? sum.p.x + sum.p.y : 0.f));
+            }
+            continue;
+        }
         if (!(nm1.y & me)) continue;
         const float4 A = meta[2 * e], B = meta[2 * e + 1];
         const float2 rx = splat((xh + A.x) + (xl + B.x));
@@ -426,43 +505,12 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
         np += num - (self ? 1 : 0);
         // place of the target's own particle among the leaf's halves, or none
         const int tp = self ? t - (begin & ~1) : -1;
-        float2 px = splat(0.f), py = px, pz = px, pp = px;
+        PairSums sum;
         auto pair = [&](const float4 F, const float4 Q, bool ok0, bool ok1) {
-            const float2 dx = __fadd2_rn(rx, make_float2(F.x, F.y));
-            const float2 dy = __fadd2_rn(ry, make_float2(F.z, F.w));
-            const float2 dz = __fadd2_rn(rz, make_float2(Q.x, Q.y));
-            const float2 q = make_float2(Q.z, Q.w);
-            if (kKelbg) {
-                // unlike charges (electron-ion) take the Kelbg form, unsoftened
-                const bool un0 = q.x != qt, un1 = q.y != qt;
-                const float2 d2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
-                const float2 r2 = __fadd2_rn(d2, make_float2(un0 ? 0.f : eps2,
-                                                             un1 ? 0.f : eps2));
-                float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
-                                        ok1 ? rsqrt_ftz(r2.y) : 0.f);
-                float2 fp = splat(1.f), fg = fp;
-                if (un0 && ok0) kelbg_factors(d2.x, ri.x, inv_lambda, fp.x, fg.x);
-                if (un1 && ok1) kelbg_factors(d2.y, ri.y, inv_lambda, fp.y, fg.y);
-                const float2 qi = __fmul2_rn(q, ri);
-                const float2 qr3 = __fmul2_rn(__fmul2_rn(__fmul2_rn(qi, ri), ri), fg);
-                px = __ffma2_rn(qr3, dx, px);
-                py = __ffma2_rn(qr3, dy, py);
-                pz = __ffma2_rn(qr3, dz, pz);
-                pp = __ffma2_rn(qi, fp, pp);
-            } else {
-                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
-                const float2 ri = make_float2(ok0 ? rsqrt_ftz(r2.x) : 0.f,
-                                              ok1 ? rsqrt_ftz(r2.y) : 0.f);
-                const float2 qi = __fmul2_rn(q, ri);
-                const float2 qr3 = __fmul2_rn(__fmul2_rn(qi, ri), ri);
-                px = __ffma2_rn(qr3, dx, px);
-                py = __ffma2_rn(qr3, dy, py);
-                pz = __ffma2_rn(qr3, dz, pz);
-                if (kPhi) pp = __fadd2_rn(pp, qi);
-            }
+            add_pair<kKelbg, kPhi>(F, Q, rx, ry, rz, g_, ok0, ok1, sum);
         };
         if (pairs > 16) {
-            // longer than the buffer: straight from memory
+            // 32 sources from an odd place: one pair more than the buffer, straight from memory
             const float4* F = S + __float_as_int(A.w);
 #pragma unroll 1
             for (int p = 0; p < pairs; ++p)
@@ -476,8 +524,8 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
 #pragma unroll 2
             for (int p = 0; p < pairs; ++p) pair(P[2 * p], P[2 * p + 1], true, true);
         }
-        add(e, make_float2(px.x + px.y, py.x + py.y),
-            make_float2(pz.x + pz.y, kPhi ? pp.x + pp.y : 0.f));
+        add(e, make_float2(sum.x.x + sum.x.y, sum.y.x + sum.y.y),
+            make_float2(sum.z.x + sum.z.y, kPhi ? sum.p.x + sum.p.y : 0.f));
     }
     __syncwarp();
 }
