@@ -579,11 +579,60 @@ __device__ __forceinline__ double halve(bool bit, double a, double b, int mask)
     return (bit ? b : a) + __shfl_xor_sync(0xffffffffu, bit ? a : b, mask);
 }
 
+// Sums of child ch, in slot o of a twig, about the twig's geometric centre: shifted by the
+// difference of the centres, h = a quarter of the twig's side along each axis, signed by the
+// octant bit.  The child was written by another thread of the same launch: its record is
+// read through L2 (__ldcg) after the acquire of the bottom-up sweep.
+__device__ __forceinline__ void child_sums_f64(const Tree& t, int ch, int o, double h, double* a)
+{
+    const double2* r = reinterpret_cast<const double2*>(t.mom + (size_t)ch * kMom);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+        const double2 v = __ldcg(r + k);
+        a[2 * k] = v.x;
+        a[2 * k + 1] = v.y;
+    }
+    const double e[3] = {o & 1 ? h : -h, o & 2 ? h : -h, o & 4 ? h : -h};
+    const double me[3] = {a[1] * e[0], a[1] * e[1], a[1] * e[2]};
+    // P + d e^T + e d^T + M e e^T
+    a[8] += (2.0 * a[5] + me[0]) * e[0];
+    a[9] += a[5] * e[1] + (a[6] + me[1]) * e[0];
+    a[10] += a[5] * e[2] + (a[7] + me[2]) * e[0];
+    a[11] += (2.0 * a[6] + me[1]) * e[1];
+    a[12] += a[6] * e[2] + (a[7] + me[2]) * e[1];
+    a[13] += (2.0 * a[7] + me[2]) * e[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        a[2 + k] += a[0] * e[k];
+        a[5 + k] += me[k];
+    }
+}
+
+// Sums of a twig with one or two children by one lane (the same bits as by eight: the other
+// slots add zeros).  The first child follows the twig.
+__device__ __forceinline__ void narrow_sums_f64(const Cube* __restrict__ cube, const Tree& t,
+                                                const Twig& w)
+{
+    const double h = ldexp(cube_of(cube, t, w.first).L, -(w.depth + 2));
+    double a[14];
+#pragma unroll
+    for (int k = 0; k < 14; ++k) a[k] = 0.0;
+#pragma unroll 1
+    for (int c = 0; c < w.nch; ++c) {
+        const int ch = c ? w.last : w.id + 1;
+        double b[14];
+        child_sums_f64(t, ch, (int)(t.cell[ch] & 7ull), h, b);
+#pragma unroll
+        for (int k = 0; k < 14; ++k) a[k] += b[k];
+    }
+    double2* r = reinterpret_cast<double2*>(t.mom + (size_t)w.id * kMom);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) r[k] = make_double2(a[2 * k], a[2 * k + 1]);
+    t.delta[w.id] = kSumsDelta;
+}
+
 // Sums of a twig about its geometric centre by a group of eight lanes, one child slot o
-// each (ch < 0: empty): the child's sums shifted by the difference of the centres,
-// a quarter of the twig's side along each axis, signed by the octant bit.  The children
-// were written by other threads of the same launch: their records are read through L2
-// (__ldcg) after the acquire of the bottom-up sweep.  A level costs its latency and the
+// each (ch < 0: empty).  A level costs its latency and the
 // FP64 pipe's 16 cycles per warp instruction, so nothing but the sums goes up the tree
 // (moments follow from them with the walk's records, one box per lane), and they are
 // added by halving exchanges, 14 additions for 14 values instead of 42, which leave sums
@@ -596,30 +645,7 @@ __device__ __forceinline__ void twig_sums_f64(const Cube* __restrict__ cube, con
     double a[14];
 #pragma unroll
     for (int k = 0; k < 14; ++k) a[k] = 0.0;
-    if (ch >= 0) {
-        const double2* r = reinterpret_cast<const double2*>(t.mom + (size_t)ch * kMom);
-#pragma unroll
-        for (int k = 0; k < 7; ++k) {
-            const double2 v = __ldcg(r + k);
-            a[2 * k] = v.x;
-            a[2 * k + 1] = v.y;
-        }
-        const double h = ldexp(cube_of(cube, t, w.first).L, -(w.depth + 2));
-        const double e[3] = {o & 1 ? h : -h, o & 2 ? h : -h, o & 4 ? h : -h};
-        const double me[3] = {a[1] * e[0], a[1] * e[1], a[1] * e[2]};
-        // P + d e^T + e d^T + M e e^T
-        a[8] += (2.0 * a[5] + me[0]) * e[0];
-        a[9] += a[5] * e[1] + (a[6] + me[1]) * e[0];
-        a[10] += a[5] * e[2] + (a[7] + me[2]) * e[0];
-        a[11] += (2.0 * a[6] + me[1]) * e[1];
-        a[12] += a[6] * e[2] + (a[7] + me[2]) * e[1];
-        a[13] += (2.0 * a[7] + me[2]) * e[2];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            a[2 + k] += a[0] * e[k];
-            a[5 + k] += me[k];
-        }
-    }
+    if (ch >= 0) child_sums_f64(t, ch, o, ldexp(cube_of(cube, t, w.first).L, -(w.depth + 2)), a);
     // ((s0 + s4) + (s2 + s6)) + ((s1 + s5) + (s3 + s7)) of each value
     const bool b4 = o & 4, b2 = o & 2, b1 = o & 1;
     double u[8];
@@ -659,9 +685,14 @@ __device__ __forceinline__ int atomic_add_acq_rel(int* ctr, int v)
 // counts its finished children (t.arrive, cleared with the topology); the lane that
 // finishes the last child has the parent combined, four parents at a time by groups of
 // eight lanes, and carries on upwards.  No thread waits for another, and every twig is
-// combined once, from all its children, whichever warp does it.
-template <class Combine>
-__device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combine)
+// combined once, from all its children, whichever warp does it.  Where more than eight of a
+// warp's twigs have one or two children, each of those lanes combines its own, narrow(twig),
+// in the time of two rounds of the groups: close pairs in small leaves hang on chains of up to
+// 20 boxes with a single child, and particles on a line have two to a box.  A build with
+// leaves of 1 and all particles in pairs 1e-6 apart: 131,072 particles FP64 FIX1 and FP32C
+// FIX2 us by groups alone FIX3.
+template <bool kNarrow, class Combine, class Narrow>
+__device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combine, Narrow narrow)
 {
     const int lane = threadIdx.x & 31;
     // (a parent comes before its child: the sweep ends, also in tables that are no tree since
@@ -680,6 +711,13 @@ __device__ __forceinline__ void sweep_up(const Tree& t, int node, Combine combin
         const Twig up = load_twig(t, ready && w.parent < w.id ? w.parent : -1);
         int4 lc;
         if (ready) lc = __ldcg(&t.info[max(w.last, 0)]);
+        if (kNarrow) {
+            const unsigned int few = __ballot_sync(0xffffffffu, ready && w.nch <= 2);
+            if (__popc(few) > 8) {
+                if (ready && w.nch <= 2) narrow(w);
+                todo &= ~few;
+            }
+        }
         while (todo) {
             // the (lane / 8)-th of the lanes that are left
             unsigned int m = todo;
@@ -782,8 +820,10 @@ k_moments(const double* __restrict__ x, const double* __restrict__ y,
             for (int k = 0; k < 7; ++k) r[k] = make_double2(a[2 * k], a[2 * k + 1]);
             t.delta[node] = kSumsDelta;
         }
-        sweep_up(t, node,
-                 [&](const Twig& w, int o, int ch) { twig_sums_f64(cube, t, w, o, ch); });
+        // (a small system's blocks of 32 positions gain less by it than its test costs)
+        sweep_up<(kPos > 32)>(
+            t, node, [&](const Twig& w, int o, int ch) { twig_sums_f64(cube, t, w, o, ch); },
+            [&](const Twig& w) { narrow_sums_f64(cube, t, w); });
     }
 }
 
@@ -854,6 +894,17 @@ __device__ __forceinline__ void twig_child_f32(const Tree& t, int ch, int o, flo
     a[13] = qk[5] + (2.f * dk[2] + me2) * e[2];
 }
 
+// A twig's records from its sums.
+__device__ __forceinline__ void put_twig_f32(const Tree& t, const Twig& w, const float* a,
+                                             const double zp[3])
+{
+    float m32[16];
+    finish_box_f32(a, zp, m32, t.mom + (size_t)w.id * kCentre, t.delta + w.id);
+    float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)w.id * 16);
+    for (int k = 0; k < 4; ++k)
+        w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
+}
+
 // FP32 moments of a twig by a group of eight lanes, one child
 // slot each, summed by an xor butterfly over the slots.
 __device__ __forceinline__ void twig_combine_f32(const Cube* __restrict__ cube, const Tree& t,
@@ -865,13 +916,28 @@ __device__ __forceinline__ void twig_combine_f32(const Cube* __restrict__ cube, 
     twig_child_f32(t, ch, o, (float)(0.25 * ps), a);
 #pragma unroll
     for (int k = 0; k < 14; ++k) a[k] = sum8(a[k]);
-    if (w.id >= 0 && o == 0) {
-        float m32[16];
-        finish_box_f32(a, zp, m32, t.mom + (size_t)w.id * kCentre, t.delta + w.id);
-        float4* w32 = reinterpret_cast<float4*>(t.mom32 + (size_t)w.id * 16);
-        for (int k = 0; k < 4; ++k)
-            w32[k] = make_float4(m32[4 * k], m32[4 * k + 1], m32[4 * k + 2], m32[4 * k + 3]);
+    if (w.id >= 0 && o == 0) put_twig_f32(t, w, a, zp);
+}
+
+// The same for a twig with one or two children, by one lane (the same bits: the other slots
+// add zeros).  The first child follows the twig.
+__device__ __forceinline__ void narrow_combine_f32(const Cube* __restrict__ cube, const Tree& t,
+                                                   const Twig& w)
+{
+    double zp[3], ps;
+    box_centre(cube_of(cube, t, w.first), w.cell, w.depth, zp, &ps);
+    float a[14];
+#pragma unroll
+    for (int k = 0; k < 14; ++k) a[k] = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < w.nch; ++c) {
+        const int ch = c ? w.last : w.id + 1;
+        float b[14];
+        twig_child_f32(t, ch, (int)(t.cell[ch] & 7ull), (float)(0.25 * ps), b);
+#pragma unroll
+        for (int k = 0; k < 14; ++k) a[k] += b[k];
     }
+    put_twig_f32(t, w, a, zp);
 }
 
 // One particle's source record, and the empty halves of its leaf's pairs.
@@ -1039,8 +1105,9 @@ k_moments_f32(const double* __restrict__ x, const double* __restrict__ y,
                                (float)(cz - z[j]), sp[j] ? q1 : q0);
             }
         }
-        sweep_up(t, node,
-                 [&](const Twig& w, int o, int ch) { twig_combine_f32(cube, t, w, o, ch); });
+        sweep_up<true>(
+            t, node, [&](const Twig& w, int o, int ch) { twig_combine_f32(cube, t, w, o, ch); },
+            [&](const Twig& w) { narrow_combine_f32(cube, t, w); });
     }
 }
 
