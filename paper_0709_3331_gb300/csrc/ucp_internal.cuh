@@ -259,6 +259,7 @@ struct WalkArgs {
     const int* pos_off;     // first box started at each sorted position (the roots)
     const Cube* cubes;      // per cloud: FP32C coordinates are taken relative to the centre
     double eps2;
+    int leaf_cap;           // of the context
     int kelbg;              // electron-ion pairs use the Kelbg form (Sec. 2.1 Eq. 3)
     double lambda;          // its fixed lambda_ei
     double* ax; double* ay; double* az; double* phi;  // key order; phi may be NULL

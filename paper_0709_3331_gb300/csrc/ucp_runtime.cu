@@ -302,6 +302,7 @@ int force(ucp_ctx* c, double theta, double eps, int electrons_only, bool want_ph
     a.pos_off = c->pos_off;
     a.cubes = c->cube;
     a.eps2 = eps * eps;
+    a.leaf_cap = c->leaf_cap;
     a.kelbg = c->potential == UCP_POT_KELBG;
     a.lambda = c->lambda_ei;
     a.ax = c->ax;

@@ -424,10 +424,48 @@ __device__ __forceinline__ void add_pair(const float4 F, const float4 Q, float2 
     }
 }
 
+// A leaf of more than 32 sources, part by part: 16 pairs at a time from F through the buffer P
+// (which holds the first) by the whole warp; mine: this lane's target opens it.  Out of line,
+// so that the walks over shorter leaves do not pay for its registers (N = 524,288, leaves of
+// 32, no potential: 2.28 ms, in line 2.32).  Straight from memory, pair by pair, a walk over
+// 131,072 particles in leaves of 300 took 2.08 ms, now 1.26; over 524,288 with 52,428 of them
+// at one place 6.4, now 4.2.
+template <bool kKelbg, bool kPhi>
+static __device__ __noinline__ PairSums long_leaf(const float4* F, float4* P, int pairs, float3 r,
+                                                  float q, float eps2, float inv_lambda, int tp,
+                                                  bool mine)
+{
+    const int lane = threadIdx.x & 31;
+    LaneTarget g;
+    g.q = q;
+    g.eps2 = eps2;
+    g.inv_lambda = inv_lambda;
+    const float2 rx = splat(r.x), ry = splat(r.y), rz = splat(r.z);
+    PairSums sum;
+#pragma unroll 1
+    for (int p0 = 0; p0 < pairs; p0 += 16) {
+        float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p0 + 16 < pairs) u = __ldg(F + 2 * (p0 + 16) + lane);
+        if (mine) {
+            const int last = min(16, pairs - p0);
+#pragma unroll 2
+            for (int p = 0; p < last; ++p)
+                add_pair<kKelbg, kPhi>(P[2 * p], P[2 * p + 1], rx, ry, rz, g, 2 * (p0 + p) != tp,
+                                       2 * (p0 + p) + 1 != tp, sum);
+        }
+        __syncwarp();
+        P[lane] = u;
+        __syncwarp();
+    }
+    return sum;
+}
+
 // Direct pairs, lanes over targets: cnt <= 32 opened leaves, each one's sources brought
 // into shared memory (32 float4 at a time) while the leaf or the part before is summed;
-// add(e, {x, y}, {z, potential}) takes leaf e's sums in the lanes of its mask.
-template <bool kKelbg, bool kPhi, class Add>
+// add(e, {x, y}, {z, potential}) takes leaf e's sums in the lanes of its mask.  kParts: leaves
+// of more than 32 sources come in parts (long_leaf), else straight from memory (walks that
+// would pay for it with shorter leaves: the Kelbg law's 1.5 %, and see below).
+template <bool kKelbg, bool kPhi, bool kParts, class Add>
 __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2* leaves, int cnt,
                                            const LaneTarget& g_, int& np, Add add)
 {
@@ -459,34 +497,16 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
         if (e + 1 < cnt) v = __ldg(S + __float_as_int(meta[2 * e + 2].w) + lane);
         __syncwarp();
         const int2 nm1 = leaves[e];
-        if (nm1.x > 32) {
-            // part by part, 16 pairs at a time through the buffer, by the whole warp
+        if (kParts && nm1.x > 32) {
             const float4 A = meta[2 * e], B = meta[2 * e + 1];
-            const float2 rx = splat((xh + A.x) + (xl + B.x));
-            const float2 ry = splat((yh + A.y) + (yl + B.y));
-            const float2 rz = splat((zh + A.z) + (zl + B.z));
             const int begin = __float_as_int(B.w), num = nm1.x;
-            const int pairs = ((begin & 1) + num + 1) >> 1;
             const bool mine = (nm1.y & me) != 0;
             const bool self = (unsigned int)(t - begin) < (unsigned int)num;
-            const int tp = self ? t - (begin & ~1) : -1;
-            const float4* F = S + __float_as_int(A.w);
-            PairSums sum;
-#pragma unroll 1
-            for (int p0 = 0; p0 < pairs; p0 += 16) {
-                float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (p0 + 16 < pairs) u = __ldg(F + 2 * (p0 + 16) + lane);
-                if (mine) {
-                    const int last = min(16, pairs - p0);
-#pragma unroll 2
-                    for (int p = 0; p < last; ++p)
-                        add_pair<kKelbg, kPhi>(P[2 * p], P[2 * p + 1], rx, ry, rz, g_,
-                                               2 * (p0 + p) != tp, 2 * (p0 + p) + 1 != tp, sum);
-                }
-                __syncwarp();
-                P[lane] = u;
-                __syncwarp();
-            }
+            const PairSums sum = long_leaf<kKelbg, kPhi>(
+                S + __float_as_int(A.w), P, ((begin & 1) + num + 1) >> 1,
+                make_float3((xh + A.x) + (xl + B.x), (yh + A.y) + (yl + B.y),
+                            (zh + A.z) + (zl + B.z)),
+                qt, eps2, inv_lambda, self ? t - (begin & ~1) : -1, mine);
             if (mine) {
                 np += num - (self ? 1 : 0);
                 add(e, make_float2(sum.x.x + sum.x.y, sum.y.x + sum.y.y),
@@ -510,7 +530,8 @@ __device__ __forceinline__ void leaf_batch(const WalkArgs& a, float* stage, int2
             add_pair<kKelbg, kPhi>(F, Q, rx, ry, rz, g_, ok0, ok1, sum);
         };
         if (pairs > 16) {
-            // 32 sources from an odd place: one pair more than the buffer, straight from memory
+            // one pair more than the buffer (32 sources from an odd place), or a long leaf
+            // without parts: straight from memory
             const float4* F = S + __float_as_int(A.w);
 #pragma unroll 1
             for (int p = 0; p < pairs; ++p)
@@ -622,7 +643,7 @@ k_walk_fp32c(WalkArgs a)
         // a leaf's pairs are summed in FP32 and enter the total by a compensated add
         // (folding every fourth leaf only is 1.5 % faster and 1 % less exact)
         auto direct_pairs = [&](int2* leaves, int cnt) {
-            leaf_batch<kKelbg, kPhi>(a, W.stage, leaves, cnt, lt, np,
+            leaf_batch<kKelbg, kPhi, !kKelbg>(a, W.stage, leaves, cnt, lt, np,
                                      [&](int, const float2 fxy, const float2 fzp) {
                                          two_sum_acc2(sxy, cxy, fxy);
                                          two_sum_acc2(szp, czp, fzp);
@@ -664,7 +685,11 @@ struct SplitShared {
     int filled[2];                       // slots of a round; ~slots: the last round
 };
 
-template <bool kKelbg, bool kPhi, int kWays, int kBlocks>
+//
+// kParts (of contexts with leaf_cap > 32): long leaves in parts, 2.2 times as fast (30,000
+// particles in leaves of 300: 960 -> 430 us), which costs walks over shorter leaves 5 to 12 %
+// here (20,000 particles: 172 -> 192 us).
+template <bool kKelbg, bool kPhi, int kWays, int kBlocks, bool kParts>
 __global__ void __launch_bounds__((kWays + 1) * 32, kBlocks)
 k_walk_fp32c_split(WalkArgs a)
 {
@@ -706,7 +731,7 @@ k_walk_fp32c_split(WalkArgs a)
                     const int c = min(kSplitLeaves, cnt - e0);
                     if (lane < kSplitLeaves)
                         s.mask[lane] = lane < c ? (unsigned int)leaves[e0 + lane].y : 0u;
-                    leaf_batch<kKelbg, kPhi>(a, W.stage, leaves + e0, c, lt, np,
+                    leaf_batch<kKelbg, kPhi, kParts>(a, W.stage, leaves + e0, c, lt, np,
                                              [&](int e, const float2 fxy, const float2 fzp) {
                                                  s.v[e][lane] = make_float4(fxy.x, fxy.y, fzp.x, fzp.y);
                                              });
@@ -843,7 +868,7 @@ __device__ __forceinline__ void box_batch_in_order(const WalkArgs& a, float* sta
     __syncwarp();
 }
 
-template <bool kTwo>
+template <bool kTwo, bool kParts>
 __global__ void __launch_bounds__(kTwo ? 64 : 32, visit_blocks(kTwo))
 k_walk_fp32c_visits(WalkArgs a)
 {
@@ -884,7 +909,7 @@ k_walk_fp32c_visits(WalkArgs a)
                     const int m = min(32, upto - done);
                     if (lane < m) sh.leaf[lane] = sh.ring[(done + lane) & (kVisitRing - 1)];
                     __syncwarp();
-                    leaf_batch<false, false>(a, sh.stage, sh.leaf, m, lt, np,
+                    leaf_batch<false, false, kParts>(a, sh.stage, sh.leaf, m, lt, np,
                                              [&](int, const float2 fxy, const float2 fzp) {
                                                  two_sum_acc2(sxy, cxy, fxy);
                                                  two_sum_acc2(sz0, cz0, fzp);
@@ -1129,14 +1154,22 @@ static void walk_fp32c_shape(const WalkArgs& a, int per_sm, int b, Queue s)
     }
 }
 
+template <bool kKelbg, bool kPhi, int kWays, int kBlocks, bool kParts>
+static void walk_fp32c_split_form(const WalkArgs& a, Queue s)
+{
+    const int bytes = (int)sizeof(SplitShared<kWays>);
+    cudaFuncSetAttribute(k_walk_fp32c_split<kKelbg, kPhi, kWays, kBlocks, kParts>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    launch_shared(k_walk_fp32c_split<kKelbg, kPhi, kWays, kBlocks, kParts>, a.nchunks,
+                  (kWays + 1) * 32, bytes, s.whole(), a);
+}
+
 template <bool kKelbg, bool kPhi, int kWays, int kBlocks>
 static void walk_fp32c_split(const WalkArgs& a, Queue s)
 {
-    const int bytes = (int)sizeof(SplitShared<kWays>);
-    cudaFuncSetAttribute(k_walk_fp32c_split<kKelbg, kPhi, kWays, kBlocks>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    launch_shared(k_walk_fp32c_split<kKelbg, kPhi, kWays, kBlocks>, a.nchunks, (kWays + 1) * 32,
-                  bytes, s.whole(), a);
+    if (!kKelbg && a.leaf_cap > 32)
+        walk_fp32c_split_form<kKelbg, kPhi, kWays, kBlocks, !kKelbg>(a, s);
+    else walk_fp32c_split_form<kKelbg, kPhi, kWays, kBlocks, false>(a, s);
 }
 
 // Walks whose chunks are few enough for several warps each: a block per chunk, all of them
@@ -1174,15 +1207,21 @@ void launch_walk_fp32c(const WalkArgs& a, int nsm, Queue s, int shape)
     else walk_fp32c_shape<false, false>(a, per_sm, b, s);
 }
 
+template <bool kTwo>
+static void walk_fp32c_visits(const WalkArgs& a, int nsm, Queue s)
+{
+    const int b = walk_blocks(a.nchunks, nsm, visit_blocks(kTwo)), threads = kTwo ? 64 : 32;
+    // (long leaves in parts: gradients of 30,000 and 131,072 particles in leaves of 300 11.2 and
+    // 19.6 -> 7.9 and 16.0 ms; the form costs a gradient at 262,144 in leaves of 32 1.7 %)
+    if (a.leaf_cap > 32) launch(k_walk_fp32c_visits<kTwo, true>, b, threads, s.whole(), a);
+    else launch(k_walk_fp32c_visits<kTwo, false>, b, threads, s.whole(), a);
+}
+
 void launch_walk_fp32c_visits(const WalkArgs& a, int nsm, Queue s)
 {
     count_launch(1);
-    if (a.nchunks <= 4 * nsm)
-        launch(k_walk_fp32c_visits<true>, walk_blocks(a.nchunks, nsm, visit_blocks(true)), 64,
-               s.whole(), a);
-    else
-        launch(k_walk_fp32c_visits<false>, walk_blocks(a.nchunks, nsm, visit_blocks(false)), 32,
-               s.whole(), a);
+    if (a.nchunks <= 4 * nsm) walk_fp32c_visits<true>(a, nsm, s);
+    else walk_fp32c_visits<false>(a, nsm, s);
 }
 
 }  // namespace ucp
