@@ -36,12 +36,30 @@ __device__ __forceinline__ void box_centre(const Cube& cb, unsigned long long ce
     }
 }
 
-// FP64 moments of one box from sums about its geometric centre z:
-//   a = {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)},  y = x - z.
-// The expansion centre is the |q|-weighted centroid c = z + e, e = sum|q|y / S0
-// (z when S0 = 0); shifting to c: D = sum q y - M e,
-// Q = sum q y y^T - (sum q y) e^T - e (sum q y)^T + M e e^T.  delta = |e|.
-__device__ __forceinline__ void finish_box(const double* a, const double z[3],
+// The same with what rounding took from z: the exact centre is z + rho (to 2^-106 L; for
+// the cube's corner as it is stored).
+__device__ __forceinline__ void box_centre_exact(const Cube& cb, unsigned long long cell, int d,
+                                                 double z[3], double rho[3])
+{
+    const double s = ldexp(cb.L, -d);
+    const unsigned int ic[3] = {compact3(cell), compact3(cell >> 1), compact3(cell >> 2)};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double lo = __dsub_rn(cb.c[a], __dmul_rn(cb.L, 0.5));
+        const double k = __dadd_rn((double)ic[a], 0.5), t = __dmul_rn(k, s);
+        z[a] = __dadd_rn(lo, t);
+        const double b = __dsub_rn(z[a], lo);            // TwoSum
+        rho[a] = __dadd_rn(__dadd_rn(__dsub_rn(lo, __dsub_rn(z[a], b)), __dsub_rn(t, b)),
+                           __fma_rn(k, s, -t));
+    }
+}
+
+// FP64 moments of one box from sums about its exact geometric centre z + rho:
+//   a = {S0, M, sum|q|y (3), sum q y (3), sum q y y^T (6)},  y = x - z - rho.
+// The expansion centre is the |q|-weighted centroid c = z + rho + e, e = sum|q|y / S0
+// (0 when S0 = 0); shifting to c: D = sum q y - M e,
+// Q = sum q y y^T - (sum q y) e^T - e (sum q y)^T + M e e^T.  delta = |c - z|.
+__device__ __forceinline__ void finish_box(const double* a, const double z[3], const double rho[3],
                                            double* __restrict__ m, double* __restrict__ delta)
 {
     double S0 = a[0], M = a[1];
@@ -50,9 +68,7 @@ __device__ __forceinline__ void finish_box(const double* a, const double z[3],
     for (int k = 0; k < 3; ++k) e[k] = a[2 + k] * inv;
     double d[3];
     for (int k = 0; k < 3; ++k) d[k] = a[5 + k];
-    m[MC + 0] = z[0] + e[0];
-    m[MC + 1] = z[1] + e[1];
-    m[MC + 2] = z[2] + e[2];
+    for (int k = 0; k < 3; ++k) m[MC + k] = z[k] + (e[k] + rho[k]);
     m[MM] = M;
     for (int k = 0; k < 3; ++k) m[MD + k] = d[k] - M * e[k];
     const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};

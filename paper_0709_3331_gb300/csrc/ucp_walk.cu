@@ -1055,9 +1055,9 @@ k_mac_prepare(Tree t, const Cube* __restrict__ cube, double theta, int* work, in
             }
         }
         if (kFp64 && delta == kSumsDelta) {
-            double z[3], side, rec[kMom];
-            box_centre(cb, t.cell[nd], dl & 255, z, &side);
-            finish_box(a, z, rec, &delta);
+            double z[3], rho[3], rec[kMom];
+            box_centre_exact(cb, t.cell[nd], dl & 255, z, rho);
+            finish_box(a, z, rho, rec, &delta);
             t.delta[nd] = delta;
 #pragma unroll
             for (int k = 0; k < 3; ++k) c[k] = rec[MC + k];
