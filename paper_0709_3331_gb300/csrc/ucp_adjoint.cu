@@ -20,6 +20,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 namespace ucp {
 
 namespace {
@@ -282,6 +284,19 @@ k_walk_adjoint_f32(WalkArgs a, int group, const double* __restrict__ lam,
             __syncwarp();
         }
         const int groups = (ck.y + 3) >> 2;
+        // Targets relative to the middle of the group keep a box's distance to as many bits as
+        // the group is larger than that distance.  Where most neighbours in the group lie
+        // within an eighth of its extent (a group over the gap between two clusters), the boxes
+        // near them are taken from float pairs, as the direct pairs are.
+        bool wide;
+        {
+            const float ext = 2.f * fmaxf(tg.ex, fmaxf(tg.ey, tg.ez));
+            const float gap = fmaxf(fabsf(__shfl_down_sync(0xffffffffu, tg.xh, 1) - tg.xh),
+                                    fmaxf(fabsf(__shfl_down_sync(0xffffffffu, tg.yh, 1) - tg.yh),
+                                          fabsf(__shfl_down_sync(0xffffffffu, tg.zh, 1) - tg.zh)));
+            const bool near = lane + 1 < ck.y && gap < 0.125f * ext;
+            wide = 2 * __popc(__ballot_sync(0xffffffffu, near)) > ck.y - 1;
+        }
 
         // Accepted boxes, one per lane.  With g = (R.R + eps^2)^-1/2 and every l replaced
         // by w:  H = aR R + al w + aD D + k,  k = 1/2 T4(w),
@@ -308,67 +323,82 @@ k_walk_adjoint_f32(WalkArgs a, int group, const double* __restrict__ lam,
 #pragma unroll
             for (int k = 0; k < 6; ++k) ga[k] = splat(0.f);
             tr = splat(0.f);
+            auto targets = [&](auto from_pairs) {
 #pragma unroll 1
-            for (int g4 = 0; g4 < groups; ++g4) {
-                float v[16];
+                for (int g4 = 0; g4 < groups; ++g4) {
+                    float v[16];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float4* T = W.tgt[2 * g4 + h];
-                    const float4 f0 = T[0], f1 = T[1], f2 = T[2];
-                    const float2 R[3] = {add2(cx, make_float2(f0.x, f0.y)),
-                                         add2(cy, make_float2(f0.z, f0.w)),
-                                         add2(cz, make_float2(f1.x, f1.y))};
-                    const float2 w[3] = {make_float2(f1.z, f1.w), make_float2(f2.x, f2.y),
-                                         make_float2(f2.z, f2.w)};
-                    const float2 rr = fma2(R[0], R[0], fma2(R[1], R[1], fma2(R[2], R[2], e2)));
-                    const unsigned int in = mask >> (4 * g4 + 2 * h);
-                    const float2 g = make_float2((in & 1u) ? rsqrt_ftz(rr.x) : 0.f,
-                                                 (in & 2u) ? rsqrt_ftz(rr.y) : 0.f);
-                    const float2 u = mul2(g, g), g3 = mul2(g, u), g5 = mul2(g3, u),
-                                 g7 = mul2(g5, u), g9 = mul2(g7, u);
-                    const float2 rw = dot2(R, w), rd = dot2(R, nD), wd = dot2(w, nD);
-                    const float2 q[3] = {
-                        fma2(qxx, R[0], fma2(qxy, R[1], mul2(qxz, R[2]))),
-                        fma2(qxy, R[0], fma2(qyy, R[1], mul2(qyz, R[2]))),
-                        fma2(qxz, R[0], fma2(qyz, R[1], mul2(qzz, R[2])))};
-                    const float2 qw[3] = {
-                        fma2(qxx, w[0], fma2(qxy, w[1], mul2(qxz, w[2]))),
-                        fma2(qxy, w[0], fma2(qyy, w[1], mul2(qyz, w[2]))),
-                        fma2(qxz, w[0], fma2(qyz, w[1], mul2(qzz, w[2])))};
-                    const float2 rqr = dot2(R, q), wqr = dot2(w, q);
-                    const float2 p5 = mul2(g5, rw), p7 = mul2(g7, rw);
-                    // k = kr R + kq q + kw w + 6 g^5 (Q/2) w
-                    const float2 kw = fma2(g7, mul2(splat(-15.f), rqr), mul2(g5, t3));
-                    const float2 kr = fma2(mul2(splat(105.f), rqr), mul2(g9, rw),
-                                           fma2(g7, mul2(splat(-30.f), wqr), mul2(t15, p7)));
-                    const float2 kq = mul2(splat(-30.f), p7), k6 = mul2(splat(6.f), g5);
-                    const float2 aR = fma2(mul2(splat(-5.f), p7), rd, mul2(g5, fma2(M3, rw, wd)));
-                    const float2 aw = fma2(g5, rd, mul2(nM, g3));
-                    const float2 p53 = mul2(splat(3.f), p5), g53 = mul2(splat(3.f), g5),
-                                 ng3 = mul2(splat(-1.f), g3), p75 = mul2(splat(-7.5f), p7);
-                    float2 b[3];
+                    for (int h = 0; h < 2; ++h) {
+                        const float4* T = W.tgt[2 * g4 + h];
+                        const float4 f0 = T[0], f1 = T[1], f2 = T[2];
+                        float2 R[3];
+                        if (decltype(from_pairs)::value) {
+                            const float4 f3 = T[3], f4 = T[4], f5 = T[5];
+                            R[0] = add2(add2(splat(r0.x), make_float2(f3.x, f3.y)),
+                                        add2(splat(lo.x), make_float2(f4.z, f4.w)));
+                            R[1] = add2(add2(splat(r0.y), make_float2(f3.z, f3.w)),
+                                        add2(splat(lo.y), make_float2(f5.x, f5.y)));
+                            R[2] = add2(add2(splat(r0.z), make_float2(f4.x, f4.y)),
+                                        add2(splat(lo.z), make_float2(f5.z, f5.w)));
+                        } else {
+                            R[0] = add2(cx, make_float2(f0.x, f0.y));
+                            R[1] = add2(cy, make_float2(f0.z, f0.w));
+                            R[2] = add2(cz, make_float2(f1.x, f1.y));
+                        }
+                        const float2 w[3] = {make_float2(f1.z, f1.w), make_float2(f2.x, f2.y),
+                                             make_float2(f2.z, f2.w)};
+                        const float2 rr = fma2(R[0], R[0], fma2(R[1], R[1], fma2(R[2], R[2], e2)));
+                        const unsigned int in = mask >> (4 * g4 + 2 * h);
+                        const float2 g = make_float2((in & 1u) ? rsqrt_ftz(rr.x) : 0.f,
+                                                     (in & 2u) ? rsqrt_ftz(rr.y) : 0.f);
+                        const float2 u = mul2(g, g), g3 = mul2(g, u), g5 = mul2(g3, u),
+                                     g7 = mul2(g5, u), g9 = mul2(g7, u);
+                        const float2 rw = dot2(R, w), rd = dot2(R, nD), wd = dot2(w, nD);
+                        const float2 q[3] = {
+                            fma2(qxx, R[0], fma2(qxy, R[1], mul2(qxz, R[2]))),
+                            fma2(qxy, R[0], fma2(qyy, R[1], mul2(qyz, R[2]))),
+                            fma2(qxz, R[0], fma2(qyz, R[1], mul2(qzz, R[2])))};
+                        const float2 qw[3] = {
+                            fma2(qxx, w[0], fma2(qxy, w[1], mul2(qxz, w[2]))),
+                            fma2(qxy, w[0], fma2(qyy, w[1], mul2(qyz, w[2]))),
+                            fma2(qxz, w[0], fma2(qyz, w[1], mul2(qzz, w[2])))};
+                        const float2 rqr = dot2(R, q), wqr = dot2(w, q);
+                        const float2 p5 = mul2(g5, rw), p7 = mul2(g7, rw);
+                        // k = kr R + kq q + kw w + 6 g^5 (Q/2) w
+                        const float2 kw = fma2(g7, mul2(splat(-15.f), rqr), mul2(g5, t3));
+                        const float2 kr = fma2(mul2(splat(105.f), rqr), mul2(g9, rw),
+                                               fma2(g7, mul2(splat(-30.f), wqr), mul2(t15, p7)));
+                        const float2 kq = mul2(splat(-30.f), p7), k6 = mul2(splat(6.f), g5);
+                        const float2 aR = fma2(mul2(splat(-5.f), p7), rd, mul2(g5, fma2(M3, rw, wd)));
+                        const float2 aw = fma2(g5, rd, mul2(nM, g3));
+                        const float2 p53 = mul2(splat(3.f), p5), g53 = mul2(splat(3.f), g5),
+                                     ng3 = mul2(splat(-1.f), g3), p75 = mul2(splat(-7.5f), p7);
+                        float2 b[3];
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        const float2 kk = fma2(kr, R[k], fma2(kq, q[k], fma2(kw, w[k], mul2(k6, qw[k]))));
-                        const float2 hh = fma2(aR, R[k], fma2(aw, w[k], fma2(p5, nD[k], kk)));
-                        v[6 * h + k] = hh.x;
-                        v[6 * h + 3 + k] = hh.y;
-                        ka[k] = add2(ka[k], kk);
-                        al[k] = fma2(p53, R[k], fma2(ng3, w[k], al[k]));
-                        b[k] = fma2(g53, w[k], mul2(p75, R[k]));
+                        for (int k = 0; k < 3; ++k) {
+                            const float2 kk = fma2(kr, R[k], fma2(kq, q[k], fma2(kw, w[k], mul2(k6, qw[k]))));
+                            const float2 hh = fma2(aR, R[k], fma2(aw, w[k], fma2(p5, nD[k], kk)));
+                            v[6 * h + k] = hh.x;
+                            v[6 * h + 3 + k] = hh.y;
+                            ka[k] = add2(ka[k], kk);
+                            al[k] = fma2(p53, R[k], fma2(ng3, w[k], al[k]));
+                            b[k] = fma2(g53, w[k], mul2(p75, R[k]));
+                        }
+                        tr = add2(tr, p53);
+                        ga[0] = fma2(b[0], R[0], ga[0]);
+                        ga[1] = fma2(b[0], R[1], fma2(b[1], R[0], ga[1]));
+                        ga[2] = fma2(b[0], R[2], fma2(b[2], R[0], ga[2]));
+                        ga[3] = fma2(b[1], R[1], ga[3]);
+                        ga[4] = fma2(b[1], R[2], fma2(b[2], R[1], ga[4]));
+                        ga[5] = fma2(b[2], R[2], ga[5]);
                     }
-                    tr = add2(tr, p53);
-                    ga[0] = fma2(b[0], R[0], ga[0]);
-                    ga[1] = fma2(b[0], R[1], fma2(b[1], R[0], ga[1]));
-                    ga[2] = fma2(b[0], R[2], fma2(b[2], R[0], ga[2]));
-                    ga[3] = fma2(b[1], R[1], ga[3]);
-                    ga[4] = fma2(b[1], R[2], fma2(b[2], R[1], ga[4]));
-                    ga[5] = fma2(b[2], R[2], ga[5]);
+                    v[12] = v[13] = v[14] = v[15] = 0.f;
+                    const float tot = warp_sum16(v, lane);
+                    W.mt[g4][lane] -= tot;
                 }
-                v[12] = v[13] = v[14] = v[15] = 0.f;
-                const float tot = warp_sum16(v, lane);
-                W.mt[g4][lane] -= tot;
-            }
+            };
+            if (wide) targets(std::true_type{});
+            else targets(std::false_type{});
             if (mask) {
                 float* d = adj + (size_t)bm.x * 12;
                 const float T = tr.x + tr.y;
