@@ -48,9 +48,10 @@ __device__ __forceinline__ void box_centre_exact(const Cube& cb, unsigned long l
         const double lo = __dsub_rn(cb.c[a], __dmul_rn(cb.L, 0.5));
         const double k = __dadd_rn((double)ic[a], 0.5), t = __dmul_rn(k, s);
         z[a] = __dadd_rn(lo, t);
-        const double b = __dsub_rn(z[a], lo);            // TwoSum
-        rho[a] = __dadd_rn(__dadd_rn(__dsub_rn(lo, __dsub_rn(z[a], b)), __dsub_rn(t, b)),
-                           __fma_rn(k, s, -t));
+        // Dekker's fast two-sum: the larger first (by exponents, on the integer units)
+        const bool lo_first = (__double2hiint(lo) & 0x7fffffff) >= (__double2hiint(t) & 0x7fffffff);
+        const double p = lo_first ? lo : t, q = lo_first ? t : lo;
+        rho[a] = __dadd_rn(__dsub_rn(q, __dsub_rn(z[a], p)), __fma_rn(k, s, -t));
     }
 }
 
